@@ -101,7 +101,7 @@ struct simrank_ctx {
   struct Buf {
     void* p = nullptr;
     size_t bytes = 0;
-  } ob[28];
+  } ob[32];
   // column mode: per-tile nonzeros of the in-lists (host), the work-item table
   // of the chain steps and its partial-sum accumulators (device)
   std::vector<int64_t> col_tnnz;
@@ -1111,19 +1111,27 @@ simrank_status run_one_shot(simrank_ctx* h, const std::map<int32_t, std::vector<
   return SR_OK;
 }
 
+// Chunks of a row of len nonzeros (an empty row has one, empty), and chunk c
+// of the nc of row a.
+int row_chunks(int len) { return std::max(1, (len + kChunk - 1) / kChunk); }
+RowChunk row_chunk(const HostAdj& A, int a, int c, int nc) {
+  const int len = std::min(kChunk, A.len[a] - c * kChunk);
+  return {a, nc == 1 ? (len | CH_ONLY) : len, A.start[a] + (int64_t)c * kChunk};
+}
+
 // Row chunks (at most kChunk nonzeros each) of the adjacency rows [0, n_rows);
 // first (optional) gets the index of each row's first chunk (n_rows + 1).
 void build_chunks(const HostAdj& A, int n_rows, std::vector<RowChunk>& out,
                   std::vector<int64_t>* first = nullptr) {
   out.clear();
   int64_t total = 0;
-  for (int a = 0; a < n_rows; ++a) total += (A.len[a] + kChunk - 1) / kChunk;
+  for (int a = 0; a < n_rows; ++a) total += row_chunks(A.len[a]);
   out.reserve((size_t)total);
   if (first) first->assign((size_t)n_rows + 1, 0);
   for (int a = 0; a < n_rows; ++a) {
     if (first) (*first)[a] = (int64_t)out.size();
-    for (int off = 0; off < A.len[a]; off += kChunk)
-      out.push_back({a, std::min(kChunk, A.len[a] - off), A.start[a] + off});
+    const int nc = row_chunks(A.len[a]);
+    for (int c = 0; c < nc; ++c) out.push_back(row_chunk(A, a, c, nc));
   }
   if (first) (*first)[n_rows] = (int64_t)out.size();
 }
@@ -1134,9 +1142,8 @@ void build_chunks(const HostAdj& A, int n_rows, std::vector<RowChunk>& out,
 bool patch_row_chunks(simrank_ctx* h, const HostAdj& A, int a, std::vector<RowChunk>& v,
                       const std::vector<int64_t>& first, ChunkList& L) {
   const int64_t c0 = first[a], nc = first[a + 1] - c0;
-  if ((A.len[a] + kChunk - 1) / kChunk != nc) return false;
-  for (int64_t c = 0; c < nc; ++c)
-    v[c0 + c] = {a, std::min(kChunk, A.len[a] - (int)(c * kChunk)), A.start[a] + c * kChunk};
+  if (row_chunks(A.len[a]) != nc) return false;
+  for (int64_t c = 0; c < nc; ++c) v[c0 + c] = row_chunk(A, a, (int)c, (int)nc);
   if (nc > 0 && cudaMemcpyAsync(L.chunks + c0, v.data() + c0, nc * sizeof(RowChunk),
                                 cudaMemcpyHostToDevice, h->st) != cudaSuccess)
     return false;
@@ -1154,6 +1161,19 @@ simrank_status upload_chunks(simrank_ctx* h, const std::vector<RowChunk>& v, Chu
   L.count = (int64_t)v.size();
   if (!v.empty())
     CUDA_TRY(h, cudaMemcpyAsync(L.chunks, v.data(), v.size() * sizeof(RowChunk),
+                                cudaMemcpyHostToDevice, h->st));
+  std::vector<int32_t> multi;
+  for (size_t q = 0; q < v.size(); ++q)
+    if (!(v[q].len & CH_ONLY) && (q == 0 || v[q - 1].row != v[q].row)) multi.push_back(v[q].row);
+  if ((int64_t)multi.size() > L.multi_cap) {
+    if (L.multi) cudaFree(L.multi);
+    L.multi = nullptr;
+    L.multi_cap = std::max<int64_t>((int64_t)multi.size(), 2 * L.multi_cap);
+    CUDA_TRY(h, dev_alloc(&L.multi, (size_t)L.multi_cap));
+  }
+  L.multi_count = (int64_t)multi.size();
+  if (!multi.empty())
+    CUDA_TRY(h, cudaMemcpyAsync(L.multi, multi.data(), multi.size() * sizeof(int32_t),
                                 cudaMemcpyHostToDevice, h->st));
   return SR_OK;
 }
@@ -1186,7 +1206,7 @@ simrank_status run_column_update(simrank_ctx* h, const std::vector<int32_t>& src
   if ((s = ob_ensure(h, 11, blk * 3)) != SR_OK) return s;
   unsigned char* w = (unsigned char*)h->ob[11].p;
   launch_partial_sim_block(h->cur_fwd, h->cur_hor, h->dout.col, h->din.col, h->din.len, d_cols, 2,
-                           n_pad, K, h->cfg.C, 64, h->ob[10].p, w, w + blk, w + 2 * blk, h->st,
+                           2, n_pad, K, h->cfg.C, 64, h->ob[10].p, w, w + blk, w + 2 * blk, nullptr, h->st,
                            WeightView(), delta);
   launch_col_extract(w + 2 * blk, 64, 2, 0, n_pad, h->sI, h->st);
   launch_col_extract(w + 2 * blk, 64, 2, 1, n_pad, h->sJ, h->st);
@@ -1265,8 +1285,10 @@ simrank_status column_mode_columns(simrank_ctx* h, const int32_t* cols, int ncol
   CUDA_TRY(h, cudaMemGetInfo(&free_b, &total_b));
   const size_t per_col = (size_t)n_pad * eb * (K + 4);
   int Bmax = (int)std::min<size_t>(1024, std::max<size_t>(1, (size_t)(0.6 * free_b) / per_col));
+  if (Bmax > 4) Bmax &= ~3;
   simrank_status s;
   if ((s = ob_ensure(h, 10, per_col * Bmax)) != SR_OK) return s;
+  if ((s = ob_ensure(h, 28, 3 * (size_t)n_pad * eb)) != SR_OK) return s;
   if (ncols > h->cols_cap) {
     if (h->d_cols) cudaFree(h->d_cols);
     h->d_cols = nullptr;
@@ -1284,15 +1306,17 @@ simrank_status column_mode_columns(simrank_ctx* h, const int32_t* cols, int ncol
   }
   for (int c0 = 0; c0 < ncols; c0 += Bmax) {
     const int B = std::min(Bmax, ncols - c0);
+    const int ldb = B > 4 ? (B + 3) & ~3 : B;  // wide blocks: 16-byte rows
     const int32_t* bc = h->d_cols + c0;
     unsigned char* base = (unsigned char*)h->ob[10].p;
-    const size_t blkb = (size_t)n_pad * B * eb;
+    const size_t blkb = (size_t)n_pad * ldb * eb;
     void* xs = base;
     void* y0 = base + blkb * (K + 1);
     void* y1 = base + blkb * (K + 2);
     void* res = base + blkb * (K + 3);
     launch_partial_sim_block(h->g0_fwd, h->g0_hor, h->g0_out_col, h->g0_in_col, h->g0_in_len, bc,
-                             B, n_pad, K, h->cfg.C, prec, xs, y0, y1, res, h->st);
+                             B, ldb, n_pad, K, h->cfg.C, prec, xs, y0, y1, res, h->ob[28].p,
+                             h->st);
     if (prec == 32 && !h->hist.empty()) {
       // all stored updates in one FP32 product
       const int U = (int)h->hist.size();
@@ -1301,12 +1325,13 @@ simrank_status column_mode_columns(simrank_ctx* h, const int32_t* cols, int ncol
       if ((s = ob_ensure(h, 18, gbytes)) != SR_OK) return s;
       CUDA_TRY(h, cudaMemcpyAsync(h->ob[17].p, h->hist.data(), U * sizeof(void*),
                                   cudaMemcpyHostToDevice, h->st));
-      launch_col_corr((const float* const*)h->ob[17].p, U, h->K1, bc, B, n_pad,
+      launch_col_corr((const float* const*)h->ob[17].p, U, h->K1, bc, B, ldb, n_pad,
                       (float*)h->ob[18].p, (float*)res, h->st);
     } else {
-      for (void* P : h->hist) launch_col_apply(P, prec, h->K1, bc, B, n_pad, prec, res, h->st);
+      for (void* P : h->hist)
+        launch_col_apply(P, prec, h->K1, bc, B, ldb, n_pad, prec, res, h->st);
     }
-    launch_col_out(res, prec, B, h->n_cur,
+    launch_col_out(res, prec, B, ldb, h->n_cur,
                    (unsigned char*)dst + (size_t)c0 * h->n_cur * (out_fp64 ? 8 : 4), out_fp64, h->st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -1340,7 +1365,8 @@ void free_ctx(simrank_ctx* h) {
   if (h->pXi) cudaFree(h->pXi);
   if (h->pEta) cudaFree(h->pEta);
   void* colptrs[] = {h->g0_in_col, h->g0_out_col, h->g0_in_len, h->g0_fwd.chunks,
-                     h->g0_hor.chunks, h->cur_fwd.chunks, h->cur_hor.chunks};
+                     h->g0_hor.chunks, h->cur_fwd.chunks, h->cur_hor.chunks,
+                     h->g0_fwd.multi, h->g0_hor.multi, h->cur_fwd.multi, h->cur_hor.multi};
   for (void* p : colptrs)
     if (p) cudaFree(p);
   // the panel snapshots come from the stream-ordered allocator
@@ -2084,12 +2110,14 @@ simrank_status simrank_grad(simrank_t h, const int32_t* pa, const int32_t* pb, c
   size_t free_b = 0, total_b = 0;
   CUDA_TRY(h, cudaMemGetInfo(&free_b, &total_b));
   const size_t per_col = (size_t)n_pad * 8 * (2 * (K + 1) + 2);
-  const int Eb = (int)std::max<size_t>(1, std::min<size_t>(1024, (size_t)(0.5 * free_b) / per_col));
+  const int Eb =
+      (int)std::max<size_t>(4, std::min<size_t>(1024, (size_t)(0.5 * free_b) / per_col)) & ~3;
   const size_t blkb = (size_t)n_pad * Eb * 8;
   if ((s = ob_ensure(h, 14, blkb * (K + 1))) != SR_OK) return s;
   if ((s = ob_ensure(h, 15, blkb * (K + 1))) != SR_OK) return s;
   if ((s = ob_ensure(h, 16, blkb)) != SR_OK) return s;
   if ((s = ob_ensure(h, 17, blkb)) != SR_OK) return s;
+  if ((s = ob_ensure(h, 28, 3 * (size_t)n_pad * 8)) != SR_OK) return s;
   const int64_t pool = h->din.pool_cap;
   if ((s = ob_ensure(h, 18, (size_t)pool * 8 * 2)) != SR_OK) return s;
   double* F = (double*)h->ob[14].p;
@@ -2120,6 +2148,7 @@ simrank_status simrank_grad(simrank_t h, const int32_t* pa, const int32_t* pb, c
   std::vector<double> sval(npairs, 0.0);
   for (size_t c0 = 0; c0 < bcols.size(); c0 += Eb) {
     const int B = (int)std::min<size_t>(Eb, bcols.size() - c0);
+    const int ldb = (B + 3) & ~3;
     std::vector<int32_t> cols(bcols.begin() + c0, bcols.begin() + c0 + B);
     std::vector<int32_t> rows, cidx;
     std::vector<int64_t> who;
@@ -2136,9 +2165,9 @@ simrank_status simrank_grad(simrank_t h, const int32_t* pa, const int32_t* pb, c
     if ((s = upload_i32(21, cidx)) != SR_OK) return s;
     if ((s = ob_ensure(h, 22, std::max<size_t>(rows.size(), 1) * 8)) != SR_OK) return s;
     launch_partial_sim_block(h->cur_fwd, h->cur_hor, h->dout.col, h->din.col, h->din.len,
-                             (const int32_t*)h->ob[19].p, B, n_pad, K, C, 64, F, y0, y1, Fp, h->st,
-                             wv);
-    launch_adj_pairs(Fp, B, (const int32_t*)h->ob[20].p, (const int32_t*)h->ob[21].p,
+                             (const int32_t*)h->ob[19].p, B, ldb, n_pad, K, C, 64, F, y0, y1, Fp,
+                             h->ob[28].p, h->st, wv);
+    launch_adj_pairs(Fp, ldb, (const int32_t*)h->ob[20].p, (const int32_t*)h->ob[21].p,
                      (int64_t)rows.size(), (double*)h->ob[22].p, h->st);
     std::vector<double> got(rows.size());
     if (!rows.empty())
@@ -2169,8 +2198,11 @@ simrank_status simrank_grad(simrank_t h, const int32_t* pa, const int32_t* pb, c
     psi[ib].push_back({A[p], g[p]});
   }
   CUDA_TRY(h, cudaMemsetAsync(G, 0, (size_t)pool * 8, h->st));
+  double* inv = (double*)h->ob[28].p;
+  launch_col_scales64(wv, h->din.len, n_pad, inv, h->st);
   for (size_t c0 = 0; c0 < ends.size(); c0 += Eb) {
     const int B = (int)std::min<size_t>(Eb, ends.size() - c0);
+    const int ldb = (B + 3) & ~3;
     std::vector<int32_t> un, uc, pn, pc;
     std::vector<double> ucoef, pcoef;
     for (int c = 0; c < B; ++c) {
@@ -2193,26 +2225,26 @@ simrank_status simrank_grad(simrank_t h, const int32_t* pa, const int32_t* pb, c
     if (!keep->empty())
       CUDA_TRY(h, cudaMemcpyAsync(h->ob[13].p, keep->data(), keep->size() * 8,
                                   cudaMemcpyHostToDevice, h->st));
-    const int64_t blk = (int64_t)n_pad * B;
+    const int64_t blk = (int64_t)n_pad * ldb;
     CUDA_TRY(h, cudaMemsetAsync(F, 0, (size_t)blk * 8, h->st));
     CUDA_TRY(h, cudaMemsetAsync(Fp, 0, (size_t)blk * 8, h->st));
     launch_adj_scatter((const int32_t*)h->ob[19].p, (const int32_t*)h->ob[20].p,
-                       (const double*)h->ob[22].p, B, B, F, h->st);
+                       (const double*)h->ob[22].p, B, ldb, F, h->st);
     launch_adj_scatter((const int32_t*)h->ob[21].p, (const int32_t*)h->ob[23].p,
-                       (const double*)h->ob[13].p, (int64_t)pn.size(), B, Fp, h->st);
+                       (const double*)h->ob[13].p, (int64_t)pn.size(), ldb, Fp, h->st);
     for (int l = 1; l <= K; ++l) {
-      launch_col_forward64(h->cur_fwd, h->dout.col, wv, h->din.len, F + (l - 1) * blk, F + l * blk,
-                           B, n_pad, h->st);
-      launch_col_forward64(h->cur_fwd, h->dout.col, wv, h->din.len, Fp + (l - 1) * blk,
-                           Fp + l * blk, B, n_pad, h->st);
+      launch_col_forward64(h->cur_fwd, h->dout.col, wv, inv, F + (l - 1) * blk, F + l * blk, ldb,
+                           h->st);
+      launch_col_forward64(h->cur_fwd, h->dout.col, wv, inv, Fp + (l - 1) * blk, Fp + l * blk, ldb,
+                           h->st);
     }
     CUDA_TRY(h, cudaMemsetAsync(y0, 0, (size_t)blk * 8, h->st));
     double* y = y0;
     double* yn = y1;
     for (int l = K - 1; l >= 0; --l) {
-      launch_col_horner64(h->cur_hor, h->din.col, wv, h->din.len, Fp + (l + 1) * blk,
-                          std::pow(C, l + 1), y, yn, B, n_pad, 1.0, h->st);
-      launch_adj_sddmm(h->cur_hor, h->din.col, F + l * blk, yn, B, 1.0 - C, G, h->st);
+      launch_col_horner64(h->cur_hor, h->din.col, wv, inv, Fp + (l + 1) * blk, std::pow(C, l + 1),
+                          y, yn, ldb, h->st);
+      launch_adj_sddmm(h->cur_hor, h->din.col, F + l * blk, yn, ldb, 1.0 - C, G, h->st);
       std::swap(y, yn);
     }
     LAUNCH_CHECK(h);

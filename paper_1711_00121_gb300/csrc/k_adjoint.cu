@@ -19,7 +19,7 @@ __global__ void k_adj_sddmm(const RowChunk* __restrict__ chunks, const int32_t* 
   const RowChunk ch = chunks[blockIdx.x];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double* fu = F + (int64_t)ch.row * B;
-  for (int e = warp; e < ch.len; e += (int)(blockDim.x >> 5)) {
+  for (int e = warp; e < chunk_len(ch); e += (int)(blockDim.x >> 5)) {
     const int v = col[ch.start + e];
     const double* yv = Y + (int64_t)v * B;
     double acc = 0.0;

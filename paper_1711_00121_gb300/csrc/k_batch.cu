@@ -370,7 +370,9 @@ __global__ void __launch_bounds__(256) k_spmm_chunks64(const RowChunk* __restric
   const int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LPC;
   const int c0 = 4 * ((int)blockIdx.y * LPC + (int)(threadIdx.x % LPC));
   if (q >= count || c0 >= ncols) return;
-  const RowChunk ch = chunks[q];
+  RowChunk ch = chunks[q];
+  ch.len = chunk_len(ch);
+  if (ch.len == 0) return;
   double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
   int e = 0;
   for (; e + 2 <= ch.len; e += 2) {

@@ -21,20 +21,20 @@ namespace {
 
 // X0[x_c][c] = 1 (the other entries are zero beforehand)
 template <typename T>
-__global__ void k_col_unit(const int32_t* __restrict__ cols, int B, T* __restrict__ X0) {
+__global__ void k_col_unit(const int32_t* __restrict__ cols, int B, int ldb, T* __restrict__ X0) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < B) X0[(int64_t)cols[c] * B + c] = (T)1;
+  if (c < B) X0[(int64_t)cols[c] * ldb + c] = (T)1;
 }
 
 // Column 0 of X0 = the indicator of the distinct ids cols[0 .. g0), column c
 // (1 <= c < B) = e_{cols[g0 + c - 1]}: Procedure 1 is linear in its start
 // vector, so column 0 of its result is the sum of the g0 columns.
 template <typename T>
-__global__ void k_col_unit_grouped(const int32_t* __restrict__ cols, int g0, int B,
+__global__ void k_col_unit_grouped(const int32_t* __restrict__ cols, int g0, int B, int ldb,
                                    T* __restrict__ X0) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < g0) X0[(int64_t)cols[q] * B] = (T)1;
-  else if (q < g0 + B - 1) X0[(int64_t)cols[q] * B + (q - g0 + 1)] = (T)1;
+  if (q < g0) X0[(int64_t)cols[q] * ldb] = (T)1;
+  else if (q < g0 + B - 1) X0[(int64_t)cols[q] * ldb + (q - g0 + 1)] = (T)1;
 }
 
 // Y[a][c] = s * X[a][c] (X may be null: Y = 0), a < n_rows, c < B
@@ -46,63 +46,173 @@ __global__ void k_col_fill(const T* __restrict__ X, double s, T* __restrict__ Y,
     Y[e] = X ? sv * X[e] : (T)0;
 }
 
-// One row chunk (at most CHUNK nonzeros of one adjacency row) per CTA and
-// 128 columns per thread block column:
-//   Y[row][c] += row_scale * sum_{e in chunk} w_e X[col_e][c]
-// forward (Q^T, out-lists): w_e = 1 / d_{col_e}, row_scale = 1
-// Horner  (Q,   in-lists):  w_e = 1,            row_scale = scale / d_row
-// Long rows are split over many chunks, whose partial sums meet in atomics.
-template <typename T, bool FORWARD>
-__global__ void k_col_chunk(const RowChunk* __restrict__ chunks, const int32_t* __restrict__ col,
-                            const float* __restrict__ ew, const int32_t* __restrict__ in_len,
-                            const double* __restrict__ wsum, const T* __restrict__ X,
-                            T* __restrict__ Y, int B, double scale) {
-  // weighted Q (wsum != null): Q[a][b] = w(b -> a) / wsum[a]; ew = weight of each
-  // adjacency entry (by pool position), null = 1
-  const RowChunk ch = chunks[blockIdx.x];
-  const int c = blockIdx.y * blockDim.x + threadIdx.x;
-  if (c >= B) return;
-  T acc = T(0);
-#pragma unroll 8
-  for (int e = 0; e < ch.len; ++e) {
-    const int a = col[ch.start + e];
-    T x = X[(int64_t)a * B + c];
-    if (ew) x *= (T)ew[ch.start + e];
-    if (FORWARD) x /= wsum ? (T)wsum[a] : (T)in_len[a];
-    acc += x;
+// Four (FP32) or two (FP64) adjacent columns as one 16-byte access, or half
+// of that (VEC columns of type T).
+template <typename T, int VEC>
+struct ColVec {
+  T v[VEC];
+};
+template <typename T, int VEC>
+__device__ __forceinline__ ColVec<T, VEC> ld_cols(const T* p) {
+  ColVec<T, VEC> r;
+  if constexpr (sizeof(T) * VEC == 16) {
+    const uint4 x = *reinterpret_cast<const uint4*>(p);
+    memcpy(&r, &x, 16);
+  } else {
+    const uint2 x = *reinterpret_cast<const uint2*>(p);
+    memcpy(&r, &x, 8);
   }
-  const T rs = FORWARD ? T(1) : (T)scale / (wsum ? (T)wsum[ch.row] : (T)in_len[ch.row]);
-  atomicAdd(&Y[(int64_t)ch.row * B + c], rs * acc);
+  return r;
+}
+template <typename T, int VEC>
+__device__ __forceinline__ void st_cols(T* p, const ColVec<T, VEC>& r) {
+  if constexpr (sizeof(T) * VEC == 16) {
+    uint4 x;
+    memcpy(&x, &r, 16);
+    *reinterpret_cast<uint4*>(p) = x;
+  } else {
+    uint2 x;
+    memcpy(&x, &r, 8);
+    *reinterpret_cast<uint2*>(p) = x;
+  }
+}
+template <typename T, int VEC>
+__device__ __forceinline__ void add_cols(T* p, const ColVec<T, VEC>& r) {
+  if constexpr (sizeof(T) == 4 && VEC == 4) {
+    atomicAdd(reinterpret_cast<float4*>(p), make_float4(r.v[0], r.v[1], r.v[2], r.v[3]));
+  } else if constexpr (sizeof(T) == 4 && VEC == 2) {
+    atomicAdd(reinterpret_cast<float2*>(p), make_float2(r.v[0], r.v[1]));
+  } else {
+#pragma unroll
+    for (int c = 0; c < VEC; ++c) atomicAdd(p + c, r.v[c]);
+  }
 }
 
-// The same for FP32 blocks with B a multiple of 4: each thread takes four
-// adjacent columns (one 16-byte gather per nonzero, one weight per nonzero
-// for the four) and adds its partial sums with one vector atomic.
-template <bool FORWARD>
-__global__ void k_col_chunk4(const RowChunk* __restrict__ chunks, const int32_t* __restrict__ col,
-                             const float* __restrict__ ew, const int32_t* __restrict__ in_len,
-                             const double* __restrict__ wsum, const float* __restrict__ X,
-                             float* __restrict__ Y, int B4, double scale) {
-  const RowChunk ch = chunks[blockIdx.x];
-  const int c4 = blockIdx.y * blockDim.x + threadIdx.x;
-  if (c4 >= B4) return;
-  const float4* __restrict__ X4 = reinterpret_cast<const float4*>(X);
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
-  for (int e = 0; e < ch.len; ++e) {
-    const int a = col[ch.start + e];
-    float w = ew ? ew[ch.start + e] : 1.f;
-    if (FORWARD) w /= wsum ? (float)wsum[a] : (float)in_len[a];
-    const float4 x = X4[(int64_t)a * B4 + c4];
-    acc.x += w * x.x;
-    acc.y += w * x.y;
-    acc.z += w * x.z;
-    acc.w += w * x.w;
+// One SpMM step on a block of ldb columns (ldb a multiple of 4), one warp per
+// row chunk (at most kChunk = 32 nonzeros of one adjacency row) and 32 * VEC
+// columns (blockIdx.y):
+//   forward (Q^T, out-lists): Y[row][c]  = sum_e w_e nodes[col_e] X[col_e][c]
+//   Horner  (Q,   in-lists):  Y[row][c]  = add_scale Xadd[row][c]
+//                                          + nodes[row] sum_e w_e X[col_e][c]
+// nodes holds 1 / d (or 1 / in-weight) per node, times the step's scale for
+// Horner; w_e = 1 without weights.  A row of one chunk (most rows; an empty
+// row has one empty chunk) is written once; the chunks of a longer row add
+// theirs to the row that k_col_prefill has set.
+//
+// Bound by the gathered bytes (FP32) or by GB300's FP64 rate of one FMA per
+// gathered value (FP64).  A warp takes `per` consecutive chunks; a chunk's
+// column ids and factors are loaded once, one per lane, two chunks ahead of
+// their use, and broadcast by shuffles, so that the loop holds a gather and an
+// FMA per value and no division, index load or degree load.
+template <typename T, int VEC, bool FORWARD>
+__global__ void __launch_bounds__(256, 6) k_col_rows(
+    const RowChunk* __restrict__ chunks, int64_t count, int per, const int32_t* __restrict__ col,
+    const float* __restrict__ ew, const T* __restrict__ nodes, const T* __restrict__ X,
+    const T* __restrict__ Xadd, T add_scale, T* __restrict__ Y, int ldb) {
+  constexpr unsigned full = 0xffffffffu;
+  constexpr int NB = 4;  // gathers in flight per lane
+  const int lane = threadIdx.x & 31;
+  const int64_t q0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * per;
+  if (q0 >= count) return;  // the whole warp
+  const int nq = (int)min((int64_t)per, count - q0);  // <= 32
+  const int c = ((int)blockIdx.y * 32 + lane) * VEC;
+  const bool act = c < ldb;
+  // lane i holds chunk q0 + i
+  RowChunk mine;
+  mine.row = mine.len = 0;
+  mine.start = 0;
+  if (lane < nq) mine = chunks[q0 + lane];
+  // column id of nonzero `lane` of chunk i, and its factor
+  auto col_of = [&](int i) -> int {
+    const int len = __shfl_sync(full, mine.len, i) & 0xffff;
+    const int64_t st = __shfl_sync(full, mine.start, i);
+    return (i < nq && lane < len) ? col[st + lane] : 0;
+  };
+  auto factor_of = [&](int i, int a) -> T {
+    const int len = __shfl_sync(full, mine.len, i) & 0xffff;
+    const int64_t st = __shfl_sync(full, mine.start, i);
+    T w = T(0);
+    if (i < nq && lane < len) {
+      w = FORWARD ? nodes[a] : T(1);
+      if (ew) w *= (T)ew[st + lane];
+    }
+    return w;
+  };
+  int a = col_of(0);
+  T w = factor_of(0, a);
+  int a1 = col_of(1);
+  for (int i = 0; i < nq; ++i) {
+    const T w1 = factor_of((i + 1) & 31, a1);
+    const int a2 = col_of((i + 2) & 31);
+    const int row = __shfl_sync(full, mine.row, i);
+    const int lf = __shfl_sync(full, mine.len, i);
+    const int len = lf & 0xffff;
+    const bool only = (lf & CH_ONLY) != 0;
+    const int64_t o = (int64_t)row * ldb + c;
+    ColVec<T, VEC> acc;
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) acc.v[u] = T(0);
+    for (int e = 0; e < len; e += NB) {
+      ColVec<T, VEC> x[NB];
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        const int64_t b = __shfl_sync(full, a, e + u);
+        if (act && e + u < len) {
+          x[u] = ld_cols<T, VEC>(X + b * ldb + c);
+        } else {
+#pragma unroll
+          for (int z = 0; z < VEC; ++z) x[u].v[z] = T(0);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        if (e + u >= len) break;
+        const T we = __shfl_sync(full, w, e + u);
+#pragma unroll
+        for (int z = 0; z < VEC; ++z) acc.v[z] += we * x[u].v[z];
+      }
+    }
+    if (!FORWARD && len > 0) {
+      const T rs = nodes[row];
+#pragma unroll
+      for (int z = 0; z < VEC; ++z) acc.v[z] *= rs;
+    }
+    if (act) {
+      if (only) {
+        if (!FORWARD) {
+          const ColVec<T, VEC> base = ld_cols<T, VEC>(Xadd + o);
+#pragma unroll
+          for (int z = 0; z < VEC; ++z) acc.v[z] += add_scale * base.v[z];
+        }
+        st_cols<T, VEC>(Y + o, acc);
+      } else {
+        add_cols<T, VEC>(Y + o, acc);
+      }
+    }
+    a = a1;
+    w = w1;
+    a1 = a2;
   }
-  const float rs =
-      FORWARD ? 1.f : (float)scale / (wsum ? (float)wsum[ch.row] : (float)in_len[ch.row]);
-  atomicAdd(reinterpret_cast<float4*>(Y) + (int64_t)ch.row * B4 + c4,
-            make_float4(rs * acc.x, rs * acc.y, rs * acc.z, rs * acc.w));
+}
+
+// The rows of more than one chunk before k_col_rows adds to them:
+// Y[row][c] = add_scale * Xadd[row][c] (0 without Xadd), one CTA per row.
+template <typename T>
+__global__ void k_col_prefill(const int32_t* __restrict__ rows, const T* __restrict__ Xadd,
+                              T add_scale, T* __restrict__ Y, int ldb) {
+  const int64_t o = (int64_t)rows[blockIdx.x] * ldb;
+  for (int c = threadIdx.x; c < ldb; c += blockDim.x)
+    Y[o + c] = Xadd ? add_scale * Xadd[o + c] : T(0);
+}
+
+// out[a] = scale / (in-degree or in-weight of a), 0 without in-neighbours
+template <typename T>
+__global__ void k_col_scales(const int32_t* __restrict__ in_len, const double* __restrict__ wsum,
+                             double scale, int n_rows, T* __restrict__ out) {
+  const int a = blockIdx.x * blockDim.x + threadIdx.x;
+  if (a >= n_rows) return;
+  const T d = wsum ? (T)wsum[a] : (T)in_len[a];
+  out[a] = in_len[a] > 0 ? (T)scale / d : T(0);
 }
 
 int num_sms_for_narrow() {
@@ -138,6 +248,7 @@ __global__ void __launch_bounds__(256) k_col_chunk_narrow(
     ch.len = 0;
     ch.start = 0;
     if (q < count) ch = chunks[q];
+    ch.len = chunk_len(ch);
     int a[4];
     T wt[4];
 #pragma unroll
@@ -185,7 +296,7 @@ __global__ void k_col_prescale(const T* __restrict__ X, const int32_t* __restric
 // block's columns are staged in shared memory.
 template <typename T, typename TP>
 __global__ void k_col_apply(const TP* __restrict__ P, int K1, const int32_t* __restrict__ cols,
-                            int B, int n_rows, T* __restrict__ Y) {
+                            int B, int ldb, int n_rows, T* __restrict__ Y) {
   extern __shared__ double sg[];  // [B][2*K1]: xi_k[x_c], eta_k[x_c]
   for (int e = threadIdx.x; e < B * K1; e += blockDim.x) {
     const int c = e / K1, k = e % K1;
@@ -204,7 +315,7 @@ __global__ void k_col_apply(const TP* __restrict__ P, int K1, const int32_t* __r
     for (int k = 0; k < K1; ++k)
       acc += (double)P[ba + (int64_t)k * PT] * g[K1 + k] +
              (double)P[ba + (int64_t)(K1 + k) * PT] * g[k];
-    Y[a * B + c] = (T)((double)Y[a * B + c] + acc);
+    Y[a * ldb + c] = (T)((double)Y[a * ldb + c] + acc);
   }
 }
 
@@ -235,7 +346,8 @@ __global__ void k_col_gvals(const float* const* __restrict__ hist, int K1,
 constexpr int CG_KC = 16;
 __global__ void __launch_bounds__(256) k_col_corr(const float* const* __restrict__ hist, int U,
                                                   int K1, const float* __restrict__ G, int Bp,
-                                                  int B, int n_rows, float* __restrict__ Y) {
+                                                  int B, int ldb, int n_rows,
+                                                  float* __restrict__ Y) {
   __shared__ __align__(16) float sA[CG_KC][PT];
   __shared__ __align__(16) float sG[CG_KC][PT];
   const int T = blockIdx.x, c0 = blockIdx.y * PT;
@@ -286,7 +398,7 @@ __global__ void __launch_bounds__(256) k_col_corr(const float* const* __restrict
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       const int col = c0 + ((c < 4) ? tx * 4 + c : 64 + tx * 4 + (c - 4));
-      if (col < B) Y[row * B + col] += acc[r][c];
+      if (col < B) Y[row * ldb + col] += acc[r][c];
     }
   }
 }
@@ -313,12 +425,20 @@ __global__ void k_col_scalars(DevAdj in, const double* __restrict__ si, const do
   }
 }
 
-// out[c * n + a] = Y[a][c] (column-major output, optional FP32)
+// out[c * n + a] = Y[a][c] (column-major output, optional FP32), transposed
+// in 32 x 32 blocks through shared memory so that both sides are read and
+// written in rows (200,000 x 256, FP32: 226 us when read column by column).
 template <typename T, typename TO>
-__global__ void k_col_out(const T* __restrict__ Y, int B, int n, TO* __restrict__ out) {
-  const int c = blockIdx.y;
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
-  if (a < n) out[(int64_t)c * n + a] = (TO)Y[(int64_t)a * B + c];
+__global__ void k_col_out(const T* __restrict__ Y, int B, int ldb, int n, TO* __restrict__ out) {
+  __shared__ T tile[32][33];
+  const int a0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
+  for (int r = threadIdx.y; r < 32; r += 8)
+    if (a0 + r < n && c0 + (int)threadIdx.x < B)
+      tile[r][threadIdx.x] = Y[(int64_t)(a0 + r) * ldb + c0 + threadIdx.x];
+  __syncthreads();
+  for (int r = threadIdx.y; r < 32; r += 8)
+    if (c0 + r < B && a0 + (int)threadIdx.x < n)
+      out[(int64_t)(c0 + r) * n + a0 + threadIdx.x] = (TO)tile[threadIdx.x][r];
 }
 
 // column c of a row-major [n][B] block into a contiguous FP64 vector
@@ -330,29 +450,78 @@ __global__ void k_col_extract(const T* __restrict__ Y, int B, int c, int n, doub
 
 }  // namespace
 
+// One wide step (ldb > 4) over the row chunks L; a warp covers 512 bytes of a
+// row.  Chunks per warp: up to 8 in FP32, as long as every SM keeps some 64
+// warps to run (200,000 nodes x 256 columns: 9.6 ms a query with 8, 10.8 ms
+// with 1; with 8 gathers in flight per lane instead of 4, 13-15 ms: they push
+// the rows that are gathered often out of L1).  FP64 is bound by its FMAs and
+// takes one chunk per warp (gradient, 5,000 nodes: 13.0 ms with 1, 15.1 ms
+// with 8).
+template <typename T>
+static void wide_step(const ChunkList& L, const int32_t* adj, const float* w, bool forward,
+                      const T* nodes, const T* X, const T* Xadd, double add_scale, T* Y, int ldb,
+                      cudaStream_t st) {
+  constexpr int VEC = 16 / sizeof(T);
+  if (L.multi_count > 0)
+    k_col_prefill<T><<<(unsigned)L.multi_count, 128, 0, st>>>(L.multi, Xadd, (T)add_scale, Y, ldb);
+  if (L.count <= 0) return;
+  const int groups = (ldb + 32 * VEC - 1) / (32 * VEC);
+  const int64_t warps = (int64_t)num_sms_for_narrow() * 64;
+  const int per = sizeof(T) == 8 ? 1
+                                 : (int)std::max<int64_t>(
+                                       1, std::min<int64_t>(8, L.count * groups / warps));
+  const dim3 grid((unsigned)((L.count + 8 * per - 1) / (8 * per)), (unsigned)groups);
+  if (forward)
+    k_col_rows<T, VEC, true><<<grid, 256, 0, st>>>(L.chunks, L.count, per, adj, w, nodes, X,
+                                                   nullptr, T(0), Y, ldb);
+  else
+    k_col_rows<T, VEC, false><<<grid, 256, 0, st>>>(L.chunks, L.count, per, adj, w, nodes, X, Xadd,
+                                                    (T)add_scale, Y, ldb);
+}
+
 template <typename T>
 static void partial_sim_block_t(const ChunkList& fwd, const ChunkList& hor, const int32_t* out_col,
                                 const int32_t* in_col, const WeightView& wv, const int32_t* in_len,
-                                const int32_t* cols, int B, int n_rows, int K, double C, T* xs, T* y0,
-                                T* y1, T* result, cudaStream_t st, int group0) {
-  const int64_t blk = (int64_t)n_rows * B;
+                                const int32_t* cols, int B, int ldb, int n_rows, int K, double C,
+                                T* xs, T* y0, T* y1, T* result, T* scales, cudaStream_t st,
+                                int group0) {
+  const int64_t blk = (int64_t)n_rows * ldb;
   const int fill_blocks = 4096;
   k_col_fill<T><<<fill_blocks, 256, 0, st>>>(nullptr, 0.0, xs, blk);
   if (group0 > 1)
-    k_col_unit_grouped<T><<<(group0 + B + 126) / 128, 128, 0, st>>>(cols, group0, B, xs);
+    k_col_unit_grouped<T><<<(group0 + B + 126) / 128, 128, 0, st>>>(cols, group0, B, ldb, xs);
   else
-    k_col_unit<T><<<(B + 127) / 128, 128, 0, st>>>(cols, B, xs);
-  const int ygroups = (B + 127) / 128;
-  const int tpb = B >= 128 ? 128 : (B + 31) / 32 * 32;
-  // FP32 blocks of a multiple of 4 columns: four columns per thread
-  const bool vec4 = sizeof(T) == 4 && B % 4 == 0;
-  const int B4 = B / 4;
-  const int tpb4 = B4 >= 256 ? 256 : (B4 + 31) / 32 * 32;
-  const int ygroups4 = (B4 + tpb4 - 1) / tpb4;
-  // narrow blocks: one warp per chunk; the forward input divided once per row
-  const bool narrow = B <= 4;
+    k_col_unit<T><<<(B + 127) / 128, 128, 0, st>>>(cols, B, ldb, xs);
+  if (K == 0) {
+    k_col_fill<T><<<fill_blocks, 256, 0, st>>>(xs, 1.0 - C, result, blk);
+    return;
+  }
+  T* bufs[2] = {y0, y1};
+  if (ldb > 4) {
+    // wide blocks: 1 / d per node, and C / d, (1 - C) C / d for the Horner steps
+    T* inv = scales;
+    T* hs = scales + n_rows;
+    T* hl = scales + 2 * (int64_t)n_rows;
+    const int nb = (n_rows + 255) / 256;
+    k_col_scales<T><<<nb, 256, 0, st>>>(in_len, wv.wsum, 1.0, n_rows, inv);
+    k_col_scales<T><<<nb, 256, 0, st>>>(in_len, wv.wsum, C, n_rows, hs);
+    k_col_scales<T><<<nb, 256, 0, st>>>(in_len, wv.wsum, (1.0 - C) * C, n_rows, hl);
+    for (int t = 1; t <= K; ++t)
+      wide_step<T>(fwd, out_col, wv.out_w, true, inv, xs + (int64_t)(t - 1) * blk, nullptr,
+                       0.0, xs + (int64_t)t * blk, ldb, st);
+    const T* y = xs + (int64_t)K * blk;
+    for (int t = 1; t <= K; ++t) {
+      T* dst = (t == K) ? result : bufs[t & 1];
+      wide_step<T>(hor, in_col, wv.in_w, false, t == K ? hl : hs, y,
+                       xs + (int64_t)(K - t) * blk, t == K ? 1.0 - C : 1.0, dst, ldb, st);
+      y = dst;
+    }
+    return;
+  }
+  // narrow blocks: a group of 8 lanes per chunk; the forward input divided once per row
   auto narrow_step = [&](const ChunkList& L, const int32_t* adj, const float* w, bool forward,
                          const T* X, T* Y, double scale) {
+    if (L.count <= 0) return;
     // persistent: at most 8 CTAs of 8 warps per SM, four chunks per warp at a time
     const int64_t want = (L.count + 31) / 32;
     const unsigned grid = (unsigned)std::min<int64_t>(want, (int64_t)num_sms_for_narrow() * 8);
@@ -365,7 +534,7 @@ static void partial_sim_block_t(const ChunkList& fwd, const ChunkList& hor, cons
       k_col_chunk_narrow<T, false, BW><<<grid, 256, 0, st>>>(L.chunks, L.count, adj, w, in_len, \
                                                              wv.wsum, X, Y, scale);            \
   } while (0)
-    switch (B) {
+    switch (ldb) {
       case 1: SR_NARROW(1); break;
       case 2: SR_NARROW(2); break;
       case 3: SR_NARROW(3); break;
@@ -373,93 +542,61 @@ static void partial_sim_block_t(const ChunkList& fwd, const ChunkList& hor, cons
     }
 #undef SR_NARROW
   };
-  auto chunk_step = [&](const ChunkList& L, const int32_t* adj, const float* w, bool forward,
-                        const T* X, T* Y, double scale) {
-    if (L.count <= 0) return;
-    if (narrow) {
-      if (forward) {
-        // y0 is free until the Horner steps: it holds X divided by the row degrees
-        k_col_prescale<T><<<fill_blocks, 256, 0, st>>>(X, in_len, wv.wsum, B, blk, y0);
-        narrow_step(L, adj, w, true, y0, Y, scale);
-      } else {
-        narrow_step(L, adj, w, false, X, Y, scale);
-      }
-    } else if (vec4) {
-      if (forward)
-        k_col_chunk4<true><<<dim3((unsigned)L.count, ygroups4), tpb4, 0, st>>>(
-            L.chunks, adj, w, in_len, wv.wsum, (const float*)X, (float*)Y, B4, scale);
-      else
-        k_col_chunk4<false><<<dim3((unsigned)L.count, ygroups4), tpb4, 0, st>>>(
-            L.chunks, adj, w, in_len, wv.wsum, (const float*)X, (float*)Y, B4, scale);
-    } else if (forward) {
-      k_col_chunk<T, true><<<dim3((unsigned)L.count, ygroups), tpb, 0, st>>>(
-          L.chunks, adj, w, in_len, wv.wsum, X, Y, B, scale);
-    } else {
-      k_col_chunk<T, false><<<dim3((unsigned)L.count, ygroups), tpb, 0, st>>>(
-          L.chunks, adj, w, in_len, wv.wsum, X, Y, B, scale);
-    }
-  };
   for (int t = 1; t <= K; ++t) {
     T* dst = xs + (int64_t)t * blk;
     k_col_fill<T><<<fill_blocks, 256, 0, st>>>(nullptr, 0.0, dst, blk);
-    chunk_step(fwd, out_col, wv.out_w, true, xs + (int64_t)(t - 1) * blk, dst, 1.0);
+    // y0 is free until the Horner steps: it holds X divided by the row degrees
+    k_col_prescale<T><<<fill_blocks, 256, 0, st>>>(xs + (int64_t)(t - 1) * blk, in_len, wv.wsum,
+                                                   ldb, blk, y0);
+    narrow_step(fwd, out_col, wv.out_w, true, y0, dst, 1.0);
   }
   // Horner: y = x_K; y <- x_{K-t} + C Q y; result (1-C) y (the last step folds the scale)
   const T* y = xs + (int64_t)K * blk;
-  T* bufs[2] = {y0, y1};
-  if (K == 0) {
-    k_col_fill<T><<<fill_blocks, 256, 0, st>>>(xs, 1.0 - C, result, blk);
-    return;
-  }
   for (int t = 1; t <= K; ++t) {
     T* dst = (t == K) ? result : bufs[t & 1];
     const double s = (t == K) ? 1.0 - C : 1.0;
     k_col_fill<T><<<fill_blocks, 256, 0, st>>>(xs + (int64_t)(K - t) * blk, s, dst, blk);
-    chunk_step(hor, in_col, wv.in_w, false, y, dst, s * C);
+    narrow_step(hor, in_col, wv.in_w, false, y, dst, s * C);
     y = dst;
   }
 }
 
 void launch_partial_sim_block(const ChunkList& fwd, const ChunkList& hor, const int32_t* out_col,
                               const int32_t* in_col, const int32_t* in_len, const int32_t* cols,
-                              int B, int n_rows, int K, double C, int prec, void* xs, void* y0,
-                              void* y1, void* result, cudaStream_t st, const WeightView& wv,
-                              int group0) {
+                              int B, int ldb, int n_rows, int K, double C, int prec, void* xs,
+                              void* y0, void* y1, void* result, void* scales, cudaStream_t st,
+                              const WeightView& wv, int group0) {
   if (prec == 64)
-    partial_sim_block_t<double>(fwd, hor, out_col, in_col, wv, in_len, cols, B, n_rows, K, C,
-                                (double*)xs, (double*)y0, (double*)y1, (double*)result, st, group0);
+    partial_sim_block_t<double>(fwd, hor, out_col, in_col, wv, in_len, cols, B, ldb, n_rows, K, C,
+                                (double*)xs, (double*)y0, (double*)y1, (double*)result,
+                                (double*)scales, st, group0);
   else
-    partial_sim_block_t<float>(fwd, hor, out_col, in_col, wv, in_len, cols, B, n_rows, K, C,
-                               (float*)xs, (float*)y0, (float*)y1, (float*)result, st, group0);
+    partial_sim_block_t<float>(fwd, hor, out_col, in_col, wv, in_len, cols, B, ldb, n_rows, K, C,
+                               (float*)xs, (float*)y0, (float*)y1, (float*)result, (float*)scales,
+                               st, group0);
 }
 
-// Y = Q^T X (FP64 blocks [n_rows][B])
-void launch_col_forward64(const ChunkList& fwd, const int32_t* out_col, const WeightView& wv,
-                          const int32_t* in_len, const double* X, double* Y, int B, int n_rows,
-                          cudaStream_t st) {
-  const int64_t blk = (int64_t)n_rows * B;
-  k_col_fill<double><<<4096, 256, 0, st>>>(nullptr, 0.0, Y, blk);
-  const int tpb = B >= 128 ? 128 : (B + 31) / 32 * 32;
-  if (fwd.count > 0)
-    k_col_chunk<double, true><<<dim3((unsigned)fwd.count, (B + 127) / 128), tpb, 0, st>>>(
-        fwd.chunks, out_col, wv.out_w, in_len, wv.wsum, X, Y, B, 1.0);
-}
-
-// Yn = add_scale * Xadd + scale * Q Y (FP64 blocks [n_rows][B])
-void launch_col_horner64(const ChunkList& hor, const int32_t* in_col, const WeightView& wv,
-                         const int32_t* in_len, const double* Xadd, double add_scale,
-                         const double* Y, double* Yn, int B, int n_rows, double scale,
+void launch_col_scales64(const WeightView& wv, const int32_t* in_len, int n_rows, double* inv,
                          cudaStream_t st) {
-  const int64_t blk = (int64_t)n_rows * B;
-  k_col_fill<double><<<4096, 256, 0, st>>>(Xadd, add_scale, Yn, blk);
-  const int tpb = B >= 128 ? 128 : (B + 31) / 32 * 32;
-  if (hor.count > 0)
-    k_col_chunk<double, false><<<dim3((unsigned)hor.count, (B + 127) / 128), tpb, 0, st>>>(
-        hor.chunks, in_col, wv.in_w, in_len, wv.wsum, Y, Yn, B, scale);
+  k_col_scales<double><<<(n_rows + 255) / 256, 256, 0, st>>>(in_len, wv.wsum, 1.0, n_rows, inv);
 }
 
-void launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, int B, int n_rows,
-                      int prec, void* Y, cudaStream_t st) {
+// Y = Q^T X (FP64 blocks [n_rows][ldb])
+void launch_col_forward64(const ChunkList& fwd, const int32_t* out_col, const WeightView& wv,
+                          const double* inv, const double* X, double* Y, int ldb,
+                          cudaStream_t st) {
+  wide_step<double>(fwd, out_col, wv.out_w, true, inv, X, nullptr, 0.0, Y, ldb, st);
+}
+
+// Yn = add_scale * Xadd + Q Y (FP64 blocks [n_rows][ldb])
+void launch_col_horner64(const ChunkList& hor, const int32_t* in_col, const WeightView& wv,
+                         const double* inv, const double* Xadd, double add_scale, const double* Y,
+                         double* Yn, int ldb, cudaStream_t st) {
+  wide_step<double>(hor, in_col, wv.in_w, false, inv, Y, Xadd, add_scale, Yn, ldb, st);
+}
+
+void launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, int B, int ldb,
+                      int n_rows, int prec, void* Y, cudaStream_t st) {
   const size_t smem = (size_t)B * 2 * K1 * sizeof(double);
   const int threads = 128;
   const int blocks = (n_rows + threads - 1) / threads;
@@ -467,7 +604,8 @@ void launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, in
   do {                                                                                       \
     cudaFuncSetAttribute(k_col_apply<T, TP>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
                          (int)smem);                                                         \
-    k_col_apply<T, TP><<<blocks, threads, smem, st>>>((const TP*)P, K1, cols, B, n_rows, (T*)Y); \
+    k_col_apply<T, TP><<<blocks, threads, smem, st>>>((const TP*)P, K1, cols, B, ldb, n_rows, \
+                                              (T*)Y); \
   } while (0)
   if (prec == 64 && p_prec == 64)
     SR_COL_APPLY(double, double);
@@ -480,13 +618,13 @@ void launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, in
 #undef SR_COL_APPLY
 }
 
-void launch_col_corr(const float* const* hist, int U, int K1, const int32_t* cols, int B,
+void launch_col_corr(const float* const* hist, int U, int K1, const int32_t* cols, int B, int ldb,
                      int n_rows, float* G, float* Y, cudaStream_t st) {
   if (U <= 0 || B <= 0) return;
   const int Bp = (B + 3) / 4 * 4;
   k_col_gvals<<<dim3((2 * K1 * Bp + 255) / 256, U), 256, 0, st>>>(hist, K1, cols, B, Bp, G);
-  k_col_corr<<<dim3(n_rows / PT, (B + PT - 1) / PT), 256, 0, st>>>(hist, U, K1, G, Bp, B, n_rows,
-                                                                   Y);
+  k_col_corr<<<dim3(n_rows / PT, (B + PT - 1) / PT), 256, 0, st>>>(hist, U, K1, G, Bp, B, ldb,
+                                                                   n_rows, Y);
 }
 
 void launch_col_scalars(const DevAdj& in, const double* si, const double* sj, int i, int j,
@@ -494,19 +632,19 @@ void launch_col_scalars(const DevAdj& in, const double* si, const double* sj, in
   k_col_scalars<<<1, 256, 0, st>>>(in, si, sj, i, j, scal);
 }
 
-void launch_col_out(const void* Y, int prec, int B, int n, void* out, int out_fp64,
+void launch_col_out(const void* Y, int prec, int B, int ldb, int n, void* out, int out_fp64,
                     cudaStream_t st) {
-  dim3 grid((n + 255) / 256, B);
+  const dim3 grid((n + 31) / 32, (B + 31) / 32), block(32, 8);
   if (prec == 64) {
     if (out_fp64)
-      k_col_out<double, double><<<grid, 256, 0, st>>>((const double*)Y, B, n, (double*)out);
+      k_col_out<double, double><<<grid, block, 0, st>>>((const double*)Y, B, ldb, n, (double*)out);
     else
-      k_col_out<double, float><<<grid, 256, 0, st>>>((const double*)Y, B, n, (float*)out);
+      k_col_out<double, float><<<grid, block, 0, st>>>((const double*)Y, B, ldb, n, (float*)out);
   } else {
     if (out_fp64)
-      k_col_out<float, double><<<grid, 256, 0, st>>>((const float*)Y, B, n, (double*)out);
+      k_col_out<float, double><<<grid, block, 0, st>>>((const float*)Y, B, ldb, n, (double*)out);
     else
-      k_col_out<float, float><<<grid, 256, 0, st>>>((const float*)Y, B, n, (float*)out);
+      k_col_out<float, float><<<grid, block, 0, st>>>((const float*)Y, B, ldb, n, (float*)out);
   }
 }
 

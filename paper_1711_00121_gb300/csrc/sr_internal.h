@@ -353,16 +353,24 @@ void launch_pack_f16_tiles(const float* Pp, int GK1, int nterms, int rg, int n_r
                            int64_t kd, cudaStream_t st);
 
 // ---- column mode (§7), k_column.cu
-// A piece of one adjacency row: row id, count (<= kChunk) and pool offset.
+// A piece of one adjacency row: row id, count (<= kChunk, in the low bits of
+// len) and pool offset.  CH_ONLY marks the only chunk of its row (an empty row
+// has one empty chunk).
 struct RowChunk {
   int32_t row;
   int32_t len;
   int64_t start;
 };
 constexpr int kChunk = 32;
+constexpr int32_t CH_ONLY = 1 << 16;
+#ifdef __CUDACC__
+__host__ __device__ __forceinline__ int chunk_len(const RowChunk& c) { return c.len & 0xffff; }
+#endif
 struct ChunkList {
   RowChunk* chunks = nullptr;  // device
   int64_t count = 0;
+  int32_t* multi = nullptr;  // device: the rows of more than one chunk
+  int64_t multi_count = 0, multi_cap = 0;
 };
 // Y[a][c] += scale / len(a) * sum over a's in-list of X[b][c], columns c <
 // ncols (a multiple of 4), by row chunks (FP64 atomics into Y, which the
@@ -382,31 +390,37 @@ struct WeightView {
 // (fwd chunks over out_col) and in-lists (hor chunks over in_col) are given;
 // in_len = in-degrees.  xs holds (K+1) row-major [n_rows][B] blocks, y0 / y1
 // are scratch blocks, result receives (1-C) sum_k C^k Q^k (Q^T)^k e_cols.
+// Blocks have row pitch ldb >= B: ldb <= 4, or a multiple of 4 (the columns
+// from B on stay zero); scales: 3 n_rows values of scratch when ldb > 4.
 void launch_partial_sim_block(const ChunkList& fwd, const ChunkList& hor, const int32_t* out_col,
                               const int32_t* in_col, const int32_t* in_len, const int32_t* cols,
-                              int B, int n_rows, int K, double C, int prec, void* xs, void* y0,
-                              void* y1, void* result, cudaStream_t st,
+                              int B, int ldb, int n_rows, int K, double C, int prec, void* xs,
+                              void* y0, void* y1, void* result, void* scales, cudaStream_t st,
                               const WeightView& wv = WeightView(), int group0 = 1);
+// inv[a] = 1 / (in-degree or in-weight of a); the two steps below on FP64
+// blocks of row pitch ldb (a multiple of 4)
+void launch_col_scales64(const WeightView& wv, const int32_t* in_len, int n_rows, double* inv,
+                         cudaStream_t st);
 void launch_col_forward64(const ChunkList& fwd, const int32_t* out_col, const WeightView& wv,
-                          const int32_t* in_len, const double* X, double* Y, int B, int n_rows,
+                          const double* inv, const double* X, double* Y, int ldb,
                           cudaStream_t st);
 void launch_col_horner64(const ChunkList& hor, const int32_t* in_col, const WeightView& wv,
-                         const int32_t* in_len, const double* Xadd, double add_scale,
-                         const double* Y, double* Yn, int B, int n_rows, double scale,
-                         cudaStream_t st);
+                         const double* inv, const double* Xadd, double add_scale, const double* Y,
+                         double* Yn, int ldb, cudaStream_t st);
 // Y[a][c] += sum_k xi_k[a] eta_k[cols[c]] + eta_k[a] xi_k[cols[c]] (panels P, FP32/64)
 // FP32 blocks: Y[a][c] += sum over the U stored updates (device array of
 // their panel pointers, tile-blocked FP32) of xi_k[a] eta_k[x_c] +
 // eta_k[a] xi_k[x_c], as one product; G: scratch of U * 2 * K1 * round4(B)
 // floats.  n_rows is a multiple of 128.
-void launch_col_corr(const float* const* hist, int U, int K1, const int32_t* cols, int B,
+void launch_col_corr(const float* const* hist, int U, int K1, const int32_t* cols, int B, int ldb,
                      int n_rows, float* G, float* Y, cudaStream_t st);
-void launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, int B, int n_rows,
-                      int prec, void* Y, cudaStream_t st);
+void launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, int B, int ldb,
+                      int n_rows, int prec, void* Y, cudaStream_t st);
 // scal[0] = si[i], scal[1] = sj[j], scal[2] = (1/d_j) sum_{b in I(j)} si[b]
 void launch_col_scalars(const DevAdj& in, const double* si, const double* sj, int i, int j,
                         double* scal, cudaStream_t st);
-void launch_col_out(const void* Y, int prec, int B, int n, void* out, int out_fp64, cudaStream_t st);
+void launch_col_out(const void* Y, int prec, int B, int ldb, int n, void* out, int out_fp64,
+                    cudaStream_t st);
 void launch_col_extract(const void* Y, int prec, int B, int c, int n, double* v, cudaStream_t st);
 
 // ---- adjoint (k_adjoint.cu)
