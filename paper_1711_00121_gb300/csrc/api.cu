@@ -760,13 +760,49 @@ simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, i
   return SR_OK;
 }
 
-// Jacobi sweeps of Eq. 1 starting from the current S, in FP64 work buffers
+// C / d (or 1 / d) for every row's in-degree d as a fixed-point factor: the
+// significand of C over d in 128-bit integers, normalised to 64 bits.
+std::vector<SweepScale> sweep_scales(const HostAdj& A, int n_rows, double C) {
+  int e = 0;
+  const unsigned long long m = (unsigned long long)std::ldexp(std::frexp(C, &e), 53);  // C = m 2^(e-53)
+  std::vector<SweepScale> out((size_t)n_rows);
+  for (int a = 0; a < n_rows; ++a) {
+    const unsigned d = (unsigned)std::max(1, A.len[a]);
+    SweepScale f{0ull, 0, 0};
+    if (!(C == 1.0 && d == 1)) {
+      // q = floor(m 2^74 / d) = C / d * 2^(127 - e), at least 2^(126 - 32)
+      const unsigned __int128 q = ((unsigned __int128)m << 74) / d;
+      int top = 127;
+      while (!(q >> top)) --top;  // 2^top <= q
+      // r = q rounded to 64 bits: q = r 2^(top - 63)
+      unsigned __int128 r = (q + ((unsigned __int128)1 << (top - 64))) >> (top - 63);
+      int sh = 127 - e - (top - 63) - 64;  // C / d = r 2^-(64 + sh)
+      if (r >> 64) {
+        r >>= 1;
+        --sh;
+      }
+      f.r = (unsigned long long)r;
+      f.s = sh;
+    }
+    out[(size_t)a] = f;
+  }
+  return out;
+}
+
+// Jacobi sweeps of Eq. 1 starting from the current S, in 64-bit work buffers
 // when three of them fit in `fp64_budget` bytes (or S itself is FP64), else
 // in FP32 storage with FP64 accumulation.  Stops when a sweep changes S by
 // less than `tol` (max-abs) or after max_sweeps; S is symmetrised at the end.
+//
+// The 64-bit sweeps of an unweighted graph run in fixed point (k_sweep.cu):
+// one sweep at n = 10,007, m = 100,000 takes FIXME instead of 11.2 ms.  They
+// need |S| < 1.875 and an S that is symmetric up to its rounding (1e-6 in
+// FP32, 1e-12 in FP64; both hold for every S of Eq. 1): `known` says so without
+// a look at S, otherwise a pass over S decides, and any other S (a caller's S0)
+// is swept in FP64 as it is.
 simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double* last_diff,
                              int* sweeps_done, double* tol_used = nullptr,
-                             double* first_diff = nullptr) {
+                             double* first_diff = nullptr, bool known = false) {
   const int sp = h->cfg.s_precision;
   const size_t elems = (size_t)h->n_pad * h->ld;
   const size_t fp64_budget = (size_t)48 << 30;
@@ -788,25 +824,57 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
       return fail(h, SR_ERR_OOM, "cudaMalloc of Jacobi buffers failed");
     }
   }
-  if (alias)
-    bufs[0] = h->S;
-  else
-    launch_convert(h->S, sp, bufs[0], wp, (int64_t)elems, h->st);
-  cudaMemsetAsync(bufs[1], 0, bytes, h->st);
-  cudaMemsetAsync(bufs[2], 0, bytes, h->st);
-  void *A = bufs[0], *B = bufs[1], *T = bufs[2];
   double diff = INFINITY;
   int it = 0;
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (!h->weighted && wp == 64 && !known) {
+    unsigned int flags = 0;
+    e = cudaMemsetAsync(h->diffbits, 0, sizeof(unsigned long long), h->st);
+    launch_sweep_check(h->S, sp, h->n_pad, h->ld, sp == 64 ? 1e-12 : 1e-6,
+                       (unsigned int*)h->diffbits, h->st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&flags, h->diffbits, sizeof(flags), cudaMemcpyDeviceToHost, h->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
+    known = flags == 0;
+  }
+  const bool fixed = !h->weighted && wp == 64 && known;
+  if (alias)
+    bufs[0] = h->S;
+  else if (!fixed)
+    launch_convert(h->S, sp, bufs[0], wp, (int64_t)elems, h->st);
+  void *A = bufs[0], *B = bufs[1], *T = bufs[2];
+  SweepScale* scales = nullptr;
+  if (fixed && e == cudaSuccess) {
+    // every entry of T and B is written by each sweep
+    launch_to_fixed(h->S, sp, (long long*)A, h->n_pad, h->ld, h->st);
+    std::vector<SweepScale> f = sweep_scales(h->hin, h->n_pad, h->cfg.C);
+    const std::vector<SweepScale> f1 = sweep_scales(h->hin, h->n_pad, 1.0);
+    f.insert(f.end(), f1.begin(), f1.end());
+    e = cudaMalloc(&scales, f.size() * sizeof(SweepScale));
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(scales, f.data(), f.size() * sizeof(SweepScale), cudaMemcpyHostToDevice,
+                          h->st);
+  } else if (!fixed) {
+    cudaMemsetAsync(bufs[1], 0, bytes, h->st);
+    cudaMemsetAsync(bufs[2], 0, bytes, h->st);
+  }
+  if (e == cudaSuccess) e = cudaGetLastError();
   const float* w = h->weighted ? h->d_in_w : nullptr;
   while (e == cudaSuccess && it < max_sweeps) {
-    launch_spmm_rows(h->din, w, h->d_wsum, A, wp, h->ld, B, wp, h->ld, h->n_pad, h->n_pad, 1.0,
-                     0.0, 0, h->st);
-    launch_transpose(B, T, wp, h->n_pad, h->ld, h->st);
-    launch_spmm_rows(h->din, w, h->d_wsum, T, wp, h->ld, B, wp, h->ld, h->n_pad, h->n_pad,
-                     h->cfg.C, 1.0 - h->cfg.C, h->n_cap, h->st);
     cudaMemsetAsync(h->diffbits, 0, sizeof(unsigned long long), h->st);
-    launch_maxdiff(A, B, wp, h->n_pad, h->ld, h->diffbits, h->st);
+    if (fixed) {
+      launch_sweep_fixed(h->din, scales, scales + h->n_pad, (const long long*)A, h->ld, h->n_pad,
+                         (long long*)T, (long long*)B,
+                         (long long)std::llrint(std::ldexp(1.0 - h->cfg.C, 60)), h->n_cap,
+                         h->diffbits, h->st);
+    } else {
+      launch_spmm_rows(h->din, w, h->d_wsum, A, wp, h->ld, B, wp, h->ld, h->n_pad, h->n_pad, 1.0,
+                       0.0, 0, h->st);
+      launch_transpose(B, T, wp, h->n_pad, h->ld, h->st);
+      launch_spmm_rows(h->din, w, h->d_wsum, T, wp, h->ld, B, wp, h->ld, h->n_pad, h->n_pad,
+                       h->cfg.C, 1.0 - h->cfg.C, h->n_cap, h->st);
+      launch_maxdiff(A, B, wp, h->n_pad, h->ld, h->diffbits, h->st);
+    }
     e = cudaGetLastError();
     if (e != cudaSuccess) break;
     std::swap(A, B);
@@ -815,7 +883,10 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
     e = cudaMemcpyAsync(&bits, h->diffbits, sizeof(bits), cudaMemcpyDeviceToHost, h->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
     if (e != cudaSuccess) break;
-    std::memcpy(&diff, &bits, sizeof(diff));
+    if (fixed)
+      diff = std::ldexp((double)bits, -60);
+    else
+      std::memcpy(&diff, &bits, sizeof(diff));
     if (it == 1 && first_diff) *first_diff = diff;
     if (diff < tol) break;
     if (wp == 32) {
@@ -828,11 +899,16 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
     }
   }
   if (e == cudaSuccess) {
-    launch_symmetrize(A, wp, h->n_pad, h->ld, h->st);
-    if (!alias) launch_convert(A, wp, h->S, sp, (int64_t)elems, h->st);
+    if (fixed) {
+      launch_from_fixed((const long long*)A, alias ? A : h->S, sp, (int64_t)elems, h->st);
+    } else {
+      launch_symmetrize(A, wp, h->n_pad, h->ld, h->st);
+      if (!alias) launch_convert(A, wp, h->S, sp, (int64_t)elems, h->st);
+    }
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
+  if (scales) cudaFree(scales);
   // bufs[] holds three distinct buffers (bufs[0] is the old S when aliasing);
   // keep the result as S when aliasing and free every other buffer once.
   if (alias && e == cudaSuccess) h->S = A;
@@ -1769,8 +1845,8 @@ simrank_status simrank_init(const simrank_config* cfg_in, int32_t n, int64_t m, 
     launch_set_diag(h->S, cfg.s_precision, 0, h->n_cap, h->ld, 1.0 - cfg.C, h->st);
     double diff = 0.0, tol_used = cfg.init_tol;
     int sweeps = 0;
-    if ((s = jacobi_sweeps(h, cfg.init_max_sweeps, cfg.init_tol, &diff, &sweeps, &tol_used)) !=
-        SR_OK)
+    if ((s = jacobi_sweeps(h, cfg.init_max_sweeps, cfg.init_tol, &diff, &sweeps, &tol_used,
+                           nullptr, true)) != SR_OK)
       return bail(s);
     h->stats.init_residual = diff;
     h->stats.init_sweeps = sweeps;

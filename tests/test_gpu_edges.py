@@ -47,3 +47,60 @@ def test_column_blocks_at_chunk_edges(P, prec, width, reverse):
     got = sr.columns(cols)
     want = O.partial_sim_block(O.transition_matrix(n, s, d, sparse=True), cols, K, C)
     assert np.max(np.abs(got - want)) < (1e-12 if prec == 64 else 1e-6)
+
+
+def sweeps(S, Q, C, k):
+    for _ in range(k):
+        S = C * (Q @ (Q @ S).T).T + (1.0 - C) * np.eye(S.shape[0])
+    return S
+
+
+@pytest.mark.parametrize("C", [0.6, 0.25, 0.95])
+@pytest.mark.parametrize("n,degs", [(300, [0, 1, 2, 95, 96, 97, 100, 131, 257, 0]), (1, []), (65, [64, 1])])
+def test_fixed_point_sweeps_at_row_edges(P, n, degs, C):
+    """The first S of an FP64 handle (fixed-point sweeps: rows of up to 96
+    nonzeros by one warp, longer ones by the CTA) and one sweep more, against
+    the oracle's fixed point: both stop within C / (1 - C) 1e-13 of it."""
+    s, d = degrees_graph(n, degs, 5) if n > 1 else (np.zeros(0, np.int32), np.zeros(0, np.int32))
+    sr = P.SimRank(n, s, d, C=C, K=3, s_precision=64, init_max_sweeps=2000)
+    want = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-15)
+    tol = 1e-13 * C / (1.0 - C) + 1e-14
+    assert np.max(np.abs(sr.dense() - want)) < tol
+    sr.reanchor(1)
+    assert np.max(np.abs(sr.dense() - want)) < tol
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("form", ["symmetric", "rounded", "asymmetric", "large", "negative"])
+def test_sweeps_from_any_s0(P, form, prec):
+    """Sweeps from a caller's S0: symmetric entries below 1.875 in magnitude
+    (also when symmetric only up to rounding) run in fixed point, others (an
+    asymmetric S0, one entry of 40) in FP64; all give the sweeps of the
+    symmetrised S0.  Entries are at most 40 and a sweep contracts: 1e-13 x 40
+    in FP64, 1e-6 x 40 stored in FP32."""
+    n, C = 200, 0.6
+    s, d = degrees_graph(n, [0, 1, 97, 130, 33], 7)
+    rng = np.random.default_rng(8)
+    S0 = rng.uniform(-0.5 if form == "negative" else 0.0, 1.0, (n, n))
+    if form == "asymmetric":
+        S0[3, 7] += 0.25
+    else:
+        S0 = 0.5 * (S0 + S0.T)
+    if form == "large":
+        S0[5, 5] = 40.0
+    if form == "rounded":
+        S0[9, 4] = np.nextafter(S0[9, 4], 2.0)
+    dt = np.float64 if prec == 64 else np.float32
+    S0 = S0.astype(dt)
+    Q = O.transition_matrix(n, s, d)
+    sr = P.SimRank(n, s, d, S0=S0, C=C, K=3, s_precision=prec, upper_only=0)
+    first = sr.reanchor(1)
+    got = sr.dense()
+    W = S0.astype(np.float64)
+    want = sweeps(W, Q, C, 1)
+    tol = (1e-13 if prec == 64 else 1e-6) * 40
+    assert np.max(np.abs(got - 0.5 * (want + want.T))) < tol
+    assert abs(first - np.max(np.abs(want - W))) < tol
+    sr.reanchor(3)
+    want = sweeps(0.5 * (W + W.T), Q, C, 4)
+    assert np.max(np.abs(sr.dense() - want)) < tol
