@@ -760,30 +760,29 @@ simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, i
   return SR_OK;
 }
 
-// C / d (or 1 / d) for every row's in-degree d as a fixed-point factor: the
-// significand of C over d in 128-bit integers, normalised to 64 bits.
+// C / d for every row's in-degree d (C <= 1) as a fixed-point factor: the
+// significand of C over d in 128-bit integers, rounded to 63 bits.
 std::vector<SweepScale> sweep_scales(const HostAdj& A, int n_rows, double C) {
   int e = 0;
   const unsigned long long m = (unsigned long long)std::ldexp(std::frexp(C, &e), 53);  // C = m 2^(e-53)
   std::vector<SweepScale> out((size_t)n_rows);
   for (int a = 0; a < n_rows; ++a) {
     const unsigned d = (unsigned)std::max(1, A.len[a]);
-    SweepScale f{0ull, 0, 0};
-    if (!(C == 1.0 && d == 1)) {
-      // q = floor(m 2^74 / d) = C / d * 2^(127 - e), at least 2^(126 - 32)
-      const unsigned __int128 q = ((unsigned __int128)m << 74) / d;
-      int top = 127;
-      while (!(q >> top)) --top;  // 2^top <= q
-      // r = q rounded to 64 bits: q = r 2^(top - 63)
-      unsigned __int128 r = (q + ((unsigned __int128)1 << (top - 64))) >> (top - 63);
-      int sh = 127 - e - (top - 63) - 64;  // C / d = r 2^-(64 + sh)
-      if (r >> 64) {
-        r >>= 1;
-        --sh;
-      }
-      f.r = (unsigned long long)r;
-      f.s = sh;
+    // q = floor(m 2^74 / d) = C / d * 2^(127 - e), at least 2^94
+    const unsigned __int128 q = ((unsigned __int128)m << 74) / d;
+    int top = 127;
+    while (!(q >> top)) --top;
+    unsigned __int128 r = (q + ((unsigned __int128)1 << (top - 63))) >> (top - 62);
+    int s = 126 - e - top;  // C / d = r 2^-(63 + s)
+    if (r >> 63) {
+      r >>= 1;
+      --s;
     }
+    SweepScale f;
+    f.r = (unsigned long long)r;
+    f.h = 5;
+    while (f.h > 0 && (d << f.h) > 32) --f.h;
+    f.sh = d <= 32 ? s + f.h - 1 : s - 1;
     out[(size_t)a] = f;
   }
   return out;
@@ -792,10 +791,11 @@ std::vector<SweepScale> sweep_scales(const HostAdj& A, int n_rows, double C) {
 // Jacobi sweeps of Eq. 1 starting from the current S, in 64-bit work buffers
 // when three of them fit in `fp64_budget` bytes (or S itself is FP64), else
 // in FP32 storage with FP64 accumulation.  Stops when a sweep changes S by
-// less than `tol` (max-abs) or after max_sweeps; S is symmetrised at the end.
+// less than `tol` (max-abs) or after max_sweeps; S is symmetrised at the end
+// (the lower tiles are taken from their mirrors when only the upper are kept).
 //
 // The 64-bit sweeps of an unweighted graph run in fixed point (k_sweep.cu):
-// one sweep at n = 10,007, m = 100,000 takes FIXME instead of 11.2 ms.  They
+// one sweep at n = 10,007, m = 100,000 takes 1.4 ms, in FP64 10.6 ms.  They
 // need |S| < 1.875 and an S that is symmetric up to its rounding (1e-6 in
 // FP32, 1e-12 in FP64; both hold for every S of Eq. 1): `known` says so without
 // a look at S, otherwise a pass over S decides, and any other S (a caller's S0)
@@ -827,37 +827,44 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
   double diff = INFINITY;
   int it = 0;
   cudaError_t e = cudaSuccess;
-  if (!h->weighted && wp == 64 && !known) {
-    unsigned int flags = 0;
-    e = cudaMemsetAsync(h->diffbits, 0, sizeof(unsigned long long), h->st);
-    launch_sweep_check(h->S, sp, h->n_pad, h->ld, sp == 64 ? 1e-12 : 1e-6,
-                       (unsigned int*)h->diffbits, h->st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(&flags, h->diffbits, sizeof(flags), cudaMemcpyDeviceToHost, h->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
-    known = flags == 0;
-  }
-  const bool fixed = !h->weighted && wp == 64 && known;
-  if (alias)
-    bufs[0] = h->S;
-  else if (!fixed)
-    launch_convert(h->S, sp, bufs[0], wp, (int64_t)elems, h->st);
-  void *A = bufs[0], *B = bufs[1], *T = bufs[2];
+  bool fixed = !h->weighted && wp == 64;
   SweepScale* scales = nullptr;
-  if (fixed && e == cudaSuccess) {
-    // every entry of T and B is written by each sweep
-    launch_to_fixed(h->S, sp, (long long*)A, h->n_pad, h->ld, h->st);
-    std::vector<SweepScale> f = sweep_scales(h->hin, h->n_pad, h->cfg.C);
-    const std::vector<SweepScale> f1 = sweep_scales(h->hin, h->n_pad, 1.0);
-    f.insert(f.end(), f1.begin(), f1.end());
-    e = cudaMalloc(&scales, f.size() * sizeof(SweepScale));
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(scales, f.data(), f.size() * sizeof(SweepScale), cudaMemcpyHostToDevice,
-                          h->st);
-  } else if (!fixed) {
+  if (fixed) {
+    // S into bufs[0] in fixed point, with a look at what it holds unless it is
+    // known (before the change when it is made in place)
+    unsigned int flags = 0;
+    long long* F = (long long*)(alias ? h->S : bufs[0]);
+    const double sym = sp == 64 ? 1e-12 : 1e-6;
+    unsigned int* df = (unsigned int*)h->diffbits;
+    e = cudaMemsetAsync(h->diffbits, 0, sizeof(unsigned long long), h->st);
+    if (!known)
+      launch_to_fixed(h->S, sp, alias ? nullptr : F, h->n_pad, h->ld, upper(h), true, sym, df,
+                      h->st);
+    if (e == cudaSuccess && !known)
+      e = cudaMemcpyAsync(&flags, h->diffbits, sizeof(flags), cudaMemcpyDeviceToHost, h->st);
+    if (e == cudaSuccess && !known) e = cudaStreamSynchronize(h->st);
+    fixed = flags == 0;
+    if (fixed && e == cudaSuccess) {
+      // every entry of the other two buffers is written by each sweep
+      if (known || alias)
+        launch_to_fixed(h->S, sp, F, h->n_pad, h->ld, upper(h), false, sym, df, h->st);
+      std::vector<SweepScale> f = sweep_scales(h->hin, h->n_pad, h->cfg.C);
+      const std::vector<SweepScale> f1 = sweep_scales(h->hin, h->n_pad, 1.0);
+      f.insert(f.end(), f1.begin(), f1.end());
+      e = cudaMalloc(&scales, f.size() * sizeof(SweepScale));
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(scales, f.data(), f.size() * sizeof(SweepScale),
+                            cudaMemcpyHostToDevice, h->st);
+    }
+  }
+  if (alias) bufs[0] = h->S;
+  if (!fixed) {
+    if (upper(h)) launch_mirror_lower(h->S, sp, h->n_pad, h->ld, h->st);
+    if (!alias) launch_convert(h->S, sp, bufs[0], wp, (int64_t)elems, h->st);
     cudaMemsetAsync(bufs[1], 0, bytes, h->st);
     cudaMemsetAsync(bufs[2], 0, bytes, h->st);
   }
+  void *A = bufs[0], *B = bufs[1], *T = bufs[2];
   if (e == cudaSuccess) e = cudaGetLastError();
   const float* w = h->weighted ? h->d_in_w : nullptr;
   while (e == cudaSuccess && it < max_sweeps) {
@@ -865,7 +872,7 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
     if (fixed) {
       launch_sweep_fixed(h->din, scales, scales + h->n_pad, (const long long*)A, h->ld, h->n_pad,
                          (long long*)T, (long long*)B,
-                         (long long)std::llrint(std::ldexp(1.0 - h->cfg.C, 60)), h->n_cap,
+                         (long long)std::llrint(std::ldexp(1.0 - h->cfg.C, 57)), h->n_cap,
                          h->diffbits, h->st);
     } else {
       launch_spmm_rows(h->din, w, h->d_wsum, A, wp, h->ld, B, wp, h->ld, h->n_pad, h->n_pad, 1.0,
@@ -884,7 +891,7 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
     if (e != cudaSuccess) break;
     if (fixed)
-      diff = std::ldexp((double)bits, -60);
+      diff = std::ldexp((double)bits, -57);
     else
       std::memcpy(&diff, &bits, sizeof(diff));
     if (it == 1 && first_diff) *first_diff = diff;
@@ -900,7 +907,8 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
   }
   if (e == cudaSuccess) {
     if (fixed) {
-      launch_from_fixed((const long long*)A, alias ? A : h->S, sp, (int64_t)elems, h->st);
+      launch_from_fixed((const long long*)A, alias ? A : h->S, sp, h->n_pad, h->ld, upper(h),
+                        h->st);
     } else {
       launch_symmetrize(A, wp, h->n_pad, h->ld, h->st);
       if (!alias) launch_convert(A, wp, h->S, sp, (int64_t)elems, h->st);
@@ -922,18 +930,11 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
   return SR_OK;
 }
 
-// Drift correction: Jacobi sweeps of Eq. 1 started from the current S (its
-// lower tiles restored from their mirrors first when only the upper ones are
-// kept), until a sweep changes S by less than tol or after `sweeps` sweeps.
+// Drift correction: Jacobi sweeps of Eq. 1 started from the current S, until a sweep changes S by less than tol or after `sweeps` sweeps.
 // The first sweep's change is the residual max |C Q S Q^T + (1-C) I - S| of
 // the S it started from.
 simrank_status reanchor_run(simrank_ctx* h, int sweeps, double tol, double* first, double* last,
                             int* done) {
-  if (upper(h)) {
-    launch_mirror_lower(h->S, h->cfg.s_precision, h->n_pad, h->ld, h->st);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(h, SR_ERR_CUDA, cudaGetErrorString(e));
-  }
   return jacobi_sweeps(h, sweeps, tol, last, done, nullptr, first);
 }
 

@@ -272,12 +272,14 @@ void launch_transpose(const void* A, void* B, int prec, int n_pad, int64_t ld, c
 // *out_bits = max(*out_bits, max |A - B|) over the n x n block (as double bits)
 void launch_maxdiff(const void* A, const void* B, int prec, int n, int64_t ld,
                     unsigned long long* out_bits, cudaStream_t st);
-// ---- the same sweep on a symmetric S in fixed point (value * 2^60), k_sweep.cu
-// A factor r * 2^-(64 + s) <= 1 with 2^63 <= r < 2^64 (r = 0: the factor one).
+// ---- the same sweep on a symmetric S in fixed point (value * 2^57), k_sweep.cu
+// The factor C / d of a row of d nonzeros, r * 2^-(63 + s) with 2^62 <= r < 2^63.
+// d <= 32: a row sum shifted left by h stays below 2^63, and the high word of
+// its product with r is shifted right by sh = s + h - 1 (at least 3); longer
+// rows: sh = s - 1 (at least 4).
 struct SweepScale {
   unsigned long long r;
-  int s;
-  int pad;
+  int h, sh;
 };
 // One sweep: T and Snew are n_pad x ld; s1[a] = C / in-degree of a, s2[a] =
 // 1 / in-degree; diag is added to the first n_diag diagonal entries; *maxd =
@@ -285,14 +287,15 @@ struct SweepScale {
 void launch_sweep_fixed(const DevAdj& in, const SweepScale* s1, const SweepScale* s2,
                         const long long* S, int64_t ld, int n_pad, long long* T, long long* Snew,
                         long long diag, int n_diag, unsigned long long* maxd, cudaStream_t st);
-// *flags |= 1 when an entry has magnitude >= 1.875 or is NaN, |= 2 when two
-// mirrored entries differ by more than tol
-void launch_sweep_check(const void* S, int prec, int n_pad, int64_t ld, double tol,
-                        unsigned int* flags, cudaStream_t st);
-// F = (S + S^T) / 2 in fixed point, and back (S and F may share memory)
-void launch_to_fixed(const void* S, int prec, long long* F, int n_pad, int64_t ld,
-                     cudaStream_t st);
-void launch_from_fixed(const long long* F, void* S, int prec, int64_t count, cudaStream_t st);
+// F = (S + S^T) / 2 in fixed point (F null, FP64 S: no change), and back (S and
+// F may share memory).  check (always with F null): *flags |= 1 when an entry
+// has magnitude >= 1.875 or is NaN, |= 2 when two mirrored entries differ by
+// more than tol.  upper: only the tiles on or above the block diagonal of S
+// are read, and written.
+void launch_to_fixed(const void* S, int prec, long long* F, int n_pad, int64_t ld, int upper,
+                     bool check, double tol, unsigned int* flags, cudaStream_t st);
+void launch_from_fixed(const long long* F, void* S, int prec, int n_pad, int64_t ld, int upper,
+                       cudaStream_t st);
 // S[J, I] = S[I, J]^T for all 128-tiles I < J (restores the lower triangle)
 void launch_mirror_lower(void* A, int prec, int n_pad, int64_t ld, cudaStream_t st);
 void launch_symmetrize(void* A, int prec, int n_pad, int64_t ld, cudaStream_t st);
