@@ -124,8 +124,8 @@ typedef struct simrank_config {
                              replayed from a CUDA graph; 1 = the same kernels launched graph by
                              graph (the per-graph-launch baseline) */
   int32_t prep_item;      /* chain = 0: 0 (default) = the nonzeros of all rows split evenly over
-                             the CTAs of the fused launch, two per thread (work items of 1024
-                             when that does not fit); > 0 = work items of at most this many
+                             the CTAs of the fused launch, up to two per thread (work items of
+                             1024 when that does not fit); > 0 = work items of at most this many
                              nonzeros inside one 128-row tile, a tile with more split over
                              several CTAs */
   int32_t upper_only;     /* dense mode: 1 = keep only the 128 x 128 tiles of S on or above the
@@ -133,8 +133,9 @@ typedef struct simrank_config {
                              half the bytes, and reads of a lower tile take its mirror); 0 = keep
                              both triangles.  Default 1. */
   int32_t vec_fp64;       /* chain = 0 with S in FP32: 1 = xi/eta vectors, gamma and the
-                             recurrence in FP64; 0 (default) = in FP32.  On GB300 the FP64 form
-                             makes the pre-update launch about 2.3x slower. */
+                             recurrence in FP64; 0 (default) = in FP32.  With prep_item = 0 the
+                             recurrence runs in 64-bit fixed point in both (as fast for 1 as for
+                             0) and vec_fp64 is the precision of the rows of S and of gamma. */
   int32_t init_form;      /* SR_INIT_SWEEPS (default), SR_INIT_FOREST or SR_INIT_COMPONENTS: how
                              simrank_init computes S when S0 is NULL (dense mode).  With
                              SR_INIT_FOREST the initial graph must be a forest of arborescences

@@ -74,6 +74,8 @@ struct simrank_ctx {
   void* W = nullptr;              // (xi, eta) working columns of the pre-update kernel
   void* rinv = nullptr;           // its per-row (C / in-degree, 1 / in-degree)
   int32_t* loff = nullptr;        // its per-row offsets inside the tile
+  long long* flowY = nullptr;     // its row sums of the flow form
+  SweepScale* flow_tab = nullptr; // 1 / d for d <= n_cap, then C^(k+1) for k <= K
   int* tile_nnz = nullptr;       // per-tile nonzeros (scratch of the pre-update kernel)
   // per-call staging
   int32_t* d_srcs = nullptr;
@@ -646,6 +648,7 @@ simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, i
     pp.inv_C = 1.0 / C;
     pp.inv_delta = 1.0 / (double)delta;
     pp.gq = (d_j + op * delta) != 0 ? (double)delta / (double)(d_j + op * delta) : 0.0;
+    pp.inv_ddj = d_j > 0 ? 1.0 / ((double)delta * (double)d_j) : 0.0;
     pp.K = h->cfg.K;
     pp.nT = nT;
     if (defer) {
@@ -673,6 +676,20 @@ simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, i
     pp.nT_cap = h->nT_cap;
     if (!h->W) {
       CUDA_TRY(h, cudaMalloc(&h->W, (size_t)h->K1 * h->n_pad * 2 * sizeof(double)));
+      CUDA_TRY(h, dev_alloc(&h->flowY, (size_t)h->n_pad));
+      CUDA_TRY(h, dev_alloc(&h->flow_tab, (size_t)h->n_cap + 1 + h->K1));
+      launch_flow_recip(h->flow_tab, h->n_cap + 1, h->st);
+      h->launches += 1;
+      std::vector<SweepScale> cp((size_t)h->K1);
+      for (int k = 0; k < h->K1; ++k) {
+        // C^(k+1) = r 2^-(63 + sh), 2^62 <= r < 2^63
+        int e = 0;
+        const double f = std::frexp(std::pow(C, k + 1), &e);
+        cp[k] = SweepScale{(unsigned long long)std::ldexp(f, 63), 0, -e};
+      }
+      CUDA_TRY(h, cudaMemcpyAsync(h->flow_tab + h->n_cap + 1, cp.data(),
+                                  cp.size() * sizeof(SweepScale), cudaMemcpyHostToDevice, h->st));
+      CUDA_TRY(h, cudaStreamSynchronize(h->st));
       CUDA_TRY(h, cudaMalloc(&h->rinv, (size_t)h->n_pad * 2 * sizeof(double)));
       CUDA_TRY(h, dev_alloc(&h->loff, (size_t)h->n_pad));
       CUDA_TRY(h, dev_alloc(&h->tile_nnz, (size_t)h->nT_cap));
@@ -681,8 +698,11 @@ simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, i
     pp.rinv = h->rinv;
     pp.loff = h->loff;
     pp.flat = h->cfg.prep_item == 0 ? 1 : 0;
+    pp.Y = h->flowY;
+    pp.recip = h->flow_tab;
+    pp.cpow = h->flow_tab + h->n_cap + 1;
     pp.tile_nnz = h->tile_nnz;
-    pp.bar = h->gbar + 2;
+    pp.bar = h->gbar;
     pp.limit = wait_limit(h);
     pp.counters = (unsigned long long*)h->counters;
     const int rc = launch_prep(pp, h->cfg.s_precision, h->cfg.vec_fp64 ? 1 : 0,
@@ -1431,7 +1451,7 @@ void free_ctx(simrank_ctx* h) {
                   h->dout.col,  h->d_in_w,   h->d_wsum,    h->S,          h->P64,
                   h->P32,       h->mXi,      h->mEta,      h->tiles,      h->ntiles,
                   h->sI,        h->sJ,       h->scal,      h->counters,   h->diffbits,
-                  h->gbar,      h->W,        h->rinv,       h->loff,     h->tile_nnz,  h->d_order,    h->d_order_row, h->d_jobs,
+                  h->gbar,      h->W,        h->rinv,       h->loff,     h->tile_nnz, h->flowY, h->flow_tab,  h->d_order,    h->d_order_row, h->d_jobs,
                   h->d_srcs,    h->d_ops,    h->d_cols,     h->d_ext2int, h->col_items,
                   h->col_gacc,  h->col_tcount};
   for (void* p : ptrs)
@@ -1726,14 +1746,14 @@ simrank_status simrank_init(const simrank_config* cfg_in, int32_t n, int64_t m, 
       dev_alloc(&h->ntiles, 1) != cudaSuccess || dev_alloc(&h->sI, (size_t)h->n_pad) != cudaSuccess ||
       dev_alloc(&h->sJ, (size_t)h->n_pad) != cudaSuccess || dev_alloc(&h->scal, 8) != cudaSuccess ||
       dev_alloc(&h->counters, CNT_N) != cudaSuccess || dev_alloc(&h->diffbits, 1) != cudaSuccess ||
-      dev_alloc(&h->gbar, 4) != cudaSuccess)
+      dev_alloc(&h->gbar, 8) != cudaSuccess)
     return bail(fail(h, SR_ERR_OOM, "cudaMalloc of work buffers failed"));
   cudaMemsetAsync(h->P64, 0, panel_elems * sizeof(double), h->st);
   if (h->P32) cudaMemsetAsync(h->P32, 0, panel_elems * sizeof(float), h->st);
   cudaMemsetAsync(h->mXi, 0, h->nT_cap * sizeof(uint64_t), h->st);
   cudaMemsetAsync(h->mEta, 0, h->nT_cap * sizeof(uint64_t), h->st);
   cudaMemsetAsync(h->counters, 0, CNT_N * sizeof(int64_t), h->st);
-  cudaMemsetAsync(h->gbar, 0, 4 * sizeof(unsigned int), h->st);
+  cudaMemsetAsync(h->gbar, 0, 8 * sizeof(unsigned int), h->st);
   cudaMemsetAsync(h->S, 0, s_bytes, h->st);
 
   if (h->column) {

@@ -11,37 +11,54 @@
 //            xi_{k+1} = C Q xi_k, eta_{k+1} = Q eta_k;
 //   phase 3  the affected-area mask words of every tile (Thm 4) and the list
 //            of affected tile pairs of the S pass.
-// Phases and steps are separated by a bounded grid barrier.
+// Phases are separated by a bounded grid barrier.
 //
-// Work split.  A gather of one scattered vector element per nonzero is bound
-// by the L1 throughput of the SM that issues it, and on GB300 the FP64 form
-// by the FP64 issue rate of the SM, so the nonzeros, not the rows, are spread
-// evenly.  Flat split (default): the in-lists of all rows, flattened in row
-// order, are cut into equal contiguous ranges, one per CTA, two nonzeros per
-// thread, located once per launch from the tile offsets and the in-tile row
-// offsets that phase 0 writes.  Item split (a set `item`, or too many
-// nonzeros for two per thread): every 128-row tile is cut into items of at
-// most `item` flattened nonzeros, and items go round-robin to the CTAs (a hub
-// row with thousands of in-neighbours spreads over many SMs); each CTA keeps
-// the row extents and column indices of its first items in shared memory for
-// all K steps.  Partial row sums are combined within a warp and added to the next
-// column with global atomics.  xi_k and eta_k are kept interleaved in the
-// working buffer W[k][a] (one 8- or 16-byte load per nonzero).  Row-wise work
-// (gamma; after the last step, the copy of the columns into the tile-blocked
-// panels that the S pass reads, with the masks) goes by tiles, round-robin.
+// Flow form (default).  The in-lists of all rows, flattened in row order, are
+// cut into equal contiguous ranges, one per CTA, one or two nonzeros per
+// thread, located once per launch.  Steps are not separated by barriers: a word
+// of W[k + 1] counts, in its upper bits, the parts of its row's sum that are
+// there, and a thread that gathers it reads it (from L2) until all are.  A step
+// then costs one reduction and one load through L2 instead of a reduction, a grid
+// barrier and a load.  At n = 20,000, m = 200,000 a step takes 2.6 us (with
+// barriers 4.8 in FP64, 2.9 in FP32), at n = 1,000, m = 8,000 1.7 us (2.95 and
+// 2.0): about half of it the L2 latency there and back, the rest the gather
+// (one 32-byte sector per nonzero and SM every other clock) and the sums.
+// Every CTA is co-resident and a value depends on earlier steps only, so the
+// waits end; they are bounded all the same.
+// The vectors are kept in 64-bit fixed point (xi without its factor C^(k+1),
+// in [0, 1], as value * 2^56; eta as value * 2^(56 - e), |eta| < 2^e from the
+// largest entry of the rows that gamma reads): row sums are exact, and the
+// division by the in-degree is a product with a 63-bit reciprocal.  GB300
+// issues FP64 (and conversions to and from 64-bit types) at 1/64 of the FP32
+// rate, which took 1.65 us of each step in FP64.  The absolute error is 2^-57 of
+// the largest entry a step, below the rounding of an FP64 S.
+// A row spread over the lanes of a warp is summed by shuffles, over the warps
+// of a CTA through shared memory, and the parts of a row cut by the CTA ranges
+// meet in its word by integer reductions.
+//
+// Item form (a set `item`, more than two nonzeros per thread, or an infinite or
+// NaN S).  Every 128-row tile is cut into items of at most `item` flattened
+// nonzeros, and items go round-robin to the CTAs (a hub row with thousands of
+// in-neighbours spreads over many SMs); each CTA keeps the row extents and
+// column indices of its first items in shared memory for all K steps.  Partial
+// row sums are combined within a warp and added to the next column with global
+// atomics, and a grid barrier ends each step.  The vectors and the arithmetic
+// are FP64 (vec64 = 1, or S in FP64) or FP32.
+//
+// In both forms xi_k and eta_k are interleaved in the working buffer W[k][a]
+// (one load per nonzero), and row-wise work (gamma; the copy of the columns into
+// the tile-blocked panels that the S pass reads, with the masks) goes by tiles,
+// round-robin.
 //
 // gamma needs w on the OLD graph; only row j of Q changes, so the kernel
 // gathers on the patched graph and corrects row j: the sum over the old
 // in-neighbours = the sum over the new ones - op * S_II.
 //
-// The vectors and the arithmetic are FP64 (vec64 = 1, or S in FP64) or FP32;
-// the panels the S pass reads have the precision of S, and lambda and row j
-// of gamma are always FP64.  The correction of the rows of S by pending
-// panels is summed in the precision of S (those panels are stored in it).
-// GB300 issues FP64 instructions at 1/64 of the FP32 rate, so the FP64 form
-// keeps per-row factors in shared memory, tests for zero on the integer pipe
-// and leaves the additions of the atomics to L2.  The atomic accumulation
-// makes the last bit of a result depend on the order of the additions.
+// The panels the S pass reads have the precision of S; gamma has that of the
+// vectors, its row j and lambda are always FP64.  The correction of the rows of S
+// by pending panels is summed in the precision of S (those panels are stored in
+// it).  The atomic accumulation of the item form makes the last bit of a result
+// depend on the order of the additions.
 #include <algorithm>
 
 #include "fx64.h"
@@ -498,45 +515,169 @@ __device__ __forceinline__ void pair_step_fx(const StepPair<double>& q, Gf gathe
   if ((q.fl & (1u << 7)) && (nz(tx) || nz(ty))) emit(q.kt, tx, ty);
 }
 
-// The flat split: CTA c takes the nonzeros [c E, (c + 1) E) of the in-lists of
-// all rows flattened in row order, E = ceil(nnz / CTAs), two per thread, so
-// every CTA gets the same number whatever the tiles hold.  Nonzero e is found
-// by its tile (tile offsets toff, shared) and its row in the tile (in-tile row
-// offsets loff, global); rows are keyed by their global index.
-__device__ __forceinline__ void flat_locate(const int* toff, int nT, const int* __restrict__ loff,
-                                            const DevAdj& in, int e, int& row, int& col) {
-  int lo = 0, hi = nT;  // the last tile T with toff[T] <= e
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (toff[mid] <= e) lo = mid; else hi = mid;
-  }
-  const int l = e - toff[lo];
-  const int* lt = loff + (int64_t)lo * PT;
-  int a = 0, b = PT;  // the last row of the tile with loff <= l
-  while (b - a > 1) {
-    const int mid = (a + b) >> 1;
-    if (__ldcg(lt + mid) <= l) a = mid; else b = mid;
-  }
-  row = lo * PT + a;
-  col = __ldcg(in.col + __ldcg(in.start + row) + (l - __ldcg(lt + a)));
+// ---- flow form
+
+struct I2 {
+  long long x, y;
+};
+// A word of W[k] is n 2^58 + v once n parts with the sum v, |v| < 2^57, are there.
+constexpr int FLOW_CNT = 58;
+constexpr int FLOW_CTA = 256;   // nonzeros per CTA while co-resident CTAs are left
+constexpr int FLOW_PARTS = 60;  // parts a row may have (of the 6-bit count)
+
+__device__ __forceinline__ I2 ld_flow(const I2* p) {
+  I2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p)
+               : "memory");
+  return v;
+}
+// A first look, which may be served by L1 (other warps of the CTA gather the same
+// entries): a line fetched too early shows too few parts and is read again from
+// L2.  Nothing older than the zeros of this launch can be there: the grid
+// barrier after them ordered them before every later read.
+__device__ __forceinline__ I2 look_flow(const I2* p) {
+  I2 v;
+  asm volatile("ld.relaxed.cta.global.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p)
+               : "memory");
+  return v;
+}
+// A row's sum, or one part of it, into its word.  A reduction also where a store
+// would do: it reached the readers 0.25 us sooner (a step 2.9 -> 2.6 us).
+__device__ __forceinline__ void put_flow(I2* p, const I2& v) {
+  constexpr long long one = 1ll << FLOW_CNT;
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(&p->x), "l"(v.x + one) : "memory");
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(&p->y), "l"(v.y + one) : "memory");
+}
+// Whether both words hold all n parts (the count is in the upper half's top bits)
+__device__ __forceinline__ bool flow_there(const I2& v, int n) {
+  constexpr int half = 1 << (FLOW_CNT - 33);
+  return (((int)(v.x >> 32) + half) >> (FLOW_CNT - 32)) == n &&
+         (((int)(v.y >> 32) + half) >> (FLOW_CNT - 32)) == n;
 }
 
+// v * 2^(56 - e) rounded to nearest, |v| < 2^e, on the integer pipe
+__device__ __forceinline__ long long flow_fix(uint64_t m, int sh, bool neg) {
+  long long f = 0;
+  if (sh >= 0)
+    f = (long long)(m << sh);
+  else if (sh > -60)
+    f = (long long)((m + (1ull << (-sh - 1))) >> -sh);
+  return neg ? -f : f;
+}
+__device__ __forceinline__ long long flow_of(float v, int e) {
+  const uint32_t b = __float_as_uint(v);
+  const int x = (int)((b >> 23) & 0xffu);
+  const uint32_t m = x ? (b & 0x7fffffu) | 0x800000u : b & 0x7fffffu;
+  return flow_fix(m, max(x, 1) - 150 + 56 - e, (b >> 31) != 0);
+}
+__device__ __forceinline__ long long flow_of(double v, int e) {
+  const uint64_t b = (uint64_t)__double_as_longlong(v);
+  const int x = (int)((b >> 52) & 0x7ffu);
+  const uint64_t m = x ? (b & 0xfffffffffffffull) | 0x10000000000000ull : b & 0xfffffffffffffull;
+  return flow_fix(m, max(x, 1) - 1075 + 56 - e, (b >> 63) != 0);
+}
+// out of line: instructions that a launch runs once are bound by their fetch
+__device__ __noinline__ double flow_value_slow(long long v, int e) { return ldexp((double)v, e); }
+
+// v * 2^e rounded to nearest even
+template <typename T>
+__device__ __forceinline__ T flow_value(long long v, int e) {
+  if (v == 0) return T(0);
+  const uint64_t a = v < 0 ? (uint64_t)-v : (uint64_t)v;
+  const int lz = __clzll((long long)a);
+  const int x = 63 - lz + e;  // 2^x <= |v| 2^e
+  constexpr bool F = sizeof(T) == 4;
+  if (x < (F ? -126 : -1022) || x > (F ? 126 : 1022)) return (T)flow_value_slow(v, e);
+  const uint64_t m = a << lz;
+  constexpr int DROP = F ? 40 : 11;
+  const uint64_t rem = m & ((1ull << DROP) - 1), half = 1ull << (DROP - 1);
+  uint64_t q = m >> DROP;  // leading one included
+  q += (rem > half || (rem == half && (q & 1))) ? 1 : 0;
+  // adding the significand with its leading one carries into the exponent
+  if constexpr (F)
+    return __uint_as_float((((uint32_t)(x + 126) << 23) + (uint32_t)q) |
+                           (v < 0 ? 0x80000000u : 0u));
+  else
+    return __longlong_as_double((long long)((((uint64_t)(x + 1022) << 52) + q) |
+                                            (v < 0 ? 0x8000000000000000ull : 0ull)));
+}
+
+// A sum of values of one row held by a warp times 1 / d, rounded to nearest
+__device__ __forceinline__ long long flow_scale(long long s, const SweepScale& f) {
+  const long long t = __mul64hi(s << f.h, (long long)f.r);
+  return (t + (1ll << (f.sh - 1))) >> f.sh;
+}
+
+// x / per for 0 <= x < 2^24 (inv = 1 / per)
+__device__ __forceinline__ int flow_div(int x, int per, float inv) {
+  int q = (int)((float)x * inv);
+  if (q * per > x) --q;
+  if ((q + 1) * per <= x) ++q;
+  return q;
+}
+
+// The number of parts of row a's sums: the CTAs whose ranges hold some of its
+// nonzeros (0: a row without in-neighbours, its sums are zero).
+__device__ __forceinline__ int flow_parts(int a, const int* ioff, const int* __restrict__ loff,
+                                          const DevAdj& in, int per, float inv) {
+  const int rs = ioff[a / PT] + __ldcg(loff + a), len = __ldcg(in.len + a);
+  return len > 0 ? flow_div(rs + len - 1, per, inv) - flow_div(rs, per, inv) + 1 : 0;
+}
+
+// v without its count
+__device__ __forceinline__ void flow_strip(I2& v, int n) {
+  const long long c = (long long)n << FLOW_CNT;
+  v.x -= c;
+  v.y -= c;
+}
+
+// Adds up the runs of lanes sharing a row: head sums to the first lane of their
+// run, a tail into the next lane's head when that holds the same row.  At most
+// 65 values below 2^56 each.
 template <typename V>
-__device__ __forceinline__ StepPair<V> flat_setup(const int* toff, int nT, const int* loff,
-                                                  const DevAdj& in, int e0, int e1) {
-  StepPair<V> q;
-  q.ca = q.cb = q.kh = q.kt = -1;
-  const int e = e0 + 2 * (int)threadIdx.x;
-  if (e < e1) {
-    flat_locate(toff, nT, loff, in, e, q.kh, q.ca);
-    if (e + 1 < e1) {
-      int r2;
-      flat_locate(toff, nT, loff, in, e + 1, r2, q.cb);
-      if (r2 != q.kh) q.kt = r2;
+__device__ __forceinline__ void flow_sum(const StepPair<V>& q, I2& h, const I2& t) {
+  constexpr unsigned full = 0xffffffffu;
+#pragma unroll
+  for (int b = 0; b < 5; ++b) {
+    if ((1 << b) >= q.span) break;
+    const long long x = __shfl_down_sync(full, h.x, 1 << b);
+    const long long y = __shfl_down_sync(full, h.y, 1 << b);
+    if (q.fl & (1u << b)) {
+      h.x += x;
+      h.y += y;
     }
   }
-  pair_pattern(q);
-  return q;
+  const long long x = __shfl_up_sync(full, t.x, 1), y = __shfl_up_sync(full, t.y, 1);
+  if (q.fl & (1u << 5)) {
+    h.x += x;
+    h.y += y;
+  }
+}
+
+// |v| as an FP32 value not below it
+__device__ __forceinline__ float up_abs(float v) { return fabsf(v); }
+__device__ __forceinline__ float up_abs(double v) { return __double2float_ru(fabs(v)); }
+
+// out[d] = 1 / d, r = 2^(62 + L) / d rounded to nearest with 2^(L-1) < d <= 2^L;
+// d <= 64: sums of d values below 2^56 may be shifted left by h = 6 - L
+__global__ void k_flow_recip(SweepScale* __restrict__ out, int count) {
+  const int d = blockIdx.x * blockDim.x + threadIdx.x;
+  if (d >= count) return;
+  SweepScale f{0ull, 0, 1};
+  if (d > 0) {
+    const int L = d > 1 ? 32 - __clz(d - 1) : 0;
+    const unsigned long long u = (unsigned long long)d;
+    if (L == 0) {
+      f.r = 1ull << 62;
+    } else {
+      const unsigned long long q0 = (1ull << 63) / u, r0 = (1ull << 63) % u;
+      const unsigned long long m = r0 << (L - 1);
+      f.r = (q0 << (L - 1)) + m / u + (2ull * (m % u) >= u ? 1ull : 0ull);
+    }
+    f.h = max(0, 6 - L);
+    f.sh = (L - 1) + f.h - 1;  // 1 / d = r 2^-(63 + L - 1)
+  }
+  out[d] = f;
 }
 
 __device__ void prep_patch(const PatchOp* __restrict__ ops, int64_t begin, int64_t end,
@@ -570,7 +711,10 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ V red[4][2][PT];
   __shared__ V rrc[PT], rri[PT];  // C / in-degree and 1 / in-degree of the rows of item 0
-  __shared__ V2<V> fsh[PG][2];      // flat split: the same for each thread's head / tail row
+  __shared__ SweepScale fsh[PG][2];  // flow form: 1 / in-degree of each thread's head / tail row
+  __shared__ int rowmap[2 * PG];     // flow form: the row of each of the CTA's nonzeros
+  __shared__ I2 dep[2][PG / 32];     // flow form: a warp's part of the row before it
+  __shared__ unsigned smax[3][PT / 32];
   __shared__ unsigned long long mk[PREP_MT][2];
   __shared__ int wsum[PG / 32];
   __shared__ int s_ok, s_div;
@@ -607,13 +751,20 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     if (p.op_end > p.op_begin) prep_patch(p.ops, p.op_begin, p.op_end, p.in, p.out);
     if (tid == 0 && p.tiles) *p.ntiles = 0;
   }
+  // W starts at zero in both forms
+  I2* F = static_cast<I2*>(p.W);
   {
-    // W[0 .. K] over all n_pad rows, 16 bytes per store (n_pad is a multiple of 128)
     uint4* w16 = reinterpret_cast<uint4*>(W);
-    const int64_t total = (int64_t)(K + 1) * p.n_pad * (int64_t)sizeof(V2<V>) / 16;
+    const int64_t total =
+        (int64_t)(K + 1) * p.n_pad * (p.flat ? 16 : (int64_t)sizeof(V2<V>)) / 16;
     for (int64_t e = (int64_t)blockIdx.x * PG + tid; e < total; e += (int64_t)G * PG)
       w16[e] = make_uint4(0u, 0u, 0u, 0u);
   }
+  if (p.flat)
+    for (int a = (int)blockIdx.x * PG + tid; a < p.n_pad; a += G * PG) p.Y[a] = 0;
+  int mxL = 0;                 // longest row of this thread
+  float mxI = 0.f, mxJ = 0.f;  // largest |sI|, |sJ| of the rows of this thread
+  bool bad = false;            // one of them is infinite or NaN
   if (np > 0) {
     // c_x[q] = sum_t xi_q[I_t], c_e[q] = sum_t eta_q[I_t]; the same at j
     for (int q = tid; q < np; q += PG) {
@@ -666,8 +817,17 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     if (lane == 31) wsum[warp] = incl;
     __syncthreads();
     if (tid < PT) {
-      sI[a] = (red[0][0][r] + red[1][0][r]) + (red[2][0][r] + red[3][0][r]);
-      sJ[a] = (red[0][1][r] + red[1][1][r]) + (red[2][1][r] + red[3][1][r]);
+      const V vi = (red[0][0][r] + red[1][0][r]) + (red[2][0][r] + red[3][0][r]);
+      const V vj = (red[0][1][r] + red[1][1][r]) + (red[2][1][r] + red[3][1][r]);
+      sI[a] = vi;
+      sJ[a] = vj;
+      if (p.flat) {
+        const float fi = up_abs(vi), fj = up_abs(vj);
+        bad |= !(fi <= 3.0e38f) || !(fj <= 3.0e38f);
+        mxI = fmaxf(mxI, fi);
+        mxJ = fmaxf(mxJ, fj);
+        mxL = max(mxL, L);
+      }
       int base = 0;
       for (int w = 0; w < warp; ++w) base += wsum[w];
       p.loff[a] = base + incl - L;  // nonzeros of the tile before row a
@@ -675,17 +835,52 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     if (tid == 0) p.tile_nnz[T] = (wsum[0] + wsum[1]) + (wsum[2] + wsum[3]);
     __syncthreads();
   }
+  if (p.flat) {
+    // non-negative floats order like their bits; an infinite or NaN entry puts
+    // the bits of infinity there
+    if (tid < PT) {
+      const unsigned bi = bad ? 0x7f800000u : __float_as_uint(mxI);
+      const unsigned wi = __reduce_max_sync(0xffffffffu, bi);
+      const unsigned wj = __reduce_max_sync(0xffffffffu, __float_as_uint(mxJ));
+      const unsigned wl = __reduce_max_sync(0xffffffffu, (unsigned)mxL);
+      if (lane == 0) {
+        smax[0][warp] = wi;
+        smax[1][warp] = wj;
+        smax[2][warp] = wl;
+      }
+    }
+    __syncthreads();
+    if (tid < 3) {
+      const unsigned m =
+          max(max(smax[tid][0], smax[tid][1]), max(smax[tid][2], smax[tid][3]));
+      if (m > 0u) atomicMax(p.bar + 2 + tid, m);
+    }
+  }
   alive = prep_barrier(p.bar, ++nb * G, p.limit, &s_ok);
 
   // ---- phase 1: the split of the nonzeros over the CTAs; w = Q sI summed by
   // atomics into W[0].x
   int my_items = 0;
-  bool flat = false;
+  bool flow = false;
   StepPair<V> q0;
+  int eI = 0, eG = 0;  // |sI| < 2^eI, |gamma| < 2^eG (flow form)
+  bool finite = true;
+  if (alive && p.flat) {
+    const float mI = __uint_as_float(__ldcg(p.bar + 2)), mJ = __uint_as_float(__ldcg(p.bar + 3));
+    // bounds of Thm 3 / Thm 9 / Table 2 with |w_j|, |S_II| / delta^2 <= max |sI| / delta
+    const float invC = (float)p.inv_C, gq = fabsf((float)p.gq), m1 = mI * (float)p.inv_delta;
+    const float lam = 3.f * m1 + mJ * invC + invC + 1.f;
+    const float g = fmaxf(2.f * m1, gq * (m1 + mJ * invC + 0.5f * gq * lam + invC + 1.f)) * 1.01f;
+    finite = mI <= 3.0e38f && mJ <= 3.0e38f && g <= 3.0e38f;
+    if (finite) {
+      eI = mI > 0.f ? ilogbf(mI) + 1 : 0;
+      eG = g > 0.f ? ilogbf(g) + 1 : 0;
+    }
+  }
   if (alive) {
-    // ioff[T] = the units of the tiles before T: their nonzeros (flat split,
+    // ioff[T] = the units of the tiles before T: their nonzeros (flow form,
     // tried first when allowed) or their items of at most `item` nonzeros
-    for (int pass = p.flat ? 0 : 1; pass < 2; ++pass) {
+    for (int pass = p.flat && finite ? 0 : 1; pass < 2; ++pass) {
       const int div = pass == 0 ? 1 : p.item;
       const int per = (nT + PG - 1) / PG;
       const int t0 = min(nT, tid * per), t1 = min(nT, t0 + per);
@@ -716,7 +911,10 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
           // the CTA's share, by one thread (a division would be issued by
           // every thread): nonzeros per CTA (flat pass) or this CTA's items
           const int b = (int)blockIdx.x;
-          s_div = pass == 0 ? (w + G - 1) / G : (w > b ? (w - b + G - 1) / G : 0);
+          // (so many that no row has more than FLOW_PARTS parts)
+          s_div = pass == 0 ? max((w + G - 1) / G,
+                                  ((int)__ldcg(p.bar + 4) + FLOW_PARTS - 2) / (FLOW_PARTS - 1))
+                            : (w > b ? (w - b + G - 1) / G : 0);
         }
       }
       __syncthreads();
@@ -729,21 +927,117 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
       __syncthreads();
       if (pass == 0) {
         // every CTA computes the same nnz, so the choice is uniform over the grid
-        const int nnz = ioff[nT];
-        const int per_cta = (nnz + G - 1) / G;
-        if (per_cta <= 2 * PG) {
-          flat = true;
-          const int e0 = min(nnz, (int)blockIdx.x * per_cta), e1 = min(nnz, e0 + per_cta);
-          q0 = flat_setup<V>(ioff, nT, p.loff, p.in, e0, e1);
+        if (s_div <= 2 * PG) {
+          flow = true;
           break;
         }
         __syncthreads();  // ioff is rewritten by the item pass
       }
     }
   }
-  if (alive && flat) {
-    pair_step<V>(q0, [&](int b) { return V2<V>{sI[b], V(0)}; },
-                 [&](int r, V a, V) { red_add(&W[r].x, a); });
+  // ---- flow form: the CTA's nonzeros [e0, e1), two per thread
+  const int per = flow ? max(1, s_div) : 1;
+  const float inv_per = 1.f / (float)per;
+  int na = 0, nb2 = 0;        // parts of the columns of the thread's nonzeros
+  int wait_w = 0;             // > 0: the emitted run goes on in that many warps more
+  bool wait_tail = false;     // it is the tail's (else the head's)
+  bool give = false;          // the head sum is the part of a row of an earlier warp
+  if (alive && flow) {
+    const int nnz = ioff[nT];
+    const int e0 = min(nnz, (int)blockIdx.x * per), e1 = min(nnz, e0 + per), cnt = e1 - e0;
+    const int E = per <= PG ? 1 : 2;  // nonzeros per thread
+    rowmap[tid] = -1;
+    rowmap[PG + tid] = -1;
+    __syncthreads();
+    if (cnt > 0) {
+      int T0 = 0, T1 = 0;  // the tiles of e0 and of e1 - 1
+      for (int hi = nT; hi - T0 > 1;) {
+        const int mid = (T0 + hi) >> 1;
+        if (ioff[mid] <= e0) T0 = mid; else hi = mid;
+      }
+      T1 = T0;
+      for (int hi = nT; hi - T1 > 1;) {
+        const int mid = (T1 + hi) >> 1;
+        if (ioff[mid] <= e1 - 1) T1 = mid; else hi = mid;
+      }
+      for (int a = T0 * PT + tid; a < (T1 + 1) * PT; a += PG) {
+        const int rs = ioff[a / PT] + __ldcg(p.loff + a), len = __ldcg(p.in.len + a);
+        if (len > 0 && rs < e1 && rs + len > e0) rowmap[max(rs, e0) - e0] = a;
+      }
+    }
+    __syncthreads();
+    // each position's row: the last one that starts at it or before
+    const int pos = E * tid;
+    const int v0 = rowmap[pos], v1 = E == 2 ? max(v0, rowmap[pos + 1]) : v0;
+    int incl = v1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl = max(incl, y);
+    }
+    int before = __shfl_up_sync(0xffffffffu, incl, 1);
+    if (lane == 0) before = -1;
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) before = max(before, wsum[w]);
+    const int ra = max(before, v0), rb = max(before, v1);
+    rowmap[pos] = ra;
+    if (E == 2) rowmap[pos + 1] = rb;
+    q0.ca = q0.cb = q0.kh = q0.kt = -1;
+    int rsh = 0, rst = 0;
+    if (pos < cnt) {
+      q0.kh = ra;
+      rsh = ioff[ra / PT] + __ldcg(p.loff + ra);
+      q0.ca = __ldcg(p.in.col + __ldcg(p.in.start + ra) + (e0 + pos - rsh));
+    }
+    if (E == 2 && pos + 1 < cnt) {
+      if (rb != ra) {
+        q0.kt = rb;
+        rst = ioff[rb / PT] + __ldcg(p.loff + rb);
+      }
+      q0.cb = __ldcg(p.in.col + __ldcg(p.in.start + rb) +
+                     (e0 + pos + 1 - (rb != ra ? rst : rsh)));
+    }
+    pair_pattern(q0);
+    __syncthreads();  // rowmap
+    const int w0 = 32 * E * warp, w1 = min(cnt, w0 + 32 * E);  // the warp's positions
+    if (w0 < cnt) {
+      const int rf = rowmap[w0], rl = rowmap[w1 - 1];
+      const bool from = w0 > 0 && rowmap[w0 - 1] == rf;
+      give = from && lane == 0;
+      if (w1 < cnt && rowmap[w1] == rl && !(from && rf == rl)) {
+        // the run of rl ends this warp and goes on: whoever emits it waits
+        const bool mine_h = (q0.fl & (1u << 6)) && q0.kh == rl;
+        const bool mine_t = (q0.fl & (1u << 7)) && q0.kt == rl;
+        if (mine_h || mine_t) {
+          wait_tail = mine_t;
+          for (int x = w1; x < cnt && rowmap[x] == rl; x += 32 * E) ++wait_w;
+        }
+      }
+    }
+    fsh[tid][0] = fsh[tid][1] = SweepScale{0ull, 0, 1};
+    if (q0.kh >= 0) {
+      const int len = __ldcg(p.in.len + q0.kh);
+      fsh[tid][0] = p.recip[len];
+    }
+    if (q0.kt >= 0) {
+      const int len = __ldcg(p.in.len + q0.kt);
+      fsh[tid][1] = p.recip[len];
+    }
+    if (q0.ca >= 0) na = flow_parts(q0.ca, ioff, p.loff, p.in, per, inv_per);
+    if (q0.cb >= 0) nb2 = flow_parts(q0.cb, ioff, p.loff, p.in, per, inv_per);
+    // w = Q sI: the parts of each row's mean, in units of 2^(eI - 56), into Y
+    I2 h{0, 0}, t{0, 0};
+    if (q0.ca >= 0) h.x = flow_of(sI[q0.ca], eI);
+    if (q0.cb >= 0) {
+      const long long v = flow_of(sI[q0.cb], eI);
+      if (q0.kt >= 0) t.x = v; else h.x += v;
+    }
+    flow_sum(q0, h, t);
+    if (q0.fl & (1u << 6))
+      atomicAdd((unsigned long long*)p.Y + q0.kh, (unsigned long long)flow_scale(h.x, fsh[tid][0]));
+    if (q0.fl & (1u << 7))
+      atomicAdd((unsigned long long*)p.Y + q0.kt, (unsigned long long)flow_scale(t.x, fsh[tid][1]));
     alive = prep_barrier(p.bar, ++nb * G, p.limit, &s_ok);
   } else if (alive) {
     my_items = s_div;
@@ -790,38 +1084,30 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
         const int64_t a = (int64_t)T * PT + tid;
         const int len = __ldcg(p.in.len + a);
         // the factors of row a of Q on the new graph, for every step below
-        const V inv = len > 0 ? V(1) / (V)len : V(0);
-        const V y = __ldcg(&W[a].x);
-        const double dl = (double)p.delta;
+        const V inv = len > 0 && !flow ? V(1) / (V)len : V(0);
+        // sum (item form) or mean (flow form) of sI over the new in-neighbours
+        const V y = flow ? flow_value<V>(__ldcg(p.Y + a), eI - 56) : __ldcg(&W[a].x);
         V g;
         if (a == p.j) {
           // row j: lambda (Eq. 29b) and w_j on the old row j, in FP64
           double S_II = 0.0;
           for (int u = 0; u < p.delta; ++u) S_II += (double)__ldcg(sI + p.I[u]);
           const double S_jj = (double)__ldcg(sJ + p.j);
-          const double C = p.C;
-          const double wj =
-              (p.d_j > 0) ? ((double)y - (double)p.op * S_II) / (dl * (double)p.d_j) : 0.0;
-          const double lam = S_II / (dl * dl) + S_jj / C - 2.0 * wj - 1.0 / C + 1.0;
+          const double ys =
+              flow ? flow_value<double>(__ldcg(p.Y + a), eI - 56) * (double)len : (double)y;
+          const double wj = (ys - (double)p.op * S_II) * p.inv_ddj;  // 0 when d_j = 0
+          const double id = p.inv_delta, iC = p.inv_C;
+          const double lam = S_II * id * id + S_jj * iC - 2.0 * wj - iC + 1.0;
+          // gq = delta / (d_j + op delta)
+          const double gj = p.gq * (wj - S_jj * iC + iC - 1.0), gl = 0.5 * p.gq * p.gq * lam;
           double gd;
-          if (p.op > 0) {
-            if (p.d_j == 0) {
-              gd = wj + S_II / (2.0 * dl * dl);
-            } else {
-              const double dd = (double)p.d_j + dl;
-              gd = (dl / dd) * (wj - S_jj / C + lam * dl / (2.0 * dd) + 1.0 / C - 1.0);
-            }
-          } else {
-            if (p.d_j == p.delta) {
-              gd = -wj + S_II / (2.0 * dl * dl);
-            } else {
-              const double dd = (double)p.d_j - dl;
-              gd = (dl / dd) * (S_jj / C - wj + lam * dl / (2.0 * dd) - 1.0 / C + 1.0);
-            }
-          }
+          if (p.op > 0)
+            gd = p.d_j == 0 ? wj + 0.5 * S_II * id * id : gj + gl;
+          else
+            gd = p.d_j == p.delta ? -wj + 0.5 * S_II * id * id : gl - gj;
           g = (V)gd;
         } else {
-          const V w = y * inv * (V)p.inv_delta;
+          const V w = flow ? y * (V)p.inv_delta : y * inv * (V)p.inv_delta;
           const V sJa = __ldcg(sJ + a);
           const V sc = sJa * (V)p.inv_C;
           if (p.op > 0) {
@@ -831,8 +1117,12 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
           }
         }
         const V x0 = (a == p.j) ? Cv : V(0);
-        W[a] = V2<V>{x0, g};
-        rinv[a] = V2<V>{Cv * inv, inv};
+        if (flow) {
+          put_flow(F + a, I2{a == p.j ? 1ll << 56 : 0ll, flow_of(g, eG)});
+        } else {
+          W[a] = V2<V>{x0, g};
+          rinv[a] = V2<V>{Cv * inv, inv};
+        }
         P[pidx(a, 0, koff)] = (TS)x0;
         P[pidx(a, 1, koff)] = (TS)g;
         pe = nz(g);
@@ -843,18 +1133,13 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
         mk[t][1] = any_e ? 1ull : 0ull;
       }
     }
-    if (K > 0) alive = prep_barrier(p.bar, ++nb * G, p.limit, &s_ok);
+    if (K > 0 && !flow) alive = prep_barrier(p.bar, ++nb * G, p.limit, &s_ok);
   }
 
   // ---- phase 2: K steps
   // the CTA's first item takes the fixed per-thread form when it can
-  const bool pair0 = !flat && my_items > 0 && items[0].e1 - items[0].e0 <= 2 * PG;
+  const bool pair0 = !flow && my_items > 0 && items[0].e1 - items[0].e0 <= 2 * PG;
   int64_t rb0 = 0;
-  if (flat) {
-    // flat split: the factors of each thread's head and tail rows
-    fsh[tid][0] = q0.kh >= 0 ? ld_v2cg(rinv + q0.kh) : V2<V>{V(0), V(0)};
-    fsh[tid][1] = q0.kt >= 0 ? ld_v2cg(rinv + q0.kt) : V2<V>{V(0), V(0)};
-  }
   if (pair0) {
     q0 = pair_setup<V>(items[0], cc, p.in.col);
     rb0 = (int64_t)items[0].T * PT;
@@ -865,14 +1150,84 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     }
     __syncthreads();
   }
-  for (int k = 0; alive && k < K; ++k) {
+  // Waits of the flow form: a warp reads its entries of W[k] again until all of
+  // them hold their parts (together: lanes that waited on their own would read
+  // one after the other).  Bounded: a wait that runs out sets the status word,
+  // and one that sees it set gives up as well (the steps then stop in the whole
+  // CTA).  True to go on waiting.
+  bool stop = false;
+  auto flow_again = [&](bool there, long long& it) -> bool {
+    if (__all_sync(0xffffffffu, there)) return false;
+    ++it;
+    bool out = it > p.limit;
+    if ((it & 255) == 0)
+      out |= __any_sync(0xffffffffu,
+                        *(volatile unsigned long long*)(p.counters + CNT_STATUS) != 0ull);
+    if (out) {
+      if (lane == 0)
+        atomicExch(&p.counters[CNT_STATUS], (unsigned long long)SR_ERR_TIMEOUT);
+      stop = true;
+    }
+    return !out;
+  };
+  if (alive && flow) {
+    for (int k = 0; k < K; ++k) {
+      const I2* Fk = F + (int64_t)k * p.n_pad;
+      I2* Fn = F + (int64_t)(k + 1) * p.n_pad;
+      I2 h{0, 0}, t{0, 0}, u{0, 0};
+      // both loads are on their way before the first is looked at; W[0] is
+      // written row by row, in one part
+      const int ma = k ? na : 1, mb = k ? nb2 : 1;
+      if (q0.ca >= 0) h = look_flow(Fk + q0.ca);
+      if (q0.cb >= 0) u = look_flow(Fk + q0.cb);
+      for (long long it = 0;;) {
+        const bool wa = q0.ca >= 0 && !flow_there(h, ma), wb = q0.cb >= 0 && !flow_there(u, mb);
+        if (!flow_again(!(wa || wb), it)) break;
+        if (wa) h = ld_flow(Fk + q0.ca);
+        if (wb) u = ld_flow(Fk + q0.cb);
+      }
+      if (q0.ca >= 0) flow_strip(h, ma);
+      if (q0.cb >= 0) flow_strip(u, mb);
+      if (q0.kt >= 0) {
+        t = u;
+      } else {
+        h.x += u.x;
+        h.y += u.y;
+      }
+      flow_sum(q0, h, t);
+      if (q0.fl & (1u << 6)) {
+        const SweepScale f = fsh[tid][0];
+        h.x = flow_scale(h.x, f);
+        h.y = flow_scale(h.y, f);
+        if (give)
+          dep[k & 1][warp] = h;
+        else if (wait_w == 0 || wait_tail)
+          put_flow(Fn + q0.kh, h);
+      }
+      if (q0.fl & (1u << 7)) {
+        const SweepScale f = fsh[tid][1];
+        t.x = flow_scale(t.x, f);
+        t.y = flow_scale(t.y, f);
+        if (!wait_tail) put_flow(Fn + q0.kt, t);
+      }
+      if (__syncthreads_or(stop)) {
+        alive = false;  // on every thread of the CTA
+        break;
+      }
+      if (wait_w) {
+        if (wait_tail) h = t;
+#pragma unroll 4
+        for (int x = 1; x <= wait_w; ++x) {
+          h.x += dep[k & 1][warp + x].x;
+          h.y += dep[k & 1][warp + x].y;
+        }
+        put_flow(Fn + (wait_tail ? q0.kt : q0.kh), h);
+      }
+    }
+  }
+  for (int k = 0; alive && !flow && k < K; ++k) {
     const V2<V>* Wk = W + (int64_t)k * p.n_pad;
     V2<V>* Wn = W + (int64_t)(k + 1) * p.n_pad;
-    if (flat)
-      pair_step<V>(q0, [&](int b) { return ld_v2(Wk + b); }, [&](int r, V a, V b) {
-        const V2<V> f = fsh[tid][r == q0.kh ? 0 : 1];
-        red_add2(Wn + r, a * f.x, b * f.y);
-      });
     for (int u = 0; u < my_items; ++u) {
       if (u == 0 && pair0) {
         pair_step<V>(q0, [&](int b) { return ld_v2(Wk + b); },
@@ -898,17 +1253,47 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     for (int t = 0; t < mt; ++t) {
       const int T = blockIdx.x + t * G;
       if (T >= nT) break;
+      int parts[PT / 32];
+#pragma unroll
+      for (int q = 0; q < PT / 32; ++q)
+        parts[q] =
+            flow ? flow_parts(T * PT + q * 32 + lane, ioff, p.loff, p.in, per, inv_per) : 0;
       // warp w copies columns k = 1 + w, 1 + w + 16, ...
       for (int k = 1 + warp; k <= K; k += PG / 32) {
         const V2<V>* Wk = W + (int64_t)k * p.n_pad;
+        const I2* Fk = F + (int64_t)k * p.n_pad + T * PT + lane;
+        const SweepScale ck = flow ? p.cpow[k] : SweepScale{0ull, 0, 0};
+        I2 look[PT / 32];
+#pragma unroll
+        for (int q = 0; q < PT / 32; ++q) look[q] = flow ? ld_flow(Fk + q * 32) : I2{0, 0};
+        if (flow)
+          for (long long it = 0;;) {
+            bool w = false;
+#pragma unroll
+            for (int q = 0; q < PT / 32; ++q) w |= !flow_there(look[q], parts[q]);
+            if (!flow_again(!w, it)) break;
+#pragma unroll
+            for (int q = 0; q < PT / 32; ++q)
+              if (!flow_there(look[q], parts[q])) look[q] = ld_flow(Fk + q * 32);
+          }
         bool nx = false, ne = false;
 #pragma unroll
         for (int q = 0; q < PT / 32; ++q) {
           const int64_t a = (int64_t)T * PT + q * 32 + lane;
-          const V2<V> v = ld_v2(Wk + a);
           // the mask bits follow the stored panel values (a value that rounds
           // to zero in the precision of S adds nothing to S)
-          const TS px = (TS)v.x, pe = (TS)v.y;
+          TS px, pe;
+          if (flow) {
+            // xi_k = C^(k+1) x 2^-56, C^(k+1) = r 2^-(63 + s)
+            I2 v = look[q];
+            flow_strip(v, parts[q]);
+            px = flow_value<TS>(__mul64hi(v.x << 6, (long long)ck.r), -61 - ck.sh);
+            pe = flow_value<TS>(v.y, eG - 56);
+          } else {
+            const V2<V> v = ld_v2(Wk + a);
+            px = (TS)v.x;
+            pe = (TS)v.y;
+          }
           P[pidx(a, 0, koff + k)] = px;
           P[pidx(a, 1, koff + k)] = pe;
           nx |= nz(px);
@@ -977,6 +1362,9 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     if (e == (unsigned int)G) {
       atomicExch(p.bar, 0u);
       atomicExch(p.bar + 1, 0u);
+      atomicExch(p.bar + 2, 0u);
+      atomicExch(p.bar + 3, 0u);
+      atomicExch(p.bar + 4, 0u);
     }
   }
 }
@@ -988,6 +1376,10 @@ size_t prep_smem(int cap, int nT_cap, int npend_max) {
 }
 
 }  // namespace
+
+void launch_flow_recip(SweepScale* out, int count, cudaStream_t st) {
+  k_flow_recip<<<(count + 255) / 256, 256, 0, st>>>(out, count);
+}
 
 int launch_prep(const PrepParams& prm, int s_prec, int vec64, int npend_max, int num_sms,
                 int max_ctas, int64_t nnz_bound, cudaStream_t st) {
@@ -1010,7 +1402,7 @@ int launch_prep(const PrepParams& prm, int s_prec, int vec64, int npend_max, int
   const int full = per_sm * num_sms;
   int grid = full;
   const int item = prm.item > 0 ? prm.item : 1024;
-  grid = (int)std::min<int64_t>((int64_t)prm.nT + nnz_bound / item + 1, full);
+  grid = (int)std::min<int64_t>((int64_t)prm.nT + nnz_bound / (prm.item > 0 ? item : FLOW_CTA) + 1, full);
   if (max_ctas > 0) grid = std::min(grid, max_ctas);
   grid = std::max(grid, 1);
   if ((prm.nT + grid - 1) / grid > PREP_MT) return 2;

@@ -129,6 +129,14 @@ void launch_patch(const PatchOp* ops, int64_t begin, int64_t end, DevAdj in, Dev
 void launch_chain_step(const DevAdj& in, int k, double C, int nT, int K1, double* P64, float* P32,
                        uint64_t* mXi, uint64_t* mEta, cudaStream_t st);
 
+// The factor C / d of a row of d nonzeros, r * 2^-(63 + s) with 2^62 <= r < 2^63.
+// d <= 32: a row sum shifted left by h stays below 2^63, and the high word of
+// its product with r is shifted right by sh = s + h - 1 (at least 3); longer
+// rows: sh = s - 1 (at least 4).
+struct SweepScale {
+  unsigned long long r;
+  int h, sh;
+};
 // Everything a rank-one update does before its S pass, in one cooperative
 // launch (k_prep.cu): patch ops [op_begin, op_end), the rows sI, sJ of the
 // current S (panel terms [0, npend) of P not yet in S are added in), gamma
@@ -138,9 +146,9 @@ void launch_chain_step(const DevAdj& in, int k, double C, int nT, int K1, double
 // all pairs, 1 = AFF-pruned).  P is tile-blocked [T][which][ldk][128] in the
 // precision of S; sI, sJ hold n_pad values of the vector precision (FP64 when
 // vec64 or S is FP64, else FP32); W is the working buffer [K+1][n_pad] of
-// (xi, eta) pairs of the vector precision; tile_nnz holds nT_cap ints.  Gathers are split into items of at most `item`
+// (xi, eta) pairs (16 bytes; of the vector precision in the item form); tile_nnz holds nT_cap ints.  Gathers are split into items of at most `item`
 // nonzeros; `cap` column indices are cached per CTA (a multiple of 4).
-// bar: two zeroed unsigned ints, left zeroed.  nnz_bound bounds the edges of
+// bar: five zeroed unsigned ints, left zeroed.  nnz_bound bounds the edges of
 // the new graph (it sizes the grid).  Returns 0 on launch, 2 when the graph
 // has more tiles than the co-resident CTAs can own (use the per-step path),
 // 1 on a launch error.
@@ -154,9 +162,10 @@ struct PrepParams {
   int delta, j, op, d_j;
   double C;
   // quotients that are the same for every row, computed once on the host (a
-  // division in the kernel would be issued by every thread): 1 / C, 1 / delta
-  // and delta / (d_j + op delta) (0 when that sum is 0)
-  double inv_C, inv_delta, gq;
+  // division in the kernel would be issued by every thread): 1 / C, 1 / delta,
+  // delta / (d_j + op delta) (0 when that sum is 0) and 1 / (delta d_j) (0 when
+  // d_j is 0)
+  double inv_C, inv_delta, gq, inv_ddj;
   int mt;  // tiles per CTA, ceil(nT / grid) (set by launch_prep)
   int K;
   int nT;
@@ -175,12 +184,17 @@ struct PrepParams {
   void* W;
   void* rinv;  // per row: (C / in-degree, 1 / in-degree) in the vector precision, n_pad pairs
   int* loff;   // per row: nonzeros of its tile before it (n_pad)
-  int flat;    // 1: split the nonzeros evenly over the CTAs when two per thread suffice
+  int flat;    // 1: the flow form when two nonzeros per thread suffice
+  long long* Y;             // flow form: n_pad row sums
+  const SweepScale* recip;  // flow form: 1 / d by d (h, sh for sums of up to 64 values of 2^56)
+  const SweepScale* cpow;   // flow form: C^(k+1) = r 2^-(63 + sh), k = 0 .. K
   int* tile_nnz;
-  unsigned int* bar;
+  unsigned int* bar;  // five
   long long limit;
   unsigned long long* counters;
 };
+// out[d] = 1 / d for d < count (PrepParams::recip)
+void launch_flow_recip(SweepScale* out, int count, cudaStream_t st);
 int launch_prep(const PrepParams& p, int s_prec, int vec64, int npend_max, int num_sms,
                 int max_ctas, int64_t nnz_bound, cudaStream_t st);
 
@@ -273,14 +287,6 @@ void launch_transpose(const void* A, void* B, int prec, int n_pad, int64_t ld, c
 void launch_maxdiff(const void* A, const void* B, int prec, int n, int64_t ld,
                     unsigned long long* out_bits, cudaStream_t st);
 // ---- the same sweep on a symmetric S in fixed point (value * 2^57), k_sweep.cu
-// The factor C / d of a row of d nonzeros, r * 2^-(63 + s) with 2^62 <= r < 2^63.
-// d <= 32: a row sum shifted left by h stays below 2^63, and the high word of
-// its product with r is shifted right by sh = s + h - 1 (at least 3); longer
-// rows: sh = s - 1 (at least 4).
-struct SweepScale {
-  unsigned long long r;
-  int h, sh;
-};
 // One sweep: T and Snew are n_pad x ld; s1[a] = C / in-degree of a, s2[a] =
 // 1 / in-degree; diag is added to the first n_diag diagonal entries; *maxd =
 // max(*maxd, max |Snew - S|) in fixed point.

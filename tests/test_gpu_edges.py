@@ -104,3 +104,30 @@ def test_sweeps_from_any_s0(P, form, prec):
     sr.reanchor(3)
     want = sweeps(0.5 * (W + W.T), Q, C, 4)
     assert np.max(np.abs(sr.dense() - want)) < tol
+
+
+@pytest.mark.parametrize("prec,kw", [(64, {}), (64, {"prep_ctas": 5}), (32, {"vec_fp64": 1}),
+                                     (32, {"tc": 1, "defer": 3, "prep_ctas": 7})])
+@pytest.mark.parametrize("scale", [1.0, 1e-20, 1e20])
+def test_recurrence_at_warp_and_cta_edges(P, prec, kw, scale):
+    """Updates on a graph whose rows end at the splits of the recurrence: 32 and
+    64 nonzeros (warps), 256, 512 and 1,024 (CTAs, one or two nonzeros per
+    thread), hubs over several CTAs, with fewer CTAs too (longer ranges), and
+    an S0 of other magnitudes (the fixed-point exponents).  One update changes
+    S by at most its truncated series: 1e-10 of the largest entry in FP64 and
+    1e-6 in FP32, as in the parity tests."""
+    n, C, K = 1300, 0.6, 7
+    degs = [0, 1, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025]
+    s, d = degrees_graph(n, degs, 11)
+    S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-14) * scale
+    edges = set(zip(s.tolist(), d.tolist()))
+    sr = P.SimRank(n, s, d, S0=S0, C=C, K=K, s_precision=prec, **kw)
+    want = S0.astype(np.float64 if prec == 64 else np.float32).astype(np.float64)
+    ups = []
+    for j, op in ((19, 1), (0, 1), (3, -1), (1, -1), (700, 1)):
+        cand = [x for x in range(n) if x != j and ((x, j) in edges) == (op < 0)]
+        ups.append((cand[len(cand) // 2], j, op))
+    want, _ = O.sequential_unit_updates(n, s, d, want, ups, C, K)
+    sr.apply_updates(ups)
+    err = np.max(np.abs(sr.dense() - want)) / max(1.0, np.max(np.abs(want)))
+    assert err < (1e-10 if prec == 64 else 1e-6)
