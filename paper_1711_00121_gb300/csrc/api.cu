@@ -76,6 +76,7 @@ struct simrank_ctx {
   int32_t* loff = nullptr;        // its per-row offsets inside the tile
   long long* flowY = nullptr;     // its row sums of the flow form
   SweepScale* flow_tab = nullptr; // 1 / d for d <= n_cap, then C^(k+1) for k <= K
+  std::vector<SweepScale> cpow;   // C^(k+1), k <= K
   int* tile_nnz = nullptr;       // per-tile nonzeros (scratch of the pre-update kernel)
   // per-call staging
   int32_t* d_srcs = nullptr;
@@ -597,6 +598,25 @@ simrank_status flush_pending(simrank_ctx* h) {
   return SR_OK;
 }
 
+// Factors of the fixed-point recurrences, once per handle: 1 / d for every
+// in-degree d <= n_cap and C^(k+1) for k <= K (cpow on the host too).
+simrank_status flow_tables(simrank_ctx* h) {
+  if (h->flow_tab) return SR_OK;
+  CUDA_TRY(h, dev_alloc(&h->flow_tab, (size_t)h->n_cap + 1 + h->K1));
+  launch_flow_recip(h->flow_tab, h->n_cap + 1, h->st);
+  h->launches += 1;
+  h->cpow.resize((size_t)h->K1);
+  for (int k = 0; k < h->K1; ++k) {
+    // C^(k+1) = r 2^-(63 + sh), 2^62 <= r < 2^63
+    int e = 0;
+    const double f = std::frexp(std::pow(h->cfg.C, k + 1), &e);
+    h->cpow[k] = SweepScale{(unsigned long long)std::ldexp(f, 63), 0, -e};
+  }
+  CUDA_TRY(h, cudaMemcpyAsync(h->flow_tab + h->n_cap + 1, h->cpow.data(),
+                              h->cpow.size() * sizeof(SweepScale), cudaMemcpyHostToDevice, h->st));
+  return SR_OK;
+}
+
 // One rank-one update of the current S for the sink block (srcs at d_srcs +
 // src_off, delta of them) into sink j, op = +1/-1, old in-degree d_j; the
 // graph patch ops [op_begin, op_end) turn the old graph into the new one.
@@ -674,22 +694,11 @@ simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, i
     pp.item = h->cfg.prep_item;
     pp.n_pad = h->n_pad;
     pp.nT_cap = h->nT_cap;
+    simrank_status fs = flow_tables(h);
+    if (fs != SR_OK) return fs;
     if (!h->W) {
       CUDA_TRY(h, cudaMalloc(&h->W, (size_t)h->K1 * h->n_pad * 2 * sizeof(double)));
       CUDA_TRY(h, dev_alloc(&h->flowY, (size_t)h->n_pad));
-      CUDA_TRY(h, dev_alloc(&h->flow_tab, (size_t)h->n_cap + 1 + h->K1));
-      launch_flow_recip(h->flow_tab, h->n_cap + 1, h->st);
-      h->launches += 1;
-      std::vector<SweepScale> cp((size_t)h->K1);
-      for (int k = 0; k < h->K1; ++k) {
-        // C^(k+1) = r 2^-(63 + sh), 2^62 <= r < 2^63
-        int e = 0;
-        const double f = std::frexp(std::pow(C, k + 1), &e);
-        cp[k] = SweepScale{(unsigned long long)std::ldexp(f, 63), 0, -e};
-      }
-      CUDA_TRY(h, cudaMemcpyAsync(h->flow_tab + h->n_cap + 1, cp.data(),
-                                  cp.size() * sizeof(SweepScale), cudaMemcpyHostToDevice, h->st));
-      CUDA_TRY(h, cudaStreamSynchronize(h->st));
       CUDA_TRY(h, cudaMalloc(&h->rinv, (size_t)h->n_pad * 2 * sizeof(double)));
       CUDA_TRY(h, dev_alloc(&h->loff, (size_t)h->n_pad));
       CUDA_TRY(h, dev_alloc(&h->tile_nnz, (size_t)h->nT_cap));
@@ -990,13 +999,18 @@ simrank_status ob_ensure(simrank_ctx* h, int slot, size_t bytes) {
 
 void build_chunks(const HostAdj& A, int n_rows, std::vector<RowChunk>& out,
                   std::vector<int64_t>* first);
+simrank_status upload_chunks(simrank_ctx* h, const std::vector<RowChunk>& v, ChunkList& L,
+                             int64_t* cap);
 
 // The whole batch as one rank-2r update (proof of Thm 2 with dQ = U V^T over
 // the r distinct sinks).  `plus` / `minus` hold the net insertions and
 // deletions per sink (storage ids); `ops` turn the old graph into the new one.
+// old_chunks: row chunks of the in-lists before the batch (the host mirror
+// already holds the graph after it).
 simrank_status run_one_shot(simrank_ctx* h, const std::map<int32_t, std::vector<int32_t>>& plus,
                             const std::map<int32_t, std::vector<int32_t>>& minus,
-                            const std::vector<PatchOp>& ops) {
+                            const std::vector<PatchOp>& ops,
+                            const std::vector<RowChunk>& old_chunks) {
   std::map<int32_t, std::pair<std::vector<int32_t>, std::vector<int32_t>>> sinks;
   for (auto& kv : plus) sinks[kv.first].first = kv.second;
   for (auto& kv : minus) sinks[kv.first].second = kv.second;
@@ -1077,18 +1091,28 @@ simrank_status run_one_shot(simrank_ctx* h, const std::map<int32_t, std::vector<
   double* X = (double*)h->ob[6].p;
   double* Xn = (double*)h->ob[7].p;
   CUDA_TRY(h, cudaMemsetAsync(Z, 0, (size_t)nr * 8, h->st));
-  CUDA_TRY(h, cudaMemsetAsync(Y, 0, (size_t)nr * 8, h->st));
+  if ((s = upload_chunks(h, old_chunks, h->cur_fwd, &h->cur_fwd_cap)) != SR_OK) return s;
+  if ((s = ob_ensure(h, 28, 3 * (size_t)n_pad * 8)) != SR_OK) return s;
+  double* inv = (double*)h->ob[28].p;
+  launch_col_scales64(WeightView(), h->din.len, n_pad, inv, h->st);
   // Z = sum of signed source rows, Y = Q Z on the OLD graph
   launch_signed_rows(h->S, sp, h->ld, d_src, d_sign, d_off, r, n_pad, Zc, h->st, upper(h));
   launch_transpose_rect(Zc, n_pad, Z, rp, r, n_pad, h->st);
-  launch_spmm_rows(h->din, nullptr, nullptr, Z, 64, rp, Y, 64, rp, n_pad, rp, 1.0, 0.0, 0, h->st);
+  launch_col_horner64(h->cur_fwd, h->din.col, WeightView(), inv, nullptr, 0.0, Z, Y, rp, h->st);
   launch_transpose_rect(Y, rp, Zc, n_pad, n_pad, r, h->st);  // Yc into buffer 1
   launch_lambda(h->S, sp, h->ld, d_sinks, d_av, d_bv, Y, Z, rp, d_src, d_sign, d_off, r, C, Lam,
                 h->st, upper(h));
   launch_w_assemble(h->S, sp, h->ld, d_sinks, d_av, d_bv, Zc, Lam, r, n_pad, C, Wc, h->st,
                     upper(h));
   LAUNCH_CHECK(h);
-  h->launches += 7;
+  h->launches += 9;
+  // the largest |W| gives the steps their fixed-point exponent (an infinite or
+  // NaN W: the steps run in FP64)
+  unsigned int wbits = 0;
+  CUDA_TRY(h, cudaMemsetAsync(h->diffbits, 0, sizeof(unsigned long long), h->st));
+  launch_os_absmax(Wc, (int64_t)r * n_pad, (unsigned int*)h->diffbits, h->st);
+  CUDA_TRY(h, cudaMemcpyAsync(&wbits, h->diffbits, sizeof(wbits), cudaMemcpyDeviceToHost, h->st));
+  if ((s = flow_tables(h)) != SR_OK) return s;
   // the graph becomes the new one
   CUDA_TRY(h, cudaMemcpyAsync(h->d_ops, ops.data(), ops.size() * sizeof(PatchOp),
                               cudaMemcpyHostToDevice, h->st));
@@ -1096,20 +1120,27 @@ simrank_status run_one_shot(simrank_ctx* h, const std::map<int32_t, std::vector<
   // X_0 = [C U | W] (row-major, 2 rp columns)
   const int64_t ldx = 2 * rp;
   CUDA_TRY(h, cudaMemsetAsync(X, 0, (size_t)nr * 2 * 8, h->st));
-  CUDA_TRY(h, cudaMemsetAsync(Xn, 0, (size_t)nr * 2 * 8, h->st));
-  launch_xi0(d_sinks, r, C, X, ldx, h->st);
-  launch_transpose_rect(Wc, n_pad, X + rp, ldx, r, n_pad, h->st);
-  LAUNCH_CHECK(h);
-  h->launches += 3;
   // the steps below gather by row chunks of the new graph (the host mirror
   // holds it), so that a hub row spreads over many warps
   std::vector<RowChunk> chv;
   build_chunks(h->hin, n_pad, chv, nullptr);
-  if ((s = ob_ensure(h, 26, std::max<size_t>(1, chv.size()) * sizeof(RowChunk))) != SR_OK) return s;
-  const RowChunk* d_chunks = (const RowChunk*)h->ob[26].p;
-  if (!chv.empty())
-    CUDA_TRY(h, cudaMemcpyAsync(h->ob[26].p, chv.data(), chv.size() * sizeof(RowChunk),
-                                cudaMemcpyHostToDevice, h->st));
+  if ((s = upload_chunks(h, chv, h->cur_hor, &h->cur_hor_cap)) != SR_OK) return s;
+  h->col_chunks_ok = false;
+  CUDA_TRY(h, cudaStreamSynchronize(h->st));
+  const bool fixed = wbits < 0x7f800000u;
+  float wmax;
+  std::memcpy(&wmax, &wbits, sizeof(wmax));
+  const int we = wbits ? std::ilogb(wmax) + 1 : 0;  // |W| < 2^we
+  long long* XI = (long long*)X;
+  if (fixed) {
+    launch_os_fix(Wc, n_pad, r, rp, we, d_sinks, XI, ldx, h->st);
+  } else {
+    CUDA_TRY(h, cudaMemsetAsync(Xn, 0, (size_t)nr * 2 * 8, h->st));
+    launch_xi0(d_sinks, r, C, X, ldx, h->st);
+    launch_transpose_rect(Wc, n_pad, X + rp, ldx, r, n_pad, h->st);
+  }
+  LAUNCH_CHECK(h);
+  h->launches += 3;
 
   // k-groups: as many terms per S pass as fit an operand budget
   // tc = 2: FP16 split, terms balanced by powers of two (rg a multiple of 64);
@@ -1128,7 +1159,7 @@ simrank_status run_one_shot(simrank_ctx* h, const std::map<int32_t, std::vector<
   if (tc) {
     if ((s = ob_ensure(h, 8, (size_t)n_pad * kd * eb)) != SR_OK) return s;
     if ((s = ob_ensure(h, 9, (size_t)n_pad * kd * eb)) != SR_OK) return s;
-    if (f16 && (s = ob_ensure(h, 27, 2 * (size_t)r * sizeof(unsigned int))) != SR_OK) return s;
+    if (f16 && (s = ob_ensure(h, 27, (size_t)ldx * sizeof(unsigned int))) != SR_OK) return s;
   } else {
     if ((s = ob_ensure(h, 8, (size_t)h->nT_cap * 2 * (size_t)(g * r) * PT * (sp == 64 ? 8 : 4))) !=
         SR_OK)
@@ -1137,7 +1168,13 @@ simrank_status run_one_shot(simrank_ctx* h, const std::map<int32_t, std::vector<
   const long long wait_limit = ::wait_limit(h);
   int slot = 0;
   for (int k = 0; k <= h->cfg.K; ++k) {
-    if (k > 0) {
+    if (k > 0 && fixed) {
+      launch_os_step(h->cur_hor, h->din.col, h->din.len, h->flow_tab, (const long long*)X,
+                     (long long*)Xn, (int)ldx, h->st);
+      std::swap(X, Xn);
+      h->launches += 1;
+    } else if (k > 0) {
+      const RowChunk* d_chunks = h->cur_hor.chunks;
       CUDA_TRY(h, cudaMemsetAsync(Xn, 0, (size_t)nr * 2 * 8, h->st));
       if (launch_spmm_chunks64(d_chunks, (int64_t)chv.size(), h->din.col, h->din.len, X, ldx, Xn,
                                ldx, rp, C, h->st) != 0 ||
@@ -1156,7 +1193,13 @@ simrank_status run_one_shot(simrank_ctx* h, const std::map<int32_t, std::vector<
         CUDA_TRY(h, cudaMemsetAsync(h->mEta, 0, h->nT_cap * sizeof(uint64_t), h->st));
       }
     }
-    if (f16)
+    if (fixed && tc)
+      launch_os_pack((const long long*)X, ldx, rp, r, slot, rg, n_pad, h->cpow[k], we,
+                     f16 ? 1 : 0, (unsigned int*)h->ob[27].p, h->ob[8].p, h->ob[9].p, kd, h->st);
+    else if (fixed)
+      launch_os_pack_ffma((const long long*)X, ldx, rp, r, slot, g * r, nT, h->cpow[k], we,
+                          h->ob[8].p, sp, h->mXi, h->mEta, h->st);
+    else if (f16)
       launch_pack_f16_oneshot(X, ldx, rp, r, slot, rg, n_pad, (unsigned int*)h->ob[27].p,
                               h->ob[8].p, h->ob[9].p, kd, h->st);
     else if (tc)
@@ -1993,6 +2036,8 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
     std::string msg;
     if ((s = plan_blocks(um.data(), count, n_old, blocks, msg)) != SR_OK) return fail(h, s, msg);
     std::map<int32_t, std::vector<int32_t>> plus, minus;
+    std::vector<RowChunk> old_chunks;
+    build_chunks(h->hin, h->n_pad, old_chunks);
     for (const Block& b : blocks) {
       auto& dstv = (b.op > 0 ? plus : minus)[b.sink];
       dstv.insert(dstv.end(), b.srcs.begin(), b.srcs.end());
@@ -2012,7 +2057,7 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
     if ((s = grow_pool(h, h->din, h->hin)) != SR_OK) return s;
     if ((s = grow_pool(h, h->dout, h->hout)) != SR_OK) return s;
     if ((s = ensure_dev_capacity(h, 1, (int64_t)ops.size())) != SR_OK) return s;
-    if ((s = run_one_shot(h, plus, minus, ops)) != SR_OK) return s;
+    if ((s = run_one_shot(h, plus, minus, ops, old_chunks)) != SR_OK) return s;
     h->stats.updates += count;
     return maybe_reanchor(h, count);
   }

@@ -10,6 +10,9 @@
 // operand layouts of the two S-update kernels.
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
+#include "fixed64.h"
 #include "sr_internal.h"
 
 namespace sr {
@@ -489,6 +492,261 @@ int launch_spmm_chunks64(const RowChunk* chunks, int64_t count, const int32_t* c
   else
     spmm_chunks64_t<32>(chunks, count, col, len, X, ldx, Y, ldy, ncols, scale, st);
   return 0;
+}
+
+}  // namespace sr
+
+// ---------------------------------------------------------------------------
+// The same steps in 64-bit fixed point.  A step gathers one row segment of the
+// 2 r columns per nonzero; in FP64 it was bound by the FP64 adds and by the
+// atomics that every row chunk made (k_spmm_chunks64, for an S that is not
+// finite).  Here X holds Q^k e_j (xi without its factor C^(k+1), in [0, 1]) and
+// W's columns as integers, value * 2^(56 - e): a warp takes a row chunk and 128
+// columns, sums exactly, multiplies by 1 / d once and writes a row of one chunk
+// directly.  The rounding of a step is 2^-57 of the largest entry.  n = 12,000,
+// m = 180,000, 2 x 190 columns: 49 us a step (10 TB/s of gathers), 260 us in FP64.
+// ---------------------------------------------------------------------------
+namespace sr {
+namespace {
+
+// X[j_t][t] = 1 (the xi half, zero before), X[a][rh + t] = W_t[a]
+__global__ void k_os_fix(const double* __restrict__ Wc, int n_pad, int r, int rh, int e,
+                         const int32_t* __restrict__ sinks, long long* __restrict__ X,
+                         int64_t ldx) {
+  __shared__ double tile[32][33];
+  const int a0 = blockIdx.x * 32, t0 = blockIdx.y * 32;
+  for (int q = threadIdx.y; q < 32; q += 8)
+    tile[q][threadIdx.x] =
+        t0 + q < r ? Wc[(int64_t)(t0 + q) * n_pad + a0 + threadIdx.x] : 0.0;
+  __syncthreads();
+  const int t = t0 + threadIdx.x;
+  if (t >= r) return;
+  const int j = sinks[t];
+  for (int q = threadIdx.y; q < 32; q += 8) {
+    const int a = a0 + q;
+    X[(int64_t)a * ldx + rh + t] = fixed_of(tile[threadIdx.x][q], e);
+    if (a == j) X[(int64_t)a * ldx + t] = 1ll << 56;
+  }
+}
+
+// *out = max |W| as the bits of an FP32 value not below it (infinity's for an
+// infinite or NaN entry)
+__global__ void k_os_absmax(const double* __restrict__ W, int64_t count,
+                            unsigned int* __restrict__ out) {
+  unsigned int m = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const float v = up_abs(W[i]);
+    m = max(m, v <= 3.0e38f ? __float_as_uint(v) : 0x7f800000u);
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
+}
+
+// Y[row] = Q X[row] for the row chunks: one warp per chunk and 128 columns (lane:
+// two pairs 64 columns apart).  Rows of several chunks start at zero in Y.
+__global__ void __launch_bounds__(256, 4) k_os_step(const RowChunk* __restrict__ chunks,
+                                                    int64_t count,
+                                                    const int32_t* __restrict__ col,
+                                                    const int32_t* __restrict__ len,
+                                                    const SweepScale* __restrict__ recip,
+                                                    const long long* __restrict__ X,
+                                                    long long* __restrict__ Y, int ldx) {
+  const int lane = threadIdx.x & 31;
+  const int64_t q = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (q >= count) return;  // the whole warp
+  const RowChunk ch = chunks[q];
+  const int m = chunk_len(ch);
+  const int id = lane < m ? col[ch.start + lane] : 0;
+  const int c = (int)blockIdx.y * 128 + 2 * lane;
+  const bool a0 = c < ldx, a1 = c + 64 < ldx;
+  long long s[4] = {0, 0, 0, 0};
+  for (int u = 0; u < m; u += 4) {
+    longlong2 v[4][2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t x = __shfl_sync(0xffffffffu, id, u + k);
+      const longlong2* p = reinterpret_cast<const longlong2*>(X + x * ldx + c);
+      v[k][0] = v[k][1] = make_longlong2(0, 0);
+      if (u + k < m && a0) v[k][0] = p[0];
+      if (u + k < m && a1) v[k][1] = p[32];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      s[0] += v[k][0].x;
+      s[1] += v[k][0].y;
+      s[2] += v[k][1].x;
+      s[3] += v[k][1].y;
+    }
+  }
+  const SweepScale f = recip[len[ch.row]];
+  long long* y = Y + (int64_t)ch.row * ldx + c;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) s[k] = m ? fixed_scale(s[k], f) : 0;
+  if (ch.len & CH_ONLY) {
+    if (a0) *reinterpret_cast<longlong2*>(y) = make_longlong2(s[0], s[1]);
+    if (a1) *reinterpret_cast<longlong2*>(y + 64) = make_longlong2(s[2], s[3]);
+  } else {
+    unsigned long long* z = reinterpret_cast<unsigned long long*>(y);
+    if (a0) {
+      atomicAdd(z, (unsigned long long)s[0]);
+      atomicAdd(z + 1, (unsigned long long)s[1]);
+    }
+    if (a1) {
+      atomicAdd(z + 64, (unsigned long long)s[2]);
+      atomicAdd(z + 65, (unsigned long long)s[3]);
+    }
+  }
+}
+
+// Y[row] = 0 for the rows of several chunks
+__global__ void k_os_zero(const int32_t* __restrict__ rows, long long* __restrict__ Y, int ldx) {
+  long long* y = Y + (int64_t)rows[blockIdx.x] * ldx;
+  for (int c = threadIdx.x; c < ldx; c += blockDim.x) y[c] = 0;
+}
+
+// bits[c] = the width of the largest |entry| of column c (0: all zero)
+__global__ void __launch_bounds__(256) k_os_width(const long long* __restrict__ X, int ldx,
+                                                  int n_rows, unsigned int* __restrict__ bits) {
+  __shared__ unsigned int red[8][32];
+  const int c = blockIdx.x * 32 + threadIdx.x;
+  unsigned long long m = 0;
+  if (c < ldx)
+    for (int64_t a = (int64_t)blockIdx.y * 8 + threadIdx.y; a < n_rows; a += (int64_t)gridDim.y * 8) {
+      const long long v = X[a * ldx + c];
+      m |= (unsigned long long)(v < 0 ? -v : v);
+    }
+  red[threadIdx.y][threadIdx.x] = 64 - __clzll((long long)m);
+  __syncthreads();
+  if (threadIdx.y == 0 && c < ldx) {
+    unsigned int w = red[0][threadIdx.x];
+#pragma unroll
+    for (int y = 1; y < 8; ++y) w = max(w, red[y][threadIdx.x]);
+    if (w) atomicMax(&bits[c], w);
+  }
+}
+
+// One value of term t as an integer and its exponent: xi (h = 0) is
+// C^(k+1) x 2^-56 with C^(k+1) = ck.r 2^-(63 + ck.sh), W (h = 1) y 2^(e - 56)
+__device__ __forceinline__ long long os_entry(long long v, int h, const SweepScale& ck, int e,
+                                              int& ex) {
+  ex = h ? e - 56 : -61 - ck.sh;
+  return h ? v : __mul64hi(v << 6, (long long)ck.r);
+}
+
+// FP16 operands as k_pack_f16_oneshot's, from the integers
+__global__ void k_os_pack_f16(const long long* __restrict__ X, int64_t ldx, int rh, int r,
+                              int slot, int rg, int n_rows, SweepScale ck, int e,
+                              const unsigned int* __restrict__ bits, __half* __restrict__ Ahi,
+                              __half* __restrict__ Alo, int64_t kd) {
+  const int t = blockIdx.y * blockDim.x + threadIdx.x;
+  if (t >= r) return;
+  const int wx = (int)bits[t], we = (int)bits[rh + t];
+  // exponents of the largest magnitudes, up to a common offset of one
+  const int bal = (wx && we) ? ((we + e - 56) - (wx - 56 - (ck.sh + 1))) / 2 : 0;
+  for (int64_t a = blockIdx.x; a < n_rows; a += gridDim.x) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      int ex;
+      const long long v = os_entry(X[a * ldx + (int64_t)h * rh + t], h, ck, e, ex);
+      // 24 bits rounded to odd, so that both roundings to FP16 are those of v
+      const float x = fixed_value<float, true>(v, ex + (h ? -bal : bal));
+      const __half hi = __float2half_rn(x);
+      const __half lo = __float2half_rn(x - __half2float(hi));
+      const int64_t c = (int64_t)h * rg + (int64_t)slot * r + t;
+      Ahi[a * kd + c] = hi;
+      Alo[a * kd + c] = lo;
+    }
+  }
+}
+
+__global__ void k_os_pack_tf32(const long long* __restrict__ X, int64_t ldx, int rh, int r,
+                               int slot, int rg, int n_rows, SweepScale ck, int e,
+                               float* __restrict__ Ahi, float* __restrict__ Alo, int64_t kd) {
+  const int t = blockIdx.y * blockDim.x + threadIdx.x;
+  if (t >= r) return;
+  for (int64_t a = blockIdx.x; a < n_rows; a += gridDim.x) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      int ex;
+      const long long v = os_entry(X[a * ldx + (int64_t)h * rh + t], h, ck, e, ex);
+      const float x = fixed_value<float>(v, ex);
+      const float hi = tf32_rne(x);
+      const int64_t c = (int64_t)h * rg + (int64_t)slot * r + t;
+      Ahi[a * kd + c] = hi;
+      Alo[a * kd + c] = tf32_rne(x - hi);
+    }
+  }
+}
+
+// k_pack_ffma's panels and masks from the integers
+template <typename TP>
+__global__ void k_os_pack_ffma(const long long* __restrict__ X, int64_t ldx, int rh, int r,
+                               int slot, int terms, SweepScale ck, int e, TP* __restrict__ Pn,
+                               uint64_t* __restrict__ mXi, uint64_t* __restrict__ mEta) {
+  const int T = blockIdx.x;
+  const int t = blockIdx.y * 2 + (threadIdx.x >> 7);
+  const int row = threadIdx.x & 127;
+  if (t >= r) return;  // whole warps
+  const int64_t a = (int64_t)T * PT + row;
+  const int term = slot * r + t;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int ex;
+    const long long v = os_entry(X[a * ldx + (int64_t)h * rh + t], h, ck, e, ex);
+    const TP x = fixed_value<TP>(v, ex);
+    Pn[(((int64_t)T * 2 + h) * terms + term) * PT + row] = x;
+    if (__any_sync(0xffffffffu, v != 0) && (threadIdx.x & 31) == 0)
+      atomicOr((unsigned long long*)(h ? mEta : mXi) + T, 1ull << (term & 63));
+  }
+}
+
+}  // namespace
+
+void launch_os_absmax(const double* W, int64_t count, unsigned int* out, cudaStream_t st) {
+  k_os_absmax<<<608, 256, 0, st>>>(W, count, out);
+}
+
+void launch_os_fix(const double* Wc, int n_pad, int r, int rh, int e, const int32_t* sinks,
+                   long long* X, int64_t ldx, cudaStream_t st) {
+  k_os_fix<<<dim3(n_pad / 32, (r + 31) / 32), dim3(32, 8), 0, st>>>(Wc, n_pad, r, rh, e, sinks, X,
+                                                                    ldx);
+}
+
+void launch_os_step(const ChunkList& L, const int32_t* col, const int32_t* len,
+                    const SweepScale* recip, const long long* X, long long* Y, int ldx,
+                    cudaStream_t st) {
+  if (L.multi_count > 0) k_os_zero<<<(unsigned)L.multi_count, 128, 0, st>>>(L.multi, Y, ldx);
+  const dim3 grid((unsigned)((L.count + 7) / 8), (unsigned)((ldx + 127) / 128));
+  k_os_step<<<grid, 256, 0, st>>>(L.chunks, L.count, col, len, recip, X, Y, ldx);
+}
+
+void launch_os_pack(const long long* X, int64_t ldx, int rh, int r, int slot, int rg, int n_rows,
+                    const SweepScale& ck, int e, int f16, unsigned int* bits, void* Ahi, void* Alo,
+                    int64_t kd, cudaStream_t st) {
+  const dim3 grid((unsigned)std::min(n_rows, 2432), (unsigned)((r + 127) / 128));
+  if (f16) {
+    cudaMemsetAsync(bits, 0, (size_t)ldx * sizeof(unsigned int), st);
+    k_os_width<<<dim3((unsigned)((ldx + 31) / 32), 64), dim3(32, 8), 0, st>>>(X, (int)ldx, n_rows,
+                                                                              bits);
+    k_os_pack_f16<<<grid, 128, 0, st>>>(X, ldx, rh, r, slot, rg, n_rows, ck, e, bits,
+                                        (__half*)Ahi, (__half*)Alo, kd);
+  } else {
+    k_os_pack_tf32<<<grid, 128, 0, st>>>(X, ldx, rh, r, slot, rg, n_rows, ck, e, (float*)Ahi,
+                                         (float*)Alo, kd);
+  }
+}
+
+void launch_os_pack_ffma(const long long* X, int64_t ldx, int rh, int r, int slot, int terms,
+                         int nT, const SweepScale& ck, int e, void* Pn, int p_prec, uint64_t* mXi,
+                         uint64_t* mEta, cudaStream_t st) {
+  const dim3 grid(nT, (r + 1) / 2);
+  if (p_prec == 64)
+    k_os_pack_ffma<double><<<grid, 256, 0, st>>>(X, ldx, rh, r, slot, terms, ck, e, (double*)Pn,
+                                                 mXi, mEta);
+  else
+    k_os_pack_ffma<float><<<grid, 256, 0, st>>>(X, ldx, rh, r, slot, terms, ck, e, (float*)Pn, mXi,
+                                                mEta);
 }
 
 }  // namespace sr

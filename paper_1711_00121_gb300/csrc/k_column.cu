@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(256, 6) k_col_rows(
     }
     if (act) {
       if (only) {
-        if (!FORWARD) {
+        if (!FORWARD && Xadd) {
           const ColVec<T, VEC> base = ld_cols<T, VEC>(Xadd + o);
 #pragma unroll
           for (int z = 0; z < VEC; ++z) acc.v[z] += add_scale * base.v[z];

@@ -61,6 +61,7 @@
 // depend on the order of the additions.
 #include <algorithm>
 
+#include "fixed64.h"
 #include "fx64.h"
 #include "sr_internal.h"
 
@@ -555,59 +556,6 @@ __device__ __forceinline__ bool flow_there(const I2& v, int n) {
          (((int)(v.y >> 32) + half) >> (FLOW_CNT - 32)) == n;
 }
 
-// v * 2^(56 - e) rounded to nearest, |v| < 2^e, on the integer pipe
-__device__ __forceinline__ long long flow_fix(uint64_t m, int sh, bool neg) {
-  long long f = 0;
-  if (sh >= 0)
-    f = (long long)(m << sh);
-  else if (sh > -60)
-    f = (long long)((m + (1ull << (-sh - 1))) >> -sh);
-  return neg ? -f : f;
-}
-__device__ __forceinline__ long long flow_of(float v, int e) {
-  const uint32_t b = __float_as_uint(v);
-  const int x = (int)((b >> 23) & 0xffu);
-  const uint32_t m = x ? (b & 0x7fffffu) | 0x800000u : b & 0x7fffffu;
-  return flow_fix(m, max(x, 1) - 150 + 56 - e, (b >> 31) != 0);
-}
-__device__ __forceinline__ long long flow_of(double v, int e) {
-  const uint64_t b = (uint64_t)__double_as_longlong(v);
-  const int x = (int)((b >> 52) & 0x7ffu);
-  const uint64_t m = x ? (b & 0xfffffffffffffull) | 0x10000000000000ull : b & 0xfffffffffffffull;
-  return flow_fix(m, max(x, 1) - 1075 + 56 - e, (b >> 63) != 0);
-}
-// out of line: instructions that a launch runs once are bound by their fetch
-__device__ __noinline__ double flow_value_slow(long long v, int e) { return ldexp((double)v, e); }
-
-// v * 2^e rounded to nearest even
-template <typename T>
-__device__ __forceinline__ T flow_value(long long v, int e) {
-  if (v == 0) return T(0);
-  const uint64_t a = v < 0 ? (uint64_t)-v : (uint64_t)v;
-  const int lz = __clzll((long long)a);
-  const int x = 63 - lz + e;  // 2^x <= |v| 2^e
-  constexpr bool F = sizeof(T) == 4;
-  if (x < (F ? -126 : -1022) || x > (F ? 126 : 1022)) return (T)flow_value_slow(v, e);
-  const uint64_t m = a << lz;
-  constexpr int DROP = F ? 40 : 11;
-  const uint64_t rem = m & ((1ull << DROP) - 1), half = 1ull << (DROP - 1);
-  uint64_t q = m >> DROP;  // leading one included
-  q += (rem > half || (rem == half && (q & 1))) ? 1 : 0;
-  // adding the significand with its leading one carries into the exponent
-  if constexpr (F)
-    return __uint_as_float((((uint32_t)(x + 126) << 23) + (uint32_t)q) |
-                           (v < 0 ? 0x80000000u : 0u));
-  else
-    return __longlong_as_double((long long)((((uint64_t)(x + 1022) << 52) + q) |
-                                            (v < 0 ? 0x8000000000000000ull : 0ull)));
-}
-
-// A sum of values of one row held by a warp times 1 / d, rounded to nearest
-__device__ __forceinline__ long long flow_scale(long long s, const SweepScale& f) {
-  const long long t = __mul64hi(s << f.h, (long long)f.r);
-  return (t + (1ll << (f.sh - 1))) >> f.sh;
-}
-
 // x / per for 0 <= x < 2^24 (inv = 1 / per)
 __device__ __forceinline__ int flow_div(int x, int per, float inv) {
   int q = (int)((float)x * inv);
@@ -653,10 +601,6 @@ __device__ __forceinline__ void flow_sum(const StepPair<V>& q, I2& h, const I2& 
     h.y += y;
   }
 }
-
-// |v| as an FP32 value not below it
-__device__ __forceinline__ float up_abs(float v) { return fabsf(v); }
-__device__ __forceinline__ float up_abs(double v) { return __double2float_ru(fabs(v)); }
 
 // out[d] = 1 / d, r = 2^(62 + L) / d rounded to nearest with 2^(L-1) < d <= 2^L;
 // d <= 64: sums of d values below 2^56 may be shifted left by h = 6 - L
@@ -1028,16 +972,16 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     if (q0.cb >= 0) nb2 = flow_parts(q0.cb, ioff, p.loff, p.in, per, inv_per);
     // w = Q sI: the parts of each row's mean, in units of 2^(eI - 56), into Y
     I2 h{0, 0}, t{0, 0};
-    if (q0.ca >= 0) h.x = flow_of(sI[q0.ca], eI);
+    if (q0.ca >= 0) h.x = fixed_of(sI[q0.ca], eI);
     if (q0.cb >= 0) {
-      const long long v = flow_of(sI[q0.cb], eI);
+      const long long v = fixed_of(sI[q0.cb], eI);
       if (q0.kt >= 0) t.x = v; else h.x += v;
     }
     flow_sum(q0, h, t);
     if (q0.fl & (1u << 6))
-      atomicAdd((unsigned long long*)p.Y + q0.kh, (unsigned long long)flow_scale(h.x, fsh[tid][0]));
+      atomicAdd((unsigned long long*)p.Y + q0.kh, (unsigned long long)fixed_scale(h.x, fsh[tid][0]));
     if (q0.fl & (1u << 7))
-      atomicAdd((unsigned long long*)p.Y + q0.kt, (unsigned long long)flow_scale(t.x, fsh[tid][1]));
+      atomicAdd((unsigned long long*)p.Y + q0.kt, (unsigned long long)fixed_scale(t.x, fsh[tid][1]));
     alive = prep_barrier(p.bar, ++nb * G, p.limit, &s_ok);
   } else if (alive) {
     my_items = s_div;
@@ -1086,7 +1030,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
         // the factors of row a of Q on the new graph, for every step below
         const V inv = len > 0 && !flow ? V(1) / (V)len : V(0);
         // sum (item form) or mean (flow form) of sI over the new in-neighbours
-        const V y = flow ? flow_value<V>(__ldcg(p.Y + a), eI - 56) : __ldcg(&W[a].x);
+        const V y = flow ? fixed_value<V>(__ldcg(p.Y + a), eI - 56) : __ldcg(&W[a].x);
         V g;
         if (a == p.j) {
           // row j: lambda (Eq. 29b) and w_j on the old row j, in FP64
@@ -1094,7 +1038,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
           for (int u = 0; u < p.delta; ++u) S_II += (double)__ldcg(sI + p.I[u]);
           const double S_jj = (double)__ldcg(sJ + p.j);
           const double ys =
-              flow ? flow_value<double>(__ldcg(p.Y + a), eI - 56) * (double)len : (double)y;
+              flow ? fixed_value<double>(__ldcg(p.Y + a), eI - 56) * (double)len : (double)y;
           const double wj = (ys - (double)p.op * S_II) * p.inv_ddj;  // 0 when d_j = 0
           const double id = p.inv_delta, iC = p.inv_C;
           const double lam = S_II * id * id + S_jj * iC - 2.0 * wj - iC + 1.0;
@@ -1118,7 +1062,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
         }
         const V x0 = (a == p.j) ? Cv : V(0);
         if (flow) {
-          put_flow(F + a, I2{a == p.j ? 1ll << 56 : 0ll, flow_of(g, eG)});
+          put_flow(F + a, I2{a == p.j ? 1ll << 56 : 0ll, fixed_of(g, eG)});
         } else {
           W[a] = V2<V>{x0, g};
           rinv[a] = V2<V>{Cv * inv, inv};
@@ -1197,8 +1141,8 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
       flow_sum(q0, h, t);
       if (q0.fl & (1u << 6)) {
         const SweepScale f = fsh[tid][0];
-        h.x = flow_scale(h.x, f);
-        h.y = flow_scale(h.y, f);
+        h.x = fixed_scale(h.x, f);
+        h.y = fixed_scale(h.y, f);
         if (give)
           dep[k & 1][warp] = h;
         else if (wait_w == 0 || wait_tail)
@@ -1206,8 +1150,8 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
       }
       if (q0.fl & (1u << 7)) {
         const SweepScale f = fsh[tid][1];
-        t.x = flow_scale(t.x, f);
-        t.y = flow_scale(t.y, f);
+        t.x = fixed_scale(t.x, f);
+        t.y = fixed_scale(t.y, f);
         if (!wait_tail) put_flow(Fn + q0.kt, t);
       }
       if (__syncthreads_or(stop)) {
@@ -1287,8 +1231,8 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
             // xi_k = C^(k+1) x 2^-56, C^(k+1) = r 2^-(63 + s)
             I2 v = look[q];
             flow_strip(v, parts[q]);
-            px = flow_value<TS>(__mul64hi(v.x << 6, (long long)ck.r), -61 - ck.sh);
-            pe = flow_value<TS>(v.y, eG - 56);
+            px = fixed_value<TS>(__mul64hi(v.x << 6, (long long)ck.r), -61 - ck.sh);
+            pe = fixed_value<TS>(v.y, eG - 56);
           } else {
             const V2<V> v = ld_v2(Wk + a);
             px = (TS)v.x;

@@ -22,7 +22,7 @@
 // second only the tiles that reach the diagonal or above are formed (S' is
 // symmetric), written together with their mirrors and compared with the old S
 // for the stopping test.
-#include "sr_internal.h"
+#include "fixed64.h"
 
 namespace sr {
 
@@ -50,12 +50,6 @@ __device__ __forceinline__ void acc_add(Acc96& a, const Acc96& b) {
   asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
       : "+r"(a.w0), "+r"(a.w1), "+r"(a.w2)
       : "r"(b.w0), "r"(b.w1), "r"(b.w2));
-}
-
-// The sum of a row of at most 32 values times its factor, rounded to nearest
-__device__ __forceinline__ long long sum_scale(long long s, const SweepScale& f) {
-  const long long t = __mul64hi(s << f.h, (long long)f.r);
-  return (t + (1ll << (f.sh - 1))) >> f.sh;
 }
 
 // The sum of a longer row times its factor r * 2^-(63 + s), s >= 5
@@ -162,7 +156,7 @@ __global__ void __launch_bounds__(256, 4) k_sweep(DevAdj in, const SweepScale* _
       long long s[2 * NV] = {};
       gather32(id, len, xc, pitch, s);
 #pragma unroll
-      for (int q = 0; q < 2 * NV; ++q) tile[r][64 * (q / 2) + 2 * lane + (q & 1)] = sum_scale(s[q], f);
+      for (int q = 0; q < 2 * NV; ++q) tile[r][64 * (q / 2) + 2 * lane + (q & 1)] = fixed_scale(s[q], f);
     } else if (len <= LONG_ROW) {
       Acc96 a[2 * NV];
       gather_long(in.col + __shfl_sync(0xffffffffu, my_st, i), 0, len, xc, pitch, a);
@@ -239,50 +233,6 @@ __global__ void __launch_bounds__(256, 4) k_sweep(DevAdj in, const SweepScale* _
   }
 }
 
-// x * 2^56 rounded to nearest (half away from zero), |x| < 2, on the integer
-// pipe: a conversion from or to a 64-bit type issues at the FP64 rate
-__device__ __forceinline__ long long fixed56(uint64_t mant, int sh, bool neg) {
-  long long v = 0;
-  if (sh >= 0)
-    v = (long long)(mant << sh);
-  else if (sh > -60)
-    v = (long long)((mant + (1ull << (-sh - 1))) >> -sh);
-  return neg ? -v : v;
-}
-__device__ __forceinline__ long long to_fixed56(float x) {
-  const uint32_t b = __float_as_uint(x);
-  const int e = (int)((b >> 23) & 0xffu);
-  if (e == 0) return 0;  // below 2^-126
-  return fixed56((b & 0x7fffffu) | 0x800000u, e - 127 - 23 + 56, (b >> 31) != 0);
-}
-__device__ __forceinline__ long long to_fixed56(double x) {
-  const uint64_t b = (uint64_t)__double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7ffu);
-  if (e == 0) return 0;
-  return fixed56((b & 0xfffffffffffffull) | 0x10000000000000ull, e - 1023 - 52 + 56,
-                 (b >> 63) != 0);
-}
-// v * 2^-57 rounded to nearest even
-template <typename T>
-__device__ __forceinline__ T from_fixed57(long long v) {
-  if (v == 0) return T(0);
-  const uint64_t a = v < 0 ? (uint64_t)-v : (uint64_t)v;
-  const int lz = __clzll((long long)a);
-  const uint64_t m = a << lz;
-  constexpr int DROP = sizeof(T) == 4 ? 40 : 11;
-  const uint64_t rem = m & ((1ull << DROP) - 1), half = 1ull << (DROP - 1);
-  uint64_t q = m >> DROP;  // leading one included
-  q += (rem > half || (rem == half && (q & 1))) ? 1 : 0;
-  const int e = 63 - lz - 57;
-  // adding the significand with its leading one carries into the exponent
-  if constexpr (sizeof(T) == 4)
-    return __uint_as_float((((uint32_t)(e + 126) << 23) + (uint32_t)q) |
-                           (v < 0 ? 0x80000000u : 0u));
-  else
-    return __longlong_as_double((long long)((((uint64_t)(e + 1022) << 52) + q) |
-                                            (v < 0 ? 0x8000000000000000ull : 0ull)));
-}
-
 // The mean of each pair of mirrored entries in fixed point, both places (FIX;
 // S and F may be the same memory: a CTA reads its two blocks, then writes
 // them), and what the fixed-point form cannot take (CHECK): *flags |= 1 for an
@@ -311,11 +261,11 @@ __global__ void k_to_fixed(const T* S, long long* F, int64_t ld, int upper, doub
     }
     if (FIX) {
       // value * 2^56: the sum of the two is their mean * 2^57
-      F[(int64_t)(bi * 32 + r) * ld + bj * 32 + threadIdx.x] = to_fixed56(x) + to_fixed56(y);
+      F[(int64_t)(bi * 32 + r) * ld + bj * 32 + threadIdx.x] = fixed_of(x, 0) + fixed_of(y, 0);
       if (bi != bj) {
         const T v = x1[threadIdx.x][r];
         const T w = one ? v : x2[r][threadIdx.x];
-        F[(int64_t)(bj * 32 + r) * ld + bi * 32 + threadIdx.x] = to_fixed56(v) + to_fixed56(w);
+        F[(int64_t)(bj * 32 + r) * ld + bi * 32 + threadIdx.x] = fixed_of(v, 0) + fixed_of(w, 0);
       }
     }
   }
@@ -334,7 +284,7 @@ __global__ void k_from_fixed(const long long* F, T* S, int64_t ld, int upper) {
   for (int r = threadIdx.y; r < 32; r += 8) {
     const int64_t o = (int64_t)(bi * 32 + r) * ld + bj * PT + threadIdx.x;
 #pragma unroll
-    for (int q = 0; q < PT; q += 32) S[o + q] = from_fixed57<T>(F[o + q]);
+    for (int q = 0; q < PT; q += 32) S[o + q] = fixed_value<T>(F[o + q], -57);
   }
 }
 

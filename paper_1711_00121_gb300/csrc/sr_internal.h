@@ -408,6 +408,24 @@ struct ChunkList {
 int launch_spmm_chunks64(const RowChunk* chunks, int64_t count, const int32_t* col,
                          const int32_t* len, const double* X, int64_t ldx, double* Y, int64_t ldy,
                          int ncols, double scale, cudaStream_t st);
+// ---- one-shot steps in 64-bit fixed point (k_batch.cu): X [n_rows][ldx], the xi
+// half (without C^(k+1), value * 2^56) at column 0, W's half (value * 2^(56 - e))
+// at column rh; ldx even
+void launch_os_absmax(const double* W, int64_t count, unsigned int* out, cudaStream_t st);
+void launch_os_fix(const double* Wc, int n_pad, int r, int rh, int e, const int32_t* sinks,
+                   long long* X, int64_t ldx, cudaStream_t st);
+// Y = Q X by row chunks; recip[d] = 1 / d (PrepParams::recip)
+void launch_os_step(const ChunkList& L, const int32_t* col, const int32_t* len,
+                    const SweepScale* recip, const long long* X, long long* Y, int ldx,
+                    cudaStream_t st);
+// ck: C^(k+1) (PrepParams::cpow); f16: FP16 operands (bits: ldx words of
+// scratch), else TF32; as launch_pack_f16_oneshot / launch_pack_tc
+void launch_os_pack(const long long* X, int64_t ldx, int rh, int r, int slot, int rg, int n_rows,
+                    const SweepScale& ck, int e, int f16, unsigned int* bits, void* Ahi, void* Alo,
+                    int64_t kd, cudaStream_t st);
+void launch_os_pack_ffma(const long long* X, int64_t ldx, int rh, int r, int slot, int terms,
+                         int nT, const SweepScale& ck, int e, void* Pn, int p_prec, uint64_t* mXi,
+                         uint64_t* mEta, cudaStream_t st);
 // Edge weights of a weighted Q (all null: Q[a][b] = 1 / in-degree(a)):
 // out_w / in_w give the weight of each out-list / in-list entry by pool
 // position, wsum[a] the total in-weight of a.
@@ -428,7 +446,8 @@ void launch_partial_sim_block(const ChunkList& fwd, const ChunkList& hor, const 
                               void* y0, void* y1, void* result, void* scales, cudaStream_t st,
                               const WeightView& wv = WeightView(), int group0 = 1);
 // inv[a] = 1 / (in-degree or in-weight of a); the two steps below on FP64
-// blocks of row pitch ldb (a multiple of 4)
+// blocks of row pitch ldb (a multiple of 4): Y = Q^T X, and
+// Yn = add_scale Xadd (none: Xadd null) + Q Y
 void launch_col_scales64(const WeightView& wv, const int32_t* in_len, int n_rows, double* inv,
                          cudaStream_t st);
 void launch_col_forward64(const ChunkList& fwd, const int32_t* out_col, const WeightView& wv,

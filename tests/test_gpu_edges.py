@@ -131,3 +131,25 @@ def test_recurrence_at_warp_and_cta_edges(P, prec, kw, scale):
     sr.apply_updates(ups)
     err = np.max(np.abs(sr.dense() - want)) / max(1.0, np.max(np.abs(want)))
     assert err < (1e-10 if prec == 64 else 1e-6)
+
+
+@pytest.mark.parametrize("prec,tc", [(64, 0), (32, 0), (32, 1), (32, 2)])
+@pytest.mark.parametrize("sinks", [1, 3, 33, 70])
+def test_one_shot_at_chunk_and_column_edges(P, prec, tc, sinks):
+    """A batch as one rank-2r update on rows of 31..33, 64, 65 and 200 nonzeros
+    (row chunks hold 32), with 2 r columns inside one column group of 128 and
+    over it: one insertion into every sink, one deletion.  1e-10 (FP64) and
+    1e-6 (FP32), as in the one-shot parity tests."""
+    n, C, K = 300, 0.6, 6
+    s, d = degrees_graph(n, [0, 1, 31, 32, 33, 64, 65, 200], 13)
+    edges = set(zip(s.tolist(), d.tolist()))
+    ups = [(next(x for x in range(n) if x != j and (x, j) not in edges), j, 1) for j in range(sinks)]
+    ups.append((sorted(e for e in edges if e[1] == 7)[0][0], 7, -1))
+    ups = [u for u in ups if not (u[1] == 7 and u[2] == 1)]
+    new = (edges | {(i, j) for i, j, op in ups if op > 0}) - {(i, j) for i, j, op in ups if op < 0}
+    S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-15)
+    sr = P.SimRank(n, s, d, C=C, K=K, s_precision=prec, tc=tc, apply=P.APPLY_ONE_SHOT)
+    sr.apply_updates(ups)
+    ns, nd = (np.array(v, np.int64) for v in zip(*sorted(new)))
+    want = O.one_shot_batch(n, s, d, ns, nd, S0, C, K)
+    assert np.max(np.abs(sr.dense() - want)) < (1e-10 if prec == 64 else 1e-6)
