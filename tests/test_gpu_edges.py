@@ -153,3 +153,47 @@ def test_one_shot_at_chunk_and_column_edges(P, prec, tc, sinks):
     ns, nd = (np.array(v, np.int64) for v in zip(*sorted(new)))
     want = O.one_shot_batch(n, s, d, ns, nd, S0, C, K)
     assert np.max(np.abs(sr.dense() - want)) < (1e-10 if prec == 64 else 1e-6)
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+def test_many_graphs_at_run_edges(P, prec):
+    """Many-graph rounds whose runs cut rows at their edges: graphs of one node
+    and of a few edges (most threads without a run), rows of 31..33 nonzeros (the
+    two loading forms), rows longer than a thread's, a warp's and several
+    warps' runs, and a graph too large for the index form.  1e-10 (FP64) and
+    1e-6 (FP32), as in the many-graph parity tests."""
+    C, K = 0.6, 6
+    shapes = [(1, []), (3, [1]), (200, [0, 1, 31, 32, 33, 64, 65, 130]),
+              (1100, [1023, 700, 333, 5, 0, 96]), (4700 if prec == 64 else 6500, [900, 40])]
+    graphs, ups = [], []
+    for t, (n, degs) in enumerate(shapes):
+        if n == 1:
+            s = d = np.zeros(0, np.int32)
+        elif n == 3:
+            s, d = np.array([1], np.int32), np.array([0], np.int32)
+        else:
+            s, d = degrees_graph(n, degs, 17 + t)
+        edges = set(zip(s.tolist(), d.tolist()))
+        u = []
+        for j in range(min(n, 3) if n > 1 else 0):
+            i = next((x for x in range(n - 1, -1, -1) if x != j and (x, j) not in edges), None)
+            if i is not None:
+                u.append((i, j, 1))
+        if n > 3:
+            u.append((sorted(e for e in edges if e[1] == 2)[0][0], 2, -1))
+        graphs.append((n, s, d))
+        ups.append(np.array(u, np.int32).reshape(-1, 3))
+    mh = P.MultiSimRank(graphs, C=C, K=K, s_precision=prec)
+    mh.apply_updates(ups)
+    mh.sync()
+    for g, (n, s, d) in enumerate(graphs):
+        cols = np.unique(np.r_[0, n // 2, n - 1, [u for u in ups[g][:, 1].tolist()]]).astype(np.int32)
+        got = mh.columns(g, cols)
+        if n > 2000:
+            sr = P.SimRank(n, s, d, C=C, K=K, s_precision=64)
+            sr.apply_updates(ups[g])
+            want = sr.columns(cols)
+        else:
+            S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-14)
+            want = O.sequential_unit_updates(n, s, d, S0, ups[g].tolist(), C, K)[0][:, cols]
+        assert np.max(np.abs(got - want)) < (1e-10 if prec == 64 else 1e-6), g
