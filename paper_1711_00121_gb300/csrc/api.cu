@@ -15,6 +15,7 @@
 #include <utility>
 #include <vector>
 
+#include "edge_set.h"
 #include "sr_internal.h"
 
 using namespace sr;
@@ -44,7 +45,7 @@ struct simrank_ctx {
   int32_t* d_ext2int = nullptr;
   // host mirror of the graph (storage ids)
   HostAdj hin, hout;
-  std::unordered_set<uint64_t> edges;
+  EdgeSet edges;
   // device graph
   DevAdj din, dout;
   float* d_in_w = nullptr;
@@ -85,6 +86,14 @@ struct simrank_ctx {
   int64_t ops_cap = 0;
   int32_t* d_cols = nullptr;
   int64_t cols_cap = 0;
+  // pinned copy of a call's sources and patch ops, and when it may be rewritten
+  unsigned char* stage = nullptr;
+  size_t stage_bytes = 0;
+  cudaEvent_t stage_ev = nullptr;
+  // work buffers of re-anchors (at most ANCHOR_KEEP bytes in all), kept between calls
+  void* anchor_buf[3] = {nullptr, nullptr, nullptr};
+  size_t anchor_bytes = 0;
+  PrepFit prep_fit;  // co-resident CTAs of the pre-update launch
   // column mode (§7): snapshot of the initial graph and the stored updates
   bool column = false;
   int32_t* g0_in_col = nullptr;
@@ -165,25 +174,33 @@ cudaError_t dev_alloc(T** p, size_t count) {
   return cudaMalloc((void**)p, std::max<size_t>(count, 1) * sizeof(T));
 }
 
-// Builds adjacency lists (rows indexed by `key`, entries `val`) with per-row
-// slack.  Row capacities are multiples of 4, so every row starts on a 16-byte
-// boundary of the pool (vector loads of whole rows).
-void build_adj(HostAdj& A, int n_rows, const std::vector<std::vector<int32_t>>& rows) {
+// Builds adjacency lists (row key[e] gets val[e], in the order of e) with
+// per-row slack.  Row capacities are multiples of 4, so every row starts on a
+// 16-byte boundary of the pool (vector loads of whole rows).  w (nullable): the
+// entries' weights, put at the same places of wpool.
+void build_adj(HostAdj& A, int n_rows, const std::vector<int32_t>& key,
+               const std::vector<int32_t>& val, const float* w = nullptr,
+               std::vector<float>* wpool = nullptr) {
   A.start.assign(n_rows, 0);
   A.len.assign(n_rows, 0);
   A.cap.assign(n_rows, 0);
+  for (int32_t a : key) A.len[a] += 1;
   int64_t used = 0;
   for (int a = 0; a < n_rows; ++a) {
-    const int len = (int)rows[a].size();
+    const int len = A.len[a];
     const int cap = (len + std::max(4, len / 4) + 3) & ~3;
     A.start[a] = used;
-    A.len[a] = len;
     A.cap[a] = cap;
     used += cap;
   }
   A.pool.assign((size_t)(used + used / 4 + 65536), 0);
-  for (int a = 0; a < n_rows; ++a)
-    std::copy(rows[a].begin(), rows[a].end(), A.pool.begin() + A.start[a]);
+  if (wpool) wpool->assign(A.pool.size(), 0.f);
+  std::vector<int64_t> at(A.start);
+  for (size_t e = 0; e < key.size(); ++e) {
+    const int64_t q = at[key[e]]++;
+    A.pool[q] = val[e];
+    if (wpool) (*wpool)[q] = w[e];
+  }
   A.used = used;
 }
 
@@ -306,14 +323,16 @@ simrank_status validate(simrank_ctx* h, const simrank_update* u, int64_t count, 
   std::unordered_set<int32_t> fresh;
   for (int64_t t = 0; t < count; ++t) {
     const int32_t s = u[t].src, d = u[t].dst;
-    const std::string at = " (update " + std::to_string(t) + ": " + std::to_string(s) + " -> " +
-                           std::to_string(d) + ")";
-    if (u[t].op != 1 && u[t].op != -1) return fail(h, SR_ERR_ARG, "op must be +1 or -1" + at);
-    if (s < 0 || d < 0) return fail(h, SR_ERR_ARG, "negative node id" + at);
-    if (s == d) return fail(h, SR_ERR_EDGE_EXISTS, "self-loop" + at);
+    auto at = [&]() {
+      return " (update " + std::to_string(t) + ": " + std::to_string(s) + " -> " +
+             std::to_string(d) + ")";
+    };
+    if (u[t].op != 1 && u[t].op != -1) return fail(h, SR_ERR_ARG, "op must be +1 or -1" + at());
+    if (s < 0 || d < 0) return fail(h, SR_ERR_ARG, "negative node id" + at());
+    if (s == d) return fail(h, SR_ERR_EDGE_EXISTS, "self-loop" + at());
     for (int32_t x : {s, d}) {
       if (x >= h->n_cur) {
-        if (x >= h->n_cap) return fail(h, SR_ERR_CAPACITY, "n_capacity exceeded" + at);
+        if (x >= h->n_cap) return fail(h, SR_ERR_CAPACITY, "n_capacity exceeded" + at());
         fresh.insert(x);
         max_id = std::max(max_id, (int)x);
       }
@@ -324,12 +343,12 @@ simrank_status validate(simrank_ctx* h, const simrank_update* u, int64_t count, 
     if (it != overlay.end())
       present = it->second != 0;
     else
-      present = h->edges.count(k) != 0;
+      present = h->edges.contains(k);
     if (u[t].op > 0) {
-      if (present) return fail(h, SR_ERR_EDGE_EXISTS, "inserting an existing edge" + at);
+      if (present) return fail(h, SR_ERR_EDGE_EXISTS, "inserting an existing edge" + at());
       overlay[k] = 1;
     } else {
-      if (!present) return fail(h, SR_ERR_EDGE_MISSING, "deleting an absent edge" + at);
+      if (!present) return fail(h, SR_ERR_EDGE_MISSING, "deleting an absent edge" + at());
       overlay[k] = 0;
     }
   }
@@ -351,6 +370,41 @@ simrank_status ensure_dev_capacity(simrank_ctx* h, int64_t nsrc, int64_t nops) {
     h->ops_cap = std::max<int64_t>(nops, 2 * h->ops_cap);
     CUDA_TRY(h, dev_alloc(&h->d_ops, (size_t)h->ops_cap));
   }
+  return SR_OK;
+}
+
+// The sources and patch ops of a call to d_srcs / d_ops through pinned memory
+// of the handle, so that the copies need no wait; a call of more than
+// STAGE_KEEP bytes copies from its own vectors and waits.
+constexpr size_t STAGE_KEEP = 4u << 20;
+simrank_status upload_plan(simrank_ctx* h, const std::vector<int32_t>& srcs,
+                           const std::vector<PatchOp>& ops) {
+  const size_t ob = ops.size() * sizeof(PatchOp), sb = srcs.size() * sizeof(int32_t);
+  const bool pin = ob + sb <= STAGE_KEEP;
+  const void *po = ops.data(), *ps = srcs.data();
+  if (pin) {
+    if (!h->stage_ev)
+      CUDA_TRY(h, cudaEventCreateWithFlags(&h->stage_ev, cudaEventDisableTiming));
+    CUDA_TRY(h, cudaEventSynchronize(h->stage_ev));  // the copies of the last call
+    if (ob + sb > h->stage_bytes) {
+      if (h->stage) cudaFreeHost(h->stage);
+      h->stage = nullptr;
+      h->stage_bytes = 0;
+      const size_t want = std::max<size_t>(2 * (ob + sb), 16384);
+      CUDA_TRY(h, cudaHostAlloc((void**)&h->stage, want, cudaHostAllocDefault));
+      h->stage_bytes = want;
+    }
+    if (ob) std::memcpy(h->stage, po, ob);
+    if (sb) std::memcpy(h->stage + ob, ps, sb);
+    po = h->stage;
+    ps = h->stage + ob;
+  }
+  if (sb) CUDA_TRY(h, cudaMemcpyAsync(h->d_srcs, ps, sb, cudaMemcpyHostToDevice, h->st));
+  if (ob) CUDA_TRY(h, cudaMemcpyAsync(h->d_ops, po, ob, cudaMemcpyHostToDevice, h->st));
+  if (pin)
+    CUDA_TRY(h, cudaEventRecord(h->stage_ev, h->st));
+  else
+    CUDA_TRY(h, cudaStreamSynchronize(h->st));
   return SR_OK;
 }
 
@@ -717,7 +771,7 @@ simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, i
     const int rc = launch_prep(pp, h->cfg.s_precision, h->cfg.vec_fp64 ? 1 : 0,
                                defer ? group(h) * h->K1 : 0,
                                h->num_sms, h->cfg.prep_ctas, (int64_t)h->edges.size() + delta,
-                               h->st);
+                               h->prep_fit, h->st);
     if (rc == 1) return fail(h, SR_ERR_CUDA, "fused pre-update launch failed");
     fused = (rc == 0);
     if (fused) {
@@ -829,6 +883,7 @@ std::vector<SweepScale> sweep_scales(const HostAdj& A, int n_rows, double C) {
 // FP32, 1e-12 in FP64; both hold for every S of Eq. 1): `known` says so without
 // a look at S, otherwise a pass over S decides, and any other S (a caller's S0)
 // is swept in FP64 as it is.
+constexpr size_t ANCHOR_KEEP = (size_t)4 << 30;
 simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double* last_diff,
                              int* sweeps_done, double* tol_used = nullptr,
                              double* first_diff = nullptr, bool known = false) {
@@ -846,8 +901,13 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
   double prev = INFINITY;
   void* bufs[3] = {nullptr, nullptr, nullptr};
   const bool alias = (wp == sp);
+  // buffers that a re-anchor left (see below) serve this one
+  const bool held = !alias && h->anchor_bytes == bytes;
   for (int b = (alias ? 1 : 0); b < 3; ++b) {
-    if (cudaMalloc(&bufs[b], bytes) != cudaSuccess) {
+    if (held) {
+      bufs[b] = h->anchor_buf[b];
+    } else if (cudaMalloc(&bufs[b], bytes) != cudaSuccess) {
+      cudaGetLastError();
       for (void* p : bufs)
         if (p) cudaFree(p);
       return fail(h, SR_ERR_OOM, "cudaMalloc of Jacobi buffers failed");
@@ -948,9 +1008,17 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
   if (scales) cudaFree(scales);
   // bufs[] holds three distinct buffers (bufs[0] is the old S when aliasing);
   // keep the result as S when aliasing and free every other buffer once.
+  // A re-anchor of an FP32 S keeps them when they are small (allocating and
+  // freeing 3 x 0.8 GB took 2.2 of 5.8 ms at n = 10,007).
   if (alias && e == cudaSuccess) h->S = A;
-  for (int b = 0; b < 3; ++b)
-    if (bufs[b] && bufs[b] != h->S) cudaFree(bufs[b]);
+  const bool keep = !alias && !known && 3 * bytes <= ANCHOR_KEEP;
+  for (int b = 0; b < 3; ++b) {
+    if (keep)
+      h->anchor_buf[b] = bufs[b];
+    else if (bufs[b] && bufs[b] != h->S)
+      cudaFree(bufs[b]);
+  }
+  if (keep) h->anchor_bytes = bytes;
   if (e != cudaSuccess)
     return fail(h, SR_ERR_CUDA, std::string("Jacobi sweep: ") + cudaGetErrorString(e));
   *last_diff = diff;
@@ -994,6 +1062,18 @@ simrank_status ob_ensure(simrank_ctx* h, int slot, size_t bytes) {
   b.bytes = 0;
   CUDA_TRY(h, cudaMalloc(&b.p, std::max<size_t>(bytes, 256)));
   b.bytes = bytes;
+  return SR_OK;
+}
+
+// Device memory for columns on their way to the host: the handle's own up to
+// 64 MB, else one allocation of the call (the caller frees what is not ob[29]).
+simrank_status columns_scratch(simrank_ctx* h, size_t bytes, void** p) {
+  if (bytes <= (64u << 20)) {
+    const simrank_status s = ob_ensure(h, 29, bytes);
+    *p = h->ob[29].p;
+    return s;
+  }
+  CUDA_TRY(h, cudaMalloc(p, bytes));
   return SR_OK;
 }
 
@@ -1441,9 +1521,12 @@ simrank_status column_mode_columns(simrank_ctx* h, const int32_t* cols, int ncol
   void* dst = out;
   void* tmp = nullptr;
   if (!out_on_device) {
-    CUDA_TRY(h, cudaMalloc(&tmp, ob));
+    if ((s = columns_scratch(h, ob, &tmp)) != SR_OK) return s;
     dst = tmp;
   }
+  auto drop = [&]() {
+    if (tmp && tmp != h->ob[29].p) cudaFree(tmp);
+  };
   for (int c0 = 0; c0 < ncols; c0 += Bmax) {
     const int B = std::min(Bmax, ncols - c0);
     const int ldb = B > 4 ? (B + 3) & ~3 : B;  // wide blocks: 16-byte rows
@@ -1475,14 +1558,14 @@ simrank_status column_mode_columns(simrank_ctx* h, const int32_t* cols, int ncol
                    (unsigned char*)dst + (size_t)c0 * h->n_cur * (out_fp64 ? 8 : 4), out_fp64, h->st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
-      if (tmp) cudaFree(tmp);
+      drop();
       return fail(h, SR_ERR_CUDA, std::string("column mode: ") + cudaGetErrorString(e));
     }
   }
   cudaError_t e = cudaSuccess;
   if (!out_on_device) e = cudaMemcpyAsync(out, tmp, ob, cudaMemcpyDeviceToHost, h->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
-  if (tmp) cudaFree(tmp);
+  drop();
   if (e != cudaSuccess) return fail(h, SR_ERR_CUDA, std::string("column mode: ") + cudaGetErrorString(e));
   return SR_OK;
 }
@@ -1501,6 +1584,10 @@ void free_ctx(simrank_ctx* h) {
     if (p) cudaFree(p);
   for (auto& b : h->ob)
     if (b.p) cudaFree(b.p);
+  for (void* p : h->anchor_buf)
+    if (p) cudaFree(p);
+  if (h->stage) cudaFreeHost(h->stage);
+  if (h->stage_ev) cudaEventDestroy(h->stage_ev);
   if (h->Pp) cudaFree(h->Pp);
   if (h->pXi) cudaFree(h->pXi);
   if (h->pEta) cudaFree(h->pEta);
@@ -1676,38 +1763,25 @@ simrank_status simrank_init(const simrank_config* cfg_in, int32_t n, int64_t m, 
   }
 
   // --- host graph (storage ids), validated
-  std::vector<std::vector<int32_t>> in_rows(h->n_pad), out_rows(h->n_pad);
-  std::vector<std::vector<float>> in_w(h->weighted ? h->n_pad : 0), out_w(h->weighted ? h->n_pad : 0);
-  h->edges.reserve((size_t)m * 2 + 16);
+  h->edges.reserve((size_t)m + 16);
+  h->init_src.reserve((size_t)m);
+  h->init_dst.reserve((size_t)m);
   for (int64_t e = 0; e < m; ++e) {
     const int32_t s = src[e], d = dst[e];
     if (s < 0 || d < 0 || s >= n || d >= n)
       return bail(fail(h, SR_ERR_ARG, "edge " + std::to_string(e) + " has an id outside [0, n)"));
     if (s == d) return bail(fail(h, SR_ERR_EDGE_EXISTS, "self-loop at edge " + std::to_string(e)));
-    if (!h->edges.insert(ekey(s, d)).second)
+    const int32_t si = h->ext2int[s], di = h->ext2int[d];
+    if (!h->edges.insert(ekey(si, di)))
       return bail(fail(h, SR_ERR_EDGE_EXISTS, "duplicate edge " + std::to_string(e)));
     if (h->weighted && !(weight[e] > 0.0f))
       return bail(fail(h, SR_ERR_ARG, "edge weights must be > 0"));
-    const int32_t si = h->ext2int[s], di = h->ext2int[d];
-    in_rows[di].push_back(si);
-    out_rows[si].push_back(di);
-    if (h->weighted) {
-      in_w[di].push_back(weight[e]);
-      out_w[si].push_back(weight[e]);
-    }
     h->init_src.push_back(si);
     h->init_dst.push_back(di);
   }
-  if (h->relabeled) {
-    // the duplicate check above ran on caller ids; keep the edge set in storage ids
-    std::unordered_set<uint64_t> mapped;
-    mapped.reserve(h->edges.size() * 2 + 16);
-    for (uint64_t k : h->edges)
-      mapped.insert(ekey(h->ext2int[(int32_t)(k >> 32)], h->ext2int[(int32_t)(k & 0xffffffffu)]));
-    h->edges.swap(mapped);
-  }
-  build_adj(h->hin, h->n_pad, in_rows);
-  build_adj(h->hout, h->n_pad, out_rows);
+  std::vector<float> wpool, opool;  // weights by pool position
+  build_adj(h->hin, h->n_pad, h->init_dst, h->init_src, weight, h->weighted ? &wpool : nullptr);
+  build_adj(h->hout, h->n_pad, h->init_src, h->init_dst, weight, h->weighted ? &opool : nullptr);
 
   // --- forest form of the initial S (Example 2): each node's parent (its one
   // in-neighbour) and level; nodes beyond n are isolated roots
@@ -1717,10 +1791,10 @@ simrank_status simrank_init(const simrank_config* cfg_in, int32_t n, int64_t m, 
     f_parent.assign(h->n_cap, -1);
     f_level.assign(h->n_cap, -1);
     for (int x = 0; x < n; ++x) {
-      if (in_rows[x].size() > 1)
+      if (h->hin.len[x] > 1)
         return bail(fail(h, SR_ERR_ARG, "SR_INIT_FOREST needs every in-degree <= 1 (node " +
                                             std::to_string(h->int2ext[x]) + ")"));
-      if (!in_rows[x].empty()) f_parent[x] = in_rows[x][0];
+      if (h->hin.len[x] == 1) f_parent[x] = h->hin.pool[h->hin.start[x]];
     }
     std::vector<int32_t> path;
     for (int x = 0; x < h->n_cap; ++x) {
@@ -1756,15 +1830,9 @@ simrank_status simrank_init(const simrank_config* cfg_in, int32_t n, int64_t m, 
   if ((s = upload_adj(h->din, h->hin)) != SR_OK) return bail(s);
   if ((s = upload_adj(h->dout, h->hout)) != SR_OK) return bail(s);
   if (h->weighted) {
-    std::vector<float> wpool(h->hin.pool.size(), 0.f), opool(h->hout.pool.size(), 0.f);
     std::vector<double> wsum(h->n_pad, 0.0);
-    for (int a = 0; a < h->n_pad; ++a) {
-      for (size_t e = 0; e < in_w[a].size(); ++e) {
-        wpool[h->hin.start[a] + e] = in_w[a][e];
-        wsum[a] += in_w[a][e];
-      }
-      for (size_t e = 0; e < out_w[a].size(); ++e) opool[h->hout.start[a] + e] = out_w[a][e];
-    }
+    for (int a = 0; a < h->n_pad; ++a)
+      for (int e = 0; e < h->hin.len[a]; ++e) wsum[a] += wpool[h->hin.start[a] + e];
     if (cudaMalloc(&h->d_in_w, wpool.size() * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&h->d_out_w, opool.size() * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&h->d_wsum, wsum.size() * sizeof(double)) != cudaSuccess)
@@ -2077,13 +2145,7 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
   if ((s = grow_pool(h, h->din, h->hin)) != SR_OK) return s;
   if ((s = grow_pool(h, h->dout, h->hout)) != SR_OK) return s;
   if ((s = ensure_dev_capacity(h, (int64_t)srcs.size() + 2, (int64_t)ops.size())) != SR_OK) return s;
-  CUDA_TRY(h, cudaMemcpyAsync(h->d_srcs, srcs.data(), srcs.size() * sizeof(int32_t),
-                              cudaMemcpyHostToDevice, h->st));
-  if (!ops.empty())
-    CUDA_TRY(h, cudaMemcpyAsync(h->d_ops, ops.data(), ops.size() * sizeof(PatchOp),
-                                cudaMemcpyHostToDevice, h->st));
-  // the staging vectors must outlive the asynchronous copies
-  CUDA_TRY(h, cudaStreamSynchronize(h->st));
+  if ((s = upload_plan(h, srcs, ops)) != SR_OK) return s;
   for (const R1& r : plan) {
     if ((s = run_rank_one(h, r.src_off, r.delta, r.sink, r.op, r.d_j, r.op_begin, r.op_end)) !=
         SR_OK)
@@ -2124,13 +2186,14 @@ simrank_status simrank_columns(simrank_t h, const int32_t* cols, int32_t ncols, 
     return SR_OK;
   }
   void* tmp = nullptr;
-  CUDA_TRY(h, cudaMalloc(&tmp, ob));
+  simrank_status s = columns_scratch(h, ob, &tmp);
+  if (s != SR_OK) return s;
   launch_copy_cols(h->S, h->cfg.s_precision, h->ld, h->d_cols, perm, ncols, h->n_cur, tmp,
                    out_fp64, h->st, upper(h));
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, tmp, ob, cudaMemcpyDeviceToHost, h->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
-  cudaFree(tmp);
+  if (tmp != h->ob[29].p) cudaFree(tmp);
   if (e != cudaSuccess) return fail(h, SR_ERR_CUDA, std::string("columns: ") + cudaGetErrorString(e));
   return SR_OK;
 }

@@ -1326,7 +1326,7 @@ void launch_flow_recip(SweepScale* out, int count, cudaStream_t st) {
 }
 
 int launch_prep(const PrepParams& prm, int s_prec, int vec64, int npend_max, int num_sms,
-                int max_ctas, int64_t nnz_bound, cudaStream_t st) {
+                int max_ctas, int64_t nnz_bound, PrepFit& fit, cudaStream_t st) {
   if (prm.nT <= 0) return 0;
   if (prm.item < 0 || prm.cap < 0 || (prm.cap & 3)) return 1;
   const size_t smem = (s_prec == 64) ? prep_smem<double>(prm.cap, prm.nT_cap, npend_max)
@@ -1334,12 +1334,23 @@ int launch_prep(const PrepParams& prm, int s_prec, int vec64, int npend_max, int
   const void* fn = (s_prec == 64) ? (const void*)k_prep<double, double>
                    : vec64        ? (const void*)k_prep<double, float>
                                   : (const void*)k_prep<float, float>;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
-    return 1;
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, PG, smem) != cudaSuccess)
-    return 1;
+  if (fit.fn != fn || fit.smem != smem) {
+    // the limit is the device's, not this launch's, so that no handle lowers
+    // another's (per device: smem_attr_once)
+    static std::atomic<unsigned long long> done[3];
+    cudaFuncAttributes fa;
+    int dev = 0, most = 0, per_sm = 0;
+    if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+      return 1;
+    const int which = s_prec == 64 ? 0 : vec64 ? 1 : 2;
+    if (smem_attr_once(fn, most - (int)fa.sharedSizeBytes, done[which]) != cudaSuccess) return 1;
+    if (smem > (size_t)most - fa.sharedSizeBytes) return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, PG, smem) != cudaSuccess)
+      return 1;
+    fit = PrepFit{fn, smem, per_sm};
+  }
+  const int per_sm = fit.per_sm;
   if (per_sm <= 0) return 2;
   // one CTA per item (at most nT + nnz / item of them), at most all
   // co-resident CTAs

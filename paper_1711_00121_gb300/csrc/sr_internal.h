@@ -195,8 +195,15 @@ struct PrepParams {
 };
 // out[d] = 1 / d for d < count (PrepParams::recip)
 void launch_flow_recip(SweepScale* out, int count, cudaStream_t st);
+// fit: the co-resident CTAs per SM found for a kernel and its shared memory,
+// asked for again when either changes.
+struct PrepFit {
+  const void* fn = nullptr;
+  size_t smem = 0;
+  int per_sm = 0;
+};
 int launch_prep(const PrepParams& p, int s_prec, int vec64, int npend_max, int num_sms,
-                int max_ctas, int64_t nnz_bound, cudaStream_t st);
+                int max_ctas, int64_t nnz_bound, PrepFit& fit, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Many independent graphs advanced together (k_multi.cu).
