@@ -93,7 +93,9 @@ typedef struct simrank_config {
                              an exact power-of-two balancing of each term (twice the tensor rate);
                              used, with FP32 S, for the one-shot batch form's pass and for the
                              pass of every unit / sink-block update (or of every group of `defer`
-                             pending updates); 0 = CUDA cores */
+                             pending updates); 0 = no split: FP32 FMAs, or digits whose
+                             products the tensor cores sum exactly (as for FP64 S) where
+                             that is faster */
   int32_t init_max_sweeps;/* cap on Jacobi sweeps of Eq. 1 at init / re-anchor */
   double init_tol;        /* init stops when a sweep changes S by less than this (max-abs);
                              <= 0 selects 1e-13 (sweeps stored in FP32 stop at 1e-7 or at
@@ -103,8 +105,9 @@ typedef struct simrank_config {
                              update can reach (Thm 4) fill whole tiles; ids in the ABI are unchanged */
   int64_t timeout_iters;  /* bound on any device spin-wait (0 = library default) */
   void* cuda_stream;      /* cudaStream_t for all work of this handle; NULL = default stream */
-  int32_t s_kernel;       /* CUDA-core S update with S in FP32: 0 = warp-specialised (math and
-                             memory warps overlap), 1 = single-role kernel */
+  int32_t s_kernel;       /* S update with S in FP32 and tc = 0: 0 = warp-specialised (math and
+                             memory warps overlap) or, for 12 to 16 terms and n > 4,992,
+                             exact digits; 1 = single-role CUDA-core kernel */
   int32_t defer;          /* dense FP32 S, unit / sink-block apply, fused update: 0 or 1 = apply
                              each rank-one update to S at once; G > 1 = keep up to G updates'
                              panels pending (the rows of S an update reads are corrected by them)

@@ -472,6 +472,22 @@ void* panel_for_s(simrank_ctx* h) {
   return h->cfg.s_precision == 64 ? (void*)h->P64 : (void*)h->P32;
 }
 
+simrank_status ob_ensure(simrank_ctx* h, int slot, size_t bytes);
+
+// Whether an update's pass takes the exact digits of the tensor cores: all its
+// terms at once and the upper tiles only.  In FP64 from 3 terms on (one update
+// with 2, 3 and 4 terms at n = 4,000: 73, 96 and 105 us, with FP64 FMAs 74, 122
+// and 167; at n = 120 from 2 terms on), in FP32 for 12 to 16 terms (one pass of
+// 16; its time hardly depends on their number) and n above 4,992, where the
+// digits' own 10 us are less than what the pass saves: K = 11 and 15 at n = 6,000
+// 107 and 112 us an update, with FP32 FMAs 111 and 127; at n = 4,000 86 and 91,
+// 85 and 92; K = 8 at n = 8,191 139 and 131.
+bool use_digits(const simrank_ctx* h, int k0, int k1, int nT) {
+  if (!upper(h) || k0 != 0 || k1 != h->K1) return false;
+  if (h->cfg.s_precision == 64) return h->K1 >= 3;
+  return h->cfg.s_kernel == 0 && h->K1 >= 12 && h->K1 <= 16 && nT >= 40;
+}
+
 simrank_status s_update_launch(simrank_ctx* h, int k0, int k1, int use_masks) {
   std::pair<cudaEvent_t, cudaEvent_t>* ev = nullptr;
   if (h->cfg.profile) {
@@ -484,18 +500,31 @@ simrank_status s_update_launch(simrank_ctx* h, int k0, int k1, int use_masks) {
     CUDA_TRY(h, cudaEventRecord(ev->first, h->st));
   }
   const bool ws = h->cfg.s_precision == 32 && h->cfg.s_kernel == 0;
-  launch_s_update(h->S, h->cfg.s_precision, h->ld, panel_for_s(h), h->K1, h->tiles, h->ntiles,
-                  h->mXi, h->mEta, k0, k1, use_masks, h->n_cur, h->counters,
-                  s_update_grid(h->cfg.s_precision, h->num_sms, ws), h->st,
-                  ws ? wait_limit(h) : 0, upper(h));
+  const int nT = (h->n_cur + PT - 1) / PT;
+  bool digits = use_digits(h, k0, k1, nT);
+  if (digits && ob_ensure(h, 30, digits_scratch_bytes(h->cfg.s_precision, h->n_pad)) != SR_OK) {
+    digits = false;  // no memory for the digits
+    h->err.clear();
+    cudaGetLastError();
+  }
+  if (digits) {
+    if (launch_s_update_digits(h->S, h->cfg.s_precision, h->ld, panel_for_s(h), h->K1, nT,
+                               h->n_pad, h->tiles, h->ntiles, h->mXi, h->mEta, use_masks, h->n_cur,
+                               h->ob[30].p, h->counters, h->num_sms, wait_limit(h), h->st) != 0)
+      return fail(h, SR_ERR_CUDA, "tensor-core S update: launch setup failed");
+    h->launches += 3 * ((h->K1 + 15) / 16) - 1;
+  } else {
+    launch_s_update(h->S, h->cfg.s_precision, h->ld, panel_for_s(h), h->K1, h->tiles, h->ntiles,
+                    h->mXi, h->mEta, k0, k1, use_masks, h->n_cur, h->counters,
+                    s_update_grid(h->cfg.s_precision, h->num_sms, ws), h->st,
+                    ws ? wait_limit(h) : 0, upper(h));
+  }
   LAUNCH_CHECK(h);
   if (ev) CUDA_TRY(h, cudaEventRecord(ev->second, h->st));
   h->prof_launches += 1;
   h->launches += 1;
   return SR_OK;
 }
-
-simrank_status ob_ensure(simrank_ctx* h, int slot, size_t bytes);
 
 // Updates go through the pending-panel buffer: G > 1 pending updates share
 // one S pass, or (tc = 1) each update's S pass runs on the tensor cores.

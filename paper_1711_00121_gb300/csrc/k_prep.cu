@@ -812,7 +812,9 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
   if (alive && p.flat) {
     const float mI = __uint_as_float(__ldcg(p.bar + 2)), mJ = __uint_as_float(__ldcg(p.bar + 3));
     // bounds of Thm 3 / Thm 9 / Table 2 with |w_j|, |S_II| / delta^2 <= max |sI| / delta
-    const float invC = (float)p.inv_C, gq = fabsf((float)p.gq), m1 = mI * (float)p.inv_delta;
+    // (a first in-link's gamma has no other terms)
+    const float gq = p.d_j == 0 ? 0.f : fabsf((float)p.gq);
+    const float invC = (float)p.inv_C, m1 = mI * (float)p.inv_delta;
     const float lam = 3.f * m1 + mJ * invC + invC + 1.f;
     const float g = fmaxf(2.f * m1, gq * (m1 + mJ * invC + 0.5f * gq * lam + invC + 1.f)) * 1.01f;
     finite = mI <= 3.0e38f && mJ <= 3.0e38f && g <= 3.0e38f;

@@ -23,19 +23,18 @@
 // Every mbarrier wait is bounded and every stop decision of the epilogue
 // warps is taken by all of them: on timeout the kernel records a status word,
 // skips the remaining work and still frees its TMEM.
-#include <cuda.h>
-
 #include <type_traits>
 
 #include "sr_internal.h"
+#include "tc_util.h"
 
 namespace sr {
 
 namespace {
 
-constexpr int TM = 128;             // rows of an S tile (M)
+constexpr int TM = TC_ROWS;         // rows of an S tile (M)
 constexpr int TN = 128;             // columns of an S tile (N)
-constexpr int KB = 128;             // bytes of K per stage (one 128-byte swizzle row)
+constexpr int KB = TC_KB;           // bytes of K per stage (one 128-byte swizzle row)
 constexpr int STAGES_STAGED = 2;  // stages when the epilogue stages D in shared memory
 constexpr int STAGES_DIRECT = 3;  // stages when it adds D to S straight from registers
 constexpr int OPB = TM * KB;        // bytes of one operand box: 16 KB
@@ -55,76 +54,6 @@ constexpr uint32_t IDESC_TF32_N256 = (1u << 4) | (2u << 7) | (2u << 10) |
                                      ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 constexpr uint32_t IDESC_F16_N256 = (1u << 4) | (0u << 7) | (0u << 10) |
                                     ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-// Bounded wait for the phase of `parity` to complete.  Returns false on timeout.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long limit,
-                                          volatile int* abort_flag) {
-  for (long long it = 0; it < limit; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.b32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if ((it & 1023) == 1023 && *abort_flag) return false;
-  }
-  return false;
-}
-
-// Wait with a fixed bound of its own, for draining copies and MMAs in flight
-// after a stop (their completion does not depend on any other thread).
-__device__ __forceinline__ void mbar_drain_wait(uint32_t bar, uint32_t parity) {
-  for (long long it = 0; it < (1ll << 24); ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.b32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return;
-  }
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
-                                            uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups
-// 1024 bytes apart (SBO), descriptor version 1.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)(16u >> 4) << 16;
-  d |= (uint64_t)(1024u >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
 
 template <bool F16>
 __device__ __forceinline__ void mma_k32b(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
@@ -163,12 +92,6 @@ __device__ __forceinline__ void mma_k32b_d(uint32_t tmem_d, uint64_t adesc, uint
   }
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   bar)
-               : "memory");
-}
-
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   uint32_t r[32];
   asm volatile(
@@ -186,17 +109,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
 }
 
-// true on all 256 epilogue threads iff pred is true on all of them (barrier 1)
-__device__ __forceinline__ bool ep_all(bool pred) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, 1, 256, p;\n"
-      " selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r)
-      : "r"((uint32_t)pred)
-      : "memory");
-  return r != 0;
-}
 __device__ __forceinline__ void ep_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 // One tile pair of the pass: where its S lives, the rows of its two operand
@@ -859,39 +771,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(TMEM_COLS_PAIR));
   }
-}
-
-using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
-                              CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                              CUtensorMapFloatOOBfill);
-
-EncodeFn encode_fn() {
-  static EncodeFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (EncodeFn)p;
-  }
-  return fn;
-}
-
-// Row-major [rows][kd] operand of 4-byte (FP32/TF32) or 2-byte (FP16)
-// elements; boxes of 128 rows x 128 bytes.
-bool make_map(CUtensorMap* m, const void* ptr, int64_t rows, int64_t kd, int eb) {
-  EncodeFn f = encode_fn();
-  if (!f) return false;
-  const cuuint64_t dims[2] = {(cuuint64_t)kd, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)kd * eb};
-  const cuuint32_t box[2] = {(cuuint32_t)(KB / eb), (cuuint32_t)TM};
-  const cuuint32_t estr[2] = {1, 1};
-  return f(m, eb == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-           const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace

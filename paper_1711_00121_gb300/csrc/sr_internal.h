@@ -280,6 +280,15 @@ void launch_s_update(void* S, int s_prec, int64_t ld, const void* P, int K1, con
                      const int* ntiles, const uint64_t* mXi, const uint64_t* mEta, int k0, int k1,
                      int use_masks, int n, int64_t* counters, int grid, cudaStream_t st,
                      long long ws_wait_limit = 0, int upper = 0);
+// The pass of one update's K1 terms over the upper tile pairs listed, by exact
+// digits on the tensor cores (k_digits.cu), DG_TERMS terms a pass.
+// scratch: digits_scratch_bytes.  Returns 0 on launch.
+size_t digits_scratch_bytes(int s_prec, int n_pad);
+int launch_s_update_digits(void* S, int s_prec, int64_t ld, const void* P, int K1, int nT,
+                           int n_pad, const uint32_t* tiles, const int* ntiles,
+                           const uint64_t* mXi, const uint64_t* mEta, int use_masks, int n,
+                           void* scratch, int64_t* counters, int grid, long long wait_limit,
+                           cudaStream_t st);
 // Persistent grid for launch_s_update on this device (ws: warp-specialised).
 int s_update_grid(int s_prec, int num_sms, bool ws = false);
 

@@ -197,3 +197,51 @@ def test_many_graphs_at_run_edges(P, prec):
             S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-14)
             want = O.sequential_unit_updates(n, s, d, S0, ups[g].tolist(), C, K)[0][:, cols]
         assert np.max(np.abs(got - want)) < (1e-10 if prec == 64 else 1e-6), g
+
+
+@pytest.mark.parametrize("prec,K,n,kw", [(64, 2, 2, {}), (64, 14, 2, {}), (64, 15, 700, {}),
+                                         (64, 16, 641, {"aff": 0}), (64, 32, 640, {}),
+                                         (32, 11, 5000, {}), (32, 15, 5120, {"aff": 0})])
+@pytest.mark.parametrize("form", ["plain", "huge", "tiny", "inf"])
+def test_digit_pass_at_term_and_tile_edges(P, prec, K, n, kw, form):
+    """The S pass by exact digits: 3, 15, 16, 17 and 33 terms (16 a pass), node
+    counts at and off the tiles of 128, all pairs or the affected ones, entries
+    of S0 of other magnitudes, and the direct sum at an infinite entry (inf and
+    NaN where the pass of a mirrored S has them).  Relative to the largest
+    entry, an update's terms and S are rounded to 2^-53 (FP32: 2^-24) some
+    2 (K + 1) + 1 times, as in the product of the oracle: 4 updates, K <= 32,
+    stay below 4 * 67 * 2^-52 < 1e-13 (FP32: 4 * 67 * 2^-24 < 2e-5)."""
+    C = 0.6
+    s, d = degrees_graph(n, [0, 1, 5, 64, 65][:n], 17)
+    edges = set(zip(s.tolist(), d.tolist()))
+    if n < 1000:
+        S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-14)
+    else:
+        S0 = np.random.default_rng(5).random((n, n))
+        S0 = 0.5 * (S0 + S0.T)
+    S0 *= {"huge": 1e12, "tiny": 1e-12}.get(form, 1.0)
+    if form == "inf":
+        S0[0, 0] = np.inf
+    ups = []
+    for j, op in ((0, 1), (4, 1), (3, -1), (n // 2, 1)):
+        j %= n
+        cand = [x for x in range(n) if x != j and ((x, j) in edges) == (op < 0)]
+        if cand and (cand[len(cand) // 2], j) not in [u[:2] for u in ups]:
+            ups.append((cand[len(cand) // 2], j, op))
+    sr = P.SimRank(n, s, d, S0=S0, C=C, K=K, s_precision=prec, upper_only=1, **kw)
+    sr.apply_updates(ups)
+    got = sr.dense()
+    if form == "inf":
+        old = P.SimRank(n, s, d, S0=S0, C=C, K=K, s_precision=prec, upper_only=0, **kw)
+        old.apply_updates(ups)
+        want = old.dense()
+        np.testing.assert_array_equal(np.isnan(got), np.isnan(want))
+        np.testing.assert_array_equal(np.isinf(got), np.isinf(want))
+        ok = np.isfinite(want)
+    else:
+        want = S0.astype(np.float64 if prec == 64 else np.float32).astype(np.float64)
+        want, _ = O.sequential_unit_updates(n, s, d, want, ups, C, K)
+        ok = np.ones_like(want, bool)
+    if ok.any():
+        err = np.max(np.abs(got[ok] - want[ok])) / max(1e-12, np.max(np.abs(want[ok])))
+        assert err < (1e-13 if prec == 64 else 2e-5)
