@@ -23,6 +23,10 @@
 // barriers 4.8 in FP64, 2.9 in FP32), at n = 1,000, m = 8,000 1.7 us (2.95 and
 // 2.0): about half of it the L2 latency there and back, the rest the gather
 // (one 32-byte sector per nonzero and SM every other clock) and the sums.
+// w and gamma go the same way (gamma's rows wait for the parts of their means).
+// Outside the steps an update costs 25 us at n = 20,000 and 19 us at n = 1,000
+// (27 and 21 with a grid barrier after w and a gather of every column's extent):
+// round trips to L2 that depend on each other.
 // Every CTA is co-resident and a value depends on earlier steps only, so the
 // waits end; they are bounded all the same.
 // The vectors are kept in 64-bit fixed point (xi without its factor C^(k+1),
@@ -521,10 +525,17 @@ __device__ __forceinline__ void pair_step_fx(const StepPair<double>& q, Gf gathe
 struct I2 {
   long long x, y;
 };
-// A word of W[k] is n 2^58 + v once n parts with the sum v, |v| < 2^57, are there.
+// A word of W[k] holds, above a sum v, |v| < 2^57, a count in its top 6 bits that
+// is FLOW_FULL once all parts of the sum are there: the part with the row's
+// first nonzero counts for the others that are missing (FLOW_FULL + 1 - parts),
+// each other one for 1.  So a reader needs to know nothing of the row (the
+// extents of the gathered rows cost 3 us of an update at n = 20,000), and a row
+// without nonzeros is complete from the start.
 constexpr int FLOW_CNT = 58;
 constexpr int FLOW_CTA = 256;   // nonzeros per CTA while co-resident CTAs are left
-constexpr int FLOW_PARTS = 60;  // parts a row may have (of the 6-bit count)
+constexpr int FLOW_PARTS = 60;  // parts a row may have
+constexpr unsigned FLOW_FULL = 63;
+constexpr long long FLOW_DONE = (long long)((unsigned long long)FLOW_FULL << FLOW_CNT);
 
 __device__ __forceinline__ I2 ld_flow(const I2* p) {
   I2 v;
@@ -544,16 +555,27 @@ __device__ __forceinline__ I2 look_flow(const I2* p) {
 }
 // A row's sum, or one part of it, into its word.  A reduction also where a store
 // would do: it reached the readers 0.25 us sooner (a step 2.9 -> 2.6 us).
-__device__ __forceinline__ void put_flow(I2* p, const I2& v) {
-  constexpr long long one = 1ll << FLOW_CNT;
-  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(&p->x), "l"(v.x + one) : "memory");
-  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(&p->y), "l"(v.y + one) : "memory");
+__device__ __forceinline__ void put_flow1(long long* p, long long v, unsigned w) {
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p),
+               "l"((unsigned long long)v + ((unsigned long long)w << FLOW_CNT))
+               : "memory");
 }
-// Whether both words hold all n parts (the count is in the upper half's top bits)
-__device__ __forceinline__ bool flow_there(const I2& v, int n) {
-  constexpr int half = 1 << (FLOW_CNT - 33);
-  return (((int)(v.x >> 32) + half) >> (FLOW_CNT - 32)) == n &&
-         (((int)(v.y >> 32) + half) >> (FLOW_CNT - 32)) == n;
+__device__ __forceinline__ void put_flow(I2* p, const I2& v, unsigned w) {
+  put_flow1(&p->x, v.x, w);
+  put_flow1(&p->y, v.y, w);
+}
+__device__ __forceinline__ long long ld_flow1(const long long* p) {
+  long long v;
+  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+// Whether all parts are there (the count is in the upper half's top bits)
+__device__ __forceinline__ bool flow_there(long long v) {
+  return (((unsigned)((unsigned long long)v >> 32) + (1u << (FLOW_CNT - 33))) >>
+          (FLOW_CNT - 32)) == FLOW_FULL;
+}
+__device__ __forceinline__ bool flow_there(const I2& v) {
+  return flow_there(v.x) && flow_there(v.y);
 }
 
 // x / per for 0 <= x < 2^24 (inv = 1 / per)
@@ -564,19 +586,17 @@ __device__ __forceinline__ int flow_div(int x, int per, float inv) {
   return q;
 }
 
-// The number of parts of row a's sums: the CTAs whose ranges hold some of its
-// nonzeros (0: a row without in-neighbours, its sums are zero).
-__device__ __forceinline__ int flow_parts(int a, const int* ioff, const int* __restrict__ loff,
-                                          const DevAdj& in, int per, float inv) {
-  const int rs = ioff[a / PT] + __ldcg(loff + a), len = __ldcg(in.len + a);
-  return len > 0 ? flow_div(rs + len - 1, per, inv) - flow_div(rs, per, inv) + 1 : 0;
+// What the part of nonzeros e0 .. counts for of a row with the nonzeros
+// rs .. rs + len - 1, cut at the multiples of per.
+__device__ __forceinline__ unsigned flow_weight(int rs, int len, int e0, int per, float inv) {
+  return rs < e0 ? 1u
+                 : FLOW_FULL - (unsigned)(flow_div(rs + len - 1, per, inv) - flow_div(rs, per, inv));
 }
 
 // v without its count
-__device__ __forceinline__ void flow_strip(I2& v, int n) {
-  const long long c = (long long)n << FLOW_CNT;
-  v.x -= c;
-  v.y -= c;
+__device__ __forceinline__ void flow_strip(I2& v) {
+  v.x -= FLOW_DONE;
+  v.y -= FLOW_DONE;
 }
 
 // Adds up the runs of lanes sharing a row: head sums to the first lane of their
@@ -695,17 +715,49 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     if (p.op_end > p.op_begin) prep_patch(p.ops, p.op_begin, p.op_end, p.in, p.out);
     if (tid == 0 && p.tiles) *p.ntiles = 0;
   }
-  // W starts at zero in both forms
   I2* F = static_cast<I2*>(p.W);
-  {
+  auto zero_w = [&]() {
     uint4* w16 = reinterpret_cast<uint4*>(W);
-    const int64_t total =
-        (int64_t)(K + 1) * p.n_pad * (p.flat ? 16 : (int64_t)sizeof(V2<V>)) / 16;
+    const int64_t total = (int64_t)(K + 1) * p.n_pad * (int64_t)sizeof(V2<V>) / 16;
     for (int64_t e = (int64_t)blockIdx.x * PG + tid; e < total; e += (int64_t)G * PG)
       w16[e] = make_uint4(0u, 0u, 0u, 0u);
+  };
+  if (p.flat) {
+    // rows without nonzeros are complete in all steps but the first
+    const int blocks = (nT * PT + PG - 1) / PG;
+    // (step, rows) units; step K + 1 = the means of phase 1
+#pragma unroll 4
+    for (int u = blockIdx.x; u < (K + 2) * blocks; u += G) {
+      const int k = u / blocks, a = (u - k * blocks) * PG + tid;
+      if (a < nT * PT) {
+        const int len = a == p.j ? new_len_j : p.in.len[a];
+        const long long c = len == 0 && k > 0 ? FLOW_DONE : 0ll;
+        if (k <= K)
+          *reinterpret_cast<longlong2*>(F + (int64_t)k * p.n_pad + a) = make_longlong2(c, c);
+        else
+          p.Y[a] = c;
+      }
+    }
+  } else {
+    zero_w();
   }
-  if (p.flat)
-    for (int a = (int)blockIdx.x * PG + tid; a < p.n_pad; a += G * PG) p.Y[a] = 0;
+  // rows sI, sJ of tile T, a quarter of the sources per thread, and row lengths:
+  // those of the first tile are on their way before the pending coefficients
+  // are read
+  V vI = V(0), vJ = V(0);
+  int L = 0;
+  auto s_rows = [&](int T) {
+    const int part = tid >> 7;
+    const int64_t a = (int64_t)T * PT + (tid & (PT - 1));
+    vI = vJ = V(0);
+    for (int u = part; u < p.delta; u += 4) vI += (V)s_at(S, p.ld, p.I[u], a, p.upper != 0);
+    if (part == 3) vJ = (V)s_at(S, p.ld, p.j, a, p.upper != 0);
+    // nonzeros of the tile after the patch (row j is being patched by CTA 0:
+    // it counts with its new length; no other row's length changes)
+    L = 0;
+    if (part == 0) L = (a == p.j) ? new_len_j : p.in.len[a];
+  };
+  if ((int)blockIdx.x < nT) s_rows(blockIdx.x);
   int mxL = 0;                 // longest row of this thread
   float mxI = 0.f, mxJ = 0.f;  // largest |sI|, |sJ| of the rows of this thread
   bool bad = false;            // one of them is infinite or NaN
@@ -730,27 +782,44 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     if (T >= nT) break;
     const int r = tid & (PT - 1), part = tid >> 7;
     const int64_t a = (int64_t)T * PT + r;
-    V vI = V(0), vJ = V(0);
-    for (int u = part; u < p.delta; u += 4) vI += (V)s_at(S, p.ld, p.I[u], a, p.upper != 0);
-    if (part == 3) vJ = (V)s_at(S, p.ld, p.j, a, p.upper != 0);
+    if (t) s_rows(T);
     // S_cur[x, a] = S[x, a] + sum_q xi_q[x] eta_q[a] + eta_q[x] xi_q[a]: the
     // pending terms are FP32 panels of an FP32 S, so they are added in FP32
-    // (on GB300 an FP64 FMA issues at 1/64 of the FP32 rate)
-    TS cI = TS(0), cJ = TS(0);
-    for (int q = part; q < np; q += 4) {
-      const TS xa = P[pidx(a, 0, q)];
-      const TS ea = P[pidx(a, 1, q)];
-      cI += coef[q] * ea + coef[np + q] * xa;
-      cJ += coef[2 * np + q] * ea + coef[3 * np + q] * xa;
+    // (on GB300 an FP64 FMA issues at 1/64 of the FP32 rate).  A warp takes every
+    // 16th term and four rows per lane, several loads under way: with a row and
+    // every fourth term per thread their latency was 3 us more of an update (24
+    // pending, n = 20,000, K = 20).
+    if constexpr (sizeof(TS) == 4) {
+      if (np > 0) {
+        static_assert(sizeof(fsh) >= (PG / 32) * 2 * PT * sizeof(float), "partial sums");
+        float* cs = reinterpret_cast<float*>(fsh);
+        const float* xp = P + pidx((int64_t)T * PT + 4 * lane, 0, 0);
+        const float* ep = xp + ldk * PT;
+        float4 cI = make_float4(0.f, 0.f, 0.f, 0.f), cJ = cI;
+#pragma unroll 4
+        for (int q = warp; q < np; q += PG / 32) {
+          const float4 xa = *reinterpret_cast<const float4*>(xp + (int64_t)q * PT);
+          const float4 ea = *reinterpret_cast<const float4*>(ep + (int64_t)q * PT);
+          const float c0 = coef[q], c1 = coef[np + q], c2 = coef[2 * np + q], c3 = coef[3 * np + q];
+          cI.x += c0 * ea.x + c1 * xa.x;
+          cI.y += c0 * ea.y + c1 * xa.y;
+          cI.z += c0 * ea.z + c1 * xa.z;
+          cI.w += c0 * ea.w + c1 * xa.w;
+          cJ.x += c2 * ea.x + c3 * xa.x;
+          cJ.y += c2 * ea.y + c3 * xa.y;
+          cJ.z += c2 * ea.z + c3 * xa.z;
+          cJ.w += c2 * ea.w + c3 * xa.w;
+        }
+        *reinterpret_cast<float4*>(cs + (2 * warp) * PT + 4 * lane) = cI;
+        *reinterpret_cast<float4*>(cs + (2 * warp + 1) * PT + 4 * lane) = cJ;
+        __syncthreads();
+        const float* c = cs + 8 * part * PT + r;
+        vI += (V)((c[0] + c[2 * PT]) + (c[4 * PT] + c[6 * PT]));
+        vJ += (V)((c[PT] + c[3 * PT]) + (c[5 * PT] + c[7 * PT]));
+      }
     }
-    vI += (V)cI;
-    vJ += (V)cJ;
     red[part][0][r] = vI;
     red[part][1][r] = vJ;
-    // nonzeros of the tile after the patch (row j is being patched by CTA 0:
-    // it counts with its new length; no other row's length changes)
-    int L = 0;
-    if (part == 0) L = (a == p.j) ? new_len_j : p.in.len[a];
     // inclusive scan of the row lengths over the tile (warps 0..3 hold its rows)
     int incl = L;
 #pragma unroll
@@ -809,8 +878,13 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
   StepPair<V> q0;
   int eI = 0, eG = 0;  // |sI| < 2^eI, |gamma| < 2^eG (flow form)
   bool finite = true;
+  const int tper = (nT + PG - 1) / PG;  // tiles a thread adds up
+  const int t0 = min(nT, tid * tper), t1 = min(nT, t0 + tper);
+  // read together: each is a round trip to L2
+  const unsigned b2 = __ldcg(p.bar + 2), b3 = __ldcg(p.bar + 3), b4 = __ldcg(p.bar + 4);
+  const int nnz0 = t0 < t1 ? __ldcg(p.tile_nnz + t0) : 0;
   if (alive && p.flat) {
-    const float mI = __uint_as_float(__ldcg(p.bar + 2)), mJ = __uint_as_float(__ldcg(p.bar + 3));
+    const float mI = __uint_as_float(b2), mJ = __uint_as_float(b3);
     // bounds of Thm 3 / Thm 9 / Table 2 with |w_j|, |S_II| / delta^2 <= max |sI| / delta
     // (a first in-link's gamma has no other terms)
     const float gq = p.d_j == 0 ? 0.f : fabsf((float)p.gq);
@@ -828,11 +902,9 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     // tried first when allowed) or their items of at most `item` nonzeros
     for (int pass = p.flat && finite ? 0 : 1; pass < 2; ++pass) {
       const int div = pass == 0 ? 1 : p.item;
-      const int per = (nT + PG - 1) / PG;
-      const int t0 = min(nT, tid * per), t1 = min(nT, t0 + per);
       int s = 0;
       for (int T = t0; T < t1; ++T) {
-        const int c = __ldcg(p.tile_nnz + T);
+        const int c = T == t0 ? nnz0 : __ldcg(p.tile_nnz + T);
         s += div == 1 ? c : (c + div - 1) / div;
       }
       int incl = s;
@@ -859,7 +931,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
           const int b = (int)blockIdx.x;
           // (so many that no row has more than FLOW_PARTS parts)
           s_div = pass == 0 ? max((w + G - 1) / G,
-                                  ((int)__ldcg(p.bar + 4) + FLOW_PARTS - 2) / (FLOW_PARTS - 1))
+                                  ((int)b4 + FLOW_PARTS - 2) / (FLOW_PARTS - 1))
                             : (w > b ? (w - b + G - 1) / G : 0);
         }
       }
@@ -867,7 +939,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
       int run = wsum[warp] + incl - s;
       for (int T = t0; T < t1; ++T) {
         ioff[T] = run;
-        const int c = __ldcg(p.tile_nnz + T);
+        const int c = T == t0 ? nnz0 : __ldcg(p.tile_nnz + T);
         run += div == 1 ? c : (c + div - 1) / div;
       }
       __syncthreads();
@@ -884,10 +956,11 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
   // ---- flow form: the CTA's nonzeros [e0, e1), two per thread
   const int per = flow ? max(1, s_div) : 1;
   const float inv_per = 1.f / (float)per;
-  int na = 0, nb2 = 0;        // parts of the columns of the thread's nonzeros
   int wait_w = 0;             // > 0: the emitted run goes on in that many warps more
   bool wait_tail = false;     // it is the tail's (else the head's)
   bool give = false;          // the head sum is the part of a row of an earlier warp
+  auto w_head = [&]() { return (q0.fl >> 16) & 63u; };
+  auto w_tail = [&]() { return (q0.fl >> 24) & 63u; };
   if (alive && flow) {
     const int nnz = ioff[nT];
     const int e0 = min(nnz, (int)blockIdx.x * per), e1 = min(nnz, e0 + per), cnt = e1 - e0;
@@ -930,21 +1003,41 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     rowmap[pos] = ra;
     if (E == 2) rowmap[pos + 1] = rb;
     q0.ca = q0.cb = q0.kh = q0.kt = -1;
-    int rsh = 0, rst = 0;
-    if (pos < cnt) {
+    // loads that do not depend on each other are issued together (each round is
+    // a trip to L2): the rows' extents; the columns and the rows' factors; sI
+    const bool has_a = pos < cnt, has_b = E == 2 && pos + 1 < cnt, two = has_b && rb != ra;
+    int la = 0, lb = 0, fa = 0, fb = 0;  // lengths of rows ra, rb, and their first nonzeros
+    int64_t sa = 0, sb = 0;              // their starts in the pool
+    if (has_a) {
+      fa = __ldcg(p.loff + ra);
+      sa = __ldcg(p.in.start + ra);
+      la = __ldcg(p.in.len + ra);
+    }
+    if (two) {
+      fb = __ldcg(p.loff + rb);
+      sb = __ldcg(p.in.start + rb);
+      lb = __ldcg(p.in.len + rb);
+    }
+    fsh[tid][0] = fsh[tid][1] = SweepScale{0ull, 0, 1};
+    if (has_a) {
       q0.kh = ra;
-      rsh = ioff[ra / PT] + __ldcg(p.loff + ra);
-      q0.ca = __ldcg(p.in.col + __ldcg(p.in.start + ra) + (e0 + pos - rsh));
-    }
-    if (E == 2 && pos + 1 < cnt) {
-      if (rb != ra) {
+      fa += ioff[ra / PT];
+      fb += ioff[rb / PT];
+      q0.ca = __ldcg(p.in.col + sa + (e0 + pos - fa));
+      if (has_b)
+        q0.cb = __ldcg(p.in.col + (two ? sb + (e0 + pos + 1 - fb) : sa + (e0 + pos + 1 - fa)));
+      fsh[tid][0] = p.recip[la];
+      if (two) {
         q0.kt = rb;
-        rst = ioff[rb / PT] + __ldcg(p.loff + rb);
+        fsh[tid][1] = p.recip[lb];
       }
-      q0.cb = __ldcg(p.in.col + __ldcg(p.in.start + rb) +
-                     (e0 + pos + 1 - (rb != ra ? rst : rsh)));
     }
+    V xa = V(0), xb = V(0);
+    if (q0.ca >= 0) xa = sI[q0.ca];
+    if (q0.cb >= 0) xb = sI[q0.cb];
     pair_pattern(q0);
+    if (has_a) q0.fl |= flow_weight(fa, la, e0, per, inv_per) << 16;
+    if (two) q0.fl |= flow_weight(fb, lb, e0, per, inv_per) << 24;
     __syncthreads();  // rowmap
     const int w0 = 32 * E * warp, w1 = min(cnt, w0 + 32 * E);  // the warp's positions
     if (w0 < cnt) {
@@ -961,32 +1054,37 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
         }
       }
     }
-    fsh[tid][0] = fsh[tid][1] = SweepScale{0ull, 0, 1};
-    if (q0.kh >= 0) {
-      const int len = __ldcg(p.in.len + q0.kh);
-      fsh[tid][0] = p.recip[len];
-    }
-    if (q0.kt >= 0) {
-      const int len = __ldcg(p.in.len + q0.kt);
-      fsh[tid][1] = p.recip[len];
-    }
-    if (q0.ca >= 0) na = flow_parts(q0.ca, ioff, p.loff, p.in, per, inv_per);
-    if (q0.cb >= 0) nb2 = flow_parts(q0.cb, ioff, p.loff, p.in, per, inv_per);
     // w = Q sI: the parts of each row's mean, in units of 2^(eI - 56), into Y
     I2 h{0, 0}, t{0, 0};
-    if (q0.ca >= 0) h.x = fixed_of(sI[q0.ca], eI);
+    if (q0.ca >= 0) h.x = fixed_of(xa, eI);
     if (q0.cb >= 0) {
-      const long long v = fixed_of(sI[q0.cb], eI);
+      const long long v = fixed_of(xb, eI);
       if (q0.kt >= 0) t.x = v; else h.x += v;
     }
     flow_sum(q0, h, t);
-    if (q0.fl & (1u << 6))
-      atomicAdd((unsigned long long*)p.Y + q0.kh, (unsigned long long)fixed_scale(h.x, fsh[tid][0]));
-    if (q0.fl & (1u << 7))
-      atomicAdd((unsigned long long*)p.Y + q0.kt, (unsigned long long)fixed_scale(t.x, fsh[tid][1]));
-    alive = prep_barrier(p.bar, ++nb * G, p.limit, &s_ok);
+    if (q0.fl & (1u << 6)) {
+      h.x = fixed_scale(h.x, fsh[tid][0]);
+      if (give)
+        dep[1][warp].x = h.x;
+      else if (wait_w == 0 || wait_tail)
+        put_flow1(p.Y + q0.kh, h.x, w_head());
+    }
+    if (q0.fl & (1u << 7)) {
+      t.x = fixed_scale(t.x, fsh[tid][1]);
+      if (!wait_tail) put_flow1(p.Y + q0.kt, t.x, w_tail());
+    }
+    __syncthreads();
+    if (wait_w) {
+      long long v = wait_tail ? t.x : h.x;
+      for (int x = 1; x <= wait_w; ++x) v += dep[1][warp + x].x;
+      put_flow1(p.Y + (wait_tail ? q0.kt : q0.kh), v, wait_tail ? w_tail() : w_head());
+    }
   } else if (alive) {
     my_items = s_div;
+    if (p.flat) {  // set up for the flow form above
+      zero_w();
+      alive = prep_barrier(p.bar, ++nb * G, p.limit, &s_ok);
+    }
     int cbase = 0;
     for (int u = 0; u < my_items; ++u) {
       PrepItem& it = items[min(u, MAXI)];
@@ -1020,6 +1118,26 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     alive = prep_barrier(p.bar, ++nb * G, p.limit, &s_ok);
   }
 
+  // Waits of the flow form: a warp reads its entries of W[k] again until all of
+  // them hold their parts (together: lanes that waited on their own would read
+  // one after the other).  Bounded: a wait that runs out sets the status word,
+  // and one that sees it set gives up as well (the steps then stop in the whole
+  // CTA).  True to go on waiting.
+  bool stop = false;
+  auto flow_again = [&](bool there, long long& it) -> bool {
+    if (__all_sync(0xffffffffu, there)) return false;
+    ++it;
+    bool out = it > p.limit;
+    if ((it & 255) == 0)
+      out |= __any_sync(0xffffffffu,
+                        *(volatile unsigned long long*)(p.counters + CNT_STATUS) != 0ull);
+    if (out) {
+      if (lane == 0)
+        atomicExch(&p.counters[CNT_STATUS], (unsigned long long)SR_ERR_TIMEOUT);
+      stop = true;
+    }
+    return !out;
+  };
   // ---- phase 1b: gamma per row (tiles round-robin); W[0] = (xi_0, eta_0)
   if (alive) {
     for (int t = 0; t < mt; ++t) {
@@ -1031,8 +1149,16 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
         const int len = __ldcg(p.in.len + a);
         // the factors of row a of Q on the new graph, for every step below
         const V inv = len > 0 && !flow ? V(1) / (V)len : V(0);
+        long long yw = 0;
+        if (flow) {
+          // the mean, once its parts are there
+          yw = ld_flow1(p.Y + a);
+          for (long long it = 0; flow_again(flow_there(yw), it);)
+            if (!flow_there(yw)) yw = ld_flow1(p.Y + a);
+          yw -= FLOW_DONE;
+        }
         // sum (item form) or mean (flow form) of sI over the new in-neighbours
-        const V y = flow ? fixed_value<V>(__ldcg(p.Y + a), eI - 56) : __ldcg(&W[a].x);
+        const V y = flow ? fixed_value<V>(yw, eI - 56) : __ldcg(&W[a].x);
         V g;
         if (a == p.j) {
           // row j: lambda (Eq. 29b) and w_j on the old row j, in FP64
@@ -1040,7 +1166,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
           for (int u = 0; u < p.delta; ++u) S_II += (double)__ldcg(sI + p.I[u]);
           const double S_jj = (double)__ldcg(sJ + p.j);
           const double ys =
-              flow ? fixed_value<double>(__ldcg(p.Y + a), eI - 56) * (double)len : (double)y;
+              flow ? fixed_value<double>(yw, eI - 56) * (double)len : (double)y;
           const double wj = (ys - (double)p.op * S_II) * p.inv_ddj;  // 0 when d_j = 0
           const double id = p.inv_delta, iC = p.inv_C;
           const double lam = S_II * id * id + S_jj * iC - 2.0 * wj - iC + 1.0;
@@ -1064,7 +1190,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
         }
         const V x0 = (a == p.j) ? Cv : V(0);
         if (flow) {
-          put_flow(F + a, I2{a == p.j ? 1ll << 56 : 0ll, fixed_of(g, eG)});
+          put_flow(F + a, I2{a == p.j ? 1ll << 56 : 0ll, fixed_of(g, eG)}, FLOW_FULL);
         } else {
           W[a] = V2<V>{x0, g};
           rinv[a] = V2<V>{Cv * inv, inv};
@@ -1079,6 +1205,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
         mk[t][1] = any_e ? 1ull : 0ull;
       }
     }
+    if (flow && __syncthreads_or(stop)) alive = false;
     if (K > 0 && !flow) alive = prep_barrier(p.bar, ++nb * G, p.limit, &s_ok);
   }
 
@@ -1096,44 +1223,22 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     }
     __syncthreads();
   }
-  // Waits of the flow form: a warp reads its entries of W[k] again until all of
-  // them hold their parts (together: lanes that waited on their own would read
-  // one after the other).  Bounded: a wait that runs out sets the status word,
-  // and one that sees it set gives up as well (the steps then stop in the whole
-  // CTA).  True to go on waiting.
-  bool stop = false;
-  auto flow_again = [&](bool there, long long& it) -> bool {
-    if (__all_sync(0xffffffffu, there)) return false;
-    ++it;
-    bool out = it > p.limit;
-    if ((it & 255) == 0)
-      out |= __any_sync(0xffffffffu,
-                        *(volatile unsigned long long*)(p.counters + CNT_STATUS) != 0ull);
-    if (out) {
-      if (lane == 0)
-        atomicExch(&p.counters[CNT_STATUS], (unsigned long long)SR_ERR_TIMEOUT);
-      stop = true;
-    }
-    return !out;
-  };
   if (alive && flow) {
     for (int k = 0; k < K; ++k) {
       const I2* Fk = F + (int64_t)k * p.n_pad;
       I2* Fn = F + (int64_t)(k + 1) * p.n_pad;
       I2 h{0, 0}, t{0, 0}, u{0, 0};
-      // both loads are on their way before the first is looked at; W[0] is
-      // written row by row, in one part
-      const int ma = k ? na : 1, mb = k ? nb2 : 1;
+      // both loads are on their way before the first is looked at
       if (q0.ca >= 0) h = look_flow(Fk + q0.ca);
       if (q0.cb >= 0) u = look_flow(Fk + q0.cb);
       for (long long it = 0;;) {
-        const bool wa = q0.ca >= 0 && !flow_there(h, ma), wb = q0.cb >= 0 && !flow_there(u, mb);
+        const bool wa = q0.ca >= 0 && !flow_there(h), wb = q0.cb >= 0 && !flow_there(u);
         if (!flow_again(!(wa || wb), it)) break;
         if (wa) h = ld_flow(Fk + q0.ca);
         if (wb) u = ld_flow(Fk + q0.cb);
       }
-      if (q0.ca >= 0) flow_strip(h, ma);
-      if (q0.cb >= 0) flow_strip(u, mb);
+      if (q0.ca >= 0) flow_strip(h);
+      if (q0.cb >= 0) flow_strip(u);
       if (q0.kt >= 0) {
         t = u;
       } else {
@@ -1148,13 +1253,13 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
         if (give)
           dep[k & 1][warp] = h;
         else if (wait_w == 0 || wait_tail)
-          put_flow(Fn + q0.kh, h);
+          put_flow(Fn + q0.kh, h, w_head());
       }
       if (q0.fl & (1u << 7)) {
         const SweepScale f = fsh[tid][1];
         t.x = fixed_scale(t.x, f);
         t.y = fixed_scale(t.y, f);
-        if (!wait_tail) put_flow(Fn + q0.kt, t);
+        if (!wait_tail) put_flow(Fn + q0.kt, t, w_tail());
       }
       if (__syncthreads_or(stop)) {
         alive = false;  // on every thread of the CTA
@@ -1167,7 +1272,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
           h.x += dep[k & 1][warp + x].x;
           h.y += dep[k & 1][warp + x].y;
         }
-        put_flow(Fn + (wait_tail ? q0.kt : q0.kh), h);
+        put_flow(Fn + (wait_tail ? q0.kt : q0.kh), h, wait_tail ? w_tail() : w_head());
       }
     }
   }
@@ -1199,11 +1304,6 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     for (int t = 0; t < mt; ++t) {
       const int T = blockIdx.x + t * G;
       if (T >= nT) break;
-      int parts[PT / 32];
-#pragma unroll
-      for (int q = 0; q < PT / 32; ++q)
-        parts[q] =
-            flow ? flow_parts(T * PT + q * 32 + lane, ioff, p.loff, p.in, per, inv_per) : 0;
       // warp w copies columns k = 1 + w, 1 + w + 16, ...
       for (int k = 1 + warp; k <= K; k += PG / 32) {
         const V2<V>* Wk = W + (int64_t)k * p.n_pad;
@@ -1216,11 +1316,11 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
           for (long long it = 0;;) {
             bool w = false;
 #pragma unroll
-            for (int q = 0; q < PT / 32; ++q) w |= !flow_there(look[q], parts[q]);
+            for (int q = 0; q < PT / 32; ++q) w |= !flow_there(look[q]);
             if (!flow_again(!w, it)) break;
 #pragma unroll
             for (int q = 0; q < PT / 32; ++q)
-              if (!flow_there(look[q], parts[q])) look[q] = ld_flow(Fk + q * 32);
+              if (!flow_there(look[q])) look[q] = ld_flow(Fk + q * 32);
           }
         bool nx = false, ne = false;
 #pragma unroll
@@ -1232,7 +1332,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
           if (flow) {
             // xi_k = C^(k+1) x 2^-56, C^(k+1) = r 2^-(63 + s)
             I2 v = look[q];
-            flow_strip(v, parts[q]);
+            flow_strip(v);
             px = fixed_value<TS>(__mul64hi(v.x << 6, (long long)ck.r), -61 - ck.sh);
             pe = fixed_value<TS>(v.y, eG - 56);
           } else {

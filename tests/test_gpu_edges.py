@@ -245,3 +245,21 @@ def test_digit_pass_at_term_and_tile_edges(P, prec, K, n, kw, form):
     if ok.any():
         err = np.max(np.abs(got[ok] - want[ok])) / max(1e-12, np.max(np.abs(want[ok])))
         assert err < (1e-13 if prec == 64 else 2e-5)
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+def test_recurrence_with_a_hub_over_many_ctas(P, prec):
+    """A row with a quarter of all nonzeros: its sums come in some fifty parts
+    (of at most 60), beside rows without nonzeros, whose sums are complete from the
+    start.  1e-10 (FP64) and 1e-6 (FP32), as in the parity tests."""
+    n, C, K = 9000, 0.6, 3
+    s, d = degrees_graph(n, [0, 8500, 0], 23)
+    edges = set(zip(s.tolist(), d.tolist()))
+    S0 = np.eye(n) * 0.5
+    S0[:200, :200] += 0.25
+    ups = [(next(x for x in range(2, n) if (x, 1) not in edges), 1, 1), (5, 0, 1),
+           (next(x for x, y in sorted(edges) if y == 1), 1, -1), (1, 2, 1)]
+    sr = P.SimRank(n, s, d, S0=S0, C=C, K=K, s_precision=prec)
+    sr.apply_updates(ups)
+    want, _ = O.sequential_unit_updates(n, s, d, S0, ups, C, K)
+    assert np.max(np.abs(sr.dense() - want)) < (1e-10 if prec == 64 else 1e-6)
