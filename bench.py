@@ -476,7 +476,11 @@ def run_gpu(args, rank, world):
                    "ms_per_launch": sp_ms / max(launches, 1), "launches": launches})
     # k_prep: one launch per update, latency-bound (L2-resident working set)
     prep_ms = phase[0]
-    pair_bytes = 16 if args.vec_fp64 else 8
+    # the flow form keeps the vectors in 64-bit integers in either precision; the
+    # item form has a grid barrier after each phase and step
+    flow = form.get("prep_item", 0) == 0
+    barriers = 1 if flow else K + 3
+    pair_bytes = 16 if flow or args.vec_fp64 else 8
     npend_avg = ((G - 1) / 2.0) * (K + 1) if args.defer > 1 else 0.0
     prep_bytes_1 = stream_prep_bytes(n_pad, M, K, pair_bytes, npend_avg)
     prep_us = 1000.0 * prep_ms / per_step
@@ -487,10 +491,11 @@ def run_gpu(args, rank, world):
             "frac": prep_gbs / peak, "peak_kind": peak_kind,
             "traffic": TRAFFIC_PREP if profiled else None,
             "bytes_per_launch": prep_bytes_1, "us_per_launch": prep_us,
-            "us_per_step": prep_us / (K + 4), "grid_barriers": K + 3,
+            "us_per_step": prep_us / (K + 4), "grid_barriers": barriers,
             "launches": per_step,
             "note": "algorithmic bytes as stream_prep_bytes states; L2-resident working set, so "
-                    "the time is set by K + 3 grid barriers and one L2 round trip per step"}
+                    "the time is set by a round trip to L2 per step (grid_barriers counts "
+                    "the barriers beside them)"}
     # the per-edge S pass (each update alone)
     pe_launches = e1["s_update_launches"] - e0["s_update_launches"]
     pe_ms = e1["s_update_ms"] - e0["s_update_ms"]

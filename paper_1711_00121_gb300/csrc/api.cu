@@ -2467,10 +2467,10 @@ simrank_status simrank_grad(simrank_t h, const int32_t* pa, const int32_t* pb, c
     launch_adj_scatter((const int32_t*)h->ob[21].p, (const int32_t*)h->ob[23].p,
                        (const double*)h->ob[13].p, (int64_t)pn.size(), ldb, Fp, h->st);
     for (int l = 1; l <= K; ++l) {
-      launch_col_forward64(h->cur_fwd, h->dout.col, wv, inv, F + (l - 1) * blk, F + l * blk, ldb,
-                           h->st);
-      launch_col_forward64(h->cur_fwd, h->dout.col, wv, inv, Fp + (l - 1) * blk, Fp + l * blk, ldb,
-                           h->st);
+      launch_col_forward64(h->cur_fwd, h->dout.col, wv, h->din.len, n_pad, inv, F + (l - 1) * blk,
+                           y0, F + l * blk, ldb, h->st);
+      launch_col_forward64(h->cur_fwd, h->dout.col, wv, h->din.len, n_pad, inv, Fp + (l - 1) * blk,
+                           y0, Fp + l * blk, ldb, h->st);
     }
     CUDA_TRY(h, cudaMemsetAsync(y0, 0, (size_t)blk * 8, h->st));
     double* y = y0;

@@ -92,6 +92,7 @@ __device__ __forceinline__ void add_cols(T* p, const ColVec<T, VEC>& r) {
 // row chunk (at most kChunk = 32 nonzeros of one adjacency row) and 32 * VEC
 // columns (blockIdx.y):
 //   forward (Q^T, out-lists): Y[row][c]  = sum_e w_e nodes[col_e] X[col_e][c]
+//                             (in FP64 X comes divided, k_col_quotient: no nodes)
 //   Horner  (Q,   in-lists):  Y[row][c]  = add_scale Xadd[row][c]
 //                                          + nodes[row] sum_e w_e X[col_e][c]
 // nodes holds 1 / d (or 1 / in-weight) per node, times the step's scale for
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(256, 6) k_col_rows(
     const int64_t st = __shfl_sync(full, mine.start, i);
     T w = T(0);
     if (i < nq && lane < len) {
-      w = FORWARD ? nodes[a] : T(1);
+      w = FORWARD && sizeof(T) == 4 ? nodes[a] : T(1);
       if (ew) w *= (T)ew[st + lane];
     }
     return w;
@@ -203,6 +204,23 @@ __global__ void k_col_prefill(const int32_t* __restrict__ rows, const T* __restr
   const int64_t o = (int64_t)rows[blockIdx.x] * ldb;
   for (int c = threadIdx.x; c < ldb; c += blockDim.x)
     Y[o + c] = Xadd ? add_scale * Xadd[o + c] : T(0);
+}
+
+// U[a][c] = X[a][c] / (in-degree or in-weight of a), r = its reciprocal: the
+// product with r and one correction, three FP64 operations where a division takes
+// some ten, and rounded like it.  One pass over the block before an FP64 forward
+// step (a gradient over 600 pairs at n = 5,000: 13.0 to 14.3 ms); a reciprocal inside
+// the step left twice the error of the division.  One CTA per row.
+__global__ void __launch_bounds__(128)
+    k_col_quotient(const double* __restrict__ X, const int32_t* __restrict__ in_len,
+                   const double* __restrict__ wsum, const double* __restrict__ recip, int ldb,
+                   double* __restrict__ U) {
+  const int64_t a = blockIdx.x;
+  const double r = recip[a], d = wsum ? wsum[a] : (double)in_len[a];
+  for (int c = threadIdx.x; c < ldb; c += 128) {
+    const double x = X[a * ldb + c], q = x * r;
+    U[a * ldb + c] = fma(fma(-q, d, x), r, q);
+  }
 }
 
 // out[a] = scale / (in-degree or in-weight of a), 0 without in-neighbours
@@ -403,28 +421,6 @@ __global__ void __launch_bounds__(256) k_col_corr(const float* const* __restrict
   }
 }
 
-// scal[0] = x_i[i], scal[1] = x_j[j], scal[2] = (1/d_j) sum_{b in I(j)} x_i[b]
-// (columns i and j of S as FP64 vectors, old graph)
-__global__ void k_col_scalars(DevAdj in, const double* __restrict__ si, const double* __restrict__ sj,
-                              int i, int j, double* __restrict__ scal) {
-  __shared__ double red[32];
-  const int64_t st = in.start[j];
-  const int len = in.len[j];
-  double acc = 0.0;
-  for (int e = threadIdx.x; e < len; e += blockDim.x) acc += si[in.col[st + e]];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double w = 0.0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) w += red[q];
-    scal[0] = si[i];
-    scal[1] = sj[j];
-    scal[2] = len > 0 ? w / (double)len : 0.0;
-  }
-}
-
 // out[c * n + a] = Y[a][c] (column-major output, optional FP32), transposed
 // in 32 x 32 blocks through shared memory so that both sides are read and
 // written in rows (200,000 x 256, FP32: 226 us when read column by column).
@@ -506,9 +502,14 @@ static void partial_sim_block_t(const ChunkList& fwd, const ChunkList& hor, cons
     k_col_scales<T><<<nb, 256, 0, st>>>(in_len, wv.wsum, 1.0, n_rows, inv);
     k_col_scales<T><<<nb, 256, 0, st>>>(in_len, wv.wsum, C, n_rows, hs);
     k_col_scales<T><<<nb, 256, 0, st>>>(in_len, wv.wsum, (1.0 - C) * C, n_rows, hl);
-    for (int t = 1; t <= K; ++t)
-      wide_step<T>(fwd, out_col, wv.out_w, true, inv, xs + (int64_t)(t - 1) * blk, nullptr,
-                       0.0, xs + (int64_t)t * blk, ldb, st);
+    for (int t = 1; t <= K; ++t) {
+      const T* X = xs + (int64_t)(t - 1) * blk;
+      T* Y = xs + (int64_t)t * blk;
+      if constexpr (sizeof(T) == 8)  // y0 is free until the Horner steps
+        launch_col_forward64(fwd, out_col, wv, in_len, n_rows, inv, X, y0, Y, ldb, st);
+      else
+        wide_step<T>(fwd, out_col, wv.out_w, true, inv, X, nullptr, 0.0, Y, ldb, st);
+    }
     const T* y = xs + (int64_t)K * blk;
     for (int t = 1; t <= K; ++t) {
       T* dst = (t == K) ? result : bufs[t & 1];
@@ -581,11 +582,12 @@ void launch_col_scales64(const WeightView& wv, const int32_t* in_len, int n_rows
   k_col_scales<double><<<(n_rows + 255) / 256, 256, 0, st>>>(in_len, wv.wsum, 1.0, n_rows, inv);
 }
 
-// Y = Q^T X (FP64 blocks [n_rows][ldb])
+// Y = Q^T X (FP64 blocks [n_rows][ldb]); U: X over the in-degrees or in-weights
 void launch_col_forward64(const ChunkList& fwd, const int32_t* out_col, const WeightView& wv,
-                          const double* inv, const double* X, double* Y, int ldb,
-                          cudaStream_t st) {
-  wide_step<double>(fwd, out_col, wv.out_w, true, inv, X, nullptr, 0.0, Y, ldb, st);
+                          const int32_t* in_len, int n_rows, const double* inv, const double* X,
+                          double* U, double* Y, int ldb, cudaStream_t st) {
+  k_col_quotient<<<n_rows, 128, 0, st>>>(X, in_len, wv.wsum, inv, ldb, U);
+  wide_step<double>(fwd, out_col, wv.out_w, true, nullptr, U, nullptr, 0.0, Y, ldb, st);
 }
 
 // Yn = add_scale * Xadd + Q Y (FP64 blocks [n_rows][ldb])
@@ -625,11 +627,6 @@ void launch_col_corr(const float* const* hist, int U, int K1, const int32_t* col
   k_col_gvals<<<dim3((2 * K1 * Bp + 255) / 256, U), 256, 0, st>>>(hist, K1, cols, B, Bp, G);
   k_col_corr<<<dim3(n_rows / PT, (B + PT - 1) / PT), 256, 0, st>>>(hist, U, K1, G, Bp, B, ldb,
                                                                    n_rows, Y);
-}
-
-void launch_col_scalars(const DevAdj& in, const double* si, const double* sj, int i, int j,
-                        double* scal, cudaStream_t st) {
-  k_col_scalars<<<1, 256, 0, st>>>(in, si, sj, i, j, scal);
 }
 
 void launch_col_out(const void* Y, int prec, int B, int ldb, int n, void* out, int out_fp64,

@@ -467,8 +467,8 @@ void launch_partial_sim_block(const ChunkList& fwd, const ChunkList& hor, const 
 void launch_col_scales64(const WeightView& wv, const int32_t* in_len, int n_rows, double* inv,
                          cudaStream_t st);
 void launch_col_forward64(const ChunkList& fwd, const int32_t* out_col, const WeightView& wv,
-                          const double* inv, const double* X, double* Y, int ldb,
-                          cudaStream_t st);
+                          const int32_t* in_len, int n_rows, const double* inv, const double* X,
+                          double* U, double* Y, int ldb, cudaStream_t st);
 void launch_col_horner64(const ChunkList& hor, const int32_t* in_col, const WeightView& wv,
                          const double* inv, const double* Xadd, double add_scale, const double* Y,
                          double* Yn, int ldb, cudaStream_t st);
@@ -481,9 +481,6 @@ void launch_col_corr(const float* const* hist, int U, int K1, const int32_t* col
                      int n_rows, float* G, float* Y, cudaStream_t st);
 void launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, int B, int ldb,
                       int n_rows, int prec, void* Y, cudaStream_t st);
-// scal[0] = si[i], scal[1] = sj[j], scal[2] = (1/d_j) sum_{b in I(j)} si[b]
-void launch_col_scalars(const DevAdj& in, const double* si, const double* sj, int i, int j,
-                        double* scal, cudaStream_t st);
 void launch_col_out(const void* Y, int prec, int B, int ldb, int n, void* out, int out_fp64,
                     cudaStream_t st);
 void launch_col_extract(const void* Y, int prec, int B, int c, int n, double* v, cudaStream_t st);

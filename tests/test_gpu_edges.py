@@ -263,3 +263,47 @@ def test_recurrence_with_a_hub_over_many_ctas(P, prec):
     sr.apply_updates(ups)
     want, _ = O.sequential_unit_updates(n, s, d, S0, ups, C, K)
     assert np.max(np.abs(sr.dense() - want)) < (1e-10 if prec == 64 else 1e-6)
+
+
+@pytest.mark.parametrize("prec,n", [(64, 700), (32, 5000)])
+def test_digit_pass_timeout(P, prec, n):
+    """A bound of one poll runs out in the digit pass (the work before it is the
+    per-step path, whose kernels have no waits): status 7 from sync, and the device
+    stays usable."""
+    s, d = degrees_graph(n, [0, 5], 29)
+    S0 = np.eye(n) * 0.5
+    ups = [(x, 0, 1) for x in range(2, 10)]
+    h = P.SimRank(n, s, d, S0=S0, C=0.6, K=12, s_precision=prec, chain=1, timeout_iters=1)
+    with pytest.raises(P.SimrankError) as err:
+        h.apply_updates(ups)
+        h.sync()
+    assert err.value.status == 7
+    h.close()
+    h = P.SimRank(n, s, d, S0=S0, C=0.6, K=12, s_precision=prec)
+    h.apply_updates(ups[:2])
+    h.sync()
+    want, _ = O.sequential_unit_updates(n, s, d, S0, ups[:2], 0.6, 12)
+    assert np.max(np.abs(h.dense() - want)) < (1e-10 if prec == 64 else 1e-6)
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("n,deg,npairs,K", [(300, 6, 1, 5), (300, 6, 2, 1), (300, 6, 1100, 4),
+                                            (701, 5, 257, 9), (60, 3, 400, 6)])
+def test_gradient_at_block_edges(P, n, deg, npairs, K, weighted):
+    """Value and gradient with blocks of two columns and more, repeated pairs and
+    pairs of a node with itself, column counts off the padding and off a CTA's 128
+    (the quotients before a forward step), nodes without in-links.  Bounds as in
+    the adjoint's parity tests."""
+    rng = np.random.default_rng(31)
+    s, d = degrees_graph(n, [0] + [deg] * (n - 1), 37)
+    w = rng.random(s.size).astype(np.float32) + 0.5 if weighted else None
+    a, b = rng.integers(0, n, npairs).astype(np.int32), rng.integers(0, n, npairs).astype(np.int32)
+    if npairs > 4:
+        a[1], b[1], b[2] = a[0], b[0], a[2]
+    t = rng.random(npairs)
+    sr = P.SimRank(n, s, d, C=0.6, K=K, s_precision=64, mode=1, **({"weight": w} if weighted else {}))
+    L, g = sr.grad(a, b, t, s.size)
+    L_ref, g_ref, _ = O.pair_loss_and_weight_grad(
+        n, s, d, w.astype(np.float64) if weighted else np.ones(s.size), a, b, t, 0.6, K)
+    assert abs(L - L_ref) < 1e-11 * max(1.0, abs(L_ref))
+    assert np.max(np.abs(g - g_ref)) < 1e-10 * max(1.0, np.max(np.abs(g_ref)))
