@@ -47,7 +47,7 @@ METRIC = "edge updates/sec & HBM GB/s: fused rank-2K ΔS vs plain Inc-uSR at 1e-
 UNIT = "edge updates/s"
 # DRAM bytes (read + write) per launch from one ncu capture of each kernel on
 # the default stream configuration (profiles/ holds the summaries)
-TRAFFIC_PREP = 6.137e7
+TRAFFIC_PREP = 6.244e7
 TRAFFIC_S_PASS = 1.828e9
 # the per-update S pass (--defer 0 replica, FP16 split): a typical launch
 TRAFFIC_S_PASS_EDGE = 1.417e9
@@ -339,7 +339,7 @@ def run_gpu(args, rank, world):
     # ---- value: device-timed steps of the headline form (no per-launch profiling)
     sr = handle(0)
     ms, st0, st1, clk = timed_steps(sr, clocks=True)
-    # drift re-anchor (FP64 Jacobi sweeps of Eq. 1 from the current S)
+    # drift re-anchor (Jacobi sweeps of Eq. 1 in 64 bits from the current S)
     ra0 = time.perf_counter()
     ra_change = sr.reanchor(2)
     sr.sync()
@@ -543,7 +543,7 @@ def run_gpu(args, rank, world):
         "roofline": dominant,
         "kernels": {"s_pass": s_pass, "prep": prep, "s_pass_per_edge": s_pass_per_edge},
         "reanchor": {"ms_per_sweep": reanchor_ms, "max_change_last_sweep": ra_change,
-                     "note": "FP64 Jacobi sweep of Eq. 1 on the n=20000 S after the timed steps"},
+                     "note": "64-bit Jacobi sweep of Eq. 1 on the n=20000 S after the timed steps"},
         "other_vectors": other,
         "e2e": {"value": e2e_val, "unit": UNIT,
                 "h2d_bytes_per_step": int(packed[0][1] * 16), "d2h_bytes_per_step": int(d2h)},

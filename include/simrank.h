@@ -116,7 +116,7 @@ typedef struct simrank_config {
                              G * (K + 1) <= 4096, else SR_ERR_ARG. */
   int32_t chain;          /* work of a rank-one update before its S pass: 0 = one cooperative
                              launch (graph patch, rows of S, gamma, all K recurrence steps, masks,
-                             tile list; bounded grid barriers), 1 = one launch per step (FP64
+                             tile list; bounded waits), 1 = one launch per step (FP64
                              vectors).  Graphs with more than 8 tiles of 128 nodes per
                              co-resident CTA take the per-step path. */
   int32_t prep_ctas;      /* chain = 0: cap on the CTAs of the fused launch (0 = as many as fit) */
