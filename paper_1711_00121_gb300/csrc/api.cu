@@ -944,9 +944,20 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
   }
   double diff = INFINITY;
   int it = 0;
-  cudaError_t e = cudaSuccess;
   bool fixed = !h->weighted && wp == 64;
   SweepScale* scales = nullptr;
+  // ends the call before S has been touched; a handle's kept buffers stay
+  auto give_up = [&](cudaError_t why) {
+    cudaGetLastError();
+    if (scales) cudaFree(scales);
+    if (!held)
+      for (void* p : bufs)
+        if (p) cudaFree(p);
+    return fail(h, why == cudaErrorMemoryAllocation ? SR_ERR_OOM : SR_ERR_CUDA,
+                std::string("Jacobi sweep: ") + cudaGetErrorString(why));
+  };
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return give_up(e);
   if (fixed) {
     // S into bufs[0] in fixed point, with a look at what it holds unless it is
     // known (before the change when it is made in place)
@@ -961,11 +972,12 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
     if (e == cudaSuccess && !known)
       e = cudaMemcpyAsync(&flags, h->diffbits, sizeof(flags), cudaMemcpyDeviceToHost, h->st);
     if (e == cudaSuccess && !known) e = cudaStreamSynchronize(h->st);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) return give_up(e);
     fixed = flags == 0;
-    if (fixed && e == cudaSuccess) {
-      // every entry of the other two buffers is written by each sweep
-      if (known || alias)
-        launch_to_fixed(h->S, sp, F, h->n_pad, h->ld, upper(h), false, sym, df, h->st);
+    if (fixed) {
+      // an S that is converted in place holds integers until the last sweep:
+      // whatever can fail for want of memory comes before that
       std::vector<SweepScale> f = sweep_scales(h->hin, h->n_pad, h->cfg.C);
       const std::vector<SweepScale> f1 = sweep_scales(h->hin, h->n_pad, 1.0);
       f.insert(f.end(), f1.begin(), f1.end());
@@ -973,6 +985,11 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(scales, f.data(), f.size() * sizeof(SweepScale),
                             cudaMemcpyHostToDevice, h->st);
+      if (e == cudaSuccess) e = sweep_fixed_ready(sp);
+      if (e != cudaSuccess) return give_up(e);
+      // every entry of the other two buffers is written by each sweep
+      if (known || alias)
+        launch_to_fixed(h->S, sp, F, h->n_pad, h->ld, upper(h), false, sym, df, h->st);
     }
   }
   if (alias) bufs[0] = h->S;
@@ -983,7 +1000,7 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
     cudaMemsetAsync(bufs[2], 0, bytes, h->st);
   }
   void *A = bufs[0], *B = bufs[1], *T = bufs[2];
-  if (e == cudaSuccess) e = cudaGetLastError();
+  e = cudaGetLastError();
   const float* w = h->weighted ? h->d_in_w : nullptr;
   while (e == cudaSuccess && it < max_sweeps) {
     cudaMemsetAsync(h->diffbits, 0, sizeof(unsigned long long), h->st);
@@ -1023,7 +1040,10 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
       }
     }
   }
-  if (e == cudaSuccess) {
+  // A is the last whole iterate, also after an error: an S that the sweeps ran
+  // in becomes values again in either case, one with buffers of its own keeps
+  // what it held
+  if (e == cudaSuccess || alias) {
     if (fixed) {
       launch_from_fixed((const long long*)A, alias ? A : h->S, sp, h->n_pad, h->ld, upper(h),
                         h->st);
@@ -1031,15 +1051,17 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
       launch_symmetrize(A, wp, h->n_pad, h->ld, h->st);
       if (!alias) launch_convert(A, wp, h->S, sp, (int64_t)elems, h->st);
     }
-    e = cudaGetLastError();
+    const cudaError_t f = cudaGetLastError();
+    if (e == cudaSuccess) e = f;
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
+  const cudaError_t fin = cudaStreamSynchronize(h->st);
+  if (e == cudaSuccess) e = fin;
   if (scales) cudaFree(scales);
   // bufs[] holds three distinct buffers (bufs[0] is the old S when aliasing);
   // keep the result as S when aliasing and free every other buffer once.
   // A re-anchor of an FP32 S keeps them when they are small (allocating and
   // freeing 3 x 0.8 GB took 2.2 of 5.8 ms at n = 10,007).
-  if (alias && e == cudaSuccess) h->S = A;
+  if (alias) h->S = A;
   const bool keep = !alias && !known && 3 * bytes <= ANCHOR_KEEP;
   for (int b = 0; b < 3; ++b) {
     if (keep)
@@ -1049,7 +1071,8 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
   }
   if (keep) h->anchor_bytes = bytes;
   if (e != cudaSuccess)
-    return fail(h, SR_ERR_CUDA, std::string("Jacobi sweep: ") + cudaGetErrorString(e));
+    return fail(h, e == cudaErrorMemoryAllocation ? SR_ERR_OOM : SR_ERR_CUDA,
+                std::string("Jacobi sweep: ") + cudaGetErrorString(e));
   *last_diff = diff;
   *sweeps_done = it;
   if (tol_used) *tol_used = tol;

@@ -290,6 +290,22 @@ __global__ void k_from_fixed(const long long* F, T* S, int64_t ld, int upper) {
 
 }  // namespace
 
+// Loads the kernels of the sweeps and of the way back (a kernel loaded at its
+// first launch can fail there for want of memory).
+cudaError_t sweep_fixed_ready(int prec) {
+  const void* fn[4] = {(const void*)k_sweep<false>, (const void*)k_sweep<true>,
+                       prec == 64 ? (const void*)k_to_fixed<double, false, true>
+                                  : (const void*)k_to_fixed<float, false, true>,
+                       prec == 64 ? (const void*)k_from_fixed<double>
+                                  : (const void*)k_from_fixed<float>};
+  for (const void* f : fn) {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, f);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 void launch_sweep_fixed(const DevAdj& in, const SweepScale* s1, const SweepScale* s2,
                         const long long* S, int64_t ld, int n_pad, long long* T, long long* Snew,
                         long long diag, int n_diag, unsigned long long* maxd, cudaStream_t st) {

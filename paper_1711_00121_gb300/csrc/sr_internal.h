@@ -318,6 +318,8 @@ void launch_to_fixed(const void* S, int prec, long long* F, int n_pad, int64_t l
                      bool check, double tol, unsigned int* flags, cudaStream_t st);
 void launch_from_fixed(const long long* F, void* S, int prec, int n_pad, int64_t ld, int upper,
                        cudaStream_t st);
+// Loads the kernels of the three above (prec: of S).
+cudaError_t sweep_fixed_ready(int prec);
 // S[J, I] = S[I, J]^T for all 128-tiles I < J (restores the lower triangle)
 void launch_mirror_lower(void* A, int prec, int n_pad, int64_t ld, cudaStream_t st);
 void launch_symmetrize(void* A, int prec, int n_pad, int64_t ld, cudaStream_t st);

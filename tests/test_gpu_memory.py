@@ -1,0 +1,100 @@
+"""Calls whose allocations fail, and what a handle holds afterwards.
+
+An allocation is made to fail on the host: a handle larger than the device's
+memory is refused by cudaMalloc at once, and a tensor of PyTorch's takes what is
+free but for a few MB."""
+import numpy as np
+import pytest
+
+from oracle import simrank_oracle as O
+from synth import chung_lu_digraph
+
+pytestmark = pytest.mark.gpu
+
+SR_ERR_OOM = 5
+
+
+@pytest.fixture(scope="module")
+def P():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_1711_00121_gb300 as P
+
+    return P
+
+
+def too_large(P):
+    """A handle of 1.3 TB of S."""
+    e = np.array([0], np.int32), np.array([1], np.int32)
+    with pytest.raises(P.SimrankError) as err:
+        P.SimRank(400_000, *e, C=0.6, K=1, s_precision=64)
+    assert err.value.status == SR_ERR_OOM
+
+
+class Squeeze:
+    """All free device memory but `keep` bytes is taken inside the block."""
+
+    def __init__(self, keep):
+        import torch
+
+        torch.cuda.empty_cache()
+        free, _ = torch.cuda.mem_get_info()
+        self.hold = torch.empty(max(1, free - keep), dtype=torch.uint8, device="cuda")
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        import torch
+
+        self.hold = None
+        torch.cuda.empty_cache()
+
+
+def fixed_point_handle(P, prec, n=2000, **kw):
+    C = 0.6
+    s, d = chung_lu_digraph(n, 8 * n, 2.1, 2.1, 3)
+    S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-15)
+    h = P.SimRank(n, s, d, S0=S0.astype(np.float64 if prec == 64 else np.float32), C=C, K=5,
+                  s_precision=prec, **kw)
+    return h, S0
+
+
+@pytest.mark.parametrize("upper", [0, 1])
+def test_fp64_s_after_an_error_of_another_call(P, upper):
+    """Sweeps of an FP64 S run in its own memory; whatever ends them, S stays the
+    matrix it was (here the fixed point, which sweeps keep): 1e-12."""
+    h, S0 = fixed_point_handle(P, 64, upper_only=upper)
+    too_large(P)
+    try:
+        h.reanchor(2)
+    except P.SimrankError:
+        pass
+    assert np.max(np.abs(h.dense() - S0)) < 1e-12
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+def test_reanchor_without_memory(P, prec):
+    """From too little for the first work buffer to enough for everything: a
+    re-anchor works or is refused as out of memory, and S is the fixed point
+    either way (1e-12; stored in FP32 1e-6)."""
+    h, S0 = fixed_point_handle(P, prec)
+    tol = 1e-12 if prec == 64 else 1e-6
+    buf = 2048 * 2048 * 8
+    refused = 0
+    for keep in [buf // 2, 2 * buf - (2 << 20)] + [b * buf + (k << 20) for b in (2, 3)
+                                                  for k in (0, 2, 4, 8)]:
+        with Squeeze(keep):
+            try:
+                h.reanchor(2)
+            except P.SimrankError as e:
+                assert e.status == SR_ERR_OOM, str(e)
+                refused += 1
+        assert np.max(np.abs(h.dense() - S0)) < tol, keep
+    assert refused
+    h.reanchor(2)
+    assert np.max(np.abs(h.dense() - S0)) < tol
