@@ -142,7 +142,14 @@ struct simrank_ctx {
 
 namespace {
 
+// The CUDA error that a status reports is cleared with it: the runtime keeps it
+// until it is read, and the next call's launch checks would report it again.
+void clear_reported(simrank_status s) {
+  if (s == SR_ERR_CUDA || s == SR_ERR_OOM) cudaGetLastError();
+}
+
 simrank_status fail(simrank_ctx* h, simrank_status s, const std::string& msg) {
+  clear_reported(s);
   if (h)
     h->err = msg;
   else
@@ -505,7 +512,6 @@ simrank_status s_update_launch(simrank_ctx* h, int k0, int k1, int use_masks) {
   if (digits && ob_ensure(h, 30, digits_scratch_bytes(h->cfg.s_precision, h->n_pad)) != SR_OK) {
     digits = false;  // no memory for the digits
     h->err.clear();
-    cudaGetLastError();
   }
   if (digits) {
     if (launch_s_update_digits(h->S, h->cfg.s_precision, h->ld, panel_for_s(h), h->K1, nT,
@@ -936,7 +942,6 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
     if (held) {
       bufs[b] = h->anchor_buf[b];
     } else if (cudaMalloc(&bufs[b], bytes) != cudaSuccess) {
-      cudaGetLastError();
       for (void* p : bufs)
         if (p) cudaFree(p);
       return fail(h, SR_ERR_OOM, "cudaMalloc of Jacobi buffers failed");
@@ -948,7 +953,6 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
   SweepScale* scales = nullptr;
   // ends the call before S has been touched; a handle's kept buffers stay
   auto give_up = [&](cudaError_t why) {
-    cudaGetLastError();
     if (scales) cudaFree(scales);
     if (!held)
       for (void* p : bufs)
@@ -2606,6 +2610,7 @@ struct simrank_multi {
 namespace {
 
 simrank_status mfail(simrank_multi* h, simrank_status s, const std::string& msg) {
+  clear_reported(s);
   if (h)
     h->err = msg;
   else

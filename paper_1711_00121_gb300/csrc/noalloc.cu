@@ -74,6 +74,7 @@ cudaError_t scratch_address(unsigned char** out) {
 }
 
 simrank_status na_fail(simrank_status s, const std::string& m) {
+  if (s == SR_ERR_CUDA) cudaGetLastError();  // reported once
   set_global_error(m);
   return s;
 }

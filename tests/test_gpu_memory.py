@@ -98,3 +98,21 @@ def test_reanchor_without_memory(P, prec):
     assert refused
     h.reanchor(2)
     assert np.max(np.abs(h.dense() - S0)) < tol
+
+
+def test_an_error_is_reported_once(P):
+    """After a refused handle the calls on other handles work: re-anchor,
+    update, query, many graphs."""
+    h, S0 = fixed_point_handle(P, 32)
+    n = S0.shape[0]
+    s, d = chung_lu_digraph(n, 8 * n, 2.1, 2.1, 3)
+    mh = P.MultiSimRank([(n, s, d)], C=0.6, K=5, s_precision=32, init_tol=1e-9)
+    new = next((x, 7, 1) for x in range(8, n) if (x, 7) not in set(zip(s.tolist(), d.tolist())))
+    calls = [lambda: h.reanchor(1), lambda: h.apply_updates([new]), lambda: h.columns([7]),
+             lambda: mh.apply_updates([np.array([new], np.int32)]), mh.sync, h.sync]
+    for call in calls:
+        too_large(P)
+        call()
+    want, _ = O.sequential_unit_updates(n, s, d, S0, [new], 0.6, 5)
+    assert np.max(np.abs(h.columns([7])[:, 0] - want[:, 7])) < 1e-6
+    assert np.max(np.abs(mh.columns(0, [7])[:, 0] - want[:, 7])) < 1e-6
