@@ -72,8 +72,8 @@ struct simrank_ctx {
   int order_n = 0;
   uint64_t* d_jobs = nullptr;    // the same pairs, two per job where they share I
   int jobs_n = 0;
-  void* W = nullptr;              // (xi, eta) working columns of the pre-update kernel
-  void* rinv = nullptr;           // its per-row (C / in-degree, 1 / in-degree)
+  double* W = nullptr;            // (xi, eta) working columns of the pre-update kernel
+  double* rinv = nullptr;         // its per-row (C / in-degree, 1 / in-degree)
   int32_t* loff = nullptr;        // its per-row offsets inside the tile
   long long* flowY = nullptr;     // its row sums of the flow form
   SweepScale* flow_tab = nullptr; // 1 / d for d <= n_cap, then C^(k+1) for k <= K
@@ -178,7 +178,29 @@ inline int elem_bytes(const simrank_ctx* h) { return h->cfg.s_precision == 64 ? 
 
 template <typename T>
 cudaError_t dev_alloc(T** p, size_t count) {
-  return cudaMalloc((void**)p, std::max<size_t>(count, 1) * sizeof(T));
+  const cudaError_t e = cudaMalloc((void**)p, std::max<size_t>(count, 1) * sizeof(T));
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
+
+// Memory made at the first call that needs it: *p as it is, if it is there.
+template <typename T>
+cudaError_t dev_alloc_once(T** p, size_t count) {
+  return *p ? cudaSuccess : dev_alloc(p, count);
+}
+
+// *p with room for `need` elements, without its old contents.  After a failure
+// there is no memory and no capacity, so that the next call asks again.
+template <typename T>
+cudaError_t dev_grow(T** p, int64_t* cap, int64_t need) {
+  if (need <= *cap) return cudaSuccess;
+  const int64_t want = std::max<int64_t>(need, 2 * *cap);
+  if (*p) cudaFree(*p);
+  *p = nullptr;
+  *cap = 0;
+  const cudaError_t e = dev_alloc(p, (size_t)want);
+  if (e == cudaSuccess) *cap = want;
+  return e;
 }
 
 // Builds adjacency lists (row key[e] gets val[e], in the order of e) with
@@ -367,16 +389,8 @@ simrank_status validate(simrank_ctx* h, const simrank_update* u, int64_t count, 
 }
 
 simrank_status ensure_dev_capacity(simrank_ctx* h, int64_t nsrc, int64_t nops) {
-  if (nsrc > h->srcs_cap) {
-    if (h->d_srcs) cudaFree(h->d_srcs);
-    h->srcs_cap = std::max<int64_t>(nsrc, 2 * h->srcs_cap);
-    CUDA_TRY(h, dev_alloc(&h->d_srcs, (size_t)h->srcs_cap));
-  }
-  if (nops > h->ops_cap) {
-    if (h->d_ops) cudaFree(h->d_ops);
-    h->ops_cap = std::max<int64_t>(nops, 2 * h->ops_cap);
-    CUDA_TRY(h, dev_alloc(&h->d_ops, (size_t)h->ops_cap));
-  }
+  CUDA_TRY(h, dev_grow(&h->d_srcs, &h->srcs_cap, nsrc));
+  CUDA_TRY(h, dev_grow(&h->d_ops, &h->ops_cap, nops));
   return SR_OK;
 }
 
@@ -691,9 +705,6 @@ simrank_status flush_pending(simrank_ctx* h) {
 // in-degree d <= n_cap and C^(k+1) for k <= K (cpow on the host too).
 simrank_status flow_tables(simrank_ctx* h) {
   if (h->flow_tab) return SR_OK;
-  CUDA_TRY(h, dev_alloc(&h->flow_tab, (size_t)h->n_cap + 1 + h->K1));
-  launch_flow_recip(h->flow_tab, h->n_cap + 1, h->st);
-  h->launches += 1;
   h->cpow.resize((size_t)h->K1);
   for (int k = 0; k < h->K1; ++k) {
     // C^(k+1) = r 2^-(63 + sh), 2^62 <= r < 2^63
@@ -701,6 +712,9 @@ simrank_status flow_tables(simrank_ctx* h) {
     const double f = std::frexp(std::pow(h->cfg.C, k + 1), &e);
     h->cpow[k] = SweepScale{(unsigned long long)std::ldexp(f, 63), 0, -e};
   }
+  CUDA_TRY(h, dev_alloc(&h->flow_tab, (size_t)h->n_cap + 1 + h->K1));
+  launch_flow_recip(h->flow_tab, h->n_cap + 1, h->st);
+  h->launches += 1;
   CUDA_TRY(h, cudaMemcpyAsync(h->flow_tab + h->n_cap + 1, h->cpow.data(),
                               h->cpow.size() * sizeof(SweepScale), cudaMemcpyHostToDevice, h->st));
   return SR_OK;
@@ -729,11 +743,11 @@ simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, i
   }
   const bool defer = deferring(h);
   if (defer && !h->Pp) {
-    const size_t pb = (size_t)h->nT_cap * 2 * group(h) * h->K1 * PT * sizeof(float);
-    CUDA_TRY(h, cudaMalloc(&h->Pp, pb));
-    CUDA_TRY(h, cudaMemsetAsync(h->Pp, 0, pb, h->st));
-    CUDA_TRY(h, dev_alloc(&h->pXi, (size_t)h->nT_cap));
-    CUDA_TRY(h, dev_alloc(&h->pEta, (size_t)h->nT_cap));
+    const size_t pe = (size_t)h->nT_cap * 2 * group(h) * h->K1 * PT;
+    CUDA_TRY(h, dev_alloc_once(&h->pXi, (size_t)h->nT_cap));
+    CUDA_TRY(h, dev_alloc_once(&h->pEta, (size_t)h->nT_cap));
+    CUDA_TRY(h, dev_alloc(&h->Pp, pe));
+    CUDA_TRY(h, cudaMemsetAsync(h->Pp, 0, pe * sizeof(float), h->st));
     CUDA_TRY(h, cudaMemsetAsync(h->pXi, 0, h->nT_cap * sizeof(uint64_t), h->st));
     CUDA_TRY(h, cudaMemsetAsync(h->pEta, 0, h->nT_cap * sizeof(uint64_t), h->st));
   }
@@ -785,13 +799,11 @@ simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, i
     pp.nT_cap = h->nT_cap;
     simrank_status fs = flow_tables(h);
     if (fs != SR_OK) return fs;
-    if (!h->W) {
-      CUDA_TRY(h, cudaMalloc(&h->W, (size_t)h->K1 * h->n_pad * 2 * sizeof(double)));
-      CUDA_TRY(h, dev_alloc(&h->flowY, (size_t)h->n_pad));
-      CUDA_TRY(h, cudaMalloc(&h->rinv, (size_t)h->n_pad * 2 * sizeof(double)));
-      CUDA_TRY(h, dev_alloc(&h->loff, (size_t)h->n_pad));
-      CUDA_TRY(h, dev_alloc(&h->tile_nnz, (size_t)h->nT_cap));
-    }
+    CUDA_TRY(h, dev_alloc_once(&h->W, (size_t)h->K1 * h->n_pad * 2));
+    CUDA_TRY(h, dev_alloc_once(&h->flowY, (size_t)h->n_pad));
+    CUDA_TRY(h, dev_alloc_once(&h->rinv, (size_t)h->n_pad * 2));
+    CUDA_TRY(h, dev_alloc_once(&h->loff, (size_t)h->n_pad));
+    CUDA_TRY(h, dev_alloc_once(&h->tile_nnz, (size_t)h->nT_cap));
     pp.W = h->W;
     pp.rinv = h->rinv;
     pp.loff = h->loff;
@@ -1261,7 +1273,6 @@ simrank_status run_one_shot(simrank_ctx* h, const std::map<int32_t, std::vector<
   std::vector<RowChunk> chv;
   build_chunks(h->hin, n_pad, chv, nullptr);
   if ((s = upload_chunks(h, chv, h->cur_hor, &h->cur_hor_cap)) != SR_OK) return s;
-  h->col_chunks_ok = false;
   CUDA_TRY(h, cudaStreamSynchronize(h->st));
   const bool fixed = wbits < 0x7f800000u;
   float wmax;
@@ -1428,29 +1439,22 @@ bool patch_row_chunks(simrank_ctx* h, const HostAdj& A, int a, std::vector<RowCh
 
 simrank_status upload_chunks(simrank_ctx* h, const std::vector<RowChunk>& v, ChunkList& L,
                              int64_t* cap) {
-  if ((int64_t)v.size() > *cap) {
-    if (L.chunks) cudaFree(L.chunks);
-    L.chunks = nullptr;
-    *cap = std::max<int64_t>((int64_t)v.size(), 2 * *cap);
-    CUDA_TRY(h, dev_alloc(&L.chunks, (size_t)*cap));
-  }
-  L.count = (int64_t)v.size();
+  // the lists of column updates are current again once that path says so
+  h->col_chunks_ok = false;
+  L.count = L.multi_count = 0;
+  CUDA_TRY(h, dev_grow(&L.chunks, cap, (int64_t)v.size()));
   if (!v.empty())
     CUDA_TRY(h, cudaMemcpyAsync(L.chunks, v.data(), v.size() * sizeof(RowChunk),
                                 cudaMemcpyHostToDevice, h->st));
   std::vector<int32_t> multi;
   for (size_t q = 0; q < v.size(); ++q)
     if (!(v[q].len & CH_ONLY) && (q == 0 || v[q - 1].row != v[q].row)) multi.push_back(v[q].row);
-  if ((int64_t)multi.size() > L.multi_cap) {
-    if (L.multi) cudaFree(L.multi);
-    L.multi = nullptr;
-    L.multi_cap = std::max<int64_t>((int64_t)multi.size(), 2 * L.multi_cap);
-    CUDA_TRY(h, dev_alloc(&L.multi, (size_t)L.multi_cap));
-  }
-  L.multi_count = (int64_t)multi.size();
+  CUDA_TRY(h, dev_grow(&L.multi, &L.multi_cap, (int64_t)multi.size()));
   if (!multi.empty())
     CUDA_TRY(h, cudaMemcpyAsync(L.multi, multi.data(), multi.size() * sizeof(int32_t),
                                 cudaMemcpyHostToDevice, h->st));
+  L.count = (int64_t)v.size();
+  L.multi_count = (int64_t)multi.size();
   return SR_OK;
 }
 
@@ -1515,15 +1519,10 @@ simrank_status run_column_update(simrank_ctx* h, const std::vector<int32_t>& src
   }
   const int64_t n_items = (int64_t)it_tile.size();
   const int64_t need = 2 * n_items + h->nT_cap;
-  if (need > h->col_items_cap) {
-    if (h->col_items) cudaFree(h->col_items);
-    h->col_items = nullptr;
-    CUDA_TRY(h, dev_alloc(&h->col_items, (size_t)need));
-    h->col_items_cap = need;
-  }
+  CUDA_TRY(h, dev_grow(&h->col_items, &h->col_items_cap, need));
   if (!h->col_gacc) {
+    CUDA_TRY(h, dev_alloc_once(&h->col_tcount, (size_t)h->nT_cap));
     CUDA_TRY(h, dev_alloc(&h->col_gacc, (size_t)h->nT_cap * 2 * PT));
-    CUDA_TRY(h, dev_alloc(&h->col_tcount, (size_t)h->nT_cap));
     CUDA_TRY(h, cudaMemsetAsync(h->col_gacc, 0, (size_t)h->nT_cap * 2 * PT * sizeof(double), h->st));
     CUDA_TRY(h, cudaMemsetAsync(h->col_tcount, 0, (size_t)h->nT_cap * sizeof(unsigned int), h->st));
   }
@@ -1565,12 +1564,7 @@ simrank_status column_mode_columns(simrank_ctx* h, const int32_t* cols, int ncol
   simrank_status s;
   if ((s = ob_ensure(h, 10, per_col * Bmax)) != SR_OK) return s;
   if ((s = ob_ensure(h, 28, 3 * (size_t)n_pad * eb)) != SR_OK) return s;
-  if (ncols > h->cols_cap) {
-    if (h->d_cols) cudaFree(h->d_cols);
-    h->d_cols = nullptr;
-    h->cols_cap = ncols;
-    CUDA_TRY(h, dev_alloc(&h->d_cols, (size_t)ncols));
-  }
+  CUDA_TRY(h, dev_grow(&h->d_cols, &h->cols_cap, ncols));
   CUDA_TRY(h, cudaMemcpyAsync(h->d_cols, cols, ncols * sizeof(int32_t), cudaMemcpyHostToDevice,
                               h->st));
   const size_t ob = (size_t)h->n_cur * ncols * (out_fp64 ? 8 : 4);
@@ -2226,11 +2220,7 @@ simrank_status simrank_columns(simrank_t h, const int32_t* cols, int32_t ncols, 
   for (int32_t& x : icols) x = h->ext2int[x];
   cols = icols.data();
   const int32_t* perm = h->relabeled ? h->d_ext2int : nullptr;
-  if (ncols > h->cols_cap) {
-    if (h->d_cols) cudaFree(h->d_cols);
-    h->cols_cap = ncols;
-    CUDA_TRY(h, dev_alloc(&h->d_cols, (size_t)ncols));
-  }
+  CUDA_TRY(h, dev_grow(&h->d_cols, &h->cols_cap, ncols));
   CUDA_TRY(h, cudaMemcpyAsync(h->d_cols, cols, ncols * sizeof(int32_t), cudaMemcpyHostToDevice,
                               h->st));
   const size_t ob = (size_t)h->n_cur * ncols * (out_fp64 ? 8 : 4);
@@ -2355,7 +2345,6 @@ simrank_status simrank_grad(simrank_t h, const int32_t* pa, const int32_t* pb, c
   if ((s = upload_chunks(h, ch, h->cur_fwd, &h->cur_fwd_cap)) != SR_OK) return s;
   build_chunks(h->hin, n_pad, ch);
   if ((s = upload_chunks(h, ch, h->cur_hor, &h->cur_hor_cap)) != SR_OK) return s;
-  h->col_chunks_ok = false;
   WeightView wv;
   if (h->weighted) {
     wv.in_w = h->d_in_w;
@@ -2572,7 +2561,7 @@ struct simrank_multi {
   int64_t steps_cap = 0;
   int* d_count = nullptr;  // [launch] number of steps
   int* d_ntiles = nullptr; // [launch] tile pairs listed
-  int64_t launch_cap = 0;
+  int64_t count_cap = 0, ntiles_cap = 0;
   uint64_t* d_tiles = nullptr;
   int64_t tiles_cap = 0;
   int32_t* d_srcs = nullptr;
@@ -2625,15 +2614,6 @@ simrank_status mfail(simrank_multi* h, simrank_status s, const std::string& msg)
       return mfail((h), e__ == cudaErrorMemoryAllocation ? SR_ERR_OOM : SR_ERR_CUDA,       \
                    std::string(#call) + ": " + cudaGetErrorString(e__));                   \
   } while (0)
-
-template <typename T>
-cudaError_t grow_dev(T** p, int64_t* cap, int64_t need) {
-  if (need <= *cap) return cudaSuccess;
-  if (*p) cudaFree(*p);
-  *p = nullptr;
-  *cap = std::max<int64_t>(need, 2 * *cap);
-  return dev_alloc(p, (size_t)*cap);
-}
 
 void multi_free(simrank_multi* h) {
   if (h->exec) cudaGraphExecDestroy(h->exec);
@@ -2884,19 +2864,12 @@ simrank_status simrank_multi_apply(simrank_multi_t h, const simrank_update* u,
       }
   }
   const int L = (int)h->h_count.size();
-  MCUDA_TRY(h, grow_dev(&h->d_steps, &h->steps_cap, (int64_t)h->h_steps.size()));
-  if (L > h->launch_cap) {
-    if (h->d_count) cudaFree(h->d_count);
-    if (h->d_ntiles) cudaFree(h->d_ntiles);
-    h->d_count = nullptr;
-    h->d_ntiles = nullptr;
-    h->launch_cap = std::max<int64_t>(L, 2 * h->launch_cap);
-    MCUDA_TRY(h, dev_alloc(&h->d_count, (size_t)h->launch_cap));
-    MCUDA_TRY(h, dev_alloc(&h->d_ntiles, (size_t)h->launch_cap));
-  }
-  MCUDA_TRY(h, grow_dev(&h->d_tiles, &h->tiles_cap, tiles_need));
-  MCUDA_TRY(h, grow_dev(&h->d_srcs, &h->srcs_cap, (int64_t)h->h_srcs.size()));
-  MCUDA_TRY(h, grow_dev(&h->d_ops, &h->ops_cap, (int64_t)h->h_ops.size()));
+  MCUDA_TRY(h, dev_grow(&h->d_steps, &h->steps_cap, (int64_t)h->h_steps.size()));
+  MCUDA_TRY(h, dev_grow(&h->d_count, &h->count_cap, L));
+  MCUDA_TRY(h, dev_grow(&h->d_ntiles, &h->ntiles_cap, L));
+  MCUDA_TRY(h, dev_grow(&h->d_tiles, &h->tiles_cap, tiles_need));
+  MCUDA_TRY(h, dev_grow(&h->d_srcs, &h->srcs_cap, (int64_t)h->h_srcs.size()));
+  MCUDA_TRY(h, dev_grow(&h->d_ops, &h->ops_cap, (int64_t)h->h_ops.size()));
   MCUDA_TRY(h, cudaMemcpyAsync(h->d_desc, h->h_desc.data(), G * sizeof(MultiGraphDesc),
                                cudaMemcpyHostToDevice, h->st));
   MCUDA_TRY(h, cudaMemcpyAsync(h->d_steps, h->h_steps.data(), h->h_steps.size() * sizeof(MultiStep),

@@ -116,3 +116,26 @@ def test_an_error_is_reported_once(P):
     want, _ = O.sequential_unit_updates(n, s, d, S0, [new], 0.6, 5)
     assert np.max(np.abs(h.columns([7])[:, 0] - want[:, 7])) < 1e-6
     assert np.max(np.abs(mh.columns(0, [7])[:, 0] - want[:, 7])) < 1e-6
+
+
+@pytest.mark.parametrize("mode", ["dense", "column", "many"])
+def test_query_after_a_refused_query(P, mode):
+    """A query that is refused for want of memory takes its buffers' capacities
+    with it: smaller and equal ones afterwards get memory of their own."""
+    n, C, K = 1500, 0.6, 30
+    s, d = chung_lu_digraph(n, 8 * n, 2.1, 2.1, 5)
+    if mode == "many":
+        mh = P.MultiSimRank([(n, s, d)], C=C, K=K, s_precision=32)
+        query = lambda cols: mh.columns(0, cols)  # noqa: E731
+    else:
+        h = P.SimRank(n, s, d, C=C, K=K, s_precision=32, mode=P.MODE_DENSE if mode == "dense" else P.MODE_COLUMN)
+        query = h.columns
+    want = O.partial_sim_block(O.transition_matrix(n, s, d, sparse=True), np.arange(n), K, C)
+    few = np.array([3, 700], np.int32)
+    many = np.tile(np.arange(n, dtype=np.int32), 200)  # 3.6 GB of scratch
+    for ask in (few, many[:5000], few):
+        with Squeeze(64 << 20):
+            with pytest.raises(P.SimrankError) as err:
+                query(many)
+            assert err.value.status == SR_ERR_OOM
+        assert np.max(np.abs(query(ask) - want[:, ask])) < 1e-6
