@@ -46,6 +46,9 @@ struct simrank_ctx {
   // host mirror of the graph (storage ids)
   HostAdj hin, hout;
   EdgeSet edges;
+  // an update's host graph is made before its device work is queued; true from
+  // there until all of it is, and so for good once that fails
+  bool part_way = false;
   // device graph
   DevAdj din, dout;
   float* d_in_w = nullptr;
@@ -156,6 +159,11 @@ simrank_status fail(simrank_ctx* h, simrank_status s, const std::string& msg) {
     g_init_error = msg;
   return s;
 }
+
+// What a call answers that would build on a graph the device does not hold
+// (its lists would name places of the pools that were never written).
+const char* const PART_WAY =
+    "an earlier update failed part way: this handle takes no further updates";
 
 #define CUDA_TRY(h, call)                                                                  \
   do {                                                                                     \
@@ -2045,6 +2053,7 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
   if (count < 0 || (count > 0 && !u)) return fail(h, SR_ERR_ARG, "bad update array");
   if (count == 0) return SR_OK;
   if (h->weighted) return fail(h, SR_ERR_UNSUPPORTED, "updates on a weighted graph");
+  if (h->part_way) return fail(h, SR_ERR_CUDA, PART_WAY);
   // caller ids -> storage ids (new ids >= n_cur map to themselves)
   std::vector<simrank_update> um(u, u + count);
   auto to_int = [&](int32_t x) { return (x >= 0 && x < h->n_cap) ? h->ext2int[x] : x; };
@@ -2124,6 +2133,7 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
       h->col_last_j = j;
       std::vector<PatchOp> ops1;
       const int d_j = h->hin.len[j];
+      h->part_way = true;
       for (int32_t i : b.srcs) {
         if (op > 0) {
           adj_append(h->hin, j, i, ops1, true);
@@ -2144,6 +2154,7 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
       if ((s = run_column_update(h, b.srcs, j, op, d_j, 0, (int64_t)ops1.size(), h->d_srcs)) !=
           SR_OK)
         return s;
+      h->part_way = false;
     }
     h->stats.updates += count;
     return SR_OK;
@@ -2156,6 +2167,7 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
     std::map<int32_t, std::vector<int32_t>> plus, minus;
     std::vector<RowChunk> old_chunks;
     build_chunks(h->hin, h->n_pad, old_chunks);
+    h->part_way = true;
     for (const Block& b : blocks) {
       auto& dstv = (b.op > 0 ? plus : minus)[b.sink];
       dstv.insert(dstv.end(), b.srcs.begin(), b.srcs.end());
@@ -2176,16 +2188,19 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
     if ((s = grow_pool(h, h->dout, h->hout)) != SR_OK) return s;
     if ((s = ensure_dev_capacity(h, 1, (int64_t)ops.size())) != SR_OK) return s;
     if ((s = run_one_shot(h, plus, minus, ops, old_chunks)) != SR_OK) return s;
+    h->part_way = false;
     h->stats.updates += count;
     return maybe_reanchor(h, count);
   }
   if (h->cfg.apply == SR_APPLY_UNIT) {
+    h->part_way = true;
     for (int64_t t = 0; t < count; ++t) add_r1(um[t].dst, um[t].op, {um[t].src});
   } else {
     // the canonical block order is defined on caller ids
     std::vector<Block> blocks;
     std::string msg;
     if ((s = plan_blocks(u, count, n_old, blocks, msg)) != SR_OK) return fail(h, s, msg);
+    h->part_way = true;
     for (Block& b : blocks) {
       for (int32_t& x : b.srcs) x = to_int(x);
       add_r1(to_int(b.sink), b.op, b.srcs);
@@ -2196,16 +2211,19 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
   if ((s = grow_pool(h, h->dout, h->hout)) != SR_OK) return s;
   if ((s = ensure_dev_capacity(h, (int64_t)srcs.size() + 2, (int64_t)ops.size())) != SR_OK) return s;
   if ((s = upload_plan(h, srcs, ops)) != SR_OK) return s;
+  simrank_status anchored = SR_OK;
   for (const R1& r : plan) {
     if ((s = run_rank_one(h, r.src_off, r.delta, r.sink, r.op, r.d_j, r.op_begin, r.op_end)) !=
         SR_OK)
       return s;
-    // every rank-one update (a unit update or a sink block) counts its edges
-    if ((s = maybe_reanchor(h, r.delta)) != SR_OK) return s;
+    // every rank-one update (a unit update or a sink block) counts its edges;
+    // a re-anchor that fails leaves S valid, and the updates go on
+    if (anchored == SR_OK) anchored = maybe_reanchor(h, r.delta);
   }
   if ((s = flush_pending(h)) != SR_OK) return s;
+  h->part_way = false;
   h->stats.updates += count;
-  return SR_OK;
+  return anchored;
 }
 
 simrank_status simrank_columns(simrank_t h, const int32_t* cols, int32_t ncols, void* out,
@@ -2332,6 +2350,7 @@ simrank_status simrank_grad(simrank_t h, const int32_t* pa, const int32_t* pb, c
   if (!h) return fail(nullptr, SR_ERR_ARG, "null handle");
   if (npairs < 0 || (npairs > 0 && (!pa || !pb || !target)) || !loss || !grad_weight)
     return fail(h, SR_ERR_ARG, "bad pair arrays");
+  if (h->part_way) return fail(h, SR_ERR_CUDA, PART_WAY);
   if (h->stats.updates > 0)
     return fail(h, SR_ERR_UNSUPPORTED, "simrank_grad needs the graph as initialised (no updates)");
   const int n_pad = h->n_pad, K = h->cfg.K;
@@ -2768,6 +2787,8 @@ simrank_status simrank_multi_apply(simrank_multi_t h, const simrank_update* u,
     if (c < 0) return mfail(h, SR_ERR_ARG, "update_offsets must be non-decreasing");
     if (c > 0 && !u) return mfail(h, SR_ERR_ARG, "null update array");
     simrank_ctx* x = h->g[g];
+    if (x->part_way)
+      return mfail(h, SR_ERR_CUDA, "graph " + std::to_string(g) + ": " + PART_WAY);
     um[g].assign(u + update_offsets[g], u + update_offsets[g] + c);
     if (x->relabeled)
       for (auto& v : um[g]) {
@@ -2787,6 +2808,7 @@ simrank_status simrank_multi_apply(simrank_multi_t h, const simrank_update* u,
   std::vector<std::vector<MultiStep>> per(G);
   for (int g = 0; g < G; ++g) {
     simrank_ctx* x = h->g[g];
+    x->part_way = true;
     int n_run = x->n_cur;
     for (const simrank_update& v : um[g]) {
       const int32_t i = v.src, j = v.dst;
@@ -2928,6 +2950,7 @@ simrank_status simrank_multi_apply(simrank_multi_t h, const simrank_update* u,
   }
   const cudaError_t le = cudaGetLastError();
   if (le != cudaSuccess) return mfail(h, SR_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(le));
+  for (simrank_ctx* x : h->g) x->part_way = false;
   h->launches += 2 * (int64_t)L;
   h->sup_launches += L;
   h->stats.updates += total;

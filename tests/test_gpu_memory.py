@@ -139,3 +139,46 @@ def test_query_after_a_refused_query(P, mode):
                 query(many)
             assert err.value.status == SR_ERR_OOM
         assert np.max(np.abs(query(ask) - want[:, ask])) < 1e-6
+
+
+@pytest.mark.parametrize("kw", [dict(s_precision=64), dict(s_precision=32, tc=2, defer=2),
+                                dict(s_precision=32, tc=2, apply=2), dict(many=1)])
+def test_update_without_memory(P, kw):
+    """A first update with too little memory for its work buffers is refused, and
+    the handle then takes no further updates (the host's graph is ahead of the
+    device's) but still answers queries; with enough it gives the oracle's S."""
+    n, C, K = 600, 0.6, 1000
+    s, d = chung_lu_digraph(n, 8 * n, 2.1, 2.1, 5)
+    edges = set(zip(s.tolist(), d.tolist()))
+    ups = [(next(x for x in range(n) if x != j and (x, j) not in edges), j, 1) for j in (3, 599)]
+    S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-15)
+    want, _ = O.sequential_unit_updates(n, s, d, S0, ups, C, K)
+    cols = np.array([3, 50, 599], np.int32)
+    kw = dict(kw)
+    many = kw.pop("many", 0)
+    for keep in (6, 10, 14, 20, 30, 40, 400):
+        if many:
+            h = P.MultiSimRank([(n, s, d)], C=C, K=K, s_precision=32, tc=1)
+            apply = lambda: h.apply_updates([np.array(ups, np.int32)])  # noqa: E731
+            query = lambda: h.columns(0, cols)  # noqa: E731
+        else:
+            h = P.SimRank(n, s, d, C=C, K=K, **kw)
+            apply, query = lambda: h.apply_updates(ups), lambda: h.columns(cols)  # noqa: E731
+        failed = 0
+        with Squeeze(keep << 20):
+            try:
+                apply()
+                h.sync()
+            except P.SimrankError as e:
+                failed = e.status
+        h.sync()
+        got = query()
+        if failed:
+            assert failed in (5, 6)
+            with pytest.raises(P.SimrankError) as err:
+                apply()
+            assert "part way" in str(err.value)
+        else:
+            assert np.max(np.abs(got - want[:, cols])) < (1e-10 if kw.get("s_precision") == 64 else 1e-6)
+        h.close()
+    assert not failed
