@@ -1609,8 +1609,13 @@ simrank_status column_mode_columns(simrank_ctx* h, const int32_t* cols, int ncol
       launch_col_corr((const float* const*)h->ob[17].p, U, h->K1, bc, B, ldb, n_pad,
                       (float*)h->ob[18].p, (float*)res, h->st);
     } else {
-      for (void* P : h->hist)
-        launch_col_apply(P, prec, h->K1, bc, B, ldb, n_pad, prec, res, h->st);
+      for (void* P : h->hist) {
+        const cudaError_t e = launch_col_apply(P, prec, h->K1, bc, B, ldb, n_pad, prec, res, h->st);
+        if (e != cudaSuccess) {
+          drop();
+          return fail(h, SR_ERR_CUDA, std::string("column mode: ") + cudaGetErrorString(e));
+        }
+      }
     }
     launch_col_out(res, prec, B, ldb, h->n_cur,
                    (unsigned char*)dst + (size_t)c0 * h->n_cur * (out_fp64 ? 8 : 4), out_fp64, h->st);

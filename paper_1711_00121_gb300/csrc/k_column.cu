@@ -597,27 +597,34 @@ void launch_col_horner64(const ChunkList& hor, const int32_t* in_col, const Weig
   wide_step<double>(hor, in_col, wv.in_w, false, inv, Y, Xadd, add_scale, Yn, ldb, st);
 }
 
-void launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, int B, int ldb,
-                      int n_rows, int prec, void* Y, cudaStream_t st) {
-  const size_t smem = (size_t)B * 2 * K1 * sizeof(double);
-  const int threads = 128;
-  const int blocks = (n_rows + threads - 1) / threads;
-#define SR_COL_APPLY(T, TP)                                                                  \
-  do {                                                                                       \
-    cudaFuncSetAttribute(k_col_apply<T, TP>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
-                         (int)smem);                                                         \
-    k_col_apply<T, TP><<<blocks, threads, smem, st>>>((const TP*)P, K1, cols, B, ldb, n_rows, \
-                                              (T*)Y); \
-  } while (0)
+// The columns of one update's panels staged by a CTA take 16 (K + 1) bytes each:
+// as many columns per launch as fit in its shared memory (908 at K = 15).
+template <typename T, typename TP>
+static cudaError_t col_apply_t(const TP* P, int K1, const int32_t* cols, int B, int ldb,
+                               int n_rows, T* Y, cudaStream_t st) {
+  constexpr int most = 227 * 1024;
+  static std::atomic<unsigned long long> done{0};
+  const cudaError_t e = smem_attr_once((const void*)k_col_apply<T, TP>, most, done);
+  if (e != cudaSuccess) return e;
+  const int per = std::max(1, most / (2 * K1 * (int)sizeof(double)));
+  const int threads = 128, blocks = (n_rows + threads - 1) / threads;
+  for (int c0 = 0; c0 < B; c0 += per) {
+    const int b = std::min(per, B - c0);
+    k_col_apply<T, TP><<<blocks, threads, (size_t)b * 2 * K1 * sizeof(double), st>>>(
+        P, K1, cols + c0, b, ldb, n_rows, Y + c0);
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, int B,
+                             int ldb, int n_rows, int prec, void* Y, cudaStream_t st) {
   if (prec == 64 && p_prec == 64)
-    SR_COL_APPLY(double, double);
-  else if (prec == 64)
-    SR_COL_APPLY(double, float);
-  else if (p_prec == 64)
-    SR_COL_APPLY(float, double);
-  else
-    SR_COL_APPLY(float, float);
-#undef SR_COL_APPLY
+    return col_apply_t((const double*)P, K1, cols, B, ldb, n_rows, (double*)Y, st);
+  if (prec == 64)
+    return col_apply_t((const float*)P, K1, cols, B, ldb, n_rows, (double*)Y, st);
+  if (p_prec == 64)
+    return col_apply_t((const double*)P, K1, cols, B, ldb, n_rows, (float*)Y, st);
+  return col_apply_t((const float*)P, K1, cols, B, ldb, n_rows, (float*)Y, st);
 }
 
 void launch_col_corr(const float* const* hist, int U, int K1, const int32_t* cols, int B, int ldb,

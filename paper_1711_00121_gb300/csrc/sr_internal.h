@@ -481,8 +481,8 @@ void launch_col_horner64(const ChunkList& hor, const int32_t* in_col, const Weig
 // floats.  n_rows is a multiple of 128.
 void launch_col_corr(const float* const* hist, int U, int K1, const int32_t* cols, int B, int ldb,
                      int n_rows, float* G, float* Y, cudaStream_t st);
-void launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, int B, int ldb,
-                      int n_rows, int prec, void* Y, cudaStream_t st);
+cudaError_t launch_col_apply(const void* P, int p_prec, int K1, const int32_t* cols, int B,
+                             int ldb, int n_rows, int prec, void* Y, cudaStream_t st);
 void launch_col_out(const void* Y, int prec, int B, int ldb, int n, void* out, int out_fp64,
                     cudaStream_t st);
 void launch_col_extract(const void* Y, int prec, int B, int c, int n, double* v, cudaStream_t st);

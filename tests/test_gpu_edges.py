@@ -307,3 +307,23 @@ def test_gradient_at_block_edges(P, n, deg, npairs, K, weighted):
         n, s, d, w.astype(np.float64) if weighted else np.ones(s.size), a, b, t, 0.6, K)
     assert abs(L - L_ref) < 1e-11 * max(1.0, abs(L_ref))
     assert np.max(np.abs(g - g_ref)) < 1e-10 * max(1.0, np.max(np.abs(g_ref)))
+
+
+@pytest.mark.parametrize("K,width", [(15, 908), (15, 909), (15, 1024), (56, 256), (1000, 29)])
+def test_fp64_stored_update_over_wide_blocks(P, K, width):
+    """FP64 column queries after a stored update: as many columns as one launch of
+    its correction holds in shared memory (227 KB, 16 (K + 1) bytes a column),
+    one more, a whole block, and long series.  Against Alg 7; 1e-10, as in the
+    column-mode parity tests."""
+    n, C = 1100, 0.6
+    s, d = degrees_graph(n, [0, 1, 40], 41)
+    ups = [(next(x for x in range(3, n) if (x, 2) not in set(zip(s.tolist(), d.tolist()))), 2, 1)]
+    sr = P.SimRank(n, s, d, C=C, K=K, s_precision=64, mode=P.MODE_COLUMN)
+    sr.apply_updates(ups)
+    cols = np.random.default_rng(7).choice(n, size=width, replace=False).astype(np.int32)
+    got = sr.columns(cols)
+    ask = np.unique(np.r_[0, width // 2, width - 2, width - 1])
+    base = O.partial_sim_block(O.transition_matrix(n, s, d, sparse=True), cols[ask], K, C)
+    for c, q in enumerate(ask.tolist()):
+        want = O.inc_sr_all_p(n, s, d, base[:, c], int(cols[q]), ups, C, K)
+        assert np.max(np.abs(got[:, q] - want)) < 1e-10
