@@ -1322,6 +1322,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
             for (int q = 0; q < PT / 32; ++q)
               if (!flow_there(look[q])) look[q] = ld_flow(Fk + q * 32);
           }
+        if (stop) break;  // the whole warp: parts are missing, the panel keeps its values
         bool nx = false, ne = false;
 #pragma unroll
         for (int q = 0; q < PT / 32; ++q) {
@@ -1353,6 +1354,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
         }
       }
     }
+    if (flow && __syncthreads_or(stop)) alive = false;  // no masks, no list
   }
 
   // ---- phase 3: mask words and the affected tile pairs

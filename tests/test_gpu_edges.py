@@ -327,3 +327,33 @@ def test_fp64_stored_update_over_wide_blocks(P, K, width):
     for c, q in enumerate(ask.tolist()):
         want = O.inc_sr_all_p(n, s, d, base[:, c], int(cols[q]), ups, C, K)
         assert np.max(np.abs(got[:, q] - want)) < 1e-10
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+def test_s_after_a_wait_that_ran_out(P, prec):
+    """One update under bounds of 1 to 2,048 polls: whichever wait of the update
+    runs out, in the sums, in the copy of the columns to the panels or in a
+    barrier, an entry of S is the old one or the updated one, never a partial
+    sum.  1e-10 (FP64) and 1e-6 (FP32), as in the parity tests."""
+    n, C, K = 3000, 0.6, 10
+    s, d = degrees_graph(n, [0, 1500, 64], 43)
+    rng = np.random.default_rng(9)
+    S0 = rng.random((n, n))
+    S0 = (0.5 * (S0 + S0.T)).astype(np.float64 if prec == 64 else np.float32)
+    edges = set(zip(s.tolist(), d.tolist()))
+    ups = [(next(x for x in range(3, n) if (x, 1) not in edges), 1, 1)]
+    want, _ = O.sequential_unit_updates(n, s, d, S0.astype(np.float64), ups, C, K)
+    ran_out = 0
+    for limit in [1, 2, 3, 5, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 512, 2048]:
+        h = P.SimRank(n, s, d, S0=S0, C=C, K=K, s_precision=prec, timeout_iters=limit, s_kernel=1)
+        h.apply_updates(ups)
+        try:
+            h.sync()
+        except P.SimrankError as e:
+            assert e.status == 7
+            ran_out += 1
+        got = h.dense()
+        h.close()
+        err = np.minimum(np.abs(got - S0), np.abs(got - want))
+        assert np.max(err) < (1e-10 if prec == 64 else 1e-6), limit
+    assert ran_out
