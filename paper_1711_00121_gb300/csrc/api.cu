@@ -535,11 +535,15 @@ simrank_status s_update_launch(simrank_ctx* h, int k0, int k1, int use_masks) {
     digits = false;  // no memory for the digits
     h->err.clear();
   }
+  // no tensor map, or no shared memory for it: nothing has been launched
+  if (digits &&
+      launch_s_update_digits(h->S, h->cfg.s_precision, h->ld, panel_for_s(h), h->K1, nT, h->n_pad,
+                             h->tiles, h->ntiles, h->mXi, h->mEta, use_masks, h->n_cur,
+                             h->ob[30].p, h->counters, h->num_sms, wait_limit(h), h->st) != 0) {
+    digits = false;
+    cudaGetLastError();
+  }
   if (digits) {
-    if (launch_s_update_digits(h->S, h->cfg.s_precision, h->ld, panel_for_s(h), h->K1, nT,
-                               h->n_pad, h->tiles, h->ntiles, h->mXi, h->mEta, use_masks, h->n_cur,
-                               h->ob[30].p, h->counters, h->num_sms, wait_limit(h), h->st) != 0)
-      return fail(h, SR_ERR_CUDA, "tensor-core S update: launch setup failed");
     h->launches += 3 * ((h->K1 + 15) / 16) - 1;
   } else {
     launch_s_update(h->S, h->cfg.s_precision, h->ld, panel_for_s(h), h->K1, h->tiles, h->ntiles,

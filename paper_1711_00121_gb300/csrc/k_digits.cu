@@ -513,9 +513,10 @@ bool make_digit_map(CUtensorMap* m, const void* ptr, int n_pad, int ns, int rows
 }
 
 template <typename T>
-int digits_pass(T* S, int64_t ld, const T* P, int K1, int k0, int kc, int nT, int n_pad,
-                const uint32_t* tiles, const int* ntiles, const uint64_t* mXi, const uint64_t* mEta,
-                int use_masks, int n, unsigned char* scratch, int64_t* counters, int grid, long long wait_limit, cudaStream_t st) {
+int digits_passes(T* S, int64_t ld, const T* P, int K1, int nT, int n_pad, const uint32_t* tiles,
+                  const int* ntiles, const uint64_t* mXi, const uint64_t* mEta, int use_masks,
+                  int n, unsigned char* scratch, int64_t* counters, int grid,
+                  long long wait_limit, cudaStream_t st) {
   using D = Dig<T>;
   // scratch: digits | maxes (32 words) | meta
   unsigned char* A = scratch;
@@ -527,12 +528,15 @@ int digits_pass(T* S, int64_t ld, const T* P, int K1, int k0, int kc, int nT, in
   const int smem = D::SMEM + 1024;
   static std::atomic<unsigned long long> done{0};
   if (smem_attr_once((const void*)k_s_update_digits<T>, smem, done) != cudaSuccess) return 1;
-  cudaMemsetAsync(maxes, 0, 32 * sizeof(unsigned int), st);
-  k_digits_max<T><<<dim3(nT, 2, (kc + 7) / 8), 256, 0, st>>>(P, K1, k0, kc, maxes);
-  k_digits_pack<T><<<nT * 4, 256, 0, st>>>(P, K1, k0, kc, maxes, A, meta);
-  k_s_update_digits<T><<<grid, DG_THREADS, smem, st>>>(
-      ma, mb, S, ld, tiles, ntiles, meta, P, mXi, mEta, use_masks, K1, k0, kc, n, wait_limit,
-      (unsigned long long*)counters);
+  for (int k0 = 0; k0 < K1; k0 += DG_TERMS) {
+    const int kc = K1 - k0 < DG_TERMS ? K1 - k0 : DG_TERMS;
+    cudaMemsetAsync(maxes, 0, 32 * sizeof(unsigned int), st);
+    k_digits_max<T><<<dim3(nT, 2, (kc + 7) / 8), 256, 0, st>>>(P, K1, k0, kc, maxes);
+    k_digits_pack<T><<<nT * 4, 256, 0, st>>>(P, K1, k0, kc, maxes, A, meta);
+    k_s_update_digits<T><<<grid, DG_THREADS, smem, st>>>(
+        ma, mb, S, ld, tiles, ntiles, meta, P, mXi, mEta, use_masks, K1, k0, kc, n, wait_limit,
+        (unsigned long long*)counters);
+  }
   return 0;
 }
 
@@ -548,17 +552,12 @@ int launch_s_update_digits(void* S, int s_prec, int64_t ld, const void* P, int K
                            void* scratch, int64_t* counters, int grid, long long wait_limit,
                            cudaStream_t st) {
   unsigned char* w = (unsigned char*)scratch;
-  for (int k0 = 0; k0 < K1; k0 += DG_TERMS) {
-    const int kc = K1 - k0 < DG_TERMS ? K1 - k0 : DG_TERMS;
-    const int rc =
-        s_prec == 64
-            ? digits_pass<double>((double*)S, ld, (const double*)P, K1, k0, kc, nT, n_pad, tiles,
-                                  ntiles, mXi, mEta, use_masks, n, w, counters, grid, wait_limit, st)
-            : digits_pass<float>((float*)S, ld, (const float*)P, K1, k0, kc, nT, n_pad, tiles,
-                                 ntiles, mXi, mEta, use_masks, n, w, counters, grid, wait_limit, st);
-    if (rc) return rc;
-  }
-  return 0;
+  return s_prec == 64
+             ? digits_passes<double>((double*)S, ld, (const double*)P, K1, nT, n_pad, tiles,
+                                     ntiles, mXi, mEta, use_masks, n, w, counters, grid,
+                                     wait_limit, st)
+             : digits_passes<float>((float*)S, ld, (const float*)P, K1, nT, n_pad, tiles, ntiles,
+                                    mXi, mEta, use_masks, n, w, counters, grid, wait_limit, st);
 }
 
 }  // namespace sr

@@ -282,7 +282,8 @@ void launch_s_update(void* S, int s_prec, int64_t ld, const void* P, int K1, con
                      long long ws_wait_limit = 0, int upper = 0);
 // The pass of one update's K1 terms over the upper tile pairs listed, by exact
 // digits on the tensor cores (k_digits.cu), DG_TERMS terms a pass.
-// scratch: digits_scratch_bytes.  Returns 0 on launch.
+// scratch: digits_scratch_bytes.  Returns 0 on launch, else
+// nothing has been launched.
 size_t digits_scratch_bytes(int s_prec, int n_pad);
 int launch_s_update_digits(void* S, int s_prec, int64_t ld, const void* P, int K1, int nT,
                            int n_pad, const uint32_t* tiles, const int* ntiles,
