@@ -96,7 +96,7 @@ struct simrank_ctx {
   // work buffers of re-anchors (at most ANCHOR_KEEP bytes in all), kept between calls
   void* anchor_buf[3] = {nullptr, nullptr, nullptr};
   size_t anchor_bytes = 0;
-  PrepFit prep_fit;  // co-resident CTAs of the pre-update launch
+  PrepFit prep_fit[2];  // co-resident CTAs of the pre-update launch
   // column mode (§7): snapshot of the initial graph and the stored updates
   bool column = false;
   int32_t* g0_in_col = nullptr;
@@ -734,13 +734,14 @@ simrank_status flow_tables(simrank_ctx* h) {
 
 // One rank-one update of the current S for the sink block (srcs at d_srcs +
 // src_off, delta of them) into sink j, op = +1/-1, old in-degree d_j; the
-// graph patch ops [op_begin, op_end) turn the old graph into the new one.
+// graph patch ops [op_begin, op_end) turn the old graph into the new one, of
+// nnz edges.
 // chain = 0 runs everything before the S pass in one cooperative launch
 // (k_prep.cu, arithmetic in the precision of S); chain = 1, or a graph with
 // more tiles than the co-resident CTAs can own, takes the per-step kernels
 // (FP64 vectors).
 simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, int op, int d_j,
-                            int64_t op_begin, int64_t op_end) {
+                            int64_t op_begin, int64_t op_end, int64_t nnz) {
   const int nT = (h->n_cur + PT - 1) / PT;
   const double C = h->cfg.C;
   cudaEvent_t* pe = nullptr;
@@ -829,8 +830,7 @@ simrank_status run_rank_one(simrank_ctx* h, int64_t src_off, int delta, int j, i
     pp.counters = (unsigned long long*)h->counters;
     const int rc = launch_prep(pp, h->cfg.s_precision, h->cfg.vec_fp64 ? 1 : 0,
                                defer ? group(h) * h->K1 : 0,
-                               h->num_sms, h->cfg.prep_ctas, (int64_t)h->edges.size() + delta,
-                               h->prep_fit, h->st);
+                               h->num_sms, h->cfg.prep_ctas, nnz, h->prep_fit, h->st);
     if (rc == 1) return fail(h, SR_ERR_CUDA, "fused pre-update launch failed");
     fused = (rc == 0);
     if (fused) {
@@ -2079,6 +2079,7 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
   struct R1 {
     int32_t sink, op, d_j, delta;
     int64_t src_off, op_begin, op_end;
+    int64_t nnz;  // edges after it
   };
   std::vector<R1> plan;
   std::vector<int32_t> srcs;
@@ -2105,6 +2106,7 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
       }
     }
     r.op_end = (int64_t)ops.size();
+    r.nnz = (int64_t)h->edges.size();
     plan.push_back(r);
   };
   if (h->column) {
@@ -2222,8 +2224,8 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
   if ((s = upload_plan(h, srcs, ops)) != SR_OK) return s;
   simrank_status anchored = SR_OK;
   for (const R1& r : plan) {
-    if ((s = run_rank_one(h, r.src_off, r.delta, r.sink, r.op, r.d_j, r.op_begin, r.op_end)) !=
-        SR_OK)
+    if ((s = run_rank_one(h, r.src_off, r.delta, r.sink, r.op, r.d_j, r.op_begin, r.op_end,
+                          r.nnz)) != SR_OK)
       return s;
     // every rank-one update (a unit update or a sink block) counts its edges;
     // a re-anchor that fails leaves S valid, and the updates go on

@@ -669,8 +669,12 @@ __device__ void prep_patch(const PatchOp* __restrict__ ops, int64_t begin, int64
   }
 }
 
-// V: arithmetic and vector precision; TS: storage precision of S and the panels
-template <typename V, typename TS>
+// V: arithmetic and vector precision; TS: storage precision of S and the panels.
+// FLOW: the flow form (p.flat), which falls back to the items; without it the
+// item form alone, which the larger kernel spills for (n = 30,000, m = 600,000,
+// K = 15 before the S pass: 296 and 311 us with FP64 vectors, 154 and 167 with
+// FP32).
+template <typename V, typename TS, bool FLOW>
 __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ V red[4][2][PT];
@@ -686,6 +690,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
   const int G = gridDim.x;
   const int nT = p.nT;
   const int mt = p.mt;
+  const bool flat = FLOW && p.flat;
   // dynamic shared memory: item slots, column cache, item offsets, pending coefficients
   PrepItem* items = reinterpret_cast<PrepItem*>(dsm);
   int* cc = reinterpret_cast<int*>(items + (MAXI + 1));
@@ -722,7 +727,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     for (int64_t e = (int64_t)blockIdx.x * PG + tid; e < total; e += (int64_t)G * PG)
       w16[e] = make_uint4(0u, 0u, 0u, 0u);
   };
-  if (p.flat) {
+  if (flat) {
     // rows without nonzeros are complete in all steps but the first
     const int blocks = (nT * PT + PG - 1) / PG;
     // (step, rows) units; step K + 1 = the means of phase 1
@@ -834,7 +839,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
       const V vj = (red[0][1][r] + red[1][1][r]) + (red[2][1][r] + red[3][1][r]);
       sI[a] = vi;
       sJ[a] = vj;
-      if (p.flat) {
+      if (flat) {
         const float fi = up_abs(vi), fj = up_abs(vj);
         bad |= !(fi <= 3.0e38f) || !(fj <= 3.0e38f);
         mxI = fmaxf(mxI, fi);
@@ -848,7 +853,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     if (tid == 0) p.tile_nnz[T] = (wsum[0] + wsum[1]) + (wsum[2] + wsum[3]);
     __syncthreads();
   }
-  if (p.flat) {
+  if (flat) {
     // non-negative floats order like their bits; an infinite or NaN entry puts
     // the bits of infinity there
     if (tid < PT) {
@@ -883,7 +888,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
   // read together: each is a round trip to L2
   const unsigned b2 = __ldcg(p.bar + 2), b3 = __ldcg(p.bar + 3), b4 = __ldcg(p.bar + 4);
   const int nnz0 = t0 < t1 ? __ldcg(p.tile_nnz + t0) : 0;
-  if (alive && p.flat) {
+  if (alive && flat) {
     const float mI = __uint_as_float(b2), mJ = __uint_as_float(b3);
     // bounds of Thm 3 / Thm 9 / Table 2 with |w_j|, |S_II| / delta^2 <= max |sI| / delta
     // (a first in-link's gamma has no other terms)
@@ -900,7 +905,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
   if (alive) {
     // ioff[T] = the units of the tiles before T: their nonzeros (flow form,
     // tried first when allowed) or their items of at most `item` nonzeros
-    for (int pass = p.flat && finite ? 0 : 1; pass < 2; ++pass) {
+    for (int pass = flat && finite ? 0 : 1; pass < 2; ++pass) {
       const int div = pass == 0 ? 1 : p.item;
       int s = 0;
       for (int T = t0; T < t1; ++T) {
@@ -1081,7 +1086,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     }
   } else if (alive) {
     my_items = s_div;
-    if (p.flat) {  // set up for the flow form above
+    if (flat) {  // set up for the flow form above
       zero_w();
       alive = prep_barrier(p.bar, ++nb * G, p.limit, &s_ok);
     }
@@ -1429,45 +1434,63 @@ void launch_flow_recip(SweepScale* out, int count, cudaStream_t st) {
   k_flow_recip<<<(count + 255) / 256, 256, 0, st>>>(out, count);
 }
 
+// The co-resident CTAs per SM of a kernel with smem bytes of dynamic shared
+// memory into fit (see PrepFit).  False on an error.
+static bool prep_resident(const void* fn, int which, size_t smem, PrepFit& fit) {
+  if (fit.fn == fn && fit.smem == smem) return true;
+  // the limit is the device's, not this launch's, so that no handle lowers
+  // another's (per device: smem_attr_once)
+  static std::atomic<unsigned long long> done[6];
+  cudaFuncAttributes fa;
+  int dev = 0, most = 0, per_sm = 0;
+  if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+    return false;
+  if (smem_attr_once(fn, most - (int)fa.sharedSizeBytes, done[which]) != cudaSuccess) return false;
+  if (smem > (size_t)most - fa.sharedSizeBytes) return false;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, PG, smem) != cudaSuccess)
+    return false;
+  fit = PrepFit{fn, smem, per_sm};
+  return true;
+}
+
 int launch_prep(const PrepParams& prm, int s_prec, int vec64, int npend_max, int num_sms,
-                int max_ctas, int64_t nnz_bound, PrepFit& fit, cudaStream_t st) {
+                int max_ctas, int64_t nnz, PrepFit (&fit)[2], cudaStream_t st) {
   if (prm.nT <= 0) return 0;
   if (prm.item < 0 || prm.cap < 0 || (prm.cap & 3)) return 1;
   const size_t smem = (s_prec == 64) ? prep_smem<double>(prm.cap, prm.nT_cap, npend_max)
                                      : prep_smem<float>(prm.cap, prm.nT_cap, npend_max);
-  const void* fn = (s_prec == 64) ? (const void*)k_prep<double, double>
-                   : vec64        ? (const void*)k_prep<double, float>
-                                  : (const void*)k_prep<float, float>;
-  if (fit.fn != fn || fit.smem != smem) {
-    // the limit is the device's, not this launch's, so that no handle lowers
-    // another's (per device: smem_attr_once)
-    static std::atomic<unsigned long long> done[3];
-    cudaFuncAttributes fa;
-    int dev = 0, most = 0, per_sm = 0;
-    if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-      return 1;
-    const int which = s_prec == 64 ? 0 : vec64 ? 1 : 2;
-    if (smem_attr_once(fn, most - (int)fa.sharedSizeBytes, done[which]) != cudaSuccess) return 1;
-    if (smem > (size_t)most - fa.sharedSizeBytes) return 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, PG, smem) != cudaSuccess)
-      return 1;
-    fit = PrepFit{fn, smem, per_sm};
-  }
-  const int per_sm = fit.per_sm;
-  if (per_sm <= 0) return 2;
-  // one CTA per item (at most nT + nnz / item of them), at most all
-  // co-resident CTAs
-  const int full = per_sm * num_sms;
-  int grid = full;
-  const int item = prm.item > 0 ? prm.item : 1024;
-  grid = (int)std::min<int64_t>((int64_t)prm.nT + nnz_bound / (prm.item > 0 ? item : FLOW_CTA) + 1, full);
-  if (max_ctas > 0) grid = std::min(grid, max_ctas);
-  grid = std::max(grid, 1);
-  if ((prm.nT + grid - 1) / grid > PREP_MT) return 2;
-  if (prm.npend > npend_max) return 1;
+  // item form, flow form
+  static const void* const fns[3][2] = {
+      {(const void*)k_prep<double, double, false>, (const void*)k_prep<double, double, true>},
+      {(const void*)k_prep<double, float, false>, (const void*)k_prep<double, float, true>},
+      {(const void*)k_prep<float, float, false>, (const void*)k_prep<float, float, true>}};
+  const int which = s_prec == 64 ? 0 : vec64 ? 1 : 2;
   PrepParams a = prm;
   if (a.item == 0) a.item = 1024;
+  const void* fn = nullptr;
+  int grid = 0;
+  for (int flow = prm.flat ? 1 : 0; flow >= 0; --flow) {
+    fn = fns[which][flow];
+    const bool fits = prep_resident(fn, 2 * which + flow, smem, fit[flow]);
+    if (flow && !(fits && fit[flow].per_sm > 0)) continue;
+    if (!fits) return 1;
+    if (fit[flow].per_sm <= 0) return 2;
+    // one CTA per item (at most nT + nnz / item of them), at most all
+    // co-resident CTAs
+    const int full = fit[flow].per_sm * num_sms;
+    grid = (int)std::min<int64_t>((int64_t)prm.nT + nnz / (prm.item > 0 ? prm.item : FLOW_CTA) + 1,
+                                  full);
+    if (max_ctas > 0) grid = std::min(grid, max_ctas);
+    grid = std::max(grid, 1);
+    a.flat = flow;
+    // more than two nonzeros a thread take the item form.  The flow form would
+    // find that out behind its zero fill and fill W again: n = 24,000,
+    // m = 340,000, K = 15, FP32 129 us an update before the S pass, here 111
+    if (nnz <= (int64_t)2 * PG * grid) break;
+  }
+  if ((prm.nT + grid - 1) / grid > PREP_MT) return 2;
+  if (prm.npend > npend_max) return 1;
   a.mt = (prm.nT + grid - 1) / grid;
   void* args[] = {&a};
   if (cudaLaunchCooperativeKernel(fn, grid, PG, args, smem, st) != cudaSuccess) return 1;

@@ -148,8 +148,8 @@ struct SweepScale {
 // vec64 or S is FP64, else FP32); W is the working buffer [K+1][n_pad] of
 // (xi, eta) pairs (16 bytes; of the vector precision in the item form); tile_nnz holds nT_cap ints.  Gathers are split into items of at most `item`
 // nonzeros; `cap` column indices are cached per CTA (a multiple of 4).
-// bar: five zeroed unsigned ints, left zeroed.  nnz_bound bounds the edges of
-// the new graph (it sizes the grid).  Returns 0 on launch, 2 when the graph
+// bar: five zeroed unsigned ints, left zeroed.  nnz: the edges of the
+// new graph (they size the grid and decide between the flow and the item form).  Returns 0 on launch, 2 when the graph
 // has more tiles than the co-resident CTAs can own (use the per-step path),
 // 1 on a launch error.
 struct PrepParams {
@@ -195,15 +195,15 @@ struct PrepParams {
 };
 // out[d] = 1 / d for d < count (PrepParams::recip)
 void launch_flow_recip(SweepScale* out, int count, cudaStream_t st);
-// fit: the co-resident CTAs per SM found for a kernel and its shared memory,
-// asked for again when either changes.
+// fit: the co-resident CTAs per SM found for the kernels of the item and the flow
+// form and their shared memory, asked for again when either changes.
 struct PrepFit {
   const void* fn = nullptr;
   size_t smem = 0;
   int per_sm = 0;
 };
 int launch_prep(const PrepParams& p, int s_prec, int vec64, int npend_max, int num_sms,
-                int max_ctas, int64_t nnz_bound, PrepFit& fit, cudaStream_t st);
+                int max_ctas, int64_t nnz, PrepFit (&fit)[2], cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Many independent graphs advanced together (k_multi.cu).

@@ -357,3 +357,26 @@ def test_s_after_a_wait_that_ran_out(P, prec):
         err = np.minimum(np.abs(got - S0), np.abs(got - want))
         assert np.max(err) < (1e-10 if prec == 64 else 1e-6), limit
     assert ran_out
+
+
+@pytest.mark.parametrize("prec,vec", [(64, 0), (32, 0), (32, 1)])
+@pytest.mark.parametrize("more", [-1, 0, 1, 700])
+def test_recurrence_at_the_switch_between_its_forms(P, prec, vec, more):
+    """The flow form takes up to 1,024 nonzeros a CTA; with 5 CTAs the updates
+    here go over that number and back, or stay above it.  1e-10 (FP64) and 1e-6
+    (FP32), as in the parity tests."""
+    n, C, K = 1300, 0.6, 7
+    rng = np.random.default_rng(12)
+    keys = rng.choice(n * n, 5 * 1024 + more + n, replace=False)
+    keys = keys[keys // n != keys % n][: 5 * 1024 + more]
+    s, d = (keys // n).astype(np.int32), (keys % n).astype(np.int32)
+    edges = set(zip(s.tolist(), d.tolist()))
+    ins = [x for x in ((i, j) for i in range(40) for j in (50, 900)) if x not in edges][:3]
+    dele = sorted(edges)[100:102]
+    ups = [(*ins[0], 1), (*ins[1], 1), (*dele[0], -1), (*dele[1], -1), (*ins[2], 1)]
+    S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-14)
+    want, _ = O.sequential_unit_updates(n, s, d, S0, ups, C, K)
+    sr = P.SimRank(n, s, d, S0=S0.astype(np.float64 if prec == 64 else np.float32), C=C, K=K,
+                   s_precision=prec, vec_fp64=vec, prep_ctas=5)
+    sr.apply_updates(ups)
+    assert np.max(np.abs(sr.dense() - want)) < (1e-10 if prec == 64 else 1e-6)
