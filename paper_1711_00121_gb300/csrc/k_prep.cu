@@ -669,6 +669,17 @@ __device__ void prep_patch(const PatchOp* __restrict__ ops, int64_t begin, int64
   }
 }
 
+// Shared memory of the flow form, in the place of the item form's column cache
+// (as arrays of their own they took the second CTA of an SM from launches with
+// 2,600 to 3,600 pending terms).  fsh also holds the partial sums of phase 0.
+struct FlowShared {
+  SweepScale fsh[PG][2];  // 1 / in-degree of each thread's head / tail row
+  int rowmap[2 * PG];     // the row of each of the CTA's nonzeros
+  I2 dep[2][PG / 32];     // a warp's part of the row before it
+};
+constexpr int FLOW_INTS = (int)(sizeof(FlowShared) / sizeof(int));
+static_assert(FLOW_INTS % 4 == 0 && sizeof(PrepItem) % 16 == 0, "16-byte alignment");
+
 // V: arithmetic and vector precision; TS: storage precision of S and the panels.
 // FLOW: the flow form (p.flat), which falls back to the items; without it the
 // item form alone, which the larger kernel spills for (n = 30,000, m = 600,000,
@@ -679,9 +690,6 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ V red[4][2][PT];
   __shared__ V rrc[PT], rri[PT];  // C / in-degree and 1 / in-degree of the rows of item 0
-  __shared__ SweepScale fsh[PG][2];  // flow form: 1 / in-degree of each thread's head / tail row
-  __shared__ int rowmap[2 * PG];     // flow form: the row of each of the CTA's nonzeros
-  __shared__ I2 dep[2][PG / 32];     // flow form: a warp's part of the row before it
   __shared__ unsigned smax[3][PT / 32];
   __shared__ unsigned long long mk[PREP_MT][2];
   __shared__ int wsum[PG / 32];
@@ -694,7 +702,11 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
   // dynamic shared memory: item slots, column cache, item offsets, pending coefficients
   PrepItem* items = reinterpret_cast<PrepItem*>(dsm);
   int* cc = reinterpret_cast<int*>(items + (MAXI + 1));
-  int* ioff = cc + p.cap;  // [nT + 1]
+  FlowShared& fl = *reinterpret_cast<FlowShared*>(cc);
+  auto& fsh = fl.fsh;
+  auto& rowmap = fl.rowmap;
+  auto& dep = fl.dep;
+  int* ioff = cc + max(p.cap, FLOW_INTS);  // [nT + 1]
   // the pending correction of the rows of S is summed in the storage precision of S
   TS* coef = reinterpret_cast<TS*>(ioff + ((p.nT_cap + 1 + 3) & ~3));
   const TS* __restrict__ S = static_cast<const TS*>(p.S);
@@ -796,7 +808,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
     // pending, n = 20,000, K = 20).
     if constexpr (sizeof(TS) == 4) {
       if (np > 0) {
-        static_assert(sizeof(fsh) >= (PG / 32) * 2 * PT * sizeof(float), "partial sums");
+        static_assert(sizeof(FlowShared::fsh) >= (PG / 32) * 2 * PT * sizeof(float), "partial sums");
         float* cs = reinterpret_cast<float*>(fsh);
         const float* xp = P + pidx((int64_t)T * PT + 4 * lane, 0, 0);
         const float* ep = xp + ldk * PT;
@@ -1424,7 +1436,7 @@ __global__ void __launch_bounds__(PG, 2) k_prep(PrepParams p) {
 
 template <typename TS>
 size_t prep_smem(int cap, int nT_cap, int npend_max) {
-  return (size_t)(MAXI + 1) * sizeof(PrepItem) + (size_t)cap * sizeof(int) +
+  return (size_t)(MAXI + 1) * sizeof(PrepItem) + (size_t)std::max(cap, FLOW_INTS) * sizeof(int) +
          (size_t)((nT_cap + 1 + 3) & ~3) * sizeof(int) + (size_t)4 * npend_max * sizeof(TS);
 }
 
