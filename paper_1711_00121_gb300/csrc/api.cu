@@ -1158,7 +1158,7 @@ simrank_status columns_scratch(simrank_ctx* h, size_t bytes, void** p) {
 }
 
 void build_chunks(const HostAdj& A, int n_rows, std::vector<RowChunk>& out,
-                  std::vector<int64_t>* first);
+                  std::vector<int64_t>* first, bool empty_last);
 simrank_status upload_chunks(simrank_ctx* h, const std::vector<RowChunk>& v, ChunkList& L,
                              int64_t* cap);
 
@@ -1283,7 +1283,7 @@ simrank_status run_one_shot(simrank_ctx* h, const std::map<int32_t, std::vector<
   // the steps below gather by row chunks of the new graph (the host mirror
   // holds it), so that a hub row spreads over many warps
   std::vector<RowChunk> chv;
-  build_chunks(h->hin, n_pad, chv, nullptr);
+  build_chunks(h->hin, n_pad, chv, nullptr, false);
   if ((s = upload_chunks(h, chv, h->cur_hor, &h->cur_hor_cap)) != SR_OK) return s;
   CUDA_TRY(h, cudaStreamSynchronize(h->st));
   const bool fixed = wbits < 0x7f800000u;
@@ -1410,29 +1410,34 @@ simrank_status run_one_shot(simrank_ctx* h, const std::map<int32_t, std::vector<
   return SR_OK;
 }
 
-// Chunks of a row of len nonzeros (an empty row has one, empty), and chunk c
-// of the nc of row a.
-int row_chunks(int len) { return std::max(1, (len + kChunk - 1) / kChunk); }
+// Chunks of a row of len nonzeros, and chunk c of the nc of row a.
+int row_chunks(int len) { return (len + kChunk - 1) / kChunk; }
 RowChunk row_chunk(const HostAdj& A, int a, int c, int nc) {
   const int len = std::min(kChunk, A.len[a] - c * kChunk);
   return {a, nc == 1 ? (len | CH_ONLY) : len, A.start[a] + (int64_t)c * kChunk};
 }
 
-// Row chunks (at most kChunk nonzeros each) of the adjacency rows [0, n_rows);
-// first (optional) gets the index of each row's first chunk (n_rows + 1).
+// Row chunks (at most kChunk nonzeros each) of the adjacency rows [0, n_rows),
+// for the steps that write every row with one empty chunk per empty row: in its
+// place, or behind all others when `empty_last` (so that a narrow step, which
+// adds to rows that are set before, can leave them out).  With `first`, which
+// gets the index of each row's first chunk (n_rows + 1), there are none.
 void build_chunks(const HostAdj& A, int n_rows, std::vector<RowChunk>& out,
-                  std::vector<int64_t>* first = nullptr) {
+                  std::vector<int64_t>* first = nullptr, bool empty_last = false) {
   out.clear();
+  const int least = first ? 0 : 1;
   int64_t total = 0;
-  for (int a = 0; a < n_rows; ++a) total += row_chunks(A.len[a]);
+  for (int a = 0; a < n_rows; ++a) total += std::max(least, row_chunks(A.len[a]));
   out.reserve((size_t)total);
   if (first) first->assign((size_t)n_rows + 1, 0);
   for (int a = 0; a < n_rows; ++a) {
     if (first) (*first)[a] = (int64_t)out.size();
-    const int nc = row_chunks(A.len[a]);
+    const int nc = std::max(empty_last ? 0 : least, row_chunks(A.len[a]));
     for (int c = 0; c < nc; ++c) out.push_back(row_chunk(A, a, c, nc));
   }
   if (first) (*first)[n_rows] = (int64_t)out.size();
+  for (int a = 0; empty_last && a < n_rows; ++a)
+    if (A.len[a] == 0) out.push_back(row_chunk(A, a, 0, 1));
 }
 
 // Rewrites row a's chunks of a list built by build_chunks (with first) after
@@ -1453,7 +1458,7 @@ simrank_status upload_chunks(simrank_ctx* h, const std::vector<RowChunk>& v, Chu
                              int64_t* cap) {
   // the lists of column updates are current again once that path says so
   h->col_chunks_ok = false;
-  L.count = L.multi_count = 0;
+  L.count = L.filled = L.multi_count = 0;
   CUDA_TRY(h, dev_grow(&L.chunks, cap, (int64_t)v.size()));
   if (!v.empty())
     CUDA_TRY(h, cudaMemcpyAsync(L.chunks, v.data(), v.size() * sizeof(RowChunk),
@@ -1465,7 +1470,8 @@ simrank_status upload_chunks(simrank_ctx* h, const std::vector<RowChunk>& v, Chu
   if (!multi.empty())
     CUDA_TRY(h, cudaMemcpyAsync(L.multi, multi.data(), multi.size() * sizeof(int32_t),
                                 cudaMemcpyHostToDevice, h->st));
-  L.count = (int64_t)v.size();
+  L.count = L.filled = (int64_t)v.size();
+  while (L.filled > 0 && chunk_len(v[(size_t)L.filled - 1]) == 0) --L.filled;
   L.multi_count = (int64_t)multi.size();
   return SR_OK;
 }
@@ -1946,9 +1952,9 @@ simrank_status simrank_init(const simrank_config* cfg_in, int32_t n, int64_t m, 
                     h->st);
     cudaMemcpyAsync(h->g0_in_len, h->din.len, (size_t)h->n_pad * 4, cudaMemcpyDeviceToDevice, h->st);
     int64_t cap_f = 0, cap_h = 0;
-    build_chunks(h->hout, h->n_pad, ch);
+    build_chunks(h->hout, h->n_pad, ch, nullptr, true);
     if ((s = upload_chunks(h, ch, h->g0_fwd, &cap_f)) != SR_OK) return bail(s);
-    build_chunks(h->hin, h->n_pad, ch);
+    build_chunks(h->hin, h->n_pad, ch, nullptr, true);
     if ((s = upload_chunks(h, ch, h->g0_hor, &cap_h)) != SR_OK) return bail(s);
     if (cudaStreamSynchronize(h->st) != cudaSuccess)
       return bail(fail(h, SR_ERR_CUDA, "init synchronisation failed"));

@@ -67,7 +67,7 @@ __global__ void k_adj_weights(DevAdj in, WeightView wv, int n_rows, const double
 
 void launch_adj_sddmm(const ChunkList& hor, const int32_t* in_col, const double* F, const double* Y,
                       int B, double scale, double* G, cudaStream_t st) {
-  if (hor.count > 0) k_adj_sddmm<<<(unsigned)hor.count, 256, 0, st>>>(hor.chunks, in_col, F, Y, B, scale, G);
+  if (hor.filled > 0) k_adj_sddmm<<<(unsigned)hor.filled, 256, 0, st>>>(hor.chunks, in_col, F, Y, B, scale, G);
 }
 
 void launch_adj_scatter(const int32_t* node, const int32_t* c, const double* coef, int64_t count,

@@ -522,17 +522,17 @@ static void partial_sim_block_t(const ChunkList& fwd, const ChunkList& hor, cons
   // narrow blocks: a group of 8 lanes per chunk; the forward input divided once per row
   auto narrow_step = [&](const ChunkList& L, const int32_t* adj, const float* w, bool forward,
                          const T* X, T* Y, double scale) {
-    if (L.count <= 0) return;
+    if (L.filled <= 0) return;
     // persistent: at most 8 CTAs of 8 warps per SM, four chunks per warp at a time
-    const int64_t want = (L.count + 31) / 32;
+    const int64_t want = (L.filled + 31) / 32;
     const unsigned grid = (unsigned)std::min<int64_t>(want, (int64_t)num_sms_for_narrow() * 8);
 #define SR_NARROW(BW)                                                                          \
   do {                                                                                         \
     if (forward)                                                                               \
-      k_col_chunk_narrow<T, true, BW><<<grid, 256, 0, st>>>(L.chunks, L.count, adj, w, in_len,  \
+      k_col_chunk_narrow<T, true, BW><<<grid, 256, 0, st>>>(L.chunks, L.filled, adj, w, in_len, \
                                                             wv.wsum, X, Y, scale);             \
     else                                                                                       \
-      k_col_chunk_narrow<T, false, BW><<<grid, 256, 0, st>>>(L.chunks, L.count, adj, w, in_len, \
+      k_col_chunk_narrow<T, false, BW><<<grid, 256, 0, st>>>(L.chunks, L.filled, adj, w, in_len, \
                                                              wv.wsum, X, Y, scale);            \
   } while (0)
     switch (ldb) {

@@ -403,8 +403,7 @@ void launch_pack_f16_tiles(const float* Pp, int GK1, int nterms, int rg, int n_r
 
 // ---- column mode (§7), k_column.cu
 // A piece of one adjacency row: row id, count (<= kChunk, in the low bits of
-// len) and pool offset.  CH_ONLY marks the only chunk of its row (an empty row
-// has one empty chunk).
+// len) and pool offset.  CH_ONLY marks the only chunk of its row.
 struct RowChunk {
   int32_t row;
   int32_t len;
@@ -418,6 +417,7 @@ __host__ __device__ __forceinline__ int chunk_len(const RowChunk& c) { return c.
 struct ChunkList {
   RowChunk* chunks = nullptr;  // device
   int64_t count = 0;
+  int64_t filled = 0;        // behind these there are chunks of empty rows only
   int32_t* multi = nullptr;  // device: the rows of more than one chunk
   int64_t multi_count = 0, multi_cap = 0;
 };

@@ -380,3 +380,28 @@ def test_recurrence_at_the_switch_between_its_forms(P, prec, vec, more):
                    s_precision=prec, vec_fp64=vec, prep_ctas=5)
     sr.apply_updates(ups)
     assert np.max(np.abs(sr.dense() - want)) < (1e-10 if prec == 64 else 1e-6)
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("width", [1, 4, 5])
+def test_stored_updates_of_rows_that_become_empty(P, prec, width):
+    """Stored updates that give an empty in-row and an empty out-row their first
+    nonzero and take a row's only one (the chunk lists of narrow steps hold no
+    empty rows, those of wide steps end with them), then narrow and wide
+    queries.  Against Alg 7: 1e-10 (FP64) and 1e-6 (FP32), as in the column-mode
+    parity tests."""
+    n, C, K = 140, 0.6, 6
+    s, d = degrees_graph(n, [0, 1, 33, 0], 47)
+    keep = s != 5  # node 5 has no out-neighbours
+    s, d = s[keep], d[keep]
+    only = next(x for x in zip(s.tolist(), d.tolist()) if x[1] == 1)
+    ups = [(5, 0, 1), (*only, -1), (7, 3, 1), (5, 0, -1), (only[0], 1, 1), (7, 3, -1)]
+    cols = np.array([1, 0, 3, 5, 100][:width], np.int32)
+    base = O.partial_sim_block(O.transition_matrix(n, s, d, sparse=True), cols, K, C)
+    for count in (1, 2, 4, 6):
+        sr = P.SimRank(n, s, d, C=C, K=K, s_precision=prec, mode=P.MODE_COLUMN)
+        sr.apply_updates(ups[:count])
+        got = sr.columns(cols)
+        for c, x in enumerate(cols.tolist()):
+            want = O.inc_sr_all_p(n, s, d, base[:, c], x, ups[:count], C, K)
+            assert np.max(np.abs(got[:, c] - want)) < (1e-10 if prec == 64 else 1e-6), (count, x)
