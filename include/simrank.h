@@ -168,7 +168,11 @@ simrank_status simrank_default_config(simrank_config* cfg);
  * until the max-abs change is below cfg->init_tol.  Self-loops and duplicate
  * edges return SR_ERR_EDGE_EXISTS.  Nodes n..n_capacity-1 are pre-allocated as
  * isolated nodes (S_xx = 1 - C, a valid fixed point) and become nodes when
- * an update names them.  On success *out owns device memory until simrank_destroy. */
+ * an update names them.  On success *out owns device memory until simrank_destroy.
+ * Work buffers of queries to host memory (up to 64 MB each) and of re-anchors of
+ * an FP32 S (up to 4 GB in all) stay with the process for the next call of any
+ * handle, 4 GB at most; they are freed when an allocation of the library fails
+ * for want of memory and with the last handle. */
 simrank_status simrank_init(const simrank_config* cfg, int32_t n, int64_t m,
                             const int32_t* src, const int32_t* dst, const float* weight,
                             const void* S0, simrank_t* out);

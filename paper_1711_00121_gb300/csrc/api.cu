@@ -4,10 +4,12 @@
 // launch sequence of each rank-one update.
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <new>
 #include <string>
 #include <unordered_map>
@@ -93,9 +95,6 @@ struct simrank_ctx {
   unsigned char* stage = nullptr;
   size_t stage_bytes = 0;
   cudaEvent_t stage_ev = nullptr;
-  // work buffers of re-anchors (at most ANCHOR_KEEP bytes in all), kept between calls
-  void* anchor_buf[3] = {nullptr, nullptr, nullptr};
-  size_t anchor_bytes = 0;
   PrepFit prep_fit[2];  // co-resident CTAs of the pre-update launch
   // column mode (§7): snapshot of the initial graph and the stored updates
   bool column = false;
@@ -184,10 +183,121 @@ inline uint64_t ekey(int32_t s, int32_t d) { return ((uint64_t)(uint32_t)s << 32
 
 inline int elem_bytes(const simrank_ctx* h) { return h->cfg.s_precision == 64 ? 8 : 4; }
 
+// Work buffers that no call is using, shared by the handles of the process: a
+// call takes one and gives it back when its stream has finished with it, so
+// that any thread and stream may have it next.  At most LIMIT bytes stay; they
+// go when an allocation of the library needs the room, and with the last handle.
+class Spare {
+ public:
+  static constexpr size_t LIMIT = (size_t)4 << 30;
+  void* take(size_t bytes) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(mu_);
+    for (size_t i = items_.size(); i-- > 0;)
+      if (items_[i].bytes == bytes && items_[i].dev == dev) {
+        void* p = items_[i].p;
+        items_.erase(items_.begin() + (ptrdiff_t)i);
+        held_ -= bytes;
+        return p;
+      }
+    return nullptr;
+  }
+  // the oldest buffers make room
+  void give(void* p, size_t bytes) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::vector<Item> out;
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      items_.push_back({dev, p, bytes});
+      held_ += bytes;
+      while (held_ > LIMIT) {
+        held_ -= items_.front().bytes;
+        out.push_back(items_.front());
+        items_.erase(items_.begin());
+      }
+    }
+    release(out);
+  }
+  // false if there was nothing to free
+  bool drain() {
+    std::vector<Item> out;
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      out.swap(items_);
+      held_ = 0;
+    }
+    release(out);
+    return !out.empty();
+  }
+  size_t held() {
+    std::lock_guard<std::mutex> lock(mu_);
+    return held_;
+  }
+
+ private:
+  struct Item {
+    int dev;
+    void* p;
+    size_t bytes;
+  };
+  static void release(const std::vector<Item>& v) {
+    int dev = 0;
+    if (v.empty()) return;
+    cudaGetDevice(&dev);
+    for (const Item& i : v) {
+      if (i.dev != dev) cudaSetDevice(i.dev);
+      cudaFree(i.p);
+      if (i.dev != dev) cudaSetDevice(dev);
+    }
+  }
+  std::mutex mu_;
+  std::vector<Item> items_;
+  size_t held_ = 0;
+};
+Spare& spare() {
+  static Spare* s = new Spare;  // outlives every handle
+  return *s;
+}
+std::atomic<int> g_handles{0};
+
 template <typename T>
 cudaError_t dev_alloc(T** p, size_t count) {
-  const cudaError_t e = cudaMalloc((void**)p, std::max<size_t>(count, 1) * sizeof(T));
+  const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
+  cudaError_t e = cudaMalloc((void**)p, bytes);
+  if (e == cudaErrorMemoryAllocation && spare().drain()) {
+    cudaGetLastError();
+    e = cudaMalloc((void**)p, bytes);
+  }
   if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
+
+// A call's work buffer: from the spare ones or allocated; given back once the
+// stream is idle, freed (which waits) on any other way out.
+struct WorkBuf {
+  void* p = nullptr;
+  size_t bytes = 0;
+  cudaError_t get(size_t want) {
+    bytes = want;
+    p = spare().take(want);
+    return p ? cudaSuccess : dev_alloc((unsigned char**)&p, want);
+  }
+  void give() {
+    if (p) spare().give(p, bytes);
+    p = nullptr;
+  }
+  ~WorkBuf() {
+    if (p) cudaFree(p);
+  }
+};
+
+// Free memory of the device, with what the library would free to allocate.
+cudaError_t free_memory(size_t* bytes) {
+  size_t total = 0;
+  const cudaError_t e = cudaMemGetInfo(bytes, &total);
+  if (e == cudaSuccess) *bytes += spare().held();
   return e;
 }
 
@@ -942,7 +1052,6 @@ std::vector<SweepScale> sweep_scales(const HostAdj& A, int n_rows, double C) {
 // FP32, 1e-12 in FP64; both hold for every S of Eq. 1): `known` says so without
 // a look at S, otherwise a pass over S decides, and any other S (a caller's S0)
 // is swept in FP64 as it is.
-constexpr size_t ANCHOR_KEEP = (size_t)4 << 30;
 simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double* last_diff,
                              int* sweeps_done, double* tol_used = nullptr,
                              double* first_diff = nullptr, bool known = false) {
@@ -958,29 +1067,18 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
   if (wp == 32) tol = std::max(tol, 1e-7);
   int flat_sweeps = 0;
   double prev = INFINITY;
-  void* bufs[3] = {nullptr, nullptr, nullptr};
+  WorkBuf bufs[3];  // the first is S itself when S has their type
   const bool alias = (wp == sp);
-  // buffers that a re-anchor left (see below) serve this one
-  const bool held = !alias && h->anchor_bytes == bytes;
-  for (int b = (alias ? 1 : 0); b < 3; ++b) {
-    if (held) {
-      bufs[b] = h->anchor_buf[b];
-    } else if (cudaMalloc(&bufs[b], bytes) != cudaSuccess) {
-      for (void* p : bufs)
-        if (p) cudaFree(p);
+  for (int b = (alias ? 1 : 0); b < 3; ++b)
+    if (bufs[b].get(bytes) != cudaSuccess)
       return fail(h, SR_ERR_OOM, "cudaMalloc of Jacobi buffers failed");
-    }
-  }
   double diff = INFINITY;
   int it = 0;
   bool fixed = !h->weighted && wp == 64;
+  WorkBuf tables;
   SweepScale* scales = nullptr;
-  // ends the call before S has been touched; a handle's kept buffers stay
+  // ends the call before S has been touched
   auto give_up = [&](cudaError_t why) {
-    if (scales) cudaFree(scales);
-    if (!held)
-      for (void* p : bufs)
-        if (p) cudaFree(p);
     return fail(h, why == cudaErrorMemoryAllocation ? SR_ERR_OOM : SR_ERR_CUDA,
                 std::string("Jacobi sweep: ") + cudaGetErrorString(why));
   };
@@ -990,7 +1088,7 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
     // S into bufs[0] in fixed point, with a look at what it holds unless it is
     // known (before the change when it is made in place)
     unsigned int flags = 0;
-    long long* F = (long long*)(alias ? h->S : bufs[0]);
+    long long* F = (long long*)(alias ? h->S : bufs[0].p);
     const double sym = sp == 64 ? 1e-12 : 1e-6;
     unsigned int* df = (unsigned int*)h->diffbits;
     e = cudaMemsetAsync(h->diffbits, 0, sizeof(unsigned long long), h->st);
@@ -1009,7 +1107,8 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
       std::vector<SweepScale> f = sweep_scales(h->hin, h->n_pad, h->cfg.C);
       const std::vector<SweepScale> f1 = sweep_scales(h->hin, h->n_pad, 1.0);
       f.insert(f.end(), f1.begin(), f1.end());
-      e = cudaMalloc(&scales, f.size() * sizeof(SweepScale));
+      e = tables.get(f.size() * sizeof(SweepScale));
+      scales = (SweepScale*)tables.p;
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(scales, f.data(), f.size() * sizeof(SweepScale),
                             cudaMemcpyHostToDevice, h->st);
@@ -1020,14 +1119,13 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
         launch_to_fixed(h->S, sp, F, h->n_pad, h->ld, upper(h), false, sym, df, h->st);
     }
   }
-  if (alias) bufs[0] = h->S;
   if (!fixed) {
     if (upper(h)) launch_mirror_lower(h->S, sp, h->n_pad, h->ld, h->st);
-    if (!alias) launch_convert(h->S, sp, bufs[0], wp, (int64_t)elems, h->st);
-    cudaMemsetAsync(bufs[1], 0, bytes, h->st);
-    cudaMemsetAsync(bufs[2], 0, bytes, h->st);
+    if (!alias) launch_convert(h->S, sp, bufs[0].p, wp, (int64_t)elems, h->st);
+    cudaMemsetAsync(bufs[1].p, 0, bytes, h->st);
+    cudaMemsetAsync(bufs[2].p, 0, bytes, h->st);
   }
-  void *A = bufs[0], *B = bufs[1], *T = bufs[2];
+  void *A = alias ? h->S : bufs[0].p, *B = bufs[1].p, *T = bufs[2].p;
   e = cudaGetLastError();
   const float* w = h->weighted ? h->d_in_w : nullptr;
   while (e == cudaSuccess && it < max_sweeps) {
@@ -1084,20 +1182,18 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
   }
   const cudaError_t fin = cudaStreamSynchronize(h->st);
   if (e == cudaSuccess) e = fin;
-  if (scales) cudaFree(scales);
-  // bufs[] holds three distinct buffers (bufs[0] is the old S when aliasing);
-  // keep the result as S when aliasing and free every other buffer once.
-  // A re-anchor of an FP32 S keeps them when they are small (allocating and
-  // freeing 3 x 0.8 GB took 2.2 of 5.8 ms at n = 10,007).
-  if (alias) h->S = A;
-  const bool keep = !alias && !known && 3 * bytes <= ANCHOR_KEEP;
-  for (int b = 0; b < 3; ++b) {
-    if (keep)
-      h->anchor_buf[b] = bufs[b];
-    else if (bufs[b] && bufs[b] != h->S)
-      cudaFree(bufs[b]);
+  // The result is S when S has the buffers' type: it takes its buffer along, and
+  // the old S is freed in its place.  Re-anchors of an FP32 S leave their buffers
+  // for the next one (allocating and freeing 3 x 0.8 GB took 2.2 of 5.8 ms at
+  // n = 10,007).
+  if (alias) {
+    for (WorkBuf& b : bufs)
+      if (b.p == A) b.p = h->S;
+    h->S = A;
+  } else if (!known && e == cudaSuccess && 3 * bytes <= Spare::LIMIT) {
+    for (WorkBuf& b : bufs) b.give();
   }
-  if (keep) h->anchor_bytes = bytes;
+  if (fin == cudaSuccess) tables.give();
   if (e != cudaSuccess)
     return fail(h, e == cudaErrorMemoryAllocation ? SR_ERR_OOM : SR_ERR_CUDA,
                 std::string("Jacobi sweep: ") + cudaGetErrorString(e));
@@ -1140,21 +1236,18 @@ simrank_status ob_ensure(simrank_ctx* h, int slot, size_t bytes) {
   if (b.p) cudaFree(b.p);
   b.p = nullptr;
   b.bytes = 0;
-  CUDA_TRY(h, cudaMalloc(&b.p, std::max<size_t>(bytes, 256)));
+  CUDA_TRY(h, dev_alloc((unsigned char**)&b.p, std::max<size_t>(bytes, 256)));
   b.bytes = bytes;
   return SR_OK;
 }
 
-// Device memory for columns on their way to the host: the handle's own up to
-// 64 MB, else one allocation of the call (the caller frees what is not ob[29]).
-simrank_status columns_scratch(simrank_ctx* h, size_t bytes, void** p) {
-  if (bytes <= (64u << 20)) {
-    const simrank_status s = ob_ensure(h, 29, bytes);
-    *p = h->ob[29].p;
-    return s;
-  }
-  CUDA_TRY(h, cudaMalloc(p, bytes));
-  return SR_OK;
+// Device memory for columns on their way to the host: sizes of powers of two up
+// to 64 MB, which one query can take from another, and what is needed above.
+constexpr size_t COLUMNS_KEEP = (size_t)64 << 20;
+size_t columns_scratch(size_t bytes) {
+  size_t r = (size_t)256 << 10;
+  while (r < bytes) r *= 2;
+  return r <= COLUMNS_KEEP ? r : bytes;
 }
 
 void build_chunks(const HostAdj& A, int n_rows, std::vector<RowChunk>& out,
@@ -1558,7 +1651,12 @@ simrank_status run_column_update(simrank_ctx* h, const std::vector<int32_t>& src
   h->launches += 3 + K;
   const size_t pbytes = (size_t)h->nT_cap * 2 * h->K1 * PT * (f32 ? 4 : 8);
   void* snap = nullptr;
-  CUDA_TRY(h, cudaMallocAsync(&snap, pbytes, h->st));
+  cudaError_t ae = cudaMallocAsync(&snap, pbytes, h->st);
+  if (ae == cudaErrorMemoryAllocation && spare().drain()) {
+    cudaGetLastError();
+    ae = cudaMallocAsync(&snap, pbytes, h->st);
+  }
+  CUDA_TRY(h, ae);
   h->hist.push_back(snap);
   CUDA_TRY(h, cudaMemcpyAsync(snap, f32 ? (void*)h->P32 : (void*)h->P64, pbytes,
                               cudaMemcpyDeviceToDevice, h->st));
@@ -1574,8 +1672,8 @@ simrank_status column_mode_columns(simrank_ctx* h, const int32_t* cols, int ncol
                                    int out_on_device, int out_fp64) {
   const int prec = h->cfg.s_precision, K = h->cfg.K, n_pad = h->n_pad;
   const size_t eb = prec == 64 ? 8 : 4;
-  size_t free_b = 0, total_b = 0;
-  CUDA_TRY(h, cudaMemGetInfo(&free_b, &total_b));
+  size_t free_b = 0;
+  CUDA_TRY(h, free_memory(&free_b));
   const size_t per_col = (size_t)n_pad * eb * (K + 4);
   int Bmax = (int)std::min<size_t>(1024, std::max<size_t>(1, (size_t)(0.6 * free_b) / per_col));
   if (Bmax > 4) Bmax &= ~3;
@@ -1587,14 +1685,11 @@ simrank_status column_mode_columns(simrank_ctx* h, const int32_t* cols, int ncol
                               h->st));
   const size_t ob = (size_t)h->n_cur * ncols * (out_fp64 ? 8 : 4);
   void* dst = out;
-  void* tmp = nullptr;
+  WorkBuf tmp;
   if (!out_on_device) {
-    if ((s = columns_scratch(h, ob, &tmp)) != SR_OK) return s;
-    dst = tmp;
+    CUDA_TRY(h, tmp.get(columns_scratch(ob)));
+    dst = tmp.p;
   }
-  auto drop = [&]() {
-    if (tmp && tmp != h->ob[29].p) cudaFree(tmp);
-  };
   for (int c0 = 0; c0 < ncols; c0 += Bmax) {
     const int B = std::min(Bmax, ncols - c0);
     const int ldb = B > 4 ? (B + 3) & ~3 : B;  // wide blocks: 16-byte rows
@@ -1621,24 +1716,20 @@ simrank_status column_mode_columns(simrank_ctx* h, const int32_t* cols, int ncol
     } else {
       for (void* P : h->hist) {
         const cudaError_t e = launch_col_apply(P, prec, h->K1, bc, B, ldb, n_pad, prec, res, h->st);
-        if (e != cudaSuccess) {
-          drop();
+        if (e != cudaSuccess)
           return fail(h, SR_ERR_CUDA, std::string("column mode: ") + cudaGetErrorString(e));
-        }
       }
     }
     launch_col_out(res, prec, B, ldb, h->n_cur,
                    (unsigned char*)dst + (size_t)c0 * h->n_cur * (out_fp64 ? 8 : 4), out_fp64, h->st);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      drop();
+    if (e != cudaSuccess)
       return fail(h, SR_ERR_CUDA, std::string("column mode: ") + cudaGetErrorString(e));
-    }
   }
   cudaError_t e = cudaSuccess;
-  if (!out_on_device) e = cudaMemcpyAsync(out, tmp, ob, cudaMemcpyDeviceToHost, h->st);
+  if (!out_on_device) e = cudaMemcpyAsync(out, tmp.p, ob, cudaMemcpyDeviceToHost, h->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
-  drop();
+  if (e == cudaSuccess && tmp.bytes <= COLUMNS_KEEP) tmp.give();
   if (e != cudaSuccess) return fail(h, SR_ERR_CUDA, std::string("column mode: ") + cudaGetErrorString(e));
   return SR_OK;
 }
@@ -1657,8 +1748,6 @@ void free_ctx(simrank_ctx* h) {
     if (p) cudaFree(p);
   for (auto& b : h->ob)
     if (b.p) cudaFree(b.p);
-  for (void* p : h->anchor_buf)
-    if (p) cudaFree(p);
   if (h->stage) cudaFreeHost(h->stage);
   if (h->stage_ev) cudaEventDestroy(h->stage_ev);
   if (h->Pp) cudaFree(h->Pp);
@@ -1680,6 +1769,7 @@ void free_ctx(simrank_ctx* h) {
   for (auto& a : h->phase_ev)
     for (auto& e : a) cudaEventDestroy(e);
   delete h;
+  if (g_handles.fetch_sub(1) == 1) spare().drain();
 }
 
 }  // namespace
@@ -1758,6 +1848,7 @@ simrank_status simrank_init(const simrank_config* cfg_in, int32_t n, int64_t m, 
 
   simrank_ctx* h = new (std::nothrow) simrank_ctx();
   if (!h) return fail(nullptr, SR_ERR_OOM, "host allocation failed");
+  g_handles.fetch_add(1);
   h->cfg = cfg;
   h->st = (cudaStream_t)cfg.cuda_stream;
   h->n_cur = n;
@@ -1906,9 +1997,9 @@ simrank_status simrank_init(const simrank_config* cfg_in, int32_t n, int64_t m, 
     std::vector<double> wsum(h->n_pad, 0.0);
     for (int a = 0; a < h->n_pad; ++a)
       for (int e = 0; e < h->hin.len[a]; ++e) wsum[a] += wpool[h->hin.start[a] + e];
-    if (cudaMalloc(&h->d_in_w, wpool.size() * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&h->d_out_w, opool.size() * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&h->d_wsum, wsum.size() * sizeof(double)) != cudaSuccess)
+    if (dev_alloc(&h->d_in_w, wpool.size()) != cudaSuccess ||
+        dev_alloc(&h->d_out_w, opool.size()) != cudaSuccess ||
+        dev_alloc(&h->d_wsum, wsum.size()) != cudaSuccess)
       return bail(fail(h, SR_ERR_OOM, "cudaMalloc of weights failed"));
     cudaMemcpy(h->d_in_w, wpool.data(), wpool.size() * sizeof(float), cudaMemcpyHostToDevice);
     cudaMemcpy(h->d_out_w, opool.data(), opool.size() * sizeof(float), cudaMemcpyHostToDevice);
@@ -1919,7 +2010,7 @@ simrank_status simrank_init(const simrank_config* cfg_in, int32_t n, int64_t m, 
   h->column = cfg.mode == SR_MODE_COLUMN;
   const size_t eb = (size_t)elem_bytes(h);
   const size_t s_bytes = h->column ? 256 : (size_t)h->n_pad * h->ld * eb;
-  if (cudaMalloc(&h->S, s_bytes) != cudaSuccess)
+  if (dev_alloc((unsigned char**)&h->S, s_bytes) != cudaSuccess)
     return bail(fail(h, SR_ERR_OOM, "cudaMalloc of S (" + std::to_string(s_bytes) + " bytes) failed"));
   const size_t panel_elems = (size_t)h->nT_cap * 2 * h->K1 * PT;
   if (dev_alloc(&h->P64, panel_elems) != cudaSuccess ||
@@ -2255,26 +2346,24 @@ simrank_status simrank_columns(simrank_t h, const int32_t* cols, int32_t ncols, 
   for (int32_t& x : icols) x = h->ext2int[x];
   cols = icols.data();
   const int32_t* perm = h->relabeled ? h->d_ext2int : nullptr;
-  CUDA_TRY(h, dev_grow(&h->d_cols, &h->cols_cap, ncols));
-  CUDA_TRY(h, cudaMemcpyAsync(h->d_cols, cols, ncols * sizeof(int32_t), cudaMemcpyHostToDevice,
-                              h->st));
+  // the ids, and the columns on their way to the host behind them
+  const size_t ib = ((size_t)ncols * sizeof(int32_t) + 255) & ~(size_t)255;
   const size_t ob = (size_t)h->n_cur * ncols * (out_fp64 ? 8 : 4);
-  if (out_on_device) {
-    launch_copy_cols(h->S, h->cfg.s_precision, h->ld, h->d_cols, perm, ncols, h->n_cur, out,
-                     out_fp64, h->st, upper(h));
-    LAUNCH_CHECK(h);
-    CUDA_TRY(h, cudaStreamSynchronize(h->st));  // cols staging reuse safety
-    return SR_OK;
+  WorkBuf tmp;
+  CUDA_TRY(h, tmp.get(columns_scratch(ib + (out_on_device ? 0 : ob))));
+  int32_t* d_cols = (int32_t*)tmp.p;
+  void* dst = out_on_device ? out : (void*)((unsigned char*)tmp.p + ib);
+  cudaError_t e =
+      cudaMemcpyAsync(d_cols, cols, ncols * sizeof(int32_t), cudaMemcpyHostToDevice, h->st);
+  if (e == cudaSuccess) {
+    launch_copy_cols(h->S, h->cfg.s_precision, h->ld, d_cols, perm, ncols, h->n_cur, dst, out_fp64,
+                     h->st, upper(h));
+    e = cudaGetLastError();
   }
-  void* tmp = nullptr;
-  simrank_status s = columns_scratch(h, ob, &tmp);
-  if (s != SR_OK) return s;
-  launch_copy_cols(h->S, h->cfg.s_precision, h->ld, h->d_cols, perm, ncols, h->n_cur, tmp,
-                   out_fp64, h->st, upper(h));
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(out, tmp, ob, cudaMemcpyDeviceToHost, h->st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
-  if (tmp != h->ob[29].p) cudaFree(tmp);
+  if (e == cudaSuccess && !out_on_device)
+    e = cudaMemcpyAsync(out, dst, ob, cudaMemcpyDeviceToHost, h->st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);  // ids and buffer are free again
+  if (e == cudaSuccess && tmp.bytes <= COLUMNS_KEEP) tmp.give();
   if (e != cudaSuccess) return fail(h, SR_ERR_CUDA, std::string("columns: ") + cudaGetErrorString(e));
   return SR_OK;
 }
@@ -2393,8 +2482,8 @@ simrank_status simrank_grad(simrank_t h, const int32_t* pa, const int32_t* pb, c
     Bv[p] = h->ext2int[pb[p]];
   }
   // endpoint block size from free memory: F and F_psi (K+1 blocks each), 2 y blocks
-  size_t free_b = 0, total_b = 0;
-  CUDA_TRY(h, cudaMemGetInfo(&free_b, &total_b));
+  size_t free_b = 0;
+  CUDA_TRY(h, free_memory(&free_b));
   const size_t per_col = (size_t)n_pad * 8 * (2 * (K + 1) + 2);
   const int Eb =
       (int)std::max<size_t>(4, std::min<size_t>(1024, (size_t)(0.5 * free_b) / per_col)) & ~3;

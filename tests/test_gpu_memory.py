@@ -182,3 +182,67 @@ def test_update_without_memory(P, kw):
             assert np.max(np.abs(got - want[:, cols])) < (1e-10 if kw.get("s_precision") == 64 else 1e-6)
         h.close()
     assert not failed
+
+
+def test_kept_buffers_make_room(P):
+    """What a re-anchor and queries leave for the next call goes when another
+    call, of another handle too, has no room otherwise, and with the last handle."""
+    import gc
+
+    import torch
+
+    gc.collect()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    h, S0 = fixed_point_handle(P, 32)
+    g, _ = fixed_point_handle(P, 32)
+    n = S0.shape[0]
+    wide = np.tile(np.arange(n, dtype=np.int32), 3)[:5600]  # 90 MB of scratch
+    for _ in range(2):
+        h.reanchor(1)  # 3 x 32 MB
+        h.columns(np.arange(500, dtype=np.int32))
+        with Squeeze(24 << 20):
+            assert np.max(np.abs(g.columns(wide) - S0[:, wide])) < 1e-6
+        with Squeeze(24 << 20):
+            with pytest.raises(P.SimrankError) as err:
+                h.reanchor(1)
+            assert err.value.status == SR_ERR_OOM
+    h.reanchor(1)
+    assert np.max(np.abs(h.dense() - S0)) < 1e-6
+    h.close()
+    g.close()
+    torch.cuda.empty_cache()
+    # module images and the like stay; three work buffers would be 96 MB
+    assert before - torch.cuda.mem_get_info()[0] < 64 << 20
+
+
+def test_kept_buffers_of_several_threads(P):
+    """Handles of four threads, each on a stream of its own, share the kept work
+    buffers: re-anchors from the fixed point and queries of several sizes."""
+    import threading
+
+    import torch
+
+    made = []
+    for t in range(4):
+        st = torch.cuda.Stream()
+        h, S0 = fixed_point_handle(P, 32, n=900 + 300 * (t // 2), stream=st.cuda_stream)
+        made.append((h, S0, st))
+    bad = []
+
+    def work(t):
+        h, S0, _ = made[t]
+        rng = np.random.default_rng(t)
+        for _ in range(40):
+            if rng.integers(2):
+                h.reanchor(int(rng.integers(1, 4)))
+            cols = rng.choice(S0.shape[0], int(rng.integers(1, 200)), replace=False).astype(np.int32)
+            if not np.max(np.abs(h.columns(cols) - S0[:, cols])) < 1e-6:
+                bad.append(t)
+
+    th = [threading.Thread(target=work, args=(t,)) for t in range(4)]
+    for x in th:
+        x.start()
+    for x in th:
+        x.join()
+    assert not bad
