@@ -1035,6 +1035,10 @@ std::vector<SweepScale> sweep_scales(const HostAdj& A, int n_rows, double C) {
     f.h = 5;
     while (f.h > 0 && (d << f.h) > 32) --f.h;
     f.sh = d <= 32 ? s + f.h - 1 : s - 1;
+    // a shift of the 63-bit (longer rows: 127-bit) product by more than its
+    // width leaves nothing
+    const int width = d <= 32 ? 62 : 126;
+    if (f.sh > width) f = SweepScale{0ull, f.h, width};
     out[(size_t)a] = f;
   }
   return out;

@@ -405,3 +405,20 @@ def test_stored_updates_of_rows_that_become_empty(P, prec, width):
         for c, x in enumerate(cols.tolist()):
             want = O.inc_sr_all_p(n, s, d, base[:, c], x, ups[:count], C, K)
             assert np.max(np.abs(got[:, c] - want)) < (1e-10 if prec == 64 else 1e-6), (count, x)
+
+
+@pytest.mark.parametrize("C", [1e-9, 1e-16, 1e-18, 1e-19, 1e-20, 1e-25, 1e-36, 1e-40, 1e-300])
+def test_sweeps_at_a_small_damping_factor(P, C):
+    """Sweeps whose factor C / d is near or below the last bit of the fixed-point
+    S, for short and long rows: the fixed point and one sweep from another S0.
+    Entries are at most 1: 1e-15."""
+    n = 300
+    s, d = degrees_graph(n, [0, 1, 2, 31, 32, 33, 96, 97, 250, 0], 5)
+    Q = O.transition_matrix(n, s, d)
+    sr = P.SimRank(n, s, d, C=C, K=1, s_precision=64)
+    assert np.max(np.abs(sr.dense() - sweeps(np.eye(n), Q, C, 2))) < 1e-15
+    S0 = np.random.default_rng(3).uniform(-1.0, 1.0, (n, n))
+    S0 = 0.5 * (S0 + S0.T)
+    sr = P.SimRank(n, s, d, S0=S0, C=C, K=1, s_precision=64)
+    sr.reanchor(1)
+    assert np.max(np.abs(sr.dense() - sweeps(S0, Q, C, 1))) < 1e-15
