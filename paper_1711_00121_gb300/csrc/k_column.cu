@@ -13,6 +13,7 @@
 // matching values at the block's columns.
 #include <algorithm>
 
+#include "quotient.h"
 #include "sr_internal.h"
 
 namespace sr {
@@ -206,21 +207,32 @@ __global__ void k_col_prefill(const int32_t* __restrict__ rows, const T* __restr
     Y[o + c] = Xadd ? add_scale * Xadd[o + c] : T(0);
 }
 
-// U[a][c] = X[a][c] / (in-degree or in-weight of a), r = its reciprocal: the
-// product with r and one correction, three FP64 operations where a division takes
-// some ten, and rounded like it.  One pass over the block before an FP64 forward
-// step (a gradient over 600 pairs at n = 5,000: 13.0 to 14.3 ms); a reciprocal inside
-// the step left twice the error of the division.  One CTA per row.
+// U[a][c] = X[a][c] / (in-degree or in-weight of a) by its reciprocal (quotient.h:
+// three FP64 operations where a division takes some ten), 0 for a node without
+// in-neighbours.  One pass over the block before an FP64 forward step (a gradient
+// over 600 pairs at n = 5,000: 13.0 to 14.3 ms); a product with the reciprocal
+// inside the step rounds twice.  One CTA per row.
 __global__ void __launch_bounds__(128)
     k_col_quotient(const double* __restrict__ X, const int32_t* __restrict__ in_len,
                    const double* __restrict__ wsum, const double* __restrict__ recip, int ldb,
                    double* __restrict__ U) {
   const int64_t a = blockIdx.x;
   const double r = recip[a], d = wsum ? wsum[a] : (double)in_len[a];
-  for (int c = threadIdx.x; c < ldb; c += 128) {
-    const double x = X[a * ldb + c], q = x * r;
-    U[a * ldb + c] = fma(fma(-q, d, x), r, q);
+  const double* x = X + a * ldb;
+  double* u = U + a * ldb;
+  if (fx_bits(r) == 0) {  // (a test on the FP64 pipe would count)
+    for (int c = threadIdx.x; c < ldb; c += 128) u[c] = 0.0;
+    return;
   }
+  bool again = false;
+  for (int c = threadIdx.x; c < ldb; c += 128) {
+    const double v = quotient_fast(x[c], d, r);
+    again |= !quotient_ok(v);
+    u[c] = v;
+  }
+  // a second look at the rare others, out of the loop
+  if (again)
+    for (int c = threadIdx.x; c < ldb; c += 128) u[c] = quotient(x[c], d, r);
 }
 
 // out[a] = scale / (in-degree or in-weight of a), 0 without in-neighbours

@@ -422,3 +422,19 @@ def test_sweeps_at_a_small_damping_factor(P, C):
     sr = P.SimRank(n, s, d, S0=S0, C=C, K=1, s_precision=64)
     sr.reanchor(1)
     assert np.max(np.abs(sr.dense() - sweeps(S0, Q, C, 1))) < 1e-15
+
+
+def test_gradient_of_a_huge_residual(P):
+    """Residuals near the largest FP64 number: the quotients before a forward step
+    take the division there.  Relative to the largest entry, as in the adjoint's
+    parity tests."""
+    n, C, K = 60, 0.2, 4
+    s, d = degrees_graph(n, [0, 1, 1, 2, 3, 40], 53)
+    a, b = np.array([1, 7], np.int32), np.array([5, 1], np.int32)
+    t = np.array([-8e307, 0.1])
+    sr = P.SimRank(n, s, d, C=C, K=K, s_precision=64, mode=1)
+    with np.errstate(over="ignore"):
+        L, g = sr.grad(a, b, t, s.size)
+        _, want, _ = O.pair_loss_and_weight_grad(n, s, d, np.ones(s.size), a, b, t, C, K)
+    assert np.isinf(L) and np.max(np.abs(want)) > 1e305
+    assert np.max(np.abs(g / np.max(np.abs(want)) - want / np.max(np.abs(want)))) < 1e-10
