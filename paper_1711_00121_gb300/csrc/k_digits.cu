@@ -468,8 +468,10 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
     }
     if (!ok) abort_flag = 1;
     if (et == 0 && my_tiles) {
-      atomicAdd(&counters[CNT_TILES_TOUCHED], my_tiles);
-      atomicAdd(&counters[CNT_S_BYTES], my_bytes);
+      if (k0 == 0) {  // an update's tiles and S count once, in its first pass
+        atomicAdd(&counters[CNT_TILES_TOUCHED], my_tiles);
+        atomicAdd(&counters[CNT_S_BYTES], my_bytes);
+      }
       atomicAdd(&counters[CNT_PANEL_BYTES],
                 my_tiles * 4ull * (unsigned long long)kc * PT * sizeof(T));
     }

@@ -438,3 +438,24 @@ def test_gradient_of_a_huge_residual(P):
         _, want, _ = O.pair_loss_and_weight_grad(n, s, d, np.ones(s.size), a, b, t, C, K)
     assert np.isinf(L) and np.max(np.abs(want)) > 1e305
     assert np.max(np.abs(g / np.max(np.abs(want)) - want / np.max(np.abs(want)))) < 1e-10
+
+
+@pytest.mark.parametrize("K", [3, 15, 16, 40])
+def test_counters_of_the_digit_pass(P, K):
+    """tiles_touched and s_bytes count an update's tiles once, however many passes
+    of 16 terms its digits take: the numbers of the FP32 CUDA-core pass, with twice
+    the bytes."""
+    n = 700
+    s, d = degrees_graph(n, [0, 5, 64], 59)
+    ups = [(x, 0, 1) for x in range(10, 13)]
+    nT = (n + 127) // 128
+    for aff in (0, 1):
+        sr = P.SimRank(n, s, d, C=0.6, K=K, s_precision=64, aff=aff)
+        sr.apply_updates(ups)
+        st = sr.stats()
+        f = P.SimRank(n, s, d, C=0.6, K=K, s_precision=32, s_kernel=1, aff=aff)
+        f.apply_updates(ups)
+        sf = f.stats()
+        assert st["tiles_total"] == sf["tiles_total"] == 3 * nT * (nT + 1) // 2
+        assert st["tiles_touched"] == sf["tiles_touched"] <= st["tiles_total"]
+        assert st["s_bytes"] == 2 * sf["s_bytes"] and st["panel_bytes"] == 2 * sf["panel_bytes"]
