@@ -459,3 +459,71 @@ def test_counters_of_the_digit_pass(P, K):
         assert st["tiles_total"] == sf["tiles_total"] == 3 * nT * (nT + 1) // 2
         assert st["tiles_touched"] == sf["tiles_touched"] <= st["tiles_total"]
         assert st["s_bytes"] == 2 * sf["s_bytes"] and st["panel_bytes"] == 2 * sf["panel_bytes"]
+
+
+@pytest.mark.parametrize("prec,tc", [(64, 0), (32, 0), (32, 1)])
+def test_one_shot_with_an_infinite_block(P, prec, tc):
+    """Two graphs without an edge between them, in tiles of their own, S infinite at
+    one node of the second: the batch's steps then run in FP64 instead of fixed
+    point.  The first graph's block is the oracle's, 1e-10 (FP64) and 1e-6 (FP32)
+    as in the one-shot parity tests; the second's is not finite."""
+    n, C, K = 128, 0.6, 6
+    s, d = degrees_graph(n, [0, 1, 31, 33, 65], 61)
+    edges = set(zip(s.tolist(), d.tolist()))
+    ups = [(next(x for x in range(9, n) if (x, j) not in edges), j, 1) for j in (0, 4)]
+    ups.append((sorted(e for e in edges if e[1] == 3)[0][0], 3, -1))
+    new = (edges | {u[:2] for u in ups if u[2] > 0}) - {u[:2] for u in ups if u[2] < 0}
+    S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-15)
+    ns, nd = (np.array(v, np.int64) for v in zip(*sorted(new)))
+    want = O.one_shot_batch(n, s, d, ns, nd, S0, C, K)
+    both = np.zeros((2 * n, 2 * n), np.float64 if prec == 64 else np.float32)
+    both[:n, :n] = both[n:, n:] = S0
+    both[n + 4, n + 4] = np.inf
+    sr = P.SimRank(2 * n, np.r_[s, s + n], np.r_[d, d + n], S0=both, C=C, K=K, s_precision=prec,
+                   tc=tc, apply=P.APPLY_ONE_SHOT, relabel=0)
+    sr.apply_updates(ups + [(i + n, j + n, op) for i, j, op in ups])
+    got = sr.dense()
+    assert np.max(np.abs(got[:n, :n] - want)) < (1e-10 if prec == 64 else 1e-6)
+    assert not np.all(np.isfinite(got[n:, n:]))
+
+
+@pytest.mark.parametrize("K", [11, 15])
+def test_fp32_digit_pass_rounds_like_fp32(P, K):
+    """One update by digits of FP32 panels (FP64 vectors) against the oracle.  A panel
+    value is rounded to 2^-24, and C + C^2 + .. < 1.5 of them meet in an entry from
+    either vector: 2 * 1.5 * 2 * 2^-24 of the largest |eta|; the four FMAs that join
+    the digits and the sum with S round five times more: 11 * 2^-24 of the largest
+    entry, of S or of the change."""
+    n, C = 5120, 0.6
+    s, d = degrees_graph(n, [0, 5, 64], 67)
+    S0 = np.random.default_rng(6).random((n, n))
+    S0 = (0.5 * (S0 + S0.T)).astype(np.float32)
+    edges = set(zip(s.tolist(), d.tolist()))
+    ups = [(next(x for x in range(9, n) if (x, 2) not in edges), 2, 1)]
+    sr = P.SimRank(n, s, d, S0=S0, C=C, K=K, s_precision=32, vec_fp64=1, aff=0)
+    sr.apply_updates(ups)
+    want, _ = O.sequential_unit_updates(n, s, d, S0.astype(np.float64), ups, C, K)
+    scale = max(np.max(np.abs(want)), np.max(np.abs(want - S0)))
+    assert np.max(np.abs(sr.dense() - want)) < 11 * 2.0**-24 * scale
+
+
+@pytest.mark.parametrize("kw", [{}, {"prep_ctas": 5}])
+@pytest.mark.parametrize("scale", [1e-3, 1e-6])
+def test_recurrence_of_a_small_s0(P, scale, kw):
+    """The part of an update that comes from S0 (the change is affine in S0): from a
+    small S0 less the same from S0 = 0.  Entries are of order 1 at most, rounded some
+    20 times on either side: 2 * 20 * 2^-53 < 5e-15, far below the part itself."""
+    n, C, K = 1300, 0.6, 7
+    s, d = degrees_graph(n, [0, 1, 33, 64, 257, 1023], 71)
+    edges = set(zip(s.tolist(), d.tolist()))
+    S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-14) * scale
+    ups = [(next(x for x in range(9, n) if (x, 1) not in edges), 1, 1)]
+    part, ref = [], []
+    for start in (S0, np.zeros_like(S0)):
+        sr = P.SimRank(n, s, d, S0=start, C=C, K=K, s_precision=64, **kw)
+        sr.apply_updates(ups)
+        part.append(sr.dense())
+        ref.append(O.sequential_unit_updates(n, s, d, start, ups, C, K)[0])
+    want = ref[0] - ref[1]
+    assert np.max(np.abs(want - S0)) > 1e-2 * scale
+    assert np.max(np.abs((part[0] - part[1]) - want)) < 5e-15
