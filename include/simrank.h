@@ -184,7 +184,8 @@ simrank_status simrank_init(const simrank_config* cfg, int32_t n, int64_t m,
  * the host returns once the work is queued.  A call that fails after that
  * (SR_ERR_OOM, SR_ERR_CUDA) may have applied some of the updates, and the
  * handle answers queries but takes no further updates; an automatic re-anchor
- * that fails alone is reported by the status, with all updates applied. */
+ * that fails alone is reported by the status, with all updates applied.  On a
+ * stream that is being captured it returns SR_ERR_CUDA and changes nothing. */
 simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64_t count);
 
 /* Copies columns cols[0..ncols) of the current S (n_cur rows each) to out,

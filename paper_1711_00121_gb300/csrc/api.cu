@@ -2164,6 +2164,11 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
   if (count == 0) return SR_OK;
   if (h->weighted) return fail(h, SR_ERR_UNSUPPORTED, "updates on a weighted graph");
   if (h->part_way) return fail(h, SR_ERR_CUDA, PART_WAY);
+  // a captured update would be replayed from the staging memory of a later call
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->st, &capture) != cudaSuccess ||
+      capture != cudaStreamCaptureStatusNone)
+    return fail(h, SR_ERR_CUDA, "updates cannot be captured into a CUDA graph");
   // caller ids -> storage ids (new ids >= n_cur map to themselves)
   std::vector<simrank_update> um(u, u + count);
   auto to_int = [&](int32_t x) { return (x >= 0 && x < h->n_cap) ? h->ext2int[x] : x; };

@@ -527,3 +527,38 @@ def test_recurrence_of_a_small_s0(P, scale, kw):
     want = ref[0] - ref[1]
     assert np.max(np.abs(want - S0)) > 1e-2 * scale
     assert np.max(np.abs((part[0] - part[1]) - want)) < 5e-15
+
+
+@pytest.mark.parametrize("kw", [{}, {"tc": 2, "defer": 4}, {"apply": 1}, {"apply": 2}, {"mode": 1}])
+def test_updates_are_not_captured(P, kw):
+    """An update on a capturing stream is refused and changes nothing (its sources
+    and graph changes lie in memory that the next call rewrites); outside of the
+    capture the same update works.  1e-6, as in the parity tests."""
+    import torch
+
+    n, C, K = 300, 0.6, 6
+    s, d = degrees_graph(n, [0, 1, 33], 73)
+    edges = set(zip(s.tolist(), d.tolist()))
+    ups = [(next(x for x in range(9, n) if (x, j) not in edges), j, 1) for j in (0, 2)]
+    st = torch.cuda.Stream()
+    sr = P.SimRank(n, s, d, C=C, K=K, s_precision=32, stream=st.cuda_stream, **kw)
+    sr.apply_updates(ups)
+    sr.apply_updates([(i, j, -1) for i, j, _ in ups])
+    sr.sync()
+    before = sr.dense()
+    graph = torch.cuda.CUDAGraph()
+    buf = torch.zeros(4, device="cuda")
+    status = 0
+    with torch.cuda.graph(graph, stream=st):
+        buf += 1.0
+        try:
+            sr.apply_updates(ups)
+        except P.SimrankError as e:
+            status = e.status
+    assert status == 6
+    assert np.array_equal(sr.dense(), before)
+    sr.apply_updates(ups)
+    again = P.SimRank(n, s, d, C=C, K=K, s_precision=32, **kw)
+    for u in (ups, [(i, j, -1) for i, j, _ in ups], ups):
+        again.apply_updates(u)
+    assert np.max(np.abs(sr.dense() - again.dense())) < 1e-6
