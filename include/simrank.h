@@ -83,7 +83,10 @@ typedef struct simrank_config {
   int32_t s_precision;    /* 32: S stored in FP32; 64: S stored in FP64.  The xi/eta vectors
                              have the precision of S (FP64 also with FP32 S when vec_fp64 = 1,
                              or with chain = 1); the panels the S pass reads have the precision
-                             of S. */
+                             of S.  Where the library computes in 64-bit fixed point (the
+                             recurrence with prep_item = 0, one-shot steps, Jacobi sweeps; the S
+                             pass of an FP64 S by digits) errors are 2^-57 to 2^-55 of the
+                             largest entry or product, not of each entry. */
   int32_t mode;           /* SR_MODE_DENSE or SR_MODE_COLUMN */
   int32_t n_capacity;     /* maximum number of nodes, including nodes added later; >= n at init */
   int32_t aff;            /* 1: skip S tiles outside the affected area of Thm 4; 0: touch every tile */
@@ -215,7 +218,7 @@ typedef struct simrank_stats {
   int64_t updates;          /* updates accepted by apply_updates */
   int64_t rank_one_updates; /* rank-one (sink-block / unit) updates run on the GPU */
   int64_t tiles_total;      /* 128 x 128 S tiles that an unpruned update would touch */
-  int64_t tiles_touched;    /* S tiles actually read and written */
+  int64_t tiles_touched;    /* S tiles read and written, once per update or group of pending ones */
   int64_t s_bytes;          /* algorithmic bytes of S read + written by S-update launches */
   int64_t panel_bytes;      /* algorithmic bytes of xi/eta panels read by S-update launches */
   int64_t s_update_launches;

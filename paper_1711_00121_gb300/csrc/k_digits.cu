@@ -1,4 +1,4 @@
-// S pass of one update without a loss of precision on the tensor cores
+// S pass of one update by exact products of digits on the tensor cores
 // (tcgen05), for S in FP64 and for the FP32 pass without a split (tc = 0):
 //   S[I,J] += sum_k xi_k[I] eta_k[J]^T + eta_k[I] xi_k[J]^T  (I <= J; Alg 1).
 //
@@ -18,8 +18,12 @@
 //   integer of unit 2^(M - 57) and rounded to FP64 once.
 //   FP32: NS = 5 (44 bits), 15 products; the sums are added by four FP32 FMAs,
 //   smallest weight first.
-// What is dropped or rounded is below 2^-55 (FP32: 2^-37) of 2^M a sum, and S is
-// rounded once, to 2^-53 (2^-24), where an FMA chain rounds every partial sum.
+// FP64: what is left out or rounded before the sum with S is below 2^-55 of 2^M.
+// FP32: what is left out is below 2^-37 of 2^M, each of the four FMAs rounds its
+// partial sum to 2^-24, and the scaling by 2^(M - 16) is exact.  S is rounded once
+// a pass of 16 terms, where an FMA chain rounds every partial sum.  All this is
+// relative to 2^M, the largest product of two column maxima: entries of S far below
+// it hold fewer bits than after an FMA chain.
 // An infinite or NaN panel value (meta[1]) is summed by the definition instead.
 //
 // k_s_update_digits: one CTA per SM over the list of affected tile pairs.  Warp

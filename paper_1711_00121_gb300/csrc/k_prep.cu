@@ -11,7 +11,8 @@
 //            xi_{k+1} = C Q xi_k, eta_{k+1} = Q eta_k;
 //   phase 3  the affected-area mask words of every tile (Thm 4) and the list
 //            of affected tile pairs of the S pass.
-// Phases are separated by a bounded grid barrier.
+// A bounded grid barrier follows phase 0 and comes before the tile list; what lies
+// between waits on counted words (flow form) or on further barriers (item form).
 //
 // Flow form (default).  The in-lists of all rows, flattened in row order, are
 // cut into equal contiguous ranges, one per CTA, one or two nonzeros per
@@ -34,8 +35,10 @@
 // largest entry of the rows that gamma reads): row sums are exact, and the
 // division by the in-degree is a product with a 63-bit reciprocal.  GB300
 // issues FP64 (and conversions to and from 64-bit types) at 1/64 of the FP32
-// rate, which took 1.65 us of each step in FP64.  The absolute error is 2^-57 of
-// the largest entry a step, below the rounding of an FP64 S.
+// rate, which took 1.65 us of each step in FP64.  The error is absolute, 2^-57 of
+// the largest entry a step.  An FP64 S rounds its entries above 2^-4 more than
+// that; smaller entries of xi and eta hold fewer bits than in FP64 (below 2^-33 of
+// the largest fewer than in FP32), and those that round to zero leave the masks.
 // A row spread over the lanes of a warp is summed by shuffles, over the warps
 // of a CTA through shared memory, and the parts of a row cut by the CTA ranges
 // meet in its word by integer reductions.

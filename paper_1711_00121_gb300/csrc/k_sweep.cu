@@ -7,6 +7,8 @@
 // rate).  Here the row sums are exact integer sums and the division by the
 // in-degree is a product with a 63-bit reciprocal, rounded once: an error
 // below 2^-57 a product, where one FP64 rounding of a value near 1 loses 2^-54.
+// The error is absolute: an entry below 2^-4 holds fewer bits than in FP64, one
+// below 2^-58 becomes zero (a first S stops at a change of 1e-13, some 2^-43).
 // Rows of up to 32 nonzeros sum in 64 bits (|value| < 1.875: 32 of them stay
 // below 2^63), longer ones flush such sums into 96 bits: with 96-bit sums for
 // every row the kernels were bound by instruction issue.

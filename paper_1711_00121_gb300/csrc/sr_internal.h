@@ -6,7 +6,6 @@
 #include <atomic>
 #include <cstdint>
 #include <string>
-#include <unordered_set>
 #include <vector>
 
 #include "../../include/simrank.h"
@@ -310,8 +309,8 @@ void launch_maxdiff(const void* A, const void* B, int prec, int n, int64_t ld,
 void launch_sweep_fixed(const DevAdj& in, const SweepScale* s1, const SweepScale* s2,
                         const long long* S, int64_t ld, int n_pad, long long* T, long long* Snew,
                         long long diag, int n_diag, unsigned long long* maxd, cudaStream_t st);
-// F = (S + S^T) / 2 in fixed point (F null, FP64 S: no change), and back (S and
-// F may share memory).  check (always with F null): *flags |= 1 when an entry
+// F = (S + S^T) / 2 in fixed point (F null, FP64 S with check: a look only), and
+// back (S and F may share memory).  check: *flags |= 1 when an entry
 // has magnitude >= 1.875 or is NaN, |= 2 when two mirrored entries differ by
 // more than tol.  upper: only the tiles on or above the block diagonal of S
 // are read, and written.
