@@ -164,6 +164,13 @@ simrank_status fail(simrank_ctx* h, simrank_status s, const std::string& msg) {
 const char* const PART_WAY =
     "an earlier update failed part way: this handle takes no further updates";
 
+// A captured update would be replayed from the staging memory of a later call.
+const char* const NOT_CAPTURED = "updates cannot be captured into a CUDA graph";
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &s) != cudaSuccess || s != cudaStreamCaptureStatusNone;
+}
+
 #define CUDA_TRY(h, call)                                                                  \
   do {                                                                                     \
     cudaError_t e__ = (call);                                                              \
@@ -2164,11 +2171,7 @@ simrank_status simrank_apply_updates(simrank_t h, const simrank_update* u, int64
   if (count == 0) return SR_OK;
   if (h->weighted) return fail(h, SR_ERR_UNSUPPORTED, "updates on a weighted graph");
   if (h->part_way) return fail(h, SR_ERR_CUDA, PART_WAY);
-  // a captured update would be replayed from the staging memory of a later call
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(h->st, &capture) != cudaSuccess ||
-      capture != cudaStreamCaptureStatusNone)
-    return fail(h, SR_ERR_CUDA, "updates cannot be captured into a CUDA graph");
+  if (capturing(h->st)) return fail(h, SR_ERR_CUDA, NOT_CAPTURED);
   // caller ids -> storage ids (new ids >= n_cur map to themselves)
   std::vector<simrank_update> um(u, u + count);
   auto to_int = [&](int32_t x) { return (x >= 0 && x < h->n_cap) ? h->ext2int[x] : x; };
@@ -2891,6 +2894,7 @@ simrank_status simrank_multi_apply(simrank_multi_t h, const simrank_update* u,
                                    const int64_t* update_offsets) {
   if (!h) return mfail(nullptr, SR_ERR_ARG, "null handle");
   if (!update_offsets) return mfail(h, SR_ERR_ARG, "null update_offsets");
+  if (capturing(h->st)) return mfail(h, SR_ERR_CUDA, NOT_CAPTURED);
   const int G = (int)h->g.size();
   // caller ids -> storage ids, then validation of every graph before any change
   std::vector<std::vector<simrank_update>> um(G);

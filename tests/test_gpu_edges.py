@@ -562,3 +562,32 @@ def test_updates_are_not_captured(P, kw):
     for u in (ups, [(i, j, -1) for i, j, _ in ups], ups):
         again.apply_updates(u)
     assert np.max(np.abs(sr.dense() - again.dense())) < 1e-6
+
+
+def test_many_graph_updates_are_not_captured(P):
+    """The same for many graphs."""
+    import torch
+
+    n, C, K = 300, 0.6, 6
+    s, d = degrees_graph(n, [0, 1, 33], 73)
+    edges = set(zip(s.tolist(), d.tolist()))
+    ups = [np.array([(next(x for x in range(9, n) if (x, 2) not in edges), 2, 1)], np.int32)]
+    st = torch.cuda.Stream()
+    mh = P.MultiSimRank([(n, s, d)], C=C, K=K, s_precision=32, stream=st.cuda_stream)
+    before = mh.dense(0)
+    graph = torch.cuda.CUDAGraph()
+    buf = torch.zeros(4, device="cuda")
+    status = 0
+    with torch.cuda.graph(graph, stream=st):
+        buf += 1.0
+        try:
+            mh.apply_updates(ups)
+        except P.SimrankError as e:
+            status = e.status
+    assert status == 6
+    assert np.array_equal(mh.dense(0), before)
+    mh.apply_updates(ups)
+    mh.sync()
+    S0 = O.simrank_fixed_point(O.transition_matrix(n, s, d, sparse=True), C, tol=1e-14)
+    want, _ = O.sequential_unit_updates(n, s, d, S0, ups[0].tolist(), C, K)
+    assert np.max(np.abs(mh.dense(0) - want)) < 1e-6
