@@ -47,7 +47,7 @@ METRIC = "edge updates/sec & HBM GB/s: fused rank-2K ΔS vs plain Inc-uSR at 1e-
 UNIT = "edge updates/s"
 # DRAM bytes (read + write) per launch from one ncu capture of each kernel on
 # the default stream configuration (profiles/ holds the summaries)
-TRAFFIC_PREP = 6.244e7
+TRAFFIC_PREP = 6.181e7
 TRAFFIC_S_PASS = 1.828e9
 # the per-update S pass (--defer 0 replica, FP16 split): a typical launch
 TRAFFIC_S_PASS_EDGE = 1.417e9

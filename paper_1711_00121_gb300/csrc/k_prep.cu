@@ -20,12 +20,12 @@
 // of W[k + 1] counts, in its upper bits, the parts of its row's sum that are
 // there, and a thread that gathers it reads it (from L2) until all are.  A step
 // then costs one reduction and one load through L2 instead of a reduction, a grid
-// barrier and a load.  At n = 20,000, m = 200,000 a step takes 2.6 us (with
-// barriers 4.8 in FP64, 2.9 in FP32), at n = 1,000, m = 8,000 1.7 us (2.95 and
+// barrier and a load.  At n = 20,000, m = 200,000 a step takes 2.5 us (with
+// barriers 4.8 in FP64, 2.9 in FP32), at n = 1,000, m = 8,000 1.55 us (2.95 and
 // 2.0): about half of it the L2 latency there and back, the rest the gather
 // (one 32-byte sector per nonzero and SM every other clock) and the sums.
 // w and gamma go the same way (gamma's rows wait for the parts of their means).
-// Outside the steps an update costs 25 us at n = 20,000 and 19 us at n = 1,000
+// Outside the steps an update costs 25 us at n = 20,000 and 20 us at n = 1,000
 // (27 and 21 with a grid barrier after w and a gather of every column's extent):
 // round trips to L2 that depend on each other.
 // Every CTA is co-resident and a value depends on earlier steps only, so the
@@ -673,8 +673,9 @@ __device__ void prep_patch(const PatchOp* __restrict__ ops, int64_t begin, int64
 }
 
 // Shared memory of the flow form, in the place of the item form's column cache
-// (as arrays of their own they took the second CTA of an SM from launches with
-// 2,600 to 3,600 pending terms).  fsh also holds the partial sums of phase 0.
+// (as arrays of their own they took the second CTA of an SM from launches with more
+// than 2,270 pending terms, 2,590 with FP32 vectors; now 3,580 and 3,900, at
+// n = 20,000).  fsh also holds the partial sums of phase 0.
 struct FlowShared {
   SweepScale fsh[PG][2];  // 1 / in-degree of each thread's head / tail row
   int rowmap[2 * PG];     // the row of each of the CTA's nonzeros
