@@ -1103,32 +1103,30 @@ simrank_status jacobi_sweeps(simrank_ctx* h, int max_sweeps, double tol, double*
     const double sym = sp == 64 ? 1e-12 : 1e-6;
     unsigned int* df = (unsigned int*)h->diffbits;
     e = cudaMemsetAsync(h->diffbits, 0, sizeof(unsigned long long), h->st);
-    if (!known)
-      launch_to_fixed(h->S, sp, alias ? nullptr : F, h->n_pad, h->ld, upper(h), true, sym, df,
-                      h->st);
-    if (e == cudaSuccess && !known)
+    launch_to_fixed(h->S, sp, alias && !known ? nullptr : F, h->n_pad, h->ld, upper(h), !known, sym,
+                    df, h->st);
+    // An S that is converted in place holds integers until the last sweep:
+    // whatever can fail for want of memory comes before that (a first S goes with
+    // its handle).  The host's part is under way beside the pass above.
+    std::vector<SweepScale> f = sweep_scales(h->hin, h->n_pad, h->cfg.C);
+    const std::vector<SweepScale> f1 = sweep_scales(h->hin, h->n_pad, 1.0);
+    f.insert(f.end(), f1.begin(), f1.end());
+    if (e == cudaSuccess) e = tables.get(f.size() * sizeof(SweepScale));
+    scales = (SweepScale*)tables.p;
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(scales, f.data(), f.size() * sizeof(SweepScale), cudaMemcpyHostToDevice,
+                          h->st);
+    if (e == cudaSuccess) e = sweep_fixed_ready(sp);
+    if (e == cudaSuccess && !known) {
       e = cudaMemcpyAsync(&flags, h->diffbits, sizeof(flags), cudaMemcpyDeviceToHost, h->st);
-    if (e == cudaSuccess && !known) e = cudaStreamSynchronize(h->st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
+    }
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return give_up(e);
     fixed = flags == 0;
-    if (fixed) {
-      // an S that is converted in place holds integers until the last sweep:
-      // whatever can fail for want of memory comes before that
-      std::vector<SweepScale> f = sweep_scales(h->hin, h->n_pad, h->cfg.C);
-      const std::vector<SweepScale> f1 = sweep_scales(h->hin, h->n_pad, 1.0);
-      f.insert(f.end(), f1.begin(), f1.end());
-      e = tables.get(f.size() * sizeof(SweepScale));
-      scales = (SweepScale*)tables.p;
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(scales, f.data(), f.size() * sizeof(SweepScale),
-                            cudaMemcpyHostToDevice, h->st);
-      if (e == cudaSuccess) e = sweep_fixed_ready(sp);
-      if (e != cudaSuccess) return give_up(e);
-      // every entry of the other two buffers is written by each sweep
-      if (known || alias)
-        launch_to_fixed(h->S, sp, F, h->n_pad, h->ld, upper(h), false, sym, df, h->st);
-    }
+    // every entry of the other two buffers is written by each sweep
+    if (fixed && alias && !known)
+      launch_to_fixed(h->S, sp, F, h->n_pad, h->ld, upper(h), false, sym, df, h->st);
   }
   if (!fixed) {
     if (upper(h)) launch_mirror_lower(h->S, sp, h->n_pad, h->ld, h->st);
